@@ -57,9 +57,8 @@ int fft_max_cc(int);
 void launch_blockmul(const BmulTask*, int, int, int, cudaStream_t, bool);
 void launch_eapply(const EApplyTask*, int, int, cudaStream_t);
 int eapply_grid(long long items);
-void launch_band_factor(const BandTask*, int, cudaStream_t);
+void launch_band_factor(const BandTask*, int, int, cudaStream_t);
 void launch_band_solve(const BandTask*, int, int, int, int, cudaStream_t, bool);
-int band_stage_doubles(int);
 void launch_cell_canon(const CanonTask*, int, int, int, cudaStream_t);
 void launch_gather(const GatherSeg*, int, uint32_t*, cudaStream_t);
 void launch_cell_back(const double*, int, int, int, const double*, double*, int, cudaStream_t);
@@ -448,7 +447,7 @@ struct Batch {
     double *Xc = nullptr, *THc = nullptr, *TSc = nullptr, *EHc = nullptr, *ESc = nullptr;
     int* kept = nullptr;
     cplx *CHo = nullptr, *CSo = nullptr;   // Fourier blocks of the original operator (matvec API)
-    double *band = nullptr, *sigma_band = nullptr;
+    double *band_win = nullptr, *band_fwd = nullptr, *band_bwd = nullptr, *band_dinv = nullptr, *sigma_band = nullptr;
     int *band_fail = nullptr;
     int* fail = nullptr;
   };
@@ -474,8 +473,8 @@ struct Batch {
   TL eHXP, eHW;                      // boundary blocks (H and S in one task)
   TL rfwdXP, rinvHXP, rinvSXP, rbmulHS2, reHXP;   // image refresh at the FP32 -> FP64 switch
   TL bandF, bandS;
-  int band_stage = 0;                // doubles of a band-solve shared-memory stage
-  int band_ringrow = 0;              // largest (D + 1) m0 of the staged band solves
+  int band_col = 0;                  // doubles of the largest block column of a band factorisation
+  int band_row = 0, band_step = 0;   // largest (D + 4) m0 and largest step of the band solves
   int gemm_tiles = 0;                // TN tile sizes in use: bit 0 = 16, bit 1 = 20
   bool rr_small = false, rr_big = false;   // Rayleigh-Ritz launches needed (256 / 512 threads)
   int rr_small_ld = 0;               // largest ld of the shared-memory problems
@@ -525,8 +524,9 @@ void plan(Batch& B, Slab& S, Slab& U) {
   B.maxnj_p = B.maxnj_s = 0; B.maxm0 = 1; B.maxM = 0; B.maxsort = 0; B.kmax = 0; B.maxLdft = 1;
   B.odd_m0 = false;
   B.any_mixed = false;
-  B.band_stage = 0;
-  B.band_ringrow = 0;
+  B.band_col = 0;
+  B.band_row = 0;
+  B.band_step = 0;
   B.gemm_tiles = 0;
   B.rr_small = B.rr_big = false;
   B.rr_small_ld = B.rr_big_ld = 0;
@@ -949,7 +949,10 @@ void plan(Batch& B, Slab& S, Slab& U) {
       // within ~4 GFLOP (tens of ms); above that the circulant inverse
       Q.use_band = 2.0 * Q.Lc * (double)Q.D * Q.D * (double)H.m0 * H.m0 * H.m0 <= 4e9;
       if (Q.use_band) {
-        Q.band = S.take<double>((size_t)Q.Lc * (Q.D + 1) * m2);
+        Q.band_win = S.take<double>((size_t)(Q.D + 1) * (Q.D + 1) * m2);
+        Q.band_fwd = S.take<double>((size_t)Q.Lc * std::max<size_t>(band_step(Q.D, H.m0), 2));
+        Q.band_bwd = S.take<double>((size_t)Q.Lc * band_step(Q.D + 1, H.m0));
+        Q.band_dinv = S.take<double>((size_t)Q.Lc * m2);
         Q.sigma_band = S.take<double>(1);
         Q.band_fail = S.take<int>(1);
       }
@@ -1082,14 +1085,17 @@ void plan(Batch& B, Slab& S, Slab& U) {
         std::memset(&bt, 0, sizeof(bt));
         bt.m0 = m0; bt.L = Q.Lc; bt.D = Q.D; bt.k = k; bt.n = n;
         bt.TH = Q.THc; bt.TS = Q.TSc; bt.nE = Q.nE; bt.Ek = U.put(Q.Ek); bt.Em = U.put(Q.Em);
-        bt.EH = Q.EHc; bt.ES = Q.ESc; bt.sigma0 = Q.sigma; bt.band = Q.band; bt.sigma_used = Q.sigma_band;
+        bt.EH = Q.EHc; bt.ES = Q.ESc; bt.sigma0 = Q.sigma; bt.win = Q.band_win; bt.fwd = Q.band_fwd; bt.bwd = Q.band_bwd; bt.dinv = Q.band_dinv; bt.sigma_used = Q.sigma_band;
         bt.fail = Q.band_fail; bt.R = l.R; bt.W = Yw; bt.ld = n; bt.active = l.active;
         bt.fp32 = H.f32;
+        B.band_col = std::max(B.band_col, 2 * m0 * m0 + (Q.D + 1) * m0 * (m0 + 1));
+        B.band_row = std::max(B.band_row, (Q.D + 4) * m0);
+        B.band_step = std::max(B.band_step, (int)band_step(Q.D + 1, m0));
+        std::vector<int> ef((size_t)Q.Lc * (Q.D + 1), -1);   // a position's entries lie one after another
+        for (int e = Q.nE - 1; e >= 0; --e)
+          if (Q.Ek[e] >= Q.Em[e] && Q.Ek[e] - Q.Em[e] <= Q.D) ef[(size_t)Q.Ek[e] * (Q.D + 1) + Q.Ek[e] - Q.Em[e]] = e;
+        bt.efirst = U.put(ef);
         bnd.push_back(bt);
-        if (m0 % 2 == 0 && (Q.D + 1) * m0 * m0 <= band_stage_doubles(1 << 30)) {   // stageable
-          B.band_stage = std::max(B.band_stage, (Q.D + 1) * m0 * m0);
-          B.band_ringrow = std::max(B.band_ringrow, (Q.D + 1) * m0);
-        }
       } else {
         fR.push_back(fwd(l.R, k, pcmode));
         iPW.push_back(inv(Y1, Yw, k, pcmode));
@@ -1241,7 +1247,6 @@ void plan(Batch& B, Slab& S, Slab& U) {
     TLp(nW, B.normW);
     TLp(bnd, B.bandF);
     B.bandS = B.bandF;
-    B.band_stage = band_stage_doubles(B.band_stage);
     TLp(rs, B.resid, kk);
   }
   // ---- descriptor arrays (uploaded in one copy with the parameters) ----
@@ -1433,7 +1438,7 @@ void run_struct_setup(fock_ctx* ctx, Batch& B) {
   for (auto& Q : B.pp)
     if (Q.band_fail) cudaMemsetAsync(Q.band_fail, 0, sizeof(int), st);
   if (B.bandF.n) { PROF("k_band_factor", 1);
-    launch_band_factor(reinterpret_cast<const BandTask*>(B.bandF.d), B.bandF.n, st); }
+    launch_band_factor(reinterpret_cast<const BandTask*>(B.bandF.d), B.bandF.n, B.band_col, st); }
 }
 
 template <class T> const T* tl(const Batch::TL& t) { return reinterpret_cast<const T*>(t.d); }
@@ -1575,7 +1580,7 @@ void refresh_XP(Batch& B, cudaStream_t st) {
 // Rayleigh-Ritz, P' S-orthogonal to X' in the coefficients, [X | P] <- Y Cc and
 // their fresh images.  Launches only.
 void lobpcg_body_a(Batch& B, cudaStream_t st) {
-  if (B.bandS.n) { PROF("k_band_solve", 1); launch_band_solve(tl<BandTask>(B.bandS), B.bandS.n, B.kmax, B.band_stage, B.band_ringrow, st, B.any_mixed); }
+  if (B.bandS.n) { PROF("k_band_solve", 1); launch_band_solve(tl<BandTask>(B.bandS), B.bandS.n, B.kmax, B.band_row, B.band_step, st, B.any_mixed); }
   if (B.fwdR.n) {
     mv_fwd(B, B.fwdR, st);
     { PROF("k_blockmul", 1); launch_blockmul(tl<BmulTask>(B.bmulK), B.bmulK.n, B.maxM, B.maxm0, st, B.any_mixed); }

@@ -323,6 +323,9 @@ struct CopyTask { const int* active; int n, ncols; const double* src; int lds; d
 // (4-byte words) for a single device-to-host copy.
 struct GatherSeg { const uint32_t* src; unsigned int words; unsigned int dst; };
 
+// doubles of one step of the banded solves with nd block coefficients, padded to 16 bytes
+__host__ __device__ inline size_t band_step(int nd, int m0) { return ((size_t)nd * m0 * m0 + 1) & ~(size_t)1; }
+
 struct BandTask {
   int m0, L, D, k, n;
   const double* TH; const double* TS;      // [D+1][m0*m0]
@@ -330,7 +333,9 @@ struct BandTask {
   const int* Ek; const int* Em;            // boundary block positions
   const double* EH; const double* ES;      // [nE][m0*m0]
   const double* sigma0;                    // shift from the embedding
-  double* band;                            // [L][D+1][m0*m0]
+  const int* efirst;                       // [L][D+1] first entry at (K, K-d), -1: none
+  double* win;                             // [D+1][D+1][m0*m0] factorisation window
+  double* fwd; double* bwd; double* dinv;  // the factor (k_band.cu): [L][band_step], [L][m0*m0]
   double* sigma_used;                      // out
   int* fail;                               // out: 1 if every attempt broke down
   const double* R; double* W; int ld;      // solve: W = A^-1 R (n x k, ld)

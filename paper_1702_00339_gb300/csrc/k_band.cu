@@ -1,322 +1,469 @@
-// Preconditioner of the box eigensolver: banded block Cholesky of H - sigma S.
+// Preconditioner of the box eigensolver: banded block factorisation of H - sigma S.
 //
 // The box chain matrix is block banded: H = BToepl(T) + E with generators
 // T_d = block (k+d, k), |d| <= D (Sec. 2.3, Remark 3.2) and the boundary blocks
 // E.  A = H - sigma S, sigma below the spectrum (from the circulant
 // embedding's Fourier blocks), is symmetric positive definite with the same
-// band, so it factors as L L^T with L block lower banded (bandwidth D cells).
-// W = A^-1 R is the shift-and-invert search direction of the block
-// iteration.  Storage: band[J][d] = block (J+d, J) of A (then of L), d = 0..D.
+// band, so it factors as M Delta M^T with M unit block lower banded (bandwidth
+// D cells) and Delta block diagonal.  W = A^-1 R is the shift-and-invert search
+// direction of the block iteration.  In this form (rather than L L^T) one step
+// of either substitution is one product of a block column with the row just
+// finished, without a triangular solve in between.
 //
-//  k_band_factor  one CTA per problem: fill the band from T and E, factor it
-//                 block column by block column; on a non-positive pivot lower
-//                 sigma and start again (at most 4 attempts)
-//                 (the diagonal slots then hold L_JJ^-1, which the solve
-//                 applies as a mat-vec)
-//  k_band_solve   forward and back substitution for the k columns of R:
-//                 one CTA per problem, one warp per group of 4 columns; the
-//                 next block row staged once per CTA in shared memory
-//                 (double-buffered cp.async), solution rows in per-warp rings
+//  k_band_factor  one thread-block cluster per problem: fill the band from T
+//                 and E, factor it block column by block column; on a
+//                 non-positive pivot lower sigma and start again
+//  k_band_solve   forward and back substitution, one CTA per group of columns
+//                 of a problem's R
+//
+// Storage, per problem: win, a ring of D + 1 block rows, row K holding the
+// blocks (K, K-d) of what is left of A; fwd[J], the coefficients of one step
+// down, [q][d-1][mu] = M_{J+d,J}[mu][q]; bwd[K], those of one step up,
+// [q][d][mu] = M_{K,K-d}[q][mu] for d >= 1 and Delta_{K-D-1}^-1[q][mu] for
+// d = 0; dinv[K] = Delta_K^-1.  A step's coefficients lie one after another in
+// the order its threads (d, mu) read them, padded to a multiple of 16 bytes.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace fock {
 
+namespace {
 
+__device__ __forceinline__ void cl_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cl_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ int cl_rank() { int r; asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ int cl_size() { int r; asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
 
-__device__ inline double* bblk(double* band, int D, int m2, int J, int d) {
-  return band + ((size_t)J * (D + 1) + d) * m2;
+constexpr int kFactorThreads = 256;
+
+// Row d1 (1-based) of pair number p in the order (1,1) (2,1) (2,2) (3,1) ...
+__device__ __forceinline__ int pair_row(int p) {
+  int d = (int)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);   // FP32: the loops below correct it
+  while ((d + 1) * (d + 2) / 2 <= p) ++d;
+  while (d * (d + 1) / 2 > p) --d;
+  return d + 1;
 }
 
-__global__ void k_band_factor(const BandTask* __restrict__ tasks) {
-  const BandTask T = tasks[blockIdx.x];
-  const int m0 = T.m0, m2 = m0 * m0, D = T.D, L = T.L;
-  __shared__ double inv[MAXM0 * MAXM0];
-  __shared__ double rlv[MAXM0];              // reciprocal pivots of the diagonal block's factor
-  __shared__ int bad, s_stop, s_nbis;
-  __shared__ double s_sigma, s_ok, s_bad;
-  if (threadIdx.x == 0) { s_sigma = *T.sigma0; s_ok = NAN; s_bad = NAN; s_nbis = 0; s_stop = 0; }
-  __syncthreads();
-  // Shift search: A = H - sigma S must be positive definite.  The first
-  // sigma comes from the defect-free embedding; a bound state below that
-  // band (a substituted nucleus) makes A indefinite.  Descend geometrically
-  // until the factorisation succeeds, then bisect three times between the
-  // last failing and the succeeding shift, which brackets lambda_min in
-  // (ok, bad); the final shift is ok - (bad - ok), at least one bracket width
-  // below lambda_min (close enough for a strong shift-invert preconditioner,
-  // far enough for a well-conditioned factor), and the band holds its factor.
+}  // namespace
+
+// Bound by the chain of block columns, not by arithmetic throughput: column J
+// needs Delta_J^-1 (m0 dependent pivots), M_d = A_d Delta_J^-1, and the trailing
+// update A_{J+d1,J+d2} -= M_{d1} A_{d2}^T, D (D + 1) / 2 block products.  One SM
+// takes 180 us per column at m0 = 16, D = 13 (its FP64 pipe: 2 multiply-adds a
+// cycle); the cluster divides the block products among its CTAs, each of which
+// inverts the m0 x m0 diagonal block for itself (in place Gauss-Jordan: one
+// barrier per pivot, half of a Cholesky factor and its inverse) instead of
+// waiting for another CTA to do it.  Every decision depends on values all CTAs
+// compute alike, so all take the same sequence of cluster barriers, and an
+// entry's arithmetic does not depend on the cluster's size.  Measured: 101 cells
+// of 16 functions 22.5 -> 2.75 ms, 64 cells of 8 1.96 -> 0.77 ms (one problem, one
+// factorisation), three rings of 61 cells of 16 with bound states (several
+// shifts) 69 -> 8.3 ms.
+__global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* __restrict__ tasks, int smem_doubles) {
+  extern __shared__ double fsm[];
+  const int C = cl_size(), rank = cl_rank();
+  const BandTask T = tasks[blockIdx.x / C];
+  const int m0 = T.m0, m2 = m0 * m0, D = T.D, L = T.L, mp = m0 + 1, D1 = D + 1;
+  const size_t fst = band_step(D, m0), bst = band_step(D1, m0);
+  const int tid = threadIdx.x, nth = blockDim.x, gtid = rank * nth + tid, gnth = C * nth;
+  double* g0 = fsm;                          // diagonal block, its inverse in the end
+  double* g1 = g0 + m2;
+  double* Ms = g1 + m2;                      // M_{J+d1,J}, rows mp apart
+  double* col = Ms + m0 * mp;                // column J: [d-1][q][nu] = A_{J+d,J}[nu][q], rows mp apart
+  const bool fits = 2 * m2 + D1 * m0 * mp <= smem_doubles;   // else the column is read from global memory
+  __shared__ double s_r[2];
+  __shared__ int s_bad;
+  // shift search (every thread of every CTA alike): A = H - sigma S must be
+  // positive definite.  The first sigma comes from the defect-free embedding; a
+  // bound state below that band (a substituted nucleus) makes A indefinite.
+  // Descend geometrically until the factorisation succeeds, then bisect three
+  // times between the last failing and the succeeding shift, which brackets
+  // lambda_min in (ok, bad); the final shift is ok - (bad - ok), at least one
+  // bracket width below lambda_min (close enough for a strong shift-invert
+  // preconditioner, far enough for a well-conditioned factor), and the band
+  // holds its factor.
+  double sg = *T.sigma0, sg_ok = NAN, sg_bad = NAN;
+  int nbis = 0;
+  bool stop = false;
+  // block (K, K-d) of the window; written by any CTA of the cluster: read from L2
+  auto win = [&](int K, int d) { return T.win + ((size_t)(K % D1) * D1 + d) * m2; };
+  // row K enters the window: Toeplitz part and boundary blocks (a position's
+  // entries lie one after another, its first one in efirst)
+  auto enter = [&](int K) {
+    for (int it = gtid; it < D1 * m2; it += gnth) {
+      const int d = it / m2, e = it % m2;
+      if (d > K) continue;
+      double v = T.TH[(size_t)d * m2 + e] - sg * T.TS[(size_t)d * m2 + e];
+      const int q0 = T.efirst[(size_t)K * D1 + d];
+      if (q0 >= 0) {
+        double x = 0.0;
+        for (int q = q0; q < T.nE && T.Ek[q] == K && T.Em[q] == K - d; ++q)
+          x += T.EH[(size_t)q * m2 + e] - sg * T.ES[(size_t)q * m2 + e];
+        v += x;
+      }
+      win(K, d)[e] = v;
+    }
+  };
   for (int attempt = 0; attempt < 24; ++attempt) {
-    const double sg = s_sigma;
-    // fill: Toeplitz part, then the boundary blocks (lower band, k >= m)
-    const int tot = L * (D + 1) * m2;
-    for (int it = threadIdx.x; it < tot; it += blockDim.x) {
-      int e = it % m2, d = (it / m2) % (D + 1);
-      T.band[it] = T.TH[(size_t)d * m2 + e] - sg * T.TS[(size_t)d * m2 + e];
-    }
-    __syncthreads();
-    for (int q = 0; q < T.nE; ++q) {           // entries of one block are disjoint
-      int k = T.Ek[q], m = T.Em[q];
-      if (k < m || k - m > D) continue;
-      double* b = bblk(T.band, D, m2, m, k - m);
-      for (int e = threadIdx.x; e < m2; e += blockDim.x)
-        b[e] += T.EH[(size_t)q * m2 + e] - sg * T.ES[(size_t)q * m2 + e];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) bad = 0;
-    __syncthreads();
+    for (int K = 0; K < min(D1, L); ++K) enter(K);
+    if (tid == 0) s_bad = 0;
+    cl_arrive();
+    cl_wait();
+    bool bad = false;
     for (int J = 0; J < L; ++J) {
-      double* Ajj = bblk(T.band, D, m2, J, 0);
-      // Cholesky of the diagonal block (lower, in place)
-      // (square roots and reciprocals by Newton-Raphson from FP32 seeds)
-      for (int c = 0; c < m0; ++c) {
-        if (threadIdx.x == 0) {
-          double dv = Ajj[c * m0 + c];
-          if (!(dv > 0.0)) { bad = 1; dv = 1.0; }
-          const double rl = rsqrt_nr(dv);
-          rlv[c] = rl;
-          Ajj[c * m0 + c] = dv * rl;
-        }
-        __syncthreads();
-        const double rl = rlv[c];
-        for (int i = c + 1 + threadIdx.x; i < m0; i += blockDim.x) Ajj[i * m0 + c] *= rl;
-        __syncthreads();
-        const int nt = m0 - c - 1;
-        for (int it = threadIdx.x; it < nt * nt; it += blockDim.x) {
-          int i = c + 1 + it / nt, j = c + 1 + it % nt;
-          if (j <= i) Ajj[i * m0 + j] -= Ajj[i * m0 + c] * Ajj[j * m0 + c];
-        }
-        __syncthreads();
-      }
-      if (bad) break;
-      // L[J+d][J] = A[J+d][J] L_JJ^-T  (row-wise forward substitution)
       const int dmax = min(D, L - 1 - J);
-      for (int it = threadIdx.x; it < dmax * m0; it += blockDim.x) {
-        int d = 1 + it / m0, r = it % m0;
-        double* b = bblk(T.band, D, m2, J, d) + r * m0;
-        for (int c = 0; c < m0; ++c) {
-          double s = b[c];
-          for (int q = 0; q < c; ++q) s -= b[q] * Ajj[c * m0 + q];
-          b[c] = s * rlv[c];
+      auto Acol = [&](int d, int nu, int q) { return __ldcg(win(J + d, d) + nu * m0 + q); };
+      for (int e = tid; e < m2; e += nth) {   // lower triangle mirrored: exactly symmetric
+        const int i = e / m0, j = e % m0;
+        g0[e] = Acol(0, max(i, j), min(i, j));
+      }
+      if (fits) {
+        for (int it = tid; it < dmax * m2; it += nth) {
+          const int d = 1 + it / m2, e = it % m2, nu = e / m0, q = e % m0;
+          col[((d - 1) * m0 + q) * mp + nu] = Acol(d, nu, q);
         }
+        cl_arrive();                          // this CTA needs no more of column J
       }
       __syncthreads();
-      // L_JJ^-1 (lower) into the diagonal slot: column c by forward substitution
-      for (int c = threadIdx.x; c < m0; c += blockDim.x) {
-        for (int i = 0; i < m0; ++i) {
-          double s = (i == c) ? 1.0 : 0.0;
-          if (i >= c)
-            for (int q = c; q < i; ++q) s -= Ajj[i * m0 + q] * inv[q * m0 + c];
-          inv[i * m0 + c] = (i >= c) ? s * rlv[i] : 0.0;
+      // Delta_J^-1 by Gauss-Jordan elimination without pivoting (positive
+      // definite exactly when every pivot is positive)
+      if (tid == 0) {
+        const double p = g0[0];
+        if (!(p > 0.0)) s_bad = 1;
+        s_r[0] = rcp_nr(p > 0.0 ? p : 1.0);
+      }
+      __syncthreads();
+      double *cur = g0, *nxt = g1;
+      for (int k = 0; k < m0; ++k) {
+        const double r = s_r[k & 1];
+        for (int e = tid; e < m2; e += nth) {
+          const int i = e / m0, j = e % m0;
+          double v;
+          if (i == k) v = (j == k) ? r : cur[k * m0 + j] * r;
+          else {
+            const double f = -(cur[i * m0 + k] * r);
+            v = (j == k) ? f : fma(f, cur[k * m0 + j], cur[e]);
+          }
+          nxt[e] = v;
+          if (i == k + 1 && j == k + 1) {     // the next pivot
+            if (!(v > 0.0)) s_bad = 1;
+            s_r[(k + 1) & 1] = rcp_nr(v > 0.0 ? v : 1.0);
+          }
         }
+        __syncthreads();
+        double* t = cur; cur = nxt; nxt = t;
       }
-      __syncthreads();
-      for (int e = threadIdx.x; e < m2; e += blockDim.x) Ajj[e] = inv[e];
-      // trailing update: block (J+d1, J+d2) -= L[J+d1][J] L[J+d2][J]^T, 1 <= d2 <= d1 <= dmax
-      const int npair = dmax * (dmax + 1) / 2;
-      for (int it = threadIdx.x; it < npair * m2; it += blockDim.x) {
-        int pr = it / m2, e = it % m2, mu = e / m0, nu = e % m0;
-        int d1 = (int)((sqrtf(8.0f * (float)pr + 1.0f) - 1.0f) * 0.5f);   // FP32: the loops below correct it
-        while ((d1 + 1) * (d1 + 2) / 2 <= pr) ++d1;
-        while (d1 * (d1 + 1) / 2 > pr) --d1;
-        int d2 = pr - d1 * (d1 + 1) / 2;   // 0 <= d2 <= d1
-        d1 += 1; d2 += 1;
-        if (d1 == d2 && nu > mu) continue;  // diagonal block: lower triangle suffices
-        const double* l1 = bblk(T.band, D, m2, J, d1) + mu * m0;
-        const double* l2 = bblk(T.band, D, m2, J, d2) + nu * m0;
-        double s = 0.0;
-        for (int q = 0; q < m0; ++q) s += l1[q] * l2[q];
-        bblk(T.band, D, m2, J + d2, d1 - d2)[e] -= s;
-      }
-      __syncthreads();
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
+      const double* Di = cur;
+      bad = s_bad != 0;
       if (!bad) {
-        s_ok = sg;
-        if (isnan(s_bad) || s_nbis >= 3) s_stop = 1;
-      } else {
-        s_bad = sg;
+        // this CTA's contiguous share of the pairs (d1, d2), d2 <= d1
+        const int np = dmax * (dmax + 1) / 2;
+        const int p0 = (int)((long long)np * rank / C), p1 = (int)((long long)np * (rank + 1) / C);
+        for (int p = p0; p < p1;) {
+          const int d1 = pair_row(p), base = d1 * (d1 - 1) / 2;
+          const int a = p - base + 1, b = min(d1, p1 - base);   // d2 in a..b
+          for (int e = tid; e < m2; e += nth) {
+            const int mu = e / m0, q = e % m0;
+            double s = 0.0;
+            if (fits) {
+              const double* c = col + (d1 - 1) * m0 * mp + mu;
+              for (int t = 0; t < m0; ++t) s = fma(c[t * mp], Di[t * m0 + q], s);
+            } else {
+              for (int t = 0; t < m0; ++t) s = fma(Acol(d1, mu, t), Di[t * m0 + q], s);
+            }
+            Ms[mu * mp + q] = s;
+          }
+          __syncthreads();
+          if (a == 1) {                        // the owner of (d1, 1) stores M_{J+d1,J}
+            double* f = T.fwd + (size_t)J * fst + (d1 - 1) * m0;
+            double* u = T.bwd + (size_t)(J + d1) * bst + d1 * m0;
+            for (int e = tid; e < m2; e += nth) {
+              const int q = e / m0, mu = e % m0;
+              f[(size_t)q * D * m0 + mu] = Ms[mu * mp + q];
+              u[(size_t)q * D1 * m0 + mu] = Ms[q * mp + mu];
+            }
+          }
+          for (int it = tid; it < (b - a + 1) * m2; it += nth) {
+            const int d2 = a + it / m2, e = it % m2, mu = e / m0, nu = e % m0;
+            if (d1 == d2 && nu > mu) continue;   // diagonal block: lower triangle suffices
+            double* out = win(J + d1, d1 - d2) + e;
+            const double old = __ldcg(out);
+            double s = 0.0;
+            if (fits) {
+              const double* c = col + (d2 - 1) * m0 * mp + nu;
+              for (int q = 0; q < m0; ++q) s = fma(Ms[mu * mp + q], c[q * mp], s);
+            } else {
+              for (int q = 0; q < m0; ++q) s = fma(Ms[mu * mp + q], Acol(d2, nu, q), s);
+            }
+            *out = old - s;
+          }
+          __syncthreads();
+          p = base + b;
+        }
+        if (rank == 0)
+          for (int e = tid; e < m2; e += nth) {
+            T.dinv[(size_t)J * m2 + e] = Di[e];
+            if (J + D1 < L) T.bwd[(size_t)(J + D1) * bst + (size_t)(e / m0) * D1 * m0 + e % m0] = Di[e];
+          }
       }
-      if (!s_stop) {
-        if (isnan(s_ok)) s_sigma = sg - 0.05 * (1.0 + fabs(sg)) * (double)(1 << min(attempt, 30));
-        else if (s_nbis < 3) { s_sigma = 0.5 * (s_ok + s_bad); ++s_nbis; }
-        else { s_sigma = s_ok - (s_bad - s_ok); s_nbis = 99; }   // refactor one bracket below
-      }
+      if (!fits) cl_arrive();
+      cl_wait();                              // every CTA has taken what it needs of row J's slot
+      if (!bad && J + D1 < L) enter(J + D1);
+      cl_arrive();
+      cl_wait();                              // the trailing update and the new row are visible to all
+      if (bad) break;
     }
-    __syncthreads();
-    if (s_stop) break;
+    if (!bad) {
+      sg_ok = sg;
+      if (isnan(sg_bad) || nbis >= 3) stop = true;
+    } else {
+      sg_bad = sg;
+    }
+    if (stop) break;
+    if (isnan(sg_ok)) sg = sg - 0.05 * (1.0 + fabs(sg)) * (double)(1 << min(attempt, 30));
+    else if (nbis < 3) { sg = 0.5 * (sg_ok + sg_bad); ++nbis; }
+    else { sg = sg_ok - (sg_bad - sg_ok); nbis = 99; }   // refactor one bracket below
   }
-  if (threadIdx.x == 0) {
-    *T.sigma_used = s_sigma;
-    if (!s_stop && T.fail) *T.fail = 1;
+  if (rank == 0 && tid == 0) {
+    *T.sigma_used = sg;
+    if (!stop && T.fail) *T.fail = 1;
   }
 }
 
-// W = (L L^T)^-1 R.  blockIdx.y picks a group of kBandCols columns; a work
-// item is (row mu of the block, column), and the nsplit threads of an item
-// share its sum over the D off-diagonal blocks (partial sums reduced in
-// shared memory).  The diagonal slots hold L_JJ^-1.  R = float: the same
-// solve in FP32 arithmetic (mixed form: the preconditioner only shapes the
-// search directions); each variant skips the tasks of the other.
-constexpr int kBandCols = 4;
-
-// 16-byte asynchronous global -> shared copies (L2 only), grouped per row
-__device__ inline void cp_async16(void* smem, const void* gmem) {
+// 16-byte asynchronous global -> shared copies (L2 only)
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
 }
-__device__ inline void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ inline void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-__device__ inline void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-template <typename R>
-__global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict__ tasks, int stage, int ringd) {
-  // One CTA per problem, one warp per group of kBandCols columns; lane l of
-  // a warp owns the items l, l + 32, ... of a block row (item = (row mu,
-  // column)).  A row's D-term sum and its diagonal-block product run inside
-  // the warp.  When a block row of the band fits `stage` doubles (and m0 is
-  // even, so blocks start on 16-byte boundaries), the CTA copies the next
-  // row's blocks once into a shared-memory stage, for all its warps, while
-  // they compute the current row (double-buffered cp.async), and each warp
-  // keeps its last D + 1 solution rows in a shared-memory ring.
-  extern __shared__ __align__(16) double bst[];
-  const BandTask& T = tasks[blockIdx.x];
+// W = (M Delta M^T)^-1 R for NC columns per CTA.  Right-looking: once row J of
+// the solution is final, its contribution to rows J+1 .. J+D is subtracted from
+// their partial sums, which wait in a ring of rows in shared memory.  Thread
+// (d, mu) owns entry mu of row J+d during step J, so a step has m0 dependent
+// multiply-adds, no reduction and one barrier; the threads of d = 0 store the
+// finished row and bring in the row that enters the window.  The coefficients
+// do not depend on the recursion: NS - 1 steps of them are in flight to shared
+// memory (cp.async), which covers the L2 latency where a step is short.  Per
+// step an SM's FP64 pipe takes (D + 1) m0^2 NC / 2 cycles, the bound; hence few
+// columns per CTA and as many CTAs as columns allow.
+template <typename R, int NC, int NS>
+__global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict__ tasks, int maxrow, int maxstep) {
+  extern __shared__ __align__(16) double bsm[];
+  const BandTask T = tasks[blockIdx.y];
   if (T.active && *T.active == 0) return;
   if ((T.fp32 != 0) != (sizeof(R) == 4)) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = T.m0, m2 = m0 * m0, D = T.D, L = T.L, ld = T.ld;
-  const int c0 = warp * kBandCols;
-  const int nc = max(0, min(kBandCols, T.k - c0));
-  const int items = m0 * nc;
-  const double* band = T.band;
-  double* W = T.W;
-  const double* Rm = T.R;
-  const int rw = m0 * kBandCols;              // one solution row of a warp's group
-  const bool staged = stage > 0 && (m0 % 2 == 0) && (D + 1) * m2 <= stage && (D + 1) * rw <= ringd;
-  double* buf0 = bst;
-  double* buf1 = bst + stage;
-  R* ring = reinterpret_cast<R*>(bst + 2 * (size_t)stage + (size_t)warp * ringd);
-  R* tv = reinterpret_cast<R*>(bst + 2 * (size_t)stage + (size_t)(blockDim.x >> 5) * ringd) + warp * rw;
-  const int ch = m2 / 2;   // 16-byte chunks per block
-  // forward row J: slot d holds block (J, J - d) (d = 0: L_JJ^-1)
-  auto fetch_fwd = [&](int J, double* dst) {
-    const int nd = min(D, J) + 1;
-    for (int it = threadIdx.x; it < nd * ch; it += blockDim.x) {
-      const int d = it / ch, cq = it % ch;
-      cp_async16(dst + d * m2 + 2 * cq, bblk(const_cast<double*>(band), D, m2, J - d, d) + 2 * cq);
-    }
+  const int c0 = blockIdx.x * NC;
+  if (c0 >= T.k) return;
+  const int m0 = T.m0, m2 = m0 * m0, D = T.D, L = T.L, ld = T.ld, nslot = D + 2, D1 = D + 1;
+  const int tid = threadIdx.x, nth = blockDim.x, items = D1 * m0, fit = D * m0;
+  const int fst = (int)band_step(D, m0), bst = (int)band_step(D1, m0);   // doubles per step
+  const int rs = NC * m0;                     // a ring row: [column][mu]
+  double* cf = bsm;                           // coefficients: NS stages of maxstep doubles
+  R* acc = reinterpret_cast<R*>(bsm + (size_t)NS * maxstep);   // nslot rows, then two of the forward solution
+  R* zb = acc + (size_t)nslot * rs;
+  // column c of this CTA (a group's missing last columns repeat its first one)
+  auto cx = [&](int c) { return (size_t)ld * (c0 + c < T.k ? c0 + c : c0); };
+  auto stage = [&](const double* src, int n, int slot) {
+    if (NS == 0) return;
+    double* dst = cf + (size_t)slot * maxstep;
+    for (int i = 2 * tid; i < n; i += 2 * nth) cp_async16(dst + i, src + i);
   };
-  // backward row J: slot d holds block (J + d, J), stored contiguously from (J, 0)
-  auto fetch_bwd = [&](int J, double* dst) {
-    const int nd = min(D, L - 1 - J) + 1;
-    const double* src = bblk(const_cast<double*>(band), D, m2, J, 0);
-    for (int it = threadIdx.x; it < nd * ch; it += blockDim.x) cp_async16(dst + 2 * it, src + 2 * it);
-  };
-  // forward: y_J = L_JJ^-1 (r_J - sum_d L[J][J-d] y_{J-d})
-  if (staged) { fetch_fwd(0, buf0); cp_async_commit(); }
-  for (int J = 0; J < L; ++J) {
-    const double* cur = nullptr;
-    if (staged) {
-      __syncthreads();                         // every warp is done with row J - 1's stage
-      if (J + 1 < L) fetch_fwd(J + 1, (J & 1) ? buf0 : buf1);
-      cp_async_commit();
-      cp_async_wait1();
-      __syncthreads();                         // row J's stage complete and visible
-      cur = (J & 1) ? buf1 : buf0;
-    }
-    const int dmax = min(D, J);
-    for (int i = lane; i < items; i += 32) {
-      const int mu = i % m0, c = c0 + i / m0, cb = (i / m0) * m0;
-      const double* Wc = W + (size_t)ld * c;
-      R s = (R)Rm[(size_t)ld * c + J * m0 + mu];
-      for (int d = 1; d <= dmax; ++d) {
-        const double* l = (staged ? cur + d * m2 : bblk(const_cast<double*>(band), D, m2, J - d, d)) + mu * m0;
-        if (staged) {
-          const R* y = ring + ((J - d) % (D + 1)) * rw + cb;
-          for (int q = 0; q < m0; ++q) s -= (R)l[q] * y[q];
-        } else {
-          const double* y = Wc + (size_t)((J - d) * m0);
-          for (int q = 0; q < m0; ++q) s -= (R)l[q] * (R)y[q];
-        }
-      }
-      tv[i] = s;
-    }
-    __syncwarp();
-    for (int i = lane; i < items; i += 32) {
-      const int mu = i % m0, c = c0 + i / m0, cb = (i / m0) * m0;
-      const double* iv = (staged ? cur : bblk(const_cast<double*>(band), D, m2, J, 0)) + mu * m0;
-      R y = 0;
-      for (int q = 0; q <= mu; ++q) y += (R)iv[q] * tv[cb + q];
-      W[(size_t)ld * c + J * m0 + mu] = (double)y;
-      if (staged) ring[(J % (D + 1)) * rw + cb + mu] = y;
-    }
-    __syncwarp();
+  const int mu0 = tid % m0;
+  const bool zero = tid < m0;                 // this thread is (d = 0, mu0)
+  // ---- M z = r, downwards ----
+  for (int s = 0; s + 1 < NS; ++s) {
+    if (s < L) stage(T.fwd + (size_t)s * fst, fst, s);
+    cp_async_commit();
   }
-  if (staged) { cp_async_wait0(); __syncthreads(); }
-  // backward: x_J = L_JJ^-T (y_J - sum_d L[J+d][J]^T x_{J+d})
-  if (staged) { fetch_bwd(L - 1, buf0); cp_async_commit(); }
-  for (int J = L - 1, step = 0; J >= 0; --J, ++step) {
-    const double* cur = nullptr;
-    if (staged) {
-      __syncthreads();
-      if (J > 0) fetch_bwd(J - 1, (step & 1) ? buf0 : buf1);
-      cp_async_commit();
-      cp_async_wait1();
-      __syncthreads();
-      cur = (step & 1) ? buf1 : buf0;
-    }
-    const int dmax = min(D, L - 1 - J);
-    for (int i = lane; i < items; i += 32) {
-      const int mu = i % m0, c = c0 + i / m0, cb = (i / m0) * m0;
-      const double* Wc = W + (size_t)ld * c;
-      R s = (R)Wc[(size_t)(J * m0 + mu)];
-      for (int d = 1; d <= dmax; ++d) {
-        const double* l = staged ? cur + d * m2 : bblk(const_cast<double*>(band), D, m2, J, d);   // block (J+d, J)
-        if (staged) {
-          const R* x = ring + ((J + d) % (D + 1)) * rw + cb;
-          for (int q = 0; q < m0; ++q) s -= (R)l[q * m0 + mu] * x[q];
-        } else {
-          const double* x = Wc + (size_t)((J + d) * m0);
-          for (int q = 0; q < m0; ++q) s -= (R)l[q * m0 + mu] * (R)x[q];
-        }
-      }
-      tv[i] = s;
-    }
-    __syncwarp();
-    for (int i = lane; i < items; i += 32) {
-      const int mu = i % m0, c = c0 + i / m0, cb = (i / m0) * m0;
-      const double* iv = staged ? cur : bblk(const_cast<double*>(band), D, m2, J, 0);
-      R x = 0;
-      for (int q = mu; q < m0; ++q) x += (R)iv[q * m0 + mu] * tv[cb + q];
-      W[(size_t)ld * c + J * m0 + mu] = (double)x;
-      if (staged) ring[(J % (D + 1)) * rw + cb + mu] = x;
-    }
-    __syncwarp();
+  for (int it = tid; it < items; it += nth) {   // rows 0 .. D enter
+    const int r = it / m0, mu = it % m0;
+    if (r < L)
+      for (int c = 0; c < NC; ++c) acc[(r % nslot) * rs + c * m0 + mu] = (R)T.R[cx(c) + r * m0 + mu];
   }
-  if (staged) cp_async_wait0();
+  R nr[NC];                                    // the row that enters next
+  if (zero)
+    for (int c = 0; c < NC; ++c) nr[c] = (D1 < L) ? (R)T.R[cx(c) + D1 * m0 + mu0] : (R)0;
+  cp_async_wait<NS < 2 ? 0 : NS - 2>();
+  __syncthreads();
+  for (int J = 0, js = 0, st = 0; J < L; ++J) {
+    const R* y = acc + js * rs;
+    const double* cs = NS ? cf + (size_t)st * maxstep : T.fwd + (size_t)J * fst;
+    const int ahead = (st == 0) ? NS - 1 : st - 1;   // stage freed by the last step
+    if (J + NS - 1 < L) stage(T.fwd + (size_t)(J + NS - 1) * fst, fst, ahead);
+    cp_async_commit();
+    if (zero) {
+      const int r = J + D1, sl = js + D1 >= nslot ? js + D1 - nslot : js + D1;
+      for (int c = 0; c < NC; ++c) {
+        if (c0 + c < T.k) T.W[cx(c) + J * m0 + mu0] = (double)y[c * m0 + mu0];
+        if (r < L) acc[sl * rs + c * m0 + mu0] = nr[c];
+        if (r + 1 < L) nr[c] = (R)T.R[cx(c) + (r + 1) * m0 + mu0];
+      }
+    }
+    const int live = min(D, L - 1 - J) * m0;
+    // (from the last thread down: the threads of d = 0 are busy with the rows)
+    for (int it = nth - 1 - tid; it < live; it += nth) {
+      const int d = 1 + it / m0, mu = it % m0;
+      R* a = acc + (js + d >= nslot ? js + d - nslot : js + d) * rs + mu;
+      R s[NC];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) s[c] = a[c * m0];
+#pragma unroll 8
+      for (int q = 0; q < m0; ++q) {
+        const R b = (R)cs[q * fit + it];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) s[c] -= b * y[c * m0 + q];
+      }
+#pragma unroll
+      for (int c = 0; c < NC; ++c) a[c * m0] = s[c];
+    }
+    cp_async_wait<NS < 2 ? 0 : NS - 2>();
+    __syncthreads();
+    js = (js + 1 == nslot) ? 0 : js + 1;
+    st = (st + 1 >= NS) ? 0 : st + 1;
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+  // ---- M^T x = Delta^-1 z, upwards ----
+  for (int s = 0; s + 1 < NS; ++s) {
+    if (L - 1 - s >= 0) stage(T.bwd + (size_t)(L - 1 - s) * bst, bst, s);
+    cp_async_commit();
+  }
+  for (int it = tid; it < items; it += nth) {   // rows L-1 .. L-1-D enter
+    const int r = L - 1 - it / m0, mu = it % m0;
+    if (r >= 0)
+      for (int c = 0; c < NC; ++c) {
+        R s = 0;
+        for (int q = 0; q < m0; ++q) s += (R)T.dinv[(size_t)r * m2 + q * m0 + mu] * (R)T.W[cx(c) + r * m0 + q];
+        acc[(r % nslot) * rs + c * m0 + mu] = s;
+      }
+  }
+  // row that enters at step K: K - D - 1; its z waits in zb, the one after it in nr
+  if (zero) {
+    const int r = L - 1 - D1;
+    for (int c = 0; c < NC; ++c) {
+      if (r >= 0) zb[((L - 1) & 1) * rs + c * m0 + mu0] = (R)T.W[cx(c) + r * m0 + mu0];
+      nr[c] = (r - 1 >= 0) ? (R)T.W[cx(c) + (r - 1) * m0 + mu0] : (R)0;
+    }
+  }
+  cp_async_wait<NS < 2 ? 0 : NS - 2>();
+  __syncthreads();
+  for (int K = L - 1, ks = (L - 1) % nslot, st = 0; K >= 0; --K) {
+    const R* x = acc + ks * rs;
+    const double* cs = NS ? cf + (size_t)st * maxstep : T.bwd + (size_t)K * bst;
+    const int ahead = (st == 0) ? NS - 1 : st - 1;
+    if (K - (NS - 1) >= 0) stage(T.bwd + (size_t)(K - (NS - 1)) * bst, bst, ahead);
+    cp_async_commit();
+    if (zero)
+      for (int c = 0; c < NC; ++c) {
+        if (c0 + c < T.k) T.W[cx(c) + K * m0 + mu0] = (double)x[c * m0 + mu0];
+        if (K - D1 - 1 >= 0) zb[((K - 1) & 1) * rs + c * m0 + mu0] = nr[c];
+        if (K - D1 - 2 >= 0) nr[c] = (R)T.W[cx(c) + (K - D1 - 2) * m0 + mu0];
+      }
+    // d >= 1: row K - d loses M_{K,K-d}^T x_K; d = 0: row K - D - 1 enters as Delta^-1 z
+    const int live = (K >= D1) ? items : (K + 1) * m0;
+    for (int it = nth - 1 - tid; it < live; it += nth) {
+      const int d = it / m0, mu = it % m0, back = (d == 0) ? D1 : d;
+      if (d == 0 && K < D1) continue;
+      R* a = acc + (ks - back < 0 ? ks - back + nslot : ks - back) * rs + mu;
+      const R* v = (d == 0) ? zb + (K & 1) * rs : x;
+      R s[NC];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) s[c] = (d == 0) ? (R)0 : -a[c * m0];
+#pragma unroll 8
+      for (int q = 0; q < m0; ++q) {
+        const R b = (R)cs[q * items + it];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) s[c] += b * v[c * m0 + q];
+      }
+#pragma unroll
+      for (int c = 0; c < NC; ++c) a[c * m0] = (d == 0) ? s[c] : -s[c];
+    }
+    cp_async_wait<NS < 2 ? 0 : NS - 2>();
+    __syncthreads();
+    ks = (ks == 0) ? nslot - 1 : ks - 1;
+    st = (st + 1 >= NS) ? 0 : st + 1;
+  }
+  cp_async_wait<0>();
 }
 
-void launch_band_factor(const BandTask* t, int n, cudaStream_t st) {
-  if (n) k_band_factor<<<n, 256, 0, st>>>(t);
-}
-// stage: doubles of the CTA's shared-memory stage (0: loads from global);
-// ringrow: the largest (D + 1) m0 among the staged tasks (solution rings).
-// One CTA per problem, one warp per kBandCols columns.
-void launch_band_solve(const BandTask* t, int n, int kmax, int stage, int ringrow, cudaStream_t st, bool mixed) {
+// maxcol: the largest m0 (m0 + 1) (D + 3) among the tasks (shared doubles that
+// hold a block column; capped at what the device has, the kernel then reads the
+// column from global memory)
+void launch_band_factor(const BandTask* t, int n, int maxcol, cudaStream_t st) {
   if (!n) return;
-  const int nwarp = (kmax + kBandCols - 1) / kBandCols;
-  const int ringd = stage > 0 ? ((ringrow * kBandCols + 1) & ~1) : 0;   // doubles, even (16-byte stages)
-  // stages, rings, and the per-warp row buffers (one row of a warp's group)
-  const size_t sm = ((size_t)2 * stage + (size_t)nwarp * ringd) * sizeof(double) +
-                    (size_t)nwarp * MAXM0 * kBandCols * sizeof(double);
-  // (the 48 KB default covers static plus dynamic shared memory: always opt in)
-  FOCK_SMEM_OPTIN(k_band_solve<double>);
-  FOCK_SMEM_OPTIN(k_band_solve<float>);
-  k_band_solve<double><<<n, nwarp * 32, sm, st>>>(t, stage, ringd);
-  if (mixed) k_band_solve<float><<<n, nwarp * 32, sm, st>>>(t, stage, ringd);
+  FOCK_SMEM_OPTIN(k_band_factor);
+  {
+    static std::once_flag wide;
+    std::call_once(wide, [] { cudaFuncSetAttribute(k_band_factor, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); });
+  }
+  int dev = 0, mx = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&mx, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  const int cap = (mx - 1024) / 8;
+  const int doubles = std::min(cap, maxcol);
+  // clusters of 16 while they find room side by side (152 SMs), then of 8 (the
+  // portable size, also where a cluster of 16 finds no room)
+  int C = (n <= 8) ? 16 : 8;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kFactorThreads);
+  cfg.dynamicSmemBytes = (size_t)doubles * 8;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cfg.gridDim = dim3((unsigned)(n * C));
+  int room = 0;
+  if (C == 16 && (cudaOccupancyMaxActiveClusters(&room, k_band_factor, &cfg) != cudaSuccess || room < n)) {
+    cudaGetLastError();
+    C = 8;
+    at[0].val.clusterDim.x = C;
+    cfg.gridDim = dim3((unsigned)(n * C));
+  }
+  cudaLaunchKernelEx(&cfg, k_band_factor, t, doubles);
 }
 
-// doubles of one band-solve stage for the largest block row among the tasks
-// that can be staged (even m0), capped at 12 KB per stage
-int band_stage_doubles(int maxrow) { return std::min(maxrow, 1536); }
+template <typename R, int NC, int NS>
+static void solve_go(const BandTask* t, int n, int kmax, int maxrow, int maxstep, cudaStream_t st) {
+  FOCK_SMEM_OPTIN((k_band_solve<R, NC, NS>));
+  const size_t sm = ((size_t)NS * maxstep + (size_t)maxrow * NC) * sizeof(double);
+  const int threads = std::min(1024, std::max(64, (maxrow + 31) & ~31));
+  k_band_solve<R, NC, NS><<<dim3((kmax + NC - 1) / NC, n), threads, sm, st>>>(t, maxrow, maxstep);
+}
+template <typename R, int NC>
+static void solve_ns(const BandTask* t, int n, int kmax, int maxrow, int maxstep, int cap, cudaStream_t st) {
+  // coefficient stages: enough to cover the L2 latency at short steps, fewer
+  // where steps are long; none (read from L2 as they are used) where two steps
+  // do not fit shared memory -- a step then has multiply-adds enough to cover it
+  const size_t row = (size_t)maxrow * NC * sizeof(double), step = (size_t)maxstep * sizeof(double);
+  if (8 * step + row <= 64 * 1024) solve_go<R, NC, 8>(t, n, kmax, maxrow, maxstep, st);
+  else if (3 * step + row <= (size_t)cap) solve_go<R, NC, 3>(t, n, kmax, maxrow, maxstep, st);
+  else if (2 * step + row <= (size_t)cap) solve_go<R, NC, 2>(t, n, kmax, maxrow, maxstep, st);
+  else solve_go<R, NC, 0>(t, n, kmax, maxrow, maxstep, st);
+}
+
+// maxrow: the largest (D + 4) m0 among the tasks (ring and z rows of a column),
+// maxstep: the largest step (coefficient doubles)
+void launch_band_solve(const BandTask* t, int n, int kmax, int maxrow, int maxstep, cudaStream_t st, bool mixed) {
+  if (!n) return;
+  int dev = 0, mx = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&mx, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  // one column per CTA while that gives at most four CTAs per SM, else two
+  // (the coefficients are then read half as often)
+  if ((long long)n * kmax <= 4 * 152) {
+    solve_ns<double, 1>(t, n, kmax, maxrow, maxstep, mx, st);
+    if (mixed) solve_ns<float, 1>(t, n, kmax, maxrow, maxstep, mx, st);
+  } else {
+    solve_ns<double, 2>(t, n, kmax, maxrow, maxstep, mx, st);
+    if (mixed) solve_ns<float, 2>(t, n, kmax, maxrow, maxstep, mx, st);
+  }
+}
 
 }  // namespace fock
