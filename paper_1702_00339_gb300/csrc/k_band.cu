@@ -404,9 +404,12 @@ void launch_band_factor(const BandTask* t, int n, int maxcol, cudaStream_t st) {
   cudaDeviceGetAttribute(&mx, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const int cap = (mx - 1024) / 8;
   const int doubles = std::min(cap, maxcol);
-  // clusters of 16 while they find room side by side (152 SMs), then of 8 (the
-  // portable size, also where a cluster of 16 finds no room)
-  int C = (n <= 8) ? 16 : 8;
+  // Clusters of 16 (where the device can place them) for few problems, smaller
+  // ones as the problems alone fill the GPU.  64 cells of 8 functions, clusters of
+  // 16 / 8 / 4: 1 problem 0.77 / 0.94 / 1.19 ms, 16 problems 0.88 / 1.03 / 1.19, 32
+  // 0.94 / 1.04 / 1.19, 128 3.7 / 2.3 / 1.65; 64 cells of 16, 32 problems 3.4 / 3.1 /
+  // 3.3; 64 cells of 32, 8 problems 16.0 / 11.7 / 18.4.
+  int C = (n <= 4) ? 16 : (n <= 64) ? 8 : 4;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kFactorThreads);
   cfg.dynamicSmemBytes = (size_t)doubles * 8;
@@ -438,13 +441,13 @@ static void solve_go(const BandTask* t, int n, int kmax, int maxrow, int maxstep
 }
 template <typename R, int NC>
 static void solve_ns(const BandTask* t, int n, int kmax, int maxrow, int maxstep, int cap, cudaStream_t st) {
-  // coefficient stages: enough to cover the L2 latency at short steps, fewer
-  // where steps are long; none (read from L2 as they are used) where two steps
-  // do not fit shared memory -- a step then has multiply-adds enough to cover it
+  // two stages of coefficients in shared memory; none (read from L2 as they are
+  // used) where they do not fit -- a step then has multiply-adds enough to cover
+  // most of the latency.  Two stages suffice and leave room for more CTAs: eight
+  // stages give the same 98 us on one chain of 64 cells of 8 functions, three give
+  // 929 us against 674 on 32 chains of 64 cells of 16.
   const size_t row = (size_t)maxrow * NC * sizeof(double), step = (size_t)maxstep * sizeof(double);
-  if (8 * step + row <= 64 * 1024) solve_go<R, NC, 8>(t, n, kmax, maxrow, maxstep, st);
-  else if (3 * step + row <= (size_t)cap) solve_go<R, NC, 3>(t, n, kmax, maxrow, maxstep, st);
-  else if (2 * step + row <= (size_t)cap) solve_go<R, NC, 2>(t, n, kmax, maxrow, maxstep, st);
+  if (2 * step + row <= (size_t)cap) solve_go<R, NC, 2>(t, n, kmax, maxrow, maxstep, st);
   else solve_go<R, NC, 0>(t, n, kmax, maxrow, maxstep, st);
 }
 
@@ -455,9 +458,13 @@ void launch_band_solve(const BandTask* t, int n, int kmax, int maxrow, int maxst
   int dev = 0, mx = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&mx, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  // one column per CTA while that gives at most four CTAs per SM, else two
-  // (the coefficients are then read half as often)
-  if ((long long)n * kmax <= 4 * 152) {
+  // One column per CTA while the CTAs fit the GPU about four to an SM, else two
+  // (the coefficients are then read half as often): 64 cells of 8 functions, 320
+  // columns 135 us against 185 with two, 640 columns 261 against 234.  Where the
+  // coefficients come straight from L2 (64 cells of 32 functions) one per SM:
+  // 20 columns 507 us against 892, 160 columns 1541 against 1151.
+  const size_t two = (size_t)2 * maxstep * sizeof(double) + (size_t)maxrow * sizeof(double);
+  if ((long long)n * kmax <= (two <= (size_t)mx ? 4 : 1) * 152) {
     solve_ns<double, 1>(t, n, kmax, maxrow, maxstep, mx, st);
     if (mixed) solve_ns<float, 1>(t, n, kmax, maxrow, maxstep, mx, st);
   } else {
