@@ -66,9 +66,7 @@ __global__ void k_init_x(const InitTask*);
 void launch_gemm_tn(const GemmTask*, int, int, int, int, cudaStream_t);
 __global__ void k_gemm_nn(const GemmTask*);
 __global__ void k_resid(const ResidTask*, double);
-__global__ void k_rr(const RRTask*, int, int);
-__global__ void k_rr_cl(const RRTask*);
-size_t rr_cl_smem(int, int);
+void launch_rr(const RRTask*, int, int, int, int, cudaStream_t);
 __global__ void k_copy_cols(const CopyTask*);
 __global__ void k_colnorm(const CopyTask*);
 }  // namespace fock
@@ -148,9 +146,6 @@ const double kPrecShift = 2e-5;   // sigma = min_j lambda_min(Chat_j) - kPrecShi
 // shorter sums do not repay the digit splitting: measured 56 vs 50 ms per
 // batch of 64 chains of 512 functions, 0.84 vs 1.66 s for one of 16384)
 const int kSplitMinRows = 2048;
-// Rayleigh-Ritz working matrices (3 ld^2 doubles) up to this many bytes live in
-// shared memory
-const size_t kRRSmemCap = 160 * 1024;
 // Fourier blocks (CTAs, of which about half are conjugates that return at
 // once) per piece launched beside a Rayleigh-Ritz launch: about three waves of
 // the 32 x 32 block kernel on the SMs the iteration leaves free, ~10 ms
@@ -467,6 +462,7 @@ struct Batch {
     void* d = nullptr; int n = 0; int ga = 1, gb = 1, tile = 16;
     // mixed form: the same products of mixed problems as tensor-core split tasks
     void* sd = nullptr; int sn = 0, sm = 1, snn = 1, sks = 1; bool sred = false;
+    int rn[2] = {0, 0}, rk[2] = {0, 0};   // Rayleigh-Ritz lists, per class
   };
   // basis layout Y = [X | P | W] (k columns each)
   TL fwdXP, fwdW, fwdR, bmulHS2, bmulHS1, bmulK, invHXP, invSXP, invHW, invSW, invPW;
@@ -476,13 +472,6 @@ struct Batch {
   int band_col = 0;                  // doubles of the largest block column of a band factorisation
   int band_row = 0, band_step = 0;   // largest (D + 4) m0 and largest step of the band solves
   int gemm_tiles = 0;                // TN tile sizes in use: bit 0 = 16, bit 1 = 20
-  bool rr_small = false, rr_big = false;   // Rayleigh-Ritz launches needed (256 / 512 threads)
-  int rr_small_ld = 0;               // largest ld of the shared-memory problems
-  int rr_big_ld = 0;                 // largest ld of the others
-  // the others on thread-block clusters (k_rr_cl) when the plan has no periodic
-  // problems; beside periodic problems one CTA each (k_rr), whose narrow launch
-  // leaves the other SMs to the periodic pieces (both give the same bits)
-  bool rr_cluster = false;
   bool odd_m0 = true;                // some problem has odd m0 (Fourier-block layout, k_fblocks)
   int ptab_maxT = 0, ptab_maxni = 0; // potential tables: largest term count, endpoint count
   TL init, tnCx, nnW, pcG, pcM, pcZ, g1, g3, rr1, rr3, u1, u3, cp2k, resid, normP, normW;
@@ -528,9 +517,6 @@ void plan(Batch& B, Slab& S, Slab& U) {
   B.band_row = 0;
   B.band_step = 0;
   B.gemm_tiles = 0;
-  B.rr_small = B.rr_big = false;
-  B.rr_small_ld = B.rr_big_ld = 0;
-  B.rr_cluster = false;
   B.ptab_maxT = 0; B.ptab_maxni = 0;
   size_t zs_total = 0;
   // ---- parameters, vectors, gram tasks ----
@@ -1160,13 +1146,8 @@ void plan(Batch& B, Slab& S, Slab& U) {
       gg1.push_back(sym(gt(k, k, l.Y, n, l.SY, n, l.GS, ld3, 1.0, 0.0)));
       gg3.push_back(sym(gt(3 * k, 3 * k, l.Y, n, l.HY, n, l.GH, ld3, 1.0, 0.0)));
       gg3.push_back(sym(gt(3 * k, 3 * k, l.Y, n, l.SY, n, l.GS, ld3, 1.0, 0.0)));
-      const int big = (3 * (size_t)ld3 * ld3 * sizeof(double) > kRRSmemCap) ? 1 : 0;
-      r1.push_back({l.active, k, k, ld3, l.GH, l.GS, l.work, l.lam, l.Cc, l.fail, opmode, big});
-      r3.push_back({l.active, 3 * k, k, ld3, l.GH, l.GS, l.work, l.lam, l.Cc, l.fail, opmode, big});
-      B.rr_small = B.rr_small || !big;
-      B.rr_big = B.rr_big || big;
-      if (!big) B.rr_small_ld = std::max(B.rr_small_ld, ld3);
-      else B.rr_big_ld = std::max(B.rr_big_ld, ld3);
+      r1.push_back({l.active, k, k, ld3, l.GH, l.GS, l.work, l.lam, l.Cc, l.fail, opmode, rr_class(k)});
+      r3.push_back({l.active, 3 * k, k, ld3, l.GH, l.GS, l.work, l.lam, l.Cc, l.fail, opmode, rr_class(3 * k)});
       // [X' | P'] = Y[:, :nb] Cc, then copied over [X | P]; images recomputed by a matvec
       uu1.push_back(gt(k, 2 * k, l.Y, n, l.Cc, ld3, l.T1, n, 1.0, 0.0));
       uu3.push_back(gt(3 * k, 2 * k, l.Y, n, l.Cc, ld3, l.T1, n, 1.0, 0.0));
@@ -1212,8 +1193,6 @@ void plan(Batch& B, Slab& S, Slab& U) {
       tl.d = (void*)U.put(v); tl.n = (int)v.size(); tl.ga = ga; tl.gb = gb;
     };
     const int kk = B.kmax;
-    int maxld3 = 0;
-    for (auto& l : B.lob) maxld3 = std::max(maxld3, l.ld3);
     TLp(fXP, B.fwdXP); TLp(fW, B.fwdW); TLp(fR, B.fwdR);
     TLp(iHXP, B.invHXP); TLp(iSXP, B.invSXP); TLp(iHW, B.invHW); TLp(iSW, B.invSW); TLp(iPW, B.invPW);
     TLp(bHS2, B.bmulHS2); TLp(bHS1, B.bmulHS1); TLp(bK, B.bmulK);
@@ -1228,8 +1207,15 @@ void plan(Batch& B, Slab& S, Slab& U) {
     TLp(gg1, B.g1, kk, kk);
     TLp(gg3, B.g3, 3 * kk, 3 * kk);
     B.tnCx.tile = B.pcM.tile = B.g1.tile = B.g3.tile = B.gemm_tiles;
-    TLp(r1, B.rr1, maxld3); TLp(r3, B.rr3, maxld3);
-    B.rr_cluster = B.fbp.empty();   // the periodic tasks are planned by now
+    auto TLr = [&](std::vector<RRTask>& v, Batch::TL& tl) {   // largest basis and wanted count of each launch
+      TLp(v, tl);
+      tl.rn[0] = tl.rn[1] = tl.rk[0] = tl.rk[1] = 0;
+      for (const RRTask& t : v) {
+        tl.rn[t.cls] = std::max(tl.rn[t.cls], t.nb);
+        tl.rk[t.cls] = std::max(tl.rk[t.cls], t.k);
+      }
+    };
+    TLr(r1, B.rr1); TLr(r3, B.rr3);
     TLp(uu1, B.u1); TLp(uu3, B.u3);
     auto TLs = [&](std::vector<SplitTask>& v, Batch::TL& tl) {
       tl.sd = (void*)U.put(v); tl.sn = (int)v.size();
@@ -1510,36 +1496,7 @@ void gemm_nn(Batch& B, const Batch::TL& t, cudaStream_t st) {
 }
 void rr(Batch& B, const Batch::TL& t, cudaStream_t st) {
   PROF("k_rr", 1);
-  if (!t.n) return;
-  FOCK_SMEM_OPTIN(k_rr);
-  // problems whose working matrices fit shared memory: 256 threads; the
-  // others (global memory, latency-bound): 512 threads, more warps in flight
-  if (B.rr_small) {
-    const int ld = B.rr_small_ld;
-    const size_t sm = ((size_t)3 * ld * ld + (size_t)rr_stage_extra(ld)) * sizeof(double);
-    k_rr<<<t.n, 256, sm, st>>>(tl<RRTask>(t), (int)sm, 0);
-  }
-  if (B.rr_big && !B.rr_cluster) {
-    const size_t sm = (size_t)2 * kRRBlock * B.rr_big_ld * sizeof(double);
-    k_rr<<<t.n, 512, sm, st>>>(tl<RRTask>(t), (int)sm, 1);
-  }
-  if (B.rr_big && B.rr_cluster) {
-    // one cluster of kRRCluster CTAs per problem
-    FOCK_SMEM_OPTIN(k_rr_cl);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(t.n * kRRCluster));
-    cfg.blockDim = dim3(512);
-    cfg.dynamicSmemBytes = rr_cl_smem(B.rr_big_ld, B.kmax);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = kRRCluster;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, k_rr_cl, tl<RRTask>(t));
-  }
+  for (int c = 0; c < 2; ++c) launch_rr(tl<RRTask>(t), t.n, c, t.rn[c], t.rk[c], st);
 }
 // unit 2-norm columns before a matvec: the FFT packs two real columns per
 // complex transform, and a column far smaller than its partner would get an

@@ -292,29 +292,19 @@ struct ResidTask {
   double* res;        // [k] relative residual
 };
 
-// pivot columns per block of the Rayleigh-Ritz step's triangular substitutions
-// (its shared-memory staging: 2 kRRBlock ld doubles)
-constexpr int kRRBlock = 8;
-// CTAs of the cluster that runs one large Rayleigh-Ritz step (k_rr_cl)
-constexpr int kRRCluster = 8;
-// extra doubles of staging a shared-memory Rayleigh-Ritz step needs beyond its
-// 3 ld^2 (none when its first working matrix, ld^2 doubles, can hold it)
-__host__ __device__ inline int rr_stage_extra(int ld) { return (ld * ld >= 2 * kRRBlock * ld) ? 0 : 2 * kRRBlock * ld; }
+// Rayleigh-Ritz steps are launched by size: 0 up to 64 columns, 1 above
+__host__ __device__ inline int rr_class(int nb) { return nb > 64 ? 1 : 0; }
 
 struct RRTask {
   const int* active;
   int nb, k, ld;          // current basis size, wanted pairs, leading dim of G / C
-  double* GH; double* GS; // [nb x nb] (ld), destroyed
-  double* work;           // [7 * ld * ld] scratch: C, V, Z (global when they do not fit
-                          //   shared memory), then 4 ld^2 for the tridiagonal eigensolver
+  const double* GH; const double* GS;   // [nb x nb] (ld)
+  double* work;           // [7 * ld * ld] scratch (k_rr.cu)
   double* lam;            // out [k]
   double* Cc;             // out [nb x 2k] (ld): [C | C with the first k rows zeroed]
   int* fail;              // out: 1 if Y^T S Y was not numerically positive definite
   const int* mode;        // mixed form: 1 while the images are FP32 (coarser drop threshold)
-  int big;                // 1: the working matrices (3 ld^2 doubles) exceed shared memory; the
-                          //    problem runs on a cluster of 512-thread CTAs (k_rr_cl), else in
-                          //    the 256-thread k_rr (a property of the problem alone, so results
-                          //    are batch-invariant)
+  int cls;                // rr_class(nb): the launch that handles it
 };
 
 struct CopyTask { const int* active; int n, ncols; const double* src; int lds; double* dst; int ldd; };
@@ -397,9 +387,10 @@ struct MatvecView {
 // On this part a warp-wide FP64 instruction holds a sub-partition's FP64
 // unit for ~64 cycles whether 1 or 32 lanes are active; an IEEE FP64
 // division takes ~440 cycles and a square root ~690 (measured).  Reciprocal
-// and inverse square root below: an FP32 seed refined by two Newton-Raphson
-// steps in FP64 (quadratic convergence, relative error 2^-22 -> 2^-44 ->
-// rounding level), 4 and 8 FP64 instructions.  Arguments outside
+// and inverse square root below: an FP32 seed (relative error e below 2^-22)
+// and one step of third order in FP64, which leaves e^3, below rounding: 3 and
+// 5 FP64 instructions, 3 and 4 of them in a chain (two Newton-Raphson steps
+// take 4 and 8, all in a chain).  Arguments outside
 // [2^-100, 2^100] in magnitude (where the FP32 seed could over- or
 // underflow) take the IEEE operation; the test is on the exponent bits.
 __device__ inline bool nr_range(double x) {
@@ -408,21 +399,16 @@ __device__ inline bool nr_range(double x) {
 }
 __device__ inline double rcp_nr(double x) {
   if (!nr_range(x)) return 1.0 / x;
-  double r = (double)__frcp_rn((float)x);
-  double e = fma(-x, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-x, r, 1.0);
-  return fma(r, e, r);
+  const double r = (double)__frcp_rn((float)x);
+  const double e = fma(-x, r, 1.0);              // 1/x = r / (1 - e) = r (1 + e + e^2 + ...)
+  return fma(r, fma(e, e, e), r);
 }
 // x > 0
 __device__ inline double rsqrt_nr(double x) {
   if (!nr_range(x)) return 1.0 / sqrt(x);
-  double r = (double)__frsqrt_rn((float)x);
-  // Newton for r^-2 = x: r <- r + (r / 2)(1 - x r^2)
-  double e = fma(-x * r, r, 1.0);
-  r = fma(0.5 * r, e, r);
-  e = fma(-x * r, r, 1.0);
-  return fma(0.5 * r, e, r);
+  const double r = (double)__frsqrt_rn((float)x);
+  const double e = fma(-x * r, r, 1.0);          // x^-1/2 = r (1 - e)^-1/2 = r (1 + e/2 + 3 e^2/8 + ...)
+  return fma(r * e, fma(0.375, e, 0.5), r);
 }
 // |x| as a bit pattern: orders like |x| (integer compare, no FP64 pipe)
 __device__ inline long long abs_bits(double x) { return __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll; }
