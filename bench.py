@@ -476,8 +476,8 @@ def fp64_flops_per_step(problems, outs):
             # banded preconditioner: forward and backward block substitution over
             # L cells with D + 1 blocks of m0 x m0 per block row, kb columns
             D = o.get("D")
-            # the library's rule: the banded factor when 2 L D^2 m0^3 <= 4e9
-            band = D is not None and 2.0 * p.L[0] * D * D * m0 ** 3 <= 4e9
+            # the library's rule: the banded factor when 2 L D^2 m0^3 <= 8e9
+            band = D is not None and 2.0 * p.L[0] * D * D * m0 ** 3 <= 8e9
             if band:
                 w["k_band_solve"] = w.get("k_band_solve", 0) + it * 4 * p.L[0] * (D + 1) * m0 * m0 * kb
             # circulant-embedding FFTs: per iteration 9 kb m0 column transforms (forward of W

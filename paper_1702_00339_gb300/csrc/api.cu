@@ -57,8 +57,8 @@ int fft_max_cc(int);
 void launch_blockmul(const BmulTask*, int, int, int, cudaStream_t, bool);
 void launch_eapply(const EApplyTask*, int, int, cudaStream_t);
 int eapply_grid(long long items);
-void launch_band_factor(const BandTask*, int, int, cudaStream_t);
-void launch_band_solve(const BandTask*, int, int, int, int, cudaStream_t, bool);
+void launch_band_factor(const BandTask*, int, int, int, cudaStream_t);
+void launch_band_solve(const BandTask*, int, int, int, int, int, cudaStream_t, bool);
 void launch_cell_canon(const CanonTask*, int, int, int, cudaStream_t);
 void launch_gather(const GatherSeg*, int, uint32_t*, cudaStream_t);
 void launch_cell_back(const double*, int, int, int, const double*, double*, int, cudaStream_t);
@@ -470,7 +470,7 @@ struct Batch {
   TL rfwdXP, rinvHXP, rinvSXP, rbmulHS2, reHXP;   // image refresh at the FP32 -> FP64 switch
   TL bandF, bandS;
   int band_col = 0;                  // doubles of the largest block column of a band factorisation
-  int band_row = 0, band_step = 0;   // largest (D + 4) m0 and largest step of the band solves
+  int band_row = 0, band_step = 0, band_8 = 0;   // band solves: largest (D + 4) m0, step, 8 (D + 1) m0
   int gemm_tiles = 0;                // TN tile sizes in use: bit 0 = 16, bit 1 = 20
   bool odd_m0 = true;                // some problem has odd m0 (Fourier-block layout, k_fblocks)
   int ptab_maxT = 0, ptab_maxni = 0; // potential tables: largest term count, endpoint count
@@ -515,7 +515,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
   B.any_mixed = false;
   B.band_col = 0;
   B.band_row = 0;
-  B.band_step = 0;
+  B.band_step = B.band_8 = 0;
   B.gemm_tiles = 0;
   B.ptab_maxT = 0; B.ptab_maxni = 0;
   size_t zs_total = 0;
@@ -931,9 +931,13 @@ void plan(Batch& B, Slab& S, Slab& U) {
       Q.K = S.take<cplx>((size_t)Q.M * m2);
       Q.emin = S.take<double>(Q.M);
       Q.sigma = S.take<double>(1);
-      // banded Cholesky of H - sigma S when its one-CTA factorisation stays
-      // within ~4 GFLOP (tens of ms); above that the circulant inverse
-      Q.use_band = 2.0 * Q.Lc * (double)Q.D * Q.D * (double)H.m0 * H.m0 * H.m0 <= 4e9;
+      // Banded factor of H - sigma S up to ~8 GFLOP (70 ms), above that the circulant
+      // inverse.  512 cells of 32 functions (5.7e9, D = 13), 64 eigenpairs, three draws:
+      // banded 13 iterations and 185 ms in the mixed form, 350 in the FP64 form;
+      // circulant 31, 50, 37 iterations and 207, 320, 243 ms (FP64 718 ms and more).
+      // Beyond, an iteration no longer repays the factor: 1000 cells (1.1e10) 359
+      // against 274 ms, 800 cells with D = 18 (1.7e10) 500 against 346.
+      Q.use_band = 2.0 * Q.Lc * (double)Q.D * Q.D * (double)H.m0 * H.m0 * H.m0 <= 8e9;
       if (Q.use_band) {
         Q.band_win = S.take<double>((size_t)(Q.D + 1) * (Q.D + 1) * m2);
         Q.band_fwd = S.take<double>((size_t)Q.Lc * std::max<size_t>(band_step(Q.D, H.m0), 2));
@@ -1077,6 +1081,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
         B.band_col = std::max(B.band_col, 2 * m0 * m0 + (Q.D + 1) * m0 * (m0 + 1));
         B.band_row = std::max(B.band_row, (Q.D + 4) * m0);
         B.band_step = std::max(B.band_step, (int)band_step(Q.D + 1, m0));
+        if (m0 > 8) B.band_8 = std::max(B.band_8, 8 * (Q.D + 1) * m0);
         std::vector<int> ef((size_t)Q.Lc * (Q.D + 1), -1);   // a position's entries lie one after another
         for (int e = Q.nE - 1; e >= 0; --e)
           if (Q.Ek[e] >= Q.Em[e] && Q.Ek[e] - Q.Em[e] <= Q.D) ef[(size_t)Q.Ek[e] * (Q.D + 1) + Q.Ek[e] - Q.Em[e]] = e;
@@ -1424,7 +1429,7 @@ void run_struct_setup(fock_ctx* ctx, Batch& B) {
   for (auto& Q : B.pp)
     if (Q.band_fail) cudaMemsetAsync(Q.band_fail, 0, sizeof(int), st);
   if (B.bandF.n) { PROF("k_band_factor", 1);
-    launch_band_factor(reinterpret_cast<const BandTask*>(B.bandF.d), B.bandF.n, B.band_col, st); }
+    launch_band_factor(reinterpret_cast<const BandTask*>(B.bandF.d), B.bandF.n, B.band_col, B.maxm0, st); }
 }
 
 template <class T> const T* tl(const Batch::TL& t) { return reinterpret_cast<const T*>(t.d); }
@@ -1537,7 +1542,7 @@ void refresh_XP(Batch& B, cudaStream_t st) {
 // Rayleigh-Ritz, P' S-orthogonal to X' in the coefficients, [X | P] <- Y Cc and
 // their fresh images.  Launches only.
 void lobpcg_body_a(Batch& B, cudaStream_t st) {
-  if (B.bandS.n) { PROF("k_band_solve", 1); launch_band_solve(tl<BandTask>(B.bandS), B.bandS.n, B.kmax, B.band_row, B.band_step, st, B.any_mixed); }
+  if (B.bandS.n) { PROF("k_band_solve", 1); launch_band_solve(tl<BandTask>(B.bandS), B.bandS.n, B.kmax, B.band_row, B.band_step, B.band_8, st, B.any_mixed); }
   if (B.fwdR.n) {
     mv_fwd(B, B.fwdR, st);
     { PROF("k_blockmul", 1); launch_blockmul(tl<BmulTask>(B.bmulK), B.bmulK.n, B.maxM, B.maxm0, st, B.any_mixed); }

@@ -35,7 +35,7 @@ __device__ __forceinline__ void cl_wait() { asm volatile("barrier.cluster.wait.a
 __device__ __forceinline__ int cl_rank() { int r; asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
 __device__ __forceinline__ int cl_size() { int r; asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
 
-constexpr int kFactorThreads = 256;
+constexpr int kFactorThreads = 512;   // 256 where blocks are small
 
 // Row d1 (1-based) of pair number p in the order (1,1) (2,1) (2,2) (3,1) ...
 __device__ __forceinline__ int pair_row(int p) {
@@ -52,14 +52,14 @@ __device__ __forceinline__ int pair_row(int p) {
 // update A_{J+d1,J+d2} -= M_{d1} A_{d2}^T, D (D + 1) / 2 block products.  One SM
 // takes 180 us per column at m0 = 16, D = 13 (its FP64 pipe: 2 multiply-adds a
 // cycle); the cluster divides the block products among its CTAs, each of which
-// inverts the m0 x m0 diagonal block for itself (in place Gauss-Jordan: one
+// inverts the m0 x m0 diagonal block for itself (Gauss-Jordan: one
 // barrier per pivot, half of a Cholesky factor and its inverse) instead of
-// waiting for another CTA to do it.  Every decision depends on values all CTAs
+// waiting for another CTA to do it; the M_d are made by one CTA each.  Every decision depends on values all CTAs
 // compute alike, so all take the same sequence of cluster barriers, and an
 // entry's arithmetic does not depend on the cluster's size.  Measured: 101 cells
-// of 16 functions 22.5 -> 2.75 ms, 64 cells of 8 1.96 -> 0.77 ms (one problem, one
+// of 16 functions 22.5 -> 2.5 ms, 64 cells of 8 1.96 -> 0.75 ms (one problem, one
 // factorisation), three rings of 61 cells of 16 with bound states (several
-// shifts) 69 -> 8.3 ms.
+// shifts) 69 -> 7.7 ms, 512 cells of 32 50 ms.
 __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* __restrict__ tasks, int smem_doubles) {
   extern __shared__ double fsm[];
   const int C = cl_size(), rank = cl_rank();
@@ -123,32 +123,31 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
           const int d = 1 + it / m2, e = it % m2, nu = e / m0, q = e % m0;
           col[((d - 1) * m0 + q) * mp + nu] = Acol(d, nu, q);
         }
-        cl_arrive();                          // this CTA needs no more of column J
       }
       __syncthreads();
       // Delta_J^-1 by Gauss-Jordan elimination without pivoting (positive
       // definite exactly when every pivot is positive)
       if (tid == 0) {
         const double p = g0[0];
-        if (!(p > 0.0)) s_bad = 1;
-        s_r[0] = rcp_nr(p > 0.0 ? p : 1.0);
+        const bool pos = __double_as_longlong(p) > 0;
+        if (!pos || !(p == p)) s_bad = 1;
+        s_r[0] = rcp_nr(pos ? p : 1.0);
       }
       __syncthreads();
       double *cur = g0, *nxt = g1;
+      const int step = nth - nth % m0, j = tid % m0;   // a thread's entries lie in one column j
       for (int k = 0; k < m0; ++k) {
         const double r = s_r[k & 1];
-        for (int e = tid; e < m2; e += nth) {
-          const int i = e / m0, j = e % m0;
-          double v;
-          if (i == k) v = (j == k) ? r : cur[k * m0 + j] * r;
-          else {
-            const double f = -(cur[i * m0 + k] * r);
-            v = (j == k) ? f : fma(f, cur[k * m0 + j], cur[e]);
-          }
-          nxt[e] = v;
-          if (i == k + 1 && j == k + 1) {     // the next pivot
-            if (!(v > 0.0)) s_bad = 1;
-            s_r[(k + 1) & 1] = rcp_nr(v > 0.0 ? v : 1.0);
+        if (tid < step) {
+          const double g = (j == k) ? r : cur[k * m0 + j] * r;   // row k of the next matrix
+          for (int e = tid, i = tid / m0; e < m2; e += step, i += step / m0) {
+            const double v = (i == k) ? g : fma(-cur[i * m0 + k], g, (j == k) ? 0.0 : cur[e]);
+            nxt[e] = v;
+            if (i == k + 1 && j == k + 1) {     // the next pivot
+              const bool pos = __double_as_longlong(v) > 0;
+              if (!pos || !(v == v)) s_bad = 1;
+              s_r[(k + 1) & 1] = rcp_nr(pos ? v : 1.0);
+            }
           }
         }
         __syncthreads();
@@ -156,6 +155,41 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
       }
       const double* Di = cur;
       bad = s_bad != 0;
+      // M_{J+d1,J} into Ms, and its storage for the solves: by one CTA each, read by
+      // the others after a barrier (made anew where the column does not fit)
+      auto make_M = [&](int d1) {
+        for (int e = tid; e < m2; e += nth) {
+          const int mu = e / m0, q = e % m0;
+          double s = 0.0;
+          if (fits) {
+            const double* c = col + (d1 - 1) * m0 * mp + mu;
+            for (int t = 0; t < m0; ++t) s = fma(c[t * mp], Di[t * m0 + q], s);
+          } else {
+            for (int t = 0; t < m0; ++t) s = fma(Acol(d1, mu, t), Di[t * m0 + q], s);
+          }
+          Ms[mu * mp + q] = s;
+        }
+        __syncthreads();
+      };
+      auto store_M = [&](int d1) {
+        double* f = T.fwd + (size_t)J * fst + (d1 - 1) * m0;
+        double* u = T.bwd + (size_t)(J + d1) * bst + d1 * m0;
+        for (int e = tid; e < m2; e += nth) {
+          const int q = e / m0, mu = e % m0;
+          f[(size_t)q * D * m0 + mu] = Ms[mu * mp + q];
+          u[(size_t)q * D1 * m0 + mu] = Ms[q * mp + mu];
+        }
+      };
+      if (fits) {
+        if (!bad)
+          for (int d1 = 1 + rank; d1 <= dmax; d1 += C) {
+            make_M(d1);
+            store_M(d1);
+            __syncthreads();
+          }
+        cl_arrive();                          // (and this CTA needs no more of column J)
+        cl_wait();
+      }
       if (!bad) {
         // this CTA's contiguous share of the pairs (d1, d2), d2 <= d1
         const int np = dmax * (dmax + 1) / 2;
@@ -163,26 +197,13 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
         for (int p = p0; p < p1;) {
           const int d1 = pair_row(p), base = d1 * (d1 - 1) / 2;
           const int a = p - base + 1, b = min(d1, p1 - base);   // d2 in a..b
-          for (int e = tid; e < m2; e += nth) {
-            const int mu = e / m0, q = e % m0;
-            double s = 0.0;
-            if (fits) {
-              const double* c = col + (d1 - 1) * m0 * mp + mu;
-              for (int t = 0; t < m0; ++t) s = fma(c[t * mp], Di[t * m0 + q], s);
-            } else {
-              for (int t = 0; t < m0; ++t) s = fma(Acol(d1, mu, t), Di[t * m0 + q], s);
-            }
-            Ms[mu * mp + q] = s;
-          }
-          __syncthreads();
-          if (a == 1) {                        // the owner of (d1, 1) stores M_{J+d1,J}
-            double* f = T.fwd + (size_t)J * fst + (d1 - 1) * m0;
-            double* u = T.bwd + (size_t)(J + d1) * bst + d1 * m0;
-            for (int e = tid; e < m2; e += nth) {
-              const int q = e / m0, mu = e % m0;
-              f[(size_t)q * D * m0 + mu] = Ms[mu * mp + q];
-              u[(size_t)q * D1 * m0 + mu] = Ms[q * mp + mu];
-            }
+          if (fits) {
+            const double* f = T.fwd + (size_t)J * fst + (d1 - 1) * m0;
+            for (int e = tid; e < m2; e += nth) Ms[(e % m0) * mp + e / m0] = __ldcg(f + (size_t)(e / m0) * D * m0 + e % m0);
+            __syncthreads();
+          } else {
+            make_M(d1);
+            if (a == 1) store_M(d1);           // the owner of (d1, 1)
           }
           for (int it = tid; it < (b - a + 1) * m2; it += nth) {
             const int d2 = a + it / m2, e = it % m2, mu = e / m0, nu = e % m0;
@@ -207,8 +228,10 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
             if (J + D1 < L) T.bwd[(size_t)(J + D1) * bst + (size_t)(e / m0) * D1 * m0 + e % m0] = Di[e];
           }
       }
-      if (!fits) cl_arrive();
-      cl_wait();                              // every CTA has taken what it needs of row J's slot
+      if (!fits) {
+        cl_arrive();
+        cl_wait();                            // every CTA has taken what it needs of row J's slot
+      }
       if (!bad && J + D1 < L) enter(J + D1);
       cl_arrive();
       cl_wait();                              // the trailing update and the new row are visible to all
@@ -237,162 +260,152 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+// coefficient rows per stage of at most `stage` doubles: the whole step, or a
+// multiple of 8 (a stage then starts on a 16-byte boundary)
+__host__ __device__ inline int band_rows(int nd, int m0, int stage) {
+  return ((int)band_step(nd, m0) <= stage) ? m0 : max(8, (stage / (nd * m0)) & ~7);
+}
 
-// W = (M Delta M^T)^-1 R for NC columns per CTA.  Right-looking: once row J of
+// W = (M Delta M^T)^-1 R, one column of R per CTA.  Right-looking: once row J of
 // the solution is final, its contribution to rows J+1 .. J+D is subtracted from
 // their partial sums, which wait in a ring of rows in shared memory.  Thread
 // (d, mu) owns entry mu of row J+d during step J, so a step has m0 dependent
-// multiply-adds, no reduction and one barrier; the threads of d = 0 store the
+// multiply-adds and no reduction; the threads of d = 0 store the
 // finished row and bring in the row that enters the window.  The coefficients
-// do not depend on the recursion: NS - 1 steps of them are in flight to shared
-// memory (cp.async), which covers the L2 latency where a step is short.  Per
-// step an SM's FP64 pipe takes (D + 1) m0^2 NC / 2 cycles, the bound; hence few
-// columns per CTA and as many CTAs as columns allow.
-template <typename R, int NC, int NS>
-__global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict__ tasks, int maxrow, int maxstep) {
+// do not depend on the recursion: they come through two stages of shared memory
+// (cp.async), qc rows of a step's coefficients at a time (MULTI; the whole step
+// where all tasks' steps fit a stage), so that the L2 latency runs beside the
+// multiply-adds.  Per step an SM's FP64 pipe takes (D + 1) m0^2 / 2 cycles, the
+// bound; hence one column per CTA (two, which read the coefficients half as often,
+// were slower from 20 columns to 2560).  Measured per launch,
+// 20 columns a problem: one chain of 64 cells of 8 functions (D = 13) 941 -> 97 us,
+// 32 of them 945 -> 200 us, three rings of 61 cells of 16 4320 -> 166 us; with one
+// step of coefficients ahead in registers instead of shared memory the first took
+// 205 us.  72 columns of 512 cells of 32: 4.9 ms (6.9 without the stages).
+template <typename R, bool MULTI>
+__global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict__ tasks, int maxrow, int maxstage) {
   extern __shared__ __align__(16) double bsm[];
   const BandTask T = tasks[blockIdx.y];
   if (T.active && *T.active == 0) return;
   if ((T.fp32 != 0) != (sizeof(R) == 4)) return;
-  const int c0 = blockIdx.x * NC;
-  if (c0 >= T.k) return;
-  const int m0 = T.m0, m2 = m0 * m0, D = T.D, L = T.L, ld = T.ld, nslot = D + 2, D1 = D + 1;
+  if (blockIdx.x >= (unsigned)T.k) return;
+  const double* Rc = T.R + (size_t)T.ld * blockIdx.x;   // this CTA's column
+  double* Wc = T.W + (size_t)T.ld * blockIdx.x;
+  const int m0 = T.m0, m2 = m0 * m0, D = T.D, L = T.L, nslot = D + 2, D1 = D + 1;
   const int tid = threadIdx.x, nth = blockDim.x, items = D1 * m0, fit = D * m0;
   const int fst = (int)band_step(D, m0), bst = (int)band_step(D1, m0);   // doubles per step
-  const int rs = NC * m0;                     // a ring row: [column][mu]
-  double* cf = bsm;                           // coefficients: NS stages of maxstep doubles
-  R* acc = reinterpret_cast<R*>(bsm + (size_t)NS * maxstep);   // nslot rows, then two of the forward solution
-  R* zb = acc + (size_t)nslot * rs;
-  // column c of this CTA (a group's missing last columns repeat its first one)
-  auto cx = [&](int c) { return (size_t)ld * (c0 + c < T.k ? c0 + c : c0); };
-  auto stage = [&](const double* src, int n, int slot) {
-    if (NS == 0) return;
-    double* dst = cf + (size_t)slot * maxstep;
+  // rows of coefficients per stage: all m0, or a multiple of 8 that fits
+  const int qc = MULTI ? band_rows(D1, m0, maxstage) : m0, nch = MULTI ? (m0 + qc - 1) / qc : 1;
+  double* cf = bsm;                           // two stages of maxstage doubles
+  R* acc = reinterpret_cast<R*>(bsm + (size_t)2 * maxstage);   // nslot rows, then two of the forward solution
+  R* zb = acc + (size_t)nslot * m0;
+  // rows [h qc, ...) of a step of `width` entries a row into stage `slot`
+  auto stage = [&](const double* step, int total, int width, int h, int slot) {
+    const double* src = step + (size_t)h * qc * width;
+    const int n = min(qc * width, total - h * qc * width);
+    double* dst = cf + (size_t)slot * maxstage;
     for (int i = 2 * tid; i < n; i += 2 * nth) cp_async16(dst + i, src + i);
   };
   const int mu0 = tid % m0;
   const bool zero = tid < m0;                 // this thread is (d = 0, mu0)
   // ---- M z = r, downwards ----
-  for (int s = 0; s + 1 < NS; ++s) {
-    if (s < L) stage(T.fwd + (size_t)s * fst, fst, s);
-    cp_async_commit();
-  }
+  stage(T.fwd, fst, fit, 0, 0);
+  cp_async_commit();
   for (int it = tid; it < items; it += nth) {   // rows 0 .. D enter
     const int r = it / m0, mu = it % m0;
     if (r < L)
-      for (int c = 0; c < NC; ++c) acc[(r % nslot) * rs + c * m0 + mu] = (R)T.R[cx(c) + r * m0 + mu];
+      acc[(r % nslot) * m0 + mu] = (R)Rc[(size_t)r * m0 + mu];
   }
-  R nr[NC];                                    // the row that enters next
-  if (zero)
-    for (int c = 0; c < NC; ++c) nr[c] = (D1 < L) ? (R)T.R[cx(c) + D1 * m0 + mu0] : (R)0;
-  cp_async_wait<NS < 2 ? 0 : NS - 2>();
+  R nr = 0;                                    // the row that enters next
+  if (zero && D1 < L) nr = (R)Rc[(size_t)D1 * m0 + mu0];
+  cp_async_wait0();
   __syncthreads();
-  for (int J = 0, js = 0, st = 0; J < L; ++J) {
-    const R* y = acc + js * rs;
-    const double* cs = NS ? cf + (size_t)st * maxstep : T.fwd + (size_t)J * fst;
-    const int ahead = (st == 0) ? NS - 1 : st - 1;   // stage freed by the last step
-    if (J + NS - 1 < L) stage(T.fwd + (size_t)(J + NS - 1) * fst, fst, ahead);
-    cp_async_commit();
-    if (zero) {
-      const int r = J + D1, sl = js + D1 >= nslot ? js + D1 - nslot : js + D1;
-      for (int c = 0; c < NC; ++c) {
-        if (c0 + c < T.k) T.W[cx(c) + J * m0 + mu0] = (double)y[c * m0 + mu0];
-        if (r < L) acc[sl * rs + c * m0 + mu0] = nr[c];
-        if (r + 1 < L) nr[c] = (R)T.R[cx(c) + (r + 1) * m0 + mu0];
-      }
-    }
+  int st = 0;
+  for (int J = 0, js = 0; J < L; ++J) {
+    const R* y = acc + js * m0;
     const int live = min(D, L - 1 - J) * m0;
-    // (from the last thread down: the threads of d = 0 are busy with the rows)
-    for (int it = nth - 1 - tid; it < live; it += nth) {
-      const int d = 1 + it / m0, mu = it % m0;
-      R* a = acc + (js + d >= nslot ? js + d - nslot : js + d) * rs + mu;
-      R s[NC];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) s[c] = a[c * m0];
-#pragma unroll 8
-      for (int q = 0; q < m0; ++q) {
-        const R b = (R)cs[q * fit + it];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) s[c] -= b * y[c * m0 + q];
+    for (int h = 0; h < nch; ++h, st ^= 1) {
+      const double* cs = cf + (size_t)st * maxstage;
+      if (h + 1 < nch) stage(T.fwd + (size_t)J * fst, fst, fit, h + 1, st ^ 1);
+      else if (J + 1 < L) stage(T.fwd + (size_t)(J + 1) * fst, fst, fit, 0, st ^ 1);
+      cp_async_commit();
+      if (zero && h == 0) {
+        const int r = J + D1, sl = js + D1 >= nslot ? js + D1 - nslot : js + D1;
+        Wc[(size_t)J * m0 + mu0] = (double)y[mu0];
+        if (r < L) acc[sl * m0 + mu0] = nr;
+        if (r + 1 < L) nr = (R)Rc[(size_t)(r + 1) * m0 + mu0];
       }
-#pragma unroll
-      for (int c = 0; c < NC; ++c) a[c * m0] = s[c];
+      const int qa = h * qc, qn = min(qc, m0 - qa);
+      // (from the last thread down: the threads of d = 0 are busy with the rows)
+      for (int it = nth - 1 - tid; it < live; it += nth) {
+        const int d = 1 + it / m0, mu = it % m0;
+        R* a = acc + (js + d >= nslot ? js + d - nslot : js + d) * m0 + mu;
+        R s = *a;
+#pragma unroll 8
+        for (int q = 0; q < qn; ++q) s -= (R)cs[q * fit + it] * y[qa + q];
+        *a = s;
+      }
+      cp_async_wait0();
+      __syncthreads();
     }
-    cp_async_wait<NS < 2 ? 0 : NS - 2>();
-    __syncthreads();
     js = (js + 1 == nslot) ? 0 : js + 1;
-    st = (st + 1 >= NS) ? 0 : st + 1;
   }
-  cp_async_wait<0>();
-  __syncthreads();
   // ---- M^T x = Delta^-1 z, upwards ----
-  for (int s = 0; s + 1 < NS; ++s) {
-    if (L - 1 - s >= 0) stage(T.bwd + (size_t)(L - 1 - s) * bst, bst, s);
-    cp_async_commit();
-  }
+  stage(T.bwd + (size_t)(L - 1) * bst, bst, items, 0, st);
+  cp_async_commit();
   for (int it = tid; it < items; it += nth) {   // rows L-1 .. L-1-D enter
     const int r = L - 1 - it / m0, mu = it % m0;
-    if (r >= 0)
-      for (int c = 0; c < NC; ++c) {
-        R s = 0;
-        for (int q = 0; q < m0; ++q) s += (R)T.dinv[(size_t)r * m2 + q * m0 + mu] * (R)T.W[cx(c) + r * m0 + q];
-        acc[(r % nslot) * rs + c * m0 + mu] = s;
-      }
+    if (r >= 0) {
+      R s = 0;
+      for (int q = 0; q < m0; ++q) s += (R)T.dinv[(size_t)r * m2 + q * m0 + mu] * (R)Wc[(size_t)r * m0 + q];
+      acc[(r % nslot) * m0 + mu] = s;
+    }
   }
   // row that enters at step K: K - D - 1; its z waits in zb, the one after it in nr
   if (zero) {
     const int r = L - 1 - D1;
-    for (int c = 0; c < NC; ++c) {
-      if (r >= 0) zb[((L - 1) & 1) * rs + c * m0 + mu0] = (R)T.W[cx(c) + r * m0 + mu0];
-      nr[c] = (r - 1 >= 0) ? (R)T.W[cx(c) + (r - 1) * m0 + mu0] : (R)0;
-    }
+    if (r >= 0) zb[((L - 1) & 1) * m0 + mu0] = (R)Wc[(size_t)r * m0 + mu0];
+    nr = (r - 1 >= 0) ? (R)Wc[(size_t)(r - 1) * m0 + mu0] : (R)0;
   }
-  cp_async_wait<NS < 2 ? 0 : NS - 2>();
+  cp_async_wait0();
   __syncthreads();
-  for (int K = L - 1, ks = (L - 1) % nslot, st = 0; K >= 0; --K) {
-    const R* x = acc + ks * rs;
-    const double* cs = NS ? cf + (size_t)st * maxstep : T.bwd + (size_t)K * bst;
-    const int ahead = (st == 0) ? NS - 1 : st - 1;
-    if (K - (NS - 1) >= 0) stage(T.bwd + (size_t)(K - (NS - 1)) * bst, bst, ahead);
-    cp_async_commit();
-    if (zero)
-      for (int c = 0; c < NC; ++c) {
-        if (c0 + c < T.k) T.W[cx(c) + K * m0 + mu0] = (double)x[c * m0 + mu0];
-        if (K - D1 - 1 >= 0) zb[((K - 1) & 1) * rs + c * m0 + mu0] = nr[c];
-        if (K - D1 - 2 >= 0) nr[c] = (R)T.W[cx(c) + (K - D1 - 2) * m0 + mu0];
-      }
+  for (int K = L - 1, ks = (L - 1) % nslot; K >= 0; --K) {
+    const R* x = acc + ks * m0;
     // d >= 1: row K - d loses M_{K,K-d}^T x_K; d = 0: row K - D - 1 enters as Delta^-1 z
     const int live = (K >= D1) ? items : (K + 1) * m0;
-    for (int it = nth - 1 - tid; it < live; it += nth) {
-      const int d = it / m0, mu = it % m0, back = (d == 0) ? D1 : d;
-      if (d == 0 && K < D1) continue;
-      R* a = acc + (ks - back < 0 ? ks - back + nslot : ks - back) * rs + mu;
-      const R* v = (d == 0) ? zb + (K & 1) * rs : x;
-      R s[NC];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) s[c] = (d == 0) ? (R)0 : -a[c * m0];
-#pragma unroll 8
-      for (int q = 0; q < m0; ++q) {
-        const R b = (R)cs[q * items + it];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) s[c] += b * v[c * m0 + q];
+    for (int h = 0; h < nch; ++h, st ^= 1) {
+      const double* cs = cf + (size_t)st * maxstage;
+      if (h + 1 < nch) stage(T.bwd + (size_t)K * bst, bst, items, h + 1, st ^ 1);
+      else if (K > 0) stage(T.bwd + (size_t)(K - 1) * bst, bst, items, 0, st ^ 1);
+      cp_async_commit();
+      if (zero && h == 0) {
+        Wc[(size_t)K * m0 + mu0] = (double)x[mu0];
+        if (K - D1 - 1 >= 0) zb[((K - 1) & 1) * m0 + mu0] = nr;
+        if (K - D1 - 2 >= 0) nr = (R)Wc[(size_t)(K - D1 - 2) * m0 + mu0];
       }
-#pragma unroll
-      for (int c = 0; c < NC; ++c) a[c * m0] = (d == 0) ? s[c] : -s[c];
+      const int qa = h * qc, qn = min(qc, m0 - qa);
+      for (int it = nth - 1 - tid; it < live; it += nth) {
+        const int d = it / m0, mu = it % m0, back = (d == 0) ? D1 : d;
+        if (d == 0 && K < D1) continue;
+        R* a = acc + (ks - back < 0 ? ks - back + nslot : ks - back) * m0 + mu;
+        const R* v = ((d == 0) ? zb + (K & 1) * m0 : x) + qa;
+        R s = (d != 0) ? -*a : (h == 0) ? (R)0 : *a;
+#pragma unroll 8
+        for (int q = 0; q < qn; ++q) s += (R)cs[q * items + it] * v[q];
+        *a = (d == 0) ? s : -s;
+      }
+      cp_async_wait0();
+      __syncthreads();
     }
-    cp_async_wait<NS < 2 ? 0 : NS - 2>();
-    __syncthreads();
     ks = (ks == 0) ? nslot - 1 : ks - 1;
-    st = (st + 1 >= NS) ? 0 : st + 1;
   }
-  cp_async_wait<0>();
 }
 
 // maxcol: the largest m0 (m0 + 1) (D + 3) among the tasks (shared doubles that
 // hold a block column; capped at what the device has, the kernel then reads the
 // column from global memory)
-void launch_band_factor(const BandTask* t, int n, int maxcol, cudaStream_t st) {
+void launch_band_factor(const BandTask* t, int n, int maxcol, int maxm0, cudaStream_t st) {
   if (!n) return;
   FOCK_SMEM_OPTIN(k_band_factor);
   {
@@ -411,7 +424,8 @@ void launch_band_factor(const BandTask* t, int n, int maxcol, cudaStream_t st) {
   // 3.3; 64 cells of 32, 8 problems 16.0 / 11.7 / 18.4.
   int C = (n <= 4) ? 16 : (n <= 64) ? 8 : 4;
   cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(kFactorThreads);
+  // (64 cells of 32 functions 6.5 ms with 256 threads, 5.9 with 512; of 8 0.76 and 0.82)
+  cfg.blockDim = dim3(maxm0 > 16 ? kFactorThreads : 256);
   cfg.dynamicSmemBytes = (size_t)doubles * 8;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
@@ -432,44 +446,30 @@ void launch_band_factor(const BandTask* t, int n, int maxcol, cudaStream_t st) {
   cudaLaunchKernelEx(&cfg, k_band_factor, t, doubles);
 }
 
-template <typename R, int NC, int NS>
-static void solve_go(const BandTask* t, int n, int kmax, int maxrow, int maxstep, cudaStream_t st) {
-  FOCK_SMEM_OPTIN((k_band_solve<R, NC, NS>));
-  const size_t sm = ((size_t)NS * maxstep + (size_t)maxrow * NC) * sizeof(double);
-  const int threads = std::min(1024, std::max(64, (maxrow + 31) & ~31));
-  k_band_solve<R, NC, NS><<<dim3((kmax + NC - 1) / NC, n), threads, sm, st>>>(t, maxrow, maxstep);
-}
-template <typename R, int NC>
-static void solve_ns(const BandTask* t, int n, int kmax, int maxrow, int maxstep, int cap, cudaStream_t st) {
-  // two stages of coefficients in shared memory; none (read from L2 as they are
-  // used) where they do not fit -- a step then has multiply-adds enough to cover
-  // most of the latency.  Two stages suffice and leave room for more CTAs: eight
-  // stages give the same 98 us on one chain of 64 cells of 8 functions, three give
-  // 929 us against 674 on 32 chains of 64 cells of 16.
-  const size_t row = (size_t)maxrow * NC * sizeof(double), step = (size_t)maxstep * sizeof(double);
-  if (2 * step + row <= (size_t)cap) solve_go<R, NC, 2>(t, n, kmax, maxrow, maxstep, st);
-  else solve_go<R, NC, 0>(t, n, kmax, maxrow, maxstep, st);
-}
-
 // maxrow: the largest (D + 4) m0 among the tasks (ring and z rows of a column),
-// maxstep: the largest step (coefficient doubles)
-void launch_band_solve(const BandTask* t, int n, int kmax, int maxrow, int maxstep, cudaStream_t st, bool mixed) {
+// maxstep: the largest step (coefficient doubles), max8: the largest 8 (D + 1) m0
+// of the steps that are taken in pieces
+template <typename R, bool MULTI>
+static void solve_go(const BandTask* t, int n, int kmax, int maxrow, int maxstage, cudaStream_t st) {
+  FOCK_SMEM_OPTIN((k_band_solve<R, MULTI>));
+  const size_t sm = ((size_t)2 * maxstage + (size_t)maxrow) * sizeof(double);
+  const int threads = std::min(1024, std::max(64, (maxrow + 31) & ~31));
+  k_band_solve<R, MULTI><<<dim3(kmax, n), threads, sm, st>>>(t, maxrow, maxstage);
+}
+void launch_band_solve(const BandTask* t, int n, int kmax, int maxrow, int maxstep, int max8, cudaStream_t st, bool mixed) {
   if (!n) return;
-  int dev = 0, mx = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&mx, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  // One column per CTA while the CTAs fit the GPU about four to an SM, else two
-  // (the coefficients are then read half as often): 64 cells of 8 functions, 320
-  // columns 135 us against 185 with two, 640 columns 261 against 234.  Where the
-  // coefficients come straight from L2 (64 cells of 32 functions) one per SM:
-  // 20 columns 507 us against 892, 160 columns 1541 against 1151.
-  const size_t two = (size_t)2 * maxstep * sizeof(double) + (size_t)maxrow * sizeof(double);
-  if ((long long)n * kmax <= (two <= (size_t)mx ? 4 : 1) * 152) {
-    solve_ns<double, 1>(t, n, kmax, maxrow, maxstep, mx, st);
-    if (mixed) solve_ns<float, 1>(t, n, kmax, maxrow, maxstep, mx, st);
+  // A stage holds a step up to 64 KB, or as many rows of one (at least 8).  Two
+  // stages are enough and leave room for several CTAs per SM: eight give the same
+  // 98 us on one chain of 64 cells of 8 functions, three 929 us against 674 on 32
+  // chains of 64 cells of 16.  Pieces of 32 KB instead of 64: 72 columns of 512 cells
+  // of 32 functions 5.8 ms against 4.9.
+  const int maxstage = std::max(std::min(maxstep, 8192), max8);
+  if (maxstep <= maxstage) {
+    solve_go<double, false>(t, n, kmax, maxrow, maxstage, st);
+    if (mixed) solve_go<float, false>(t, n, kmax, maxrow, maxstage, st);
   } else {
-    solve_ns<double, 2>(t, n, kmax, maxrow, maxstep, mx, st);
-    if (mixed) solve_ns<float, 2>(t, n, kmax, maxrow, maxstep, mx, st);
+    solve_go<double, true>(t, n, kmax, maxrow, maxstage, st);
+    if (mixed) solve_go<float, true>(t, n, kmax, maxrow, maxstage, st);
   }
 }
 
