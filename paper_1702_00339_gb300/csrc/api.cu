@@ -55,8 +55,7 @@ void launch_fft(const FftTask*, int, int, int, int, int, cudaStream_t, bool);
 void launch_fft_cc(const FftTask*, int, int, int, int, int, cudaStream_t, bool);
 int fft_max_cc(int);
 void launch_blockmul(const BmulTask*, int, int, int, cudaStream_t, bool);
-void launch_eapply(const EApplyTask*, int, int, cudaStream_t);
-int eapply_grid(long long items);
+void launch_eapply(const EApplyTask*, int, int, int, int, bool, cudaStream_t);
 void launch_band_factor(const BandTask*, int, int, int, cudaStream_t);
 void launch_band_solve(const BandTask*, int, int, int, int, int, cudaStream_t, bool);
 void launch_cell_canon(const CanonTask*, int, int, int, cudaStream_t);
@@ -486,7 +485,7 @@ struct Batch {
   int graph_nodes = 0;
   // periodic Fourier blocks issued in pieces: next local index, piece width
   int pchunk_next = 0, pchunk_w = 0;
-  int eapply_gx = 16;
+  int eapply_rows = 0;               // largest number of block rows with E entries
   int* d_ones = nullptr;
   int* d_active = nullptr;
   int* d_mode = nullptr;             // per structured problem: 1 while its matvecs run in FP32
@@ -515,6 +514,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
   B.any_mixed = false;
   B.band_col = 0;
   B.band_row = 0;
+  B.eapply_rows = 0;
   B.band_step = B.band_8 = 0;
   B.gemm_tiles = 0;
   B.ptab_maxT = 0; B.ptab_maxni = 0;
@@ -1041,7 +1041,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
       const int n = l.n, k = l.k, m0 = H.m0, ld3 = l.ld3;
       const size_t nk = (size_t)n * k;
       maxcols = std::max(maxcols, m0 * k);   // packed: two real columns per transform
-      B.eapply_gx = std::max(B.eapply_gx, eapply_grid((long long)Q.nErows * m0 * 2 * k));
+      B.eapply_rows = std::max(B.eapply_rows, Q.nErows);
       cplx* X = B.mvX + B.mv_off[s2];
       cplx* Y1 = B.mvY1 + B.mv_off[s2];
       cplx* Y2 = B.mvY2 + B.mv_off[s2];
@@ -1095,8 +1095,9 @@ void plan(Batch& B, Slab& S, Slab& U) {
       auto ea = [&](const double* vals, const double* x, double* y, int ncol, const int* md) {
         EApplyTask t;
         std::memset(&t, 0, sizeof(t));
+      const int* ekinds = Q.nE ? U.put(Q.Ekind) : nullptr;
         t.prob = i; t.m0 = m0; t.ncol = ncol; t.nrows = Q.nErows; t.rows = Q.Erows; t.rowptr = Q.Erowptr;
-        t.cols = Q.Ecols; t.vals = vals; t.x = x; t.ldx = n; t.y = y; t.ldy = n; t.mode = md; t.active = l.active;
+        t.cols = Q.Ecols; t.vals = vals; t.x = x; t.ldx = n; t.y = y; t.ldy = n; t.mode = md; t.active = l.active; t.kinds = ekinds;
         return t;
       };
       if (Q.nE) {
@@ -1524,7 +1525,7 @@ void mv_HS(Batch& B, bool xp, cudaStream_t st) {
   mv_inv(B, xp ? B.invHXP : B.invHW, st);
   mv_inv(B, xp ? B.invSXP : B.invSW, st);
   const Batch::TL& eh = xp ? B.eHXP : B.eHW;   // each task applies the H and the S blocks
-  if (eh.n) { PROF("k_eapply", 1); launch_eapply(tl<EApplyTask>(eh), eh.n, B.eapply_gx, st); }
+  if (eh.n) { PROF("k_eapply", 1); launch_eapply(tl<EApplyTask>(eh), eh.n, B.eapply_rows, (xp ? 2 : 1) * B.kmax, B.maxm0, true, st); }
 }
 
 // [X | P] images in FP64 for the problems flagged in d_refresh only
@@ -1533,7 +1534,7 @@ void refresh_XP(Batch& B, cudaStream_t st) {
   { PROF("k_blockmul", 1); launch_blockmul(tl<BmulTask>(B.rbmulHS2), B.rbmulHS2.n, B.maxM, B.maxm0, st, false); }
   mv_inv(B, B.rinvHXP, st);
   mv_inv(B, B.rinvSXP, st);
-  if (B.reHXP.n) { PROF("k_eapply", 1); launch_eapply(tl<EApplyTask>(B.reHXP), B.reHXP.n, B.eapply_gx, st); }
+  if (B.reHXP.n) { PROF("k_eapply", 1); launch_eapply(tl<EApplyTask>(B.reHXP), B.reHXP.n, B.eapply_rows, 2 * B.kmax, B.maxm0, true, st); }
 }
 
 // One block-iteration step after the convergence test, in two parts.  A: W = K R
@@ -2561,7 +2562,7 @@ int fock_toeplitz_matvec(fock_ctx* ctx, const fock_blocks* b, int which, const d
   launch_fft((const FftTask*)tasks, 1, chunks, Q.M, cc, +1, st, false);
   launch_blockmul((const BmulTask*)(tasks + 1024), 1, Q.M, H.m0, st, false);
   launch_fft((const FftTask*)(tasks + 512), 1, chunks, Q.M, cc, -1, st, false);
-  if (Q.nE) launch_eapply((const EApplyTask*)(tasks + 1536), 1, eapply_grid((long long)Q.nErows * H.m0 * nvec), st);
+  if (Q.nE) launch_eapply((const EApplyTask*)(tasks + 1536), 1, Q.nErows, nvec, H.m0, false, st);
   if (!on_device) CUDA_TRY(ctx, cudaMemcpyAsync(y, dy, nbytes, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(ctx, cudaStreamSynchronize(st));
   CUDA_TRY(ctx, cudaGetLastError());

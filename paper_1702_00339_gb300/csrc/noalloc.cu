@@ -21,8 +21,7 @@ int blocks_matvec_view(const fock_blocks* b, MatvecView* v);
 void set_ctx_error(fock_ctx* c, const char* msg);
 void launch_fft(const FftTask*, int, int, int, int, int, cudaStream_t, bool);
 void launch_blockmul(const BmulTask*, int, int, int, cudaStream_t, bool);
-void launch_eapply(const EApplyTask*, int, int, cudaStream_t);
-int eapply_grid(long long items);
+void launch_eapply(const EApplyTask*, int, int, int, int, bool, cudaStream_t);
 }  // namespace fock
 
 using namespace fock;
@@ -129,7 +128,7 @@ extern "C" int fock_toeplitz_matvec_noalloc(fock_ctx* ctx, const fock_blocks* b,
   launch_blockmul((const BmulTask*)(s + 2 * kDescSlot), 1, v.M, v.m0, v.stream, false);
   launch_fft((const FftTask*)(s + kDescSlot), 1, chunks, v.M, cc, -1, v.stream, false);
   if (v.nE)
-    launch_eapply((const EApplyTask*)(s + 3 * kDescSlot), 1, eapply_grid((long long)v.nErows * v.m0 * nvec), v.stream);
+    launch_eapply((const EApplyTask*)(s + 3 * kDescSlot), 1, v.nErows, nvec, v.m0, false, v.stream);
   cudaError_t e = cudaStreamSynchronize(v.stream);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
