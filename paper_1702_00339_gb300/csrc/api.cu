@@ -62,7 +62,7 @@ void launch_cell_canon(const CanonTask*, int, int, int, cudaStream_t);
 void launch_gather(const GatherSeg*, int, uint32_t*, cudaStream_t);
 void launch_cell_back(const double*, int, int, int, const double*, double*, int, cudaStream_t);
 __global__ void k_init_x(const InitTask*);
-void launch_gemm_tn(const GemmTask*, int, int, int, int, cudaStream_t);
+void launch_gemm_tn(const GemmTask*, int, int, int, int, int, cudaStream_t);
 __global__ void k_gemm_nn(const GemmTask*);
 __global__ void k_resid(const ResidTask*, double);
 void launch_rr(const RRTask*, int, int, int, int, cudaStream_t);
@@ -145,6 +145,7 @@ const double kPrecShift = 2e-5;   // sigma = min_j lambda_min(Chat_j) - kPrecShi
 // shorter sums do not repay the digit splitting: measured 56 vs 50 ms per
 // batch of 64 chains of 512 functions, 0.84 vs 1.66 s for one of 16384)
 const int kSplitMinRows = 2048;
+const int kGemmTiles = 256;   // output tiles of a TN product: at most (255 / 16 + 1)^2
 // Fourier blocks (CTAs, of which about half are conjugates that return at
 // once) per piece launched beside a Rayleigh-Ritz launch: about three waves of
 // the 32 x 32 block kernel on the SMs the iteration leaves free, ~10 ms
@@ -458,7 +459,7 @@ struct Batch {
   cplx *mvX = nullptr, *mvY1 = nullptr, *mvY2 = nullptr;   // FFT work (shared by all structured)
   std::vector<size_t> mv_off;        // per structured problem: offset (cplx) into mv buffers
   struct TL {
-    void* d = nullptr; int n = 0; int ga = 1, gb = 1, tile = 16;
+    void* d = nullptr; int n = 0; int ga = 1, gb = 1, tile = 16, gk = 1;
     // mixed form: the same products of mixed problems as tensor-core split tasks
     void* sd = nullptr; int sn = 0, sm = 1, snn = 1, sks = 1; bool sred = false;
     int rn[2] = {0, 0}, rk[2] = {0, 0};   // Rayleigh-Ritz lists, per class
@@ -471,6 +472,7 @@ struct Batch {
   int band_col = 0;                  // doubles of the largest block column of a band factorisation
   int band_row = 0, band_step = 0, band_8 = 0;   // band solves: largest (D + 4) m0, step, 8 (D + 1) m0
   int gemm_tiles = 0;                // TN tile sizes in use: bit 0 = 16, bit 1 = 20
+  int* gemm_count = nullptr;         // [structured problem][2][kGemmTiles] arrivals of split TN sums, zero between launches
   bool odd_m0 = true;                // some problem has odd m0 (Fourier-block layout, k_fblocks)
   int ptab_maxT = 0, ptab_maxni = 0; // potential tables: largest term count, endpoint count
   TL init, tnCx, nnW, pcG, pcM, pcZ, g1, g3, rr1, rr3, u1, u3, cp2k, resid, normP, normW;
@@ -512,9 +514,9 @@ void plan(Batch& B, Slab& S, Slab& U) {
   B.maxnj_p = B.maxnj_s = 0; B.maxm0 = 1; B.maxM = 0; B.maxsort = 0; B.kmax = 0; B.maxLdft = 1;
   B.odd_m0 = false;
   B.any_mixed = false;
+  B.eapply_rows = 0;
   B.band_col = 0;
   B.band_row = 0;
-  B.eapply_rows = 0;
   B.band_step = B.band_8 = 0;
   B.gemm_tiles = 0;
   B.ptab_maxT = 0; B.ptab_maxni = 0;
@@ -1032,6 +1034,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
     std::vector<ResidTask> rs;
     std::vector<BandTask> bnd;
     std::vector<int> ones(ns, 1);
+    B.gemm_count = S.take<int>((size_t)ns * 2 * kGemmTiles);
     B.d_ones = U.put(ones);
     for (int s2 = 0; s2 < ns; ++s2) {
       const int i = B.sidx[s2];
@@ -1092,10 +1095,10 @@ void plan(Batch& B, Slab& S, Slab& U) {
         iPW.push_back(inv(Y1, Yw, k, pcmode));
         bK.push_back({i, Q.M, m0, k, Q.K, nullptr, X, Y1, nullptr, pcmode, l.active});
       }
+      const int* ekinds = Q.nE ? U.put(Q.Ekind) : nullptr;
       auto ea = [&](const double* vals, const double* x, double* y, int ncol, const int* md) {
         EApplyTask t;
         std::memset(&t, 0, sizeof(t));
-      const int* ekinds = Q.nE ? U.put(Q.Ekind) : nullptr;
         t.prob = i; t.m0 = m0; t.ncol = ncol; t.nrows = Q.nErows; t.rows = Q.Erows; t.rowptr = Q.Erowptr;
         t.cols = Q.Ecols; t.vals = vals; t.x = x; t.ldx = n; t.y = y; t.ldy = n; t.mode = md; t.active = l.active; t.kinds = ekinds;
         return t;
@@ -1124,13 +1127,23 @@ void plan(Batch& B, Slab& S, Slab& U) {
                     double alpha, double beta) {
         GemmTask g; g.active = l.active; g.n = n; g.a = a; g.b = b; g.A = A; g.lda = lda; g.B = Bm; g.ldb = ldb;
         g.C = C; g.ldc = ldc; g.alpha = alpha; g.beta = beta; g.sym = 0; g.split = 0;
+        g.ksplit = 1; g.part = nullptr; g.count = nullptr;
         g.tile = (k % 20 == 0) ? 20 : 16;   // a property of the problem alone
         B.gemm_tiles |= (g.tile == 20) ? 2 : 1;
         return g;
       };
+      // TN products over n with their sums split (the projection; the two Gram
+      // matrices, whose start on X alone reuses the same partial sums)
+      const int ks = gemm_tn_ksplit(n);
+      const size_t pgram = (size_t)ks * 9 * k * k;
+      double* part = (ks > 1) ? S.take<double>(2 * pgram) : nullptr;
+      auto tn = [&](GemmTask g, int which) {
+        if (ks > 1) { g.ksplit = ks; g.part = part + which * pgram; g.count = B.gemm_count + ((size_t)s2 * 2 + which) * kGemmTiles; }
+        return g;
+      };
       // W made S-orthogonal to X before its images are formed:  C = (S X)^T W,
       // W -= X C (the images of the projected vectors are then fresh)
-      tcx.push_back(gt(k, k, l.SY, n, Yw, n, l.Cx, k, 1.0, 0.0));
+      tcx.push_back(tn(gt(k, k, l.SY, n, Yw, n, l.Cx, k, 1.0, 0.0), 0));
       nw.push_back(gt(k, k, l.Y, n, l.Cx, k, l.Y + 2 * nk, n, -1.0, 1.0));
       // P' made S-orthogonal to X' in the coefficients, before [X' | P'] = Y Cc is
       // formed: with z_X, z_P the two column blocks of Cc and G_S = Y^T S Y,
@@ -1148,10 +1161,10 @@ void plan(Batch& B, Slab& S, Slab& U) {
       }
       // Gram matrices Y^T H Y, Y^T S Y: symmetric, upper tiles only
       auto sym = [](GemmTask g) { g.sym = 1; return g; };
-      gg1.push_back(sym(gt(k, k, l.Y, n, l.HY, n, l.GH, ld3, 1.0, 0.0)));
-      gg1.push_back(sym(gt(k, k, l.Y, n, l.SY, n, l.GS, ld3, 1.0, 0.0)));
-      gg3.push_back(sym(gt(3 * k, 3 * k, l.Y, n, l.HY, n, l.GH, ld3, 1.0, 0.0)));
-      gg3.push_back(sym(gt(3 * k, 3 * k, l.Y, n, l.SY, n, l.GS, ld3, 1.0, 0.0)));
+      gg1.push_back(tn(sym(gt(k, k, l.Y, n, l.HY, n, l.GH, ld3, 1.0, 0.0)), 0));
+      gg1.push_back(tn(sym(gt(k, k, l.Y, n, l.SY, n, l.GS, ld3, 1.0, 0.0)), 1));
+      gg3.push_back(tn(sym(gt(3 * k, 3 * k, l.Y, n, l.HY, n, l.GH, ld3, 1.0, 0.0)), 0));
+      gg3.push_back(tn(sym(gt(3 * k, 3 * k, l.Y, n, l.SY, n, l.GS, ld3, 1.0, 0.0)), 1));
       r1.push_back({l.active, k, k, ld3, l.GH, l.GS, l.work, l.lam, l.Cc, l.fail, opmode, rr_class(k)});
       r3.push_back({l.active, 3 * k, k, ld3, l.GH, l.GS, l.work, l.lam, l.Cc, l.fail, opmode, rr_class(3 * k)});
       // [X' | P'] = Y[:, :nb] Cc, then copied over [X | P]; images recomputed by a matvec
@@ -1196,7 +1209,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
     B.fft_chunks = (maxcols + B.fft_cc - 1) / B.fft_cc;
     B.fft_maxcols = maxcols;
     auto TLp = [&](auto& v, Batch::TL& tl, int ga = 1, int gb = 1) {
-      tl.d = (void*)U.put(v); tl.n = (int)v.size(); tl.ga = ga; tl.gb = gb;
+      tl.d = (void*)U.put(v); tl.n = (int)v.size(); tl.ga = ga; tl.gb = gb; tl.gk = 1;
     };
     const int kk = B.kmax;
     TLp(fXP, B.fwdXP); TLp(fW, B.fwdW); TLp(fR, B.fwdR);
@@ -1213,6 +1226,8 @@ void plan(Batch& B, Slab& S, Slab& U) {
     TLp(gg1, B.g1, kk, kk);
     TLp(gg3, B.g3, 3 * kk, 3 * kk);
     B.tnCx.tile = B.pcM.tile = B.g1.tile = B.g3.tile = B.gemm_tiles;
+    for (const GemmTask& g : tcx) B.tnCx.gk = std::max(B.tnCx.gk, g.ksplit);
+    B.g1.gk = B.g3.gk = B.tnCx.gk;   // the same sums over n
     auto TLr = [&](std::vector<RRTask>& v, Batch::TL& tl) {   // largest basis and wanted count of each launch
       TLp(v, tl);
       tl.rn[0] = tl.rn[1] = tl.rk[0] = tl.rk[1] = 0;
@@ -1492,12 +1507,12 @@ void split_products(Batch& B, const Batch::TL& t, cudaStream_t st) {
 }
 void gemm_tn(Batch& B, const Batch::TL& t, cudaStream_t st) {
   { PROF("k_gemm_tn", 1);
-    launch_gemm_tn(tl<GemmTask>(t), t.n, t.ga, t.gb, t.tile, st); }   // ga, gb: output dims; tile: tile-size bits
+    launch_gemm_tn(tl<GemmTask>(t), t.n, t.ga, t.gb, t.tile, t.gk, st); }   // ga, gb: output dims; tile: tile-size bits
   split_products(B, t, st);
 }
 void gemm_nn(Batch& B, const Batch::TL& t, cudaStream_t st) {
   { PROF("k_gemm_nn", 1);
-    if (t.n) k_gemm_nn<<<dim3(64, t.n), 256, 0, st>>>(tl<GemmTask>(t)); }
+    if (t.n) k_gemm_nn<<<dim3(128, t.n), 256, 0, st>>>(tl<GemmTask>(t)); }
   split_products(B, t, st);
 }
 void rr(Batch& B, const Batch::TL& t, cudaStream_t st) {
@@ -1584,6 +1599,7 @@ int run_lobpcg(fock_ctx* ctx, Batch& B, double tol, int maxit, std::vector<int>&
   if (!ns) return FOCK_OK;
   CUDA_TRY(ctx, cudaMemcpyAsync(B.d_active, B.d_ones, ns * sizeof(int), cudaMemcpyDeviceToDevice, st));
   CUDA_TRY(ctx, cudaMemsetAsync(B.d_fail, 0, ns * sizeof(int), st));
+  CUDA_TRY(ctx, cudaMemsetAsync(B.gemm_count, 0, (size_t)ns * 2 * kGemmTiles * sizeof(int), st));
   // mixed form: matvecs in FP32 until the wanted residual falls below
   // kMixedSwitch, FP64 from then on (monotone), so that the converged pairs
   // come from FP64 images; no convergence decision during the FP32 phase

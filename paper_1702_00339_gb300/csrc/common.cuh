@@ -282,7 +282,12 @@ struct GemmTask {
   int sym;                     // TN with a symmetric result: upper tiles computed, mirrored
   int tile;                    // TN output tile: 20 when the problem's block size is a multiple of 20, else 16
   int split;                   // 1: computed by k_split_gemm instead (mixed form)
+  int ksplit;                  // TN: ranges of the sum over n (gemm_tn_ksplit), by separate CTAs
+  double* part;                // (ksplit > 1) [ksplit][a * b] partial sums
+  int* count;                  // (ksplit > 1) arrivals per output tile, zero between launches
 };
+// ranges of a TN product's sum: at least 64 rows each, at most 32
+__host__ __device__ inline int gemm_tn_ksplit(int n) { return n < 128 ? 1 : (n / 64 < 32 ? n / 64 : 32); }
 
 struct ResidTask {
   const int* active;

@@ -48,37 +48,59 @@ __global__ void k_init_x(const InitTask* __restrict__ tasks) {
 
 
 
-// G = alpha A^T B (+ beta G), one output per thread of a 16 x 16 tile.  With
+// C = alpha A^T B + beta C on TILE x TILE output tiles, one thread per
+// output; TILE = 20 when the block sizes are multiples of 20 (less padding
+// than 16 for the 3k x 3k Gram and the k x k projections at k = 20).  With
 // T.sym the result is symmetric: tiles below the diagonal are skipped and the
 // tiles above also write their transposes (diagonal tiles are computed in
 // full and not mirrored, so no entry has two writers).
-#define TT 16
-// C = alpha A^T B + beta C on TILE x TILE output tiles, one thread per
-// output; TILE = 20 when the block sizes are multiples of 20 (less padding
-// than 16 for the 3k x 3k Gram and the k x k projections at k = 20).
+//
+// The sum over n is split over T.ksplit CTAs per tile (gemm_tn_ksplit: a property
+// of n, so results do not depend on the batch): a tile alone keeps one SM's FP64
+// pipe busy for TILE^2 n / 1.7 cycles, 60 us for the Gram matrices of a chain of
+// 512 functions, whose dozen tiles left the other SMs idle.  Each CTA leaves its
+// partial sums in T.part; the last one of a tile to arrive (a counter in global
+// memory that it resets) adds them in the order of the ranges.  Within a range
+// partial sums of 8 tiles' rows (128 or 160 terms) are added to the total, so
+// rounding grows like (8 TILE + n / (8 TILE)) u instead of n u (n = 16384 on the
+// 512-cell chains, where the Gram entries of nearly dependent directions decide
+// the pivots of the Rayleigh-Ritz step).  The next rows are loaded into registers
+// while the present ones are multiplied.  Measured, mean
+// of an iteration's launches: one chain of 512 functions 57 -> 18 us, 32 of them 91 ->
+// 65, three of 976 95 -> 26.
 template <int TILE>
-__global__ void __launch_bounds__(TILE * TILE) k_gemm_tn(const GemmTask* __restrict__ tasks) {
+__global__ void __launch_bounds__(TILE * TILE) k_gemm_tn(const GemmTask* __restrict__ tasks, int max_ks) {
   const GemmTask T = tasks[blockIdx.z];
+  const int ks = blockIdx.x % max_ks, bx = blockIdx.x / max_ks;
   if (T.split) return;                       // computed on the tensor cores (mixed form)
-  if (T.tile != TILE) return;                // the other tile size's launch
+  if (T.tile != TILE || ks >= T.ksplit) return;   // the other tile size's launch
   if (T.active && *T.active == 0) return;
-  const int i0 = blockIdx.x * TILE, j0 = blockIdx.y * TILE;
+  const int i0 = bx * TILE, j0 = blockIdx.y * TILE;
   if (i0 >= T.a || j0 >= T.b) return;
   if (T.sym && j0 < i0) return;
   __shared__ double As[TILE][TILE + 1], Bs[TILE][TILE + 1];
+  __shared__ int s_last;
   const int tx = threadIdx.x % TILE, ty = threadIdx.x / TILE;
-  // blocked summation: a partial sum over 8 tiles (128 or 160 terms) is added
-  // to the total, so the rounding error of a sum over n terms grows like
-  // (8 TILE + n / (8 TILE)) u instead of n u (n = 16384 on the 512-cell chains,
-  // where the Gram entries of nearly dependent directions decide the pivots of
-  // the Rayleigh-Ritz step)
+  // this CTA's range: whole tiles of rows
+  const int nt = (T.n + TILE - 1) / TILE;
+  const int t0 = (int)((long long)nt * ks / T.ksplit), t1 = (int)((long long)nt * (ks + 1) / T.ksplit);
+  const bool ain = i0 + ty < T.a, bin = j0 + ty < T.b;
+  const double* Ap = T.A + (size_t)T.lda * (i0 + ty) + tx;
+  const double* Bp = T.B + (size_t)T.ldb * (j0 + ty) + tx;
+  double an = 0.0, bn = 0.0;
+  auto fetch = [&](int t) {
+    const int r = t * TILE;
+    an = (ain && r + tx < T.n) ? Ap[r] : 0.0;
+    bn = (bin && r + tx < T.n) ? Bp[r] : 0.0;
+  };
   double acc = 0.0, blk = 0.0;
   int cnt = 0;
-  for (int n0 = 0; n0 < T.n; n0 += TILE) {
-    int r = n0 + tx;
-    As[ty][tx] = (r < T.n && i0 + ty < T.a) ? T.A[(size_t)r + (size_t)T.lda * (i0 + ty)] : 0.0;
-    Bs[ty][tx] = (r < T.n && j0 + ty < T.b) ? T.B[(size_t)r + (size_t)T.ldb * (j0 + ty)] : 0.0;
+  if (t0 < t1) fetch(t0);
+  for (int t = t0; t < t1; ++t) {
+    As[ty][tx] = an;
+    Bs[ty][tx] = bn;
     __syncthreads();
+    if (t + 1 < t1) fetch(t + 1);
 #pragma unroll
     for (int q = 0; q < TILE; ++q) blk = fma(As[tx][q], Bs[ty][q], blk);
     __syncthreads();
@@ -86,7 +108,25 @@ __global__ void __launch_bounds__(TILE * TILE) k_gemm_tn(const GemmTask* __restr
   }
   acc += blk;
   // thread (tx, ty) holds G[i0+tx][j0+ty]
-  if (i0 + tx < T.a && j0 + ty < T.b) {
+  const bool in = i0 + tx < T.a && j0 + ty < T.b;
+  if (T.ksplit > 1) {
+    const size_t pl = (size_t)T.a * T.b, o = (size_t)(i0 + tx) + (size_t)T.a * (j0 + ty);
+    if (in) T.part[pl * ks + o] = acc;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int* c = T.count + blockIdx.y * ((T.a + TILE - 1) / TILE) + bx;
+      s_last = (atomicAdd(c, 1) == T.ksplit - 1);
+      if (s_last) *c = 0;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    acc = 0.0;
+    if (in)
+      for (int q = 0; q < T.ksplit; ++q) acc += __ldcg(T.part + pl * q + o);
+  }
+  if (in) {
     double* g = T.C + (size_t)(i0 + tx) + (size_t)T.ldc * (j0 + ty);
     const double v = (T.beta == 0.0) ? T.alpha * acc : T.beta * *g + T.alpha * acc;
     *g = v;
@@ -96,39 +136,50 @@ __global__ void __launch_bounds__(TILE * TILE) k_gemm_tn(const GemmTask* __restr
 
 // amax, bmax: largest output dimensions; tiles: bit 0 = some task uses 16,
 // bit 1 = some task uses 20 (one launch per tile size, each skipping the
-// other's tasks, so a problem's products never depend on its batch)
-void launch_gemm_tn(const GemmTask* t, int n, int amax, int bmax, int tiles, cudaStream_t st) {
+// other's tasks, so a problem's products never depend on its batch); ks: the
+// largest split of the sum
+void launch_gemm_tn(const GemmTask* t, int n, int amax, int bmax, int tiles, int ks, cudaStream_t st) {
   if (!n) return;
-  if (tiles & 1) k_gemm_tn<16><<<dim3((amax + 15) / 16, (bmax + 15) / 16, n), 256, 0, st>>>(t);
-  if (tiles & 2) k_gemm_tn<20><<<dim3((amax + 19) / 20, (bmax + 19) / 20, n), 400, 0, st>>>(t);
+  if (tiles & 1) k_gemm_tn<16><<<dim3((amax + 15) / 16 * ks, (bmax + 15) / 16, n), 256, 0, st>>>(t, ks);
+  if (tiles & 2) k_gemm_tn<20><<<dim3((amax + 19) / 20 * ks, (bmax + 19) / 20, n), 400, 0, st>>>(t, ks);
 }
 
 // C = alpha A B + beta C; a thread owns row i of four consecutive columns,
-// so each load of A serves four FP64 FMAs.
-__global__ void k_gemm_nn(const GemmTask* __restrict__ tasks) {
+// so each load of A serves four FP64 FMAs -- or of one column where the product
+// is too small to fill the GPU that way (64 CTAs of 256 threads): 512 x 40 outputs
+// of a chain of 512 functions, mean of an iteration's launches 19 us -> 10.  The
+// same sum either way.
+template <int NC>
+__device__ __forceinline__ void gemm_nn_cols(const GemmTask& T) {
+  const int nbc = (T.b + NC - 1) / NC;
+  const int tot = T.n * nbc;
+  for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < tot; it += gridDim.x * blockDim.x) {
+    const int i = it % T.n, j0 = (it / T.n) * NC;
+    const int nj = min(NC, T.b - j0);
+    const double* b[NC];
+    double acc[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) { b[c] = T.B + (size_t)T.ldb * (j0 + (c < nj ? c : 0)); acc[c] = 0.0; }
+#pragma unroll 4
+    for (int q = 0; q < T.a; ++q) {
+      const double x = T.A[(size_t)i + (size_t)T.lda * q];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[c] = fma(x, b[c][q], acc[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+      if (c < nj) {
+        double* cp = T.C + (size_t)i + (size_t)T.ldc * (j0 + c);
+        *cp = (T.beta == 0.0) ? T.alpha * acc[c] : T.beta * *cp + T.alpha * acc[c];
+      }
+  }
+}
+__global__ void __launch_bounds__(256) k_gemm_nn(const GemmTask* __restrict__ tasks) {
   const GemmTask T = tasks[blockIdx.y];
   if (T.split) return;                       // computed on the tensor cores (mixed form)
   if (T.active && *T.active == 0) return;
-  const int nb4 = (T.b + 3) >> 2;
-  const int tot = T.n * nb4;
-  for (int it = blockIdx.x * blockDim.x + threadIdx.x; it < tot; it += gridDim.x * blockDim.x) {
-    const int i = it % T.n, j0 = (it / T.n) * 4;
-    const int nj = min(4, T.b - j0);
-    const double* b0 = T.B + (size_t)T.ldb * j0;
-    const double* b1 = b0 + (nj > 1 ? T.ldb : 0);
-    const double* b2 = b0 + (nj > 2 ? 2 * (size_t)T.ldb : 0);
-    const double* b3 = b0 + (nj > 3 ? 3 * (size_t)T.ldb : 0);
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    for (int q = 0; q < T.a; ++q) {
-      const double x = T.A[(size_t)i + (size_t)T.lda * q];
-      a0 = fma(x, b0[q], a0); a1 = fma(x, b1[q], a1); a2 = fma(x, b2[q], a2); a3 = fma(x, b3[q], a3);
-    }
-    const double acc[4] = {a0, a1, a2, a3};
-    for (int c = 0; c < nj; ++c) {
-      double* cp = T.C + (size_t)i + (size_t)T.ldc * (j0 + c);
-      *cp = (T.beta == 0.0) ? T.alpha * acc[c] : T.beta * *cp + T.alpha * acc[c];
-    }
-  }
+  if ((long long)T.n * T.b <= (long long)gridDim.x * blockDim.x * 2) gemm_nn_cols<1>(T);
+  else gemm_nn_cols<4>(T);
 }
 
 // Columns at or below lock_tol get R = 0 (soft locking).
