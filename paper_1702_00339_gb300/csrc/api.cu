@@ -38,7 +38,7 @@ namespace fock {
 
 // launchers (defined in the .cu files)
 void launch_vec1d(const ProbDev*, const SegDesc*, int, const SegDesc*, int, const DefTab*, int, int, int, cudaStream_t);
-void launch_gram(const ProbDev*, const GramTask*, int, const DefTab*, cudaStream_t);
+void launch_gram(const ProbDev*, const GramTask*, int, const DefTab*, int, cudaStream_t);
 void launch_combine(const ProbDev*, const CombineTask*, int, cudaStream_t);
 void launch_defects(const ProbDev*, const DefField*, int, const DefBlock*, int, cudaStream_t);
 void launch_axis_dft(const ProbDev*, const DftTask*, int, int, cudaStream_t);
@@ -1382,7 +1382,7 @@ void run_assemble(fock_ctx* ctx, Batch& B) {
   cudaStream_t st = ctx->stream;
   { PROF("k_vec1d", 2); launch_vec1d(B.d_probs, B.d_gsegs, (int)B.gsegs.size(), B.d_psegs, (int)B.psegs.size(),
                                      B.d_dtabs, (int)B.dtabs.size(), B.ptab_maxT, B.ptab_maxni, st); }
-  { PROF("k_gram", 2); launch_gram(B.d_probs, B.d_gram, (int)B.gram.size(), B.d_dtabs, st); }
+  { PROF("k_gram", 2); launch_gram(B.d_probs, B.d_gram, (int)B.gram.size(), B.d_dtabs, B.ptab_maxT * B.maxm0 * B.maxm0, st); }
   if (!B.splits.empty()) {
     cudaMemsetAsync(B.d_split_err, 0, sizeof(int), st);
     PROF("k_split_gemm", 1);

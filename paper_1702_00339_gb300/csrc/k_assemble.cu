@@ -18,6 +18,8 @@
 //             writes its transpose into the mirror entry (E(m,k) = E(k,m)^T).
 //  k_axis_dft sparse DFT of the per-axis factors over the lattice offset
 //             (Thm. 3.3: only 1D transforms of the factors are needed).
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace fock {
@@ -177,7 +179,8 @@ __global__ void k_deftab(const ProbDev* __restrict__ probs, const DefTab* __rest
 // ---------------------------------------------------------------- K2 ----
 __device__ inline double gval(const AxisDev& A, int mode, int n0, int mu, int cell, int rho) {
   if (mode == RING) {
-    int j = posmod(rho - cell * n0, A.N);
+    int j = rho - cell * n0;
+    if ((unsigned)j >= (unsigned)A.N) j = posmod(j, A.N);   // (no division for most nodes)
     return A.g[mu * A.W + j];
   }
   if (mode == WALL && (rho < -A.pad || rho >= A.N - A.pad)) return 0.0;
@@ -186,15 +189,60 @@ __device__ inline double gval(const AxisDev& A, int mode, int n0, int mu, int ce
   return A.g[mu * A.W + j];
 }
 
-// One CTA per task: folded pair products Z[r][mu nu] and the S1 / A1 forms.
-__global__ void k_gram_fold(const ProbDev* __restrict__ probs, const GramTask* __restrict__ tasks) {
+// Folded pair products Z[r][mu nu] (shared out over blockIdx.y) and the S1 / A1
+// forms (the last blockIdx.y: lanes over an entry's nodes).  Both gram
+// kernels were one CTA per task with a thread summing each form's nodes in turn,
+// latency from end to end: 237 us for a ring of 8 cells of 4 functions (9 axis
+// forms over up to 256 nodes), 1.1 ms for a chain of 101 cells of 16; now
+// 35 us and 0.23 ms (4600 tasks of 32 chains and rings of 64 cells: 1.40 -> 1.25).
+__global__ void __launch_bounds__(256) k_gram_fold(const ProbDev* __restrict__ probs, const GramTask* __restrict__ tasks) {
   const GramTask T = tasks[blockIdx.x];
   const ProbDev& P = probs[T.prob];
   const AxisDev& A = P.ax[T.axis];
   const int m0 = P.m0, n0 = P.n0, np = m0 * m0;
   const bool direct = (T.ptab >= 0);      // defect tables: no replication
-  const int tot = T.nfold * np;
-  for (int it = threadIdx.x; it < tot; it += blockDim.x) {
+  if (blockIdx.y + 1 == gridDim.y) {
+    if (direct) return;   // defect forms carry no mass / stiffness part
+    // 8 lanes per entry (32 where entries are few) over the nodes of g_mu's own
+    // support (the others add zeros)
+    const bool ring_sup = (T.mode == RING && A.slen < A.N);
+    const int lo0 = ring_sup ? A.smin : T.rho0 - T.a * n0, len = ring_sup ? A.slen : T.rho1 - T.rho0;   // from cell a's origin
+    __shared__ float s_log;
+    if (threadIdx.x == 0) s_log = (float)log(1.0 / P.eps);
+    __syncthreads();
+    const int LN = (np <= 16) ? 32 : 8, o = threadIdx.x & (LN - 1);
+    for (int p0 = 0; p0 < np; p0 += blockDim.x / LN) {
+      const int pr = p0 + threadIdx.x / LN, mu = min(pr, np - 1) / m0, nu = pr % m0;
+      double s = 0.0, a = 0.0;
+      int t0 = 0, t1 = len;
+      if (T.mode != RING || ring_sup) {
+        const float c = (float)(P.frac[P.centre[mu] * 3 + T.axis] * (double)n0) - 0.5f;
+        const float reach = sqrtf(s_log / (float)P.alpha[mu]) / (float)P.h * 1.0001f + 1.0f;   // a node to spare
+        t0 = max(t0, (int)floorf(c - reach) - lo0);
+        t1 = min(t1, (int)ceilf(c + reach) + 1 - lo0);
+      }
+      if (pr < np)
+        for (int t = t0 + o; t < t1; t += LN) {
+          const int rho = ring_sup ? posmod(T.a * n0 + A.smin + t, A.N) : T.rho0 + t;
+          const double ga = gval(A, T.mode, n0, mu, T.a, rho);
+          const double b0 = gval(A, T.mode, n0, nu, T.b, rho);
+          const double b1 = gval(A, T.mode, n0, nu, T.b, rho - 1) + gval(A, T.mode, n0, nu, T.b, rho + 1);
+          s = fma(ga, fma(4.0, b0, b1), s);
+          a = fma(ga, fma(2.0, b0, -b1), a);
+        }
+      for (int x = 1; x < LN; x <<= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, x);
+        a += __shfl_xor_sync(0xffffffffu, a, x);
+      }
+      if (o == 0 && pr < np) {
+        T.X[0 * np + pr] = s * (P.h / 6.0);
+        T.X[1 * np + pr] = a / P.h;
+      }
+    }
+    return;
+  }
+  const int tot = T.nfold * np, nth = blockDim.x * (gridDim.y - 1);
+  for (int it = blockIdx.y * blockDim.x + threadIdx.x; it < tot; it += nth) {
     int rr = it / np, pr = it % np, mu = pr / m0, nu = pr % m0;
     int r = T.foldlo + rr;
     double acc = 0.0;
@@ -233,31 +281,15 @@ __global__ void k_gram_fold(const ProbDev* __restrict__ probs, const GramTask* _
     }
     T.Zs[it] = acc;
   }
-  if (direct) return;   // defect forms carry no mass / stiffness part
-  // RING: only the nodes of the support of g_mu(cell a) (the others add zeros)
-  const bool ring_sup = (T.mode == RING && A.slen < A.N);
-  const int nrho = ring_sup ? A.slen : T.rho1 - T.rho0;
-  for (int pr = threadIdx.x; pr < np; pr += blockDim.x) {
-    int mu = pr / m0, nu = pr % m0;
-    double s = 0.0, a = 0.0;
-    for (int t = 0; t < nrho; ++t) {
-      const int rho = ring_sup ? posmod(T.a * n0 + A.smin + t, A.N) : T.rho0 + t;
-      double ga = gval(A, T.mode, n0, mu, T.a, rho);
-      if (ga == 0.0) continue;
-      double b0 = gval(A, T.mode, n0, nu, T.b, rho);
-      double bm = gval(A, T.mode, n0, nu, T.b, rho - 1);
-      double bp = gval(A, T.mode, n0, nu, T.b, rho + 1);
-      s += ga * (4.0 * b0 + bm + bp);
-      a += ga * (2.0 * b0 - bm - bp);
-    }
-    T.X[0 * np + pr] = s * (P.h / 6.0);
-    T.X[1 * np + pr] = a / P.h;
-  }
 }
 
-// One CTA per task: X_t[mu nu] = sum_r P_t[r] Z[r][mu nu].
-__global__ void k_gram_pot(const ProbDev* __restrict__ probs, const GramTask* __restrict__ tasks,
-                           const DefTab* __restrict__ dtabs) {
+// X_t[mu nu] = sum_r P_t[r] Z[r][mu nu].  A CTA takes 64 of the task's outputs
+// (t, mu nu), four threads each: their sums over every fourth node, in registers,
+// added through shared memory; short sums (folded nodes) take a thread each, and
+// so do all, with the same four partial sums, where tasks alone fill the GPU
+// (spread = 0).
+__global__ void __launch_bounds__(256) k_gram_pot(const ProbDev* __restrict__ probs, const GramTask* __restrict__ tasks,
+                                                  const DefTab* __restrict__ dtabs, int spread) {
   const GramTask T = tasks[blockIdx.x];
   if (T.split) return;   // mixed form: contracted by k_split_gemm
   const ProbDev& P = probs[T.prob];
@@ -269,12 +301,39 @@ __global__ void k_gram_pot(const ProbDev* __restrict__ probs, const GramTask* __
   const int ld = direct ? dtabs[T.ptab].N : A.nr;
   const int off = direct ? (T.foldlo + dtabs[T.ptab].pad) : (T.foldlo - A.rlo);
   double* out = T.X + (direct ? 0 : 2 * np);
-  for (int it = threadIdx.x; it < nt * np; it += blockDim.x) {
-    int t = it / np, pr = it % np;
-    const double* pt = tab + (size_t)t * ld + off;
+  if (T.nfold <= 32 || !spread) {
+    for (int it = blockIdx.y * blockDim.x + threadIdx.x; it < nt * np; it += gridDim.y * blockDim.x) {
+      const double* pt = tab + (size_t)(it / np) * ld + off;
+      const double* z = T.Zs + it % np;
+      double acc[4] = {0.0, 0.0, 0.0, 0.0};
+      if (T.nfold <= 32) {
+        for (int rr = 0; rr < T.nfold; ++rr) acc[0] += pt[rr] * z[(size_t)rr * np];
+      } else {
+        for (int r0 = 0; r0 < T.nfold; r0 += 4)
+#pragma unroll
+          for (int g = 0; g < 4; ++g)
+            if (r0 + g < T.nfold) acc[g] += pt[r0 + g] * z[(size_t)(r0 + g) * np];
+        acc[0] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+      }
+      out[it] = acc[0];
+    }
+    return;
+  }
+  __shared__ double part[3][64];
+  const int o = threadIdx.x & 63, g = threadIdx.x >> 6, tot = nt * np;
+  for (int i0 = blockIdx.y * 64; i0 < tot; i0 += gridDim.y * 64) {
+    const int it = i0 + o;
     double acc = 0.0;
-    for (int rr = 0; rr < T.nfold; ++rr) acc += pt[rr] * T.Zs[(size_t)rr * np + pr];
-    out[(size_t)t * np + pr] = acc;
+    if (it < tot) {
+      const double* pt = tab + (size_t)(it / np) * ld + off;
+      const double* z = T.Zs + it % np;
+#pragma unroll 4
+      for (int rr = g; rr < T.nfold; rr += 4) acc += pt[rr] * z[(size_t)rr * np];
+    }
+    if (g) part[g - 1][o] = acc;
+    __syncthreads();
+    if (g == 0 && it < tot) out[it] = (acc + part[0][o]) + (part[1][o] + part[2][o]);
+    __syncthreads();
   }
 }
 
@@ -419,11 +478,15 @@ void launch_vec1d(const ProbDev* probs, const SegDesc* gsegs, int ngseg, const S
   if (ndtab) k_deftab<<<dim3(8, ndtab), 256, 0, st>>>(probs, dtabs);
 }
 
-void launch_gram(const ProbDev* probs, const GramTask* tasks, int ntask, const DefTab* dtabs,
+// maxout: the largest number of outputs (terms x m0^2) of a task
+void launch_gram(const ProbDev* probs, const GramTask* tasks, int ntask, const DefTab* dtabs, int maxout,
                  cudaStream_t st) {
   if (!ntask) return;
-  k_gram_fold<<<ntask, 256, 0, st>>>(probs, tasks);
-  k_gram_pot<<<ntask, 256, 0, st>>>(probs, tasks, dtabs);
+  // CTAs per task: the fold and the contraction spread while tasks alone do not
+  // fill the GPU
+  const int room = std::max(1, 2048 / ntask);
+  k_gram_fold<<<dim3(ntask, 1 + std::min(8, room)), 256, 0, st>>>(probs, tasks);
+  k_gram_pot<<<dim3(ntask, std::min(room, (maxout + 63) / 64)), 256, 0, st>>>(probs, tasks, dtabs, room >= 8);
 }
 
 void launch_combine(const ProbDev* probs, const CombineTask* tasks, int n, cudaStream_t st) {
