@@ -42,6 +42,8 @@ void launch_gram(const ProbDev*, const GramTask*, int, const DefTab*, int, cudaS
 void launch_combine(const ProbDev*, const CombineTask*, int, cudaStream_t);
 void launch_defects(const ProbDev*, const DefField*, int, const DefBlock*, int, cudaStream_t);
 void launch_axis_dft(const ProbDev*, const DftTask*, int, int, cudaStream_t);
+size_t pf_layout(char*, int, size_t, PfWork*);
+void launch_pf(const ProbDev*, const PfTask*, const PfGroup*, int, const PfWork&, cudaStream_t);
 void launch_fblocks(const ProbDev*, const FBlockTask*, int, int, int, cudaStream_t, bool vectors = false,
                     int x0 = 0, int nx = -1, bool any_odd = true);
 void launch_bloch_vectors(int, int, int, int, int, const int*, const cplx*, const int*, cplx*, cudaStream_t);
@@ -146,10 +148,14 @@ const double kPrecShift = 2e-5;   // sigma = min_j lambda_min(Chat_j) - kPrecShi
 // batch of 64 chains of 512 functions, 0.84 vs 1.66 s for one of 16384)
 const int kSplitMinRows = 2048;
 const int kGemmTiles = 256;   // output tiles of a TN product: at most (255 / 16 + 1)^2
-// Fourier blocks (CTAs, of which about half are conjugates that return at
-// once) per piece launched beside a Rayleigh-Ritz launch: about three waves of
-// the 32 x 32 block kernel on the SMs the iteration leaves free, ~10 ms
-const int kPeriodicPieceCTAs = 3072;
+// Fourier blocks (conjugate pairs once) per piece launched beside a Rayleigh-Ritz
+// launch: a few milliseconds of 32 x 32 blocks on the SMs the iteration leaves free
+const int kPeriodicPiece = 1024;
+// bound of the workspace of the periodic spectra's chunks (55 KB a block of order 32):
+// the kernels that give a block one thread take as long for a block as for 19 000 (a
+// lattice of 32^3 cells of 32 functions: the call takes 55 ms with 256 MB, 45 with 1 GB). A plan that would not fit its budget otherwise takes the least, 32 blocks at
+// a time; the chunks do not change a result.
+const size_t kPfWorkBytes = (size_t)1 << 30;
 
 int set_err(fock_ctx* c, int code, const std::string& m) {
   if (c) c->err = m;
@@ -299,6 +305,35 @@ uint64_t problem_seed(const HostProb& H) {
   return h;
 }
 
+// Representatives of the Fourier indices j0 .. j0 + nj - 1 of an L1 x L2 x L3 lattice,
+// as local indices: with real generators the block at -j (componentwise mod L) is the
+// conjugate of the block at j, with the same spectrum; where the range holds both,
+// the lower index stands for the pair.
+std::vector<int> pf_reps(const int* L, int j0, int nj) {
+  std::vector<int> rep;
+  rep.reserve(nj / 2 + 8);
+  int j3 = j0 % L[2], j2 = (j0 / L[2]) % L[1], j1 = j0 / (L[1] * L[2]);
+  for (int j = j0; j < j0 + nj; ++j) {
+    const int jm = ((j1 ? L[0] - j1 : 0) * L[1] + (j2 ? L[1] - j2 : 0)) * L[2] + (j3 ? L[2] - j3 : 0);
+    if (jm >= j || jm < j0) rep.push_back(j - j0);
+    if (++j3 == L[2]) {
+      j3 = 0;
+      if (++j2 == L[1]) { j2 = 0; ++j1; }
+    }
+  }
+  return rep;
+}
+
+// their groups, appended
+void pf_groups(int task, int nrep, std::vector<PfGroup>& out) {
+  for (int r = 0; r < nrep; r += kPfGroup) out.push_back({task, r});
+}
+
+// workspace for ng groups of blocks of order m, in whole 32 slots
+size_t pf_bytes_for(int m, size_t ng) {
+  return (ng * kPfGroup + 31) / 32 * pf_layout(nullptr, m, 32, nullptr);
+}
+
 inline int posmod_h(int a, int b) { int r = a % b; return r < 0 ? r + b : r; }
 
 // smallest 2^a 3^b 5^c >= n
@@ -406,7 +441,11 @@ struct Batch {
   std::vector<DefField> dfields; DefField* d_dfields = nullptr;
   std::vector<DefBlock> dblocks; DefBlock* d_dblocks = nullptr;
   std::vector<DftTask> dft; DftTask* d_dft = nullptr; int maxLdft = 1;
-  std::vector<FBlockTask> fbp, fbs; FBlockTask *d_fbp = nullptr, *d_fbs = nullptr;
+  std::vector<PfTask> pft; PfTask* d_pft = nullptr;
+  std::vector<PfGroup> pfg; PfGroup* d_pfg = nullptr;   // largest blocks first
+  size_t pf_limit = kPfWorkBytes;    // bound of the workspace below
+  char* pf_work = nullptr; size_t pf_bytes = 0;   // chunk workspace of the periodic spectra
+  std::vector<FBlockTask> fbp, fbs; FBlockTask* d_fbs = nullptr;   // fbp: templates of the vector solves
   std::vector<NullTask> nulls; NullTask* d_nulls = nullptr;   // dependency cut of each periodic problem
   int maxnj_p = 0, maxnj_s = 0, maxm0 = 1;
   std::vector<PrecTask> prec; PrecTask* d_prec = nullptr; int maxM = 0;
@@ -509,7 +548,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
   B.pp.assign(np, Batch::PerProb());
   B.gsegs.clear(); B.psegs.clear(); B.gram.clear(); B.combT.clear(); B.combE.clear();
   B.dtabs.clear(); B.dfields.clear(); B.dblocks.clear();
-  B.dft.clear(); B.fbp.clear(); B.fbs.clear(); B.nulls.clear(); B.prec.clear(); B.canon.clear(); B.fbo.clear(); B.maxcblk = 0; B.sorts.clear(); B.bigsort.clear();
+  B.dft.clear(); B.fbp.clear(); B.pft.clear(); B.pfg.clear(); B.fbs.clear(); B.nulls.clear(); B.prec.clear(); B.canon.clear(); B.fbo.clear(); B.maxcblk = 0; B.sorts.clear(); B.bigsort.clear();
   B.circs.clear(); B.lob.clear(); B.sidx.clear(); B.mv_off.clear();
   B.maxnj_p = B.maxnj_s = 0; B.maxm0 = 1; B.maxM = 0; B.maxsort = 0; B.kmax = 0; B.maxLdft = 1;
   B.odd_m0 = false;
@@ -803,6 +842,15 @@ void plan(Batch& B, Slab& S, Slab& U) {
       f.tau = nt.tau;
       B.nulls.push_back(nt);
       B.fbp.push_back(f);
+      PfTask pt;
+      std::memset(&pt, 0, sizeof(pt));
+      pt.prob = i; pt.nj = ncell;
+      for (int a = 0; a < 3; ++a) { pt.L[a] = H.L[a]; pt.Xh[a] = Q.Xh[a]; }
+      const std::vector<int> reps = pf_reps(H.L, 0, ncell);
+      pt.nrep = (int)reps.size();
+      pt.rep = U.put(reps);
+      pt.ev = Q.ev; pt.blk = Q.blk; pt.tau = f.tau; pt.neig = f.neig;
+      B.pft.push_back(pt);
       B.maxnj_p = std::max(B.maxnj_p, ncell);
       if (Q.nev <= kSmallSort) {
         B.sorts.push_back({Q.nev, Q.ev, Q.blk});
@@ -967,6 +1015,22 @@ void plan(Batch& B, Slab& S, Slab& U) {
       B.sidx.push_back(i);
       B.kmax = std::max(B.kmax, lobpcg_block(H.k_eig, Q.Lc * H.m0));
     }
+  }
+  // ---- groups and chunk workspace of the periodic spectra ----
+  if (!B.pft.empty()) {
+    std::vector<int> by(B.pft.size());
+    for (size_t i = 0; i < by.size(); ++i) by[i] = (int)i;
+    std::stable_sort(by.begin(), by.end(),
+                     [&](int a, int b) { return B.hp[B.pft[a].prob].m0 > B.hp[B.pft[b].prob].m0; });
+    size_t own = 0;   // what the problems take one by one
+    for (int t : by) {
+      const size_t n0 = B.pfg.size();
+      pf_groups(t, B.pft[t].nrep, B.pfg);
+      own += pf_bytes_for(B.hp[B.pft[t].prob].m0, B.pfg.size() - n0);
+    }
+    const size_t least = pf_bytes_for(B.hp[B.pft[by[0]].prob].m0, 1);
+    B.pf_bytes = std::max(least, std::min(own, B.pf_limit));
+    B.pf_work = S.take<char>(B.pf_bytes);
   }
   // ---- LOBPCG state ----
   size_t mv_total = 0;
@@ -1268,7 +1332,8 @@ void plan(Batch& B, Slab& S, Slab& U) {
   B.d_dfields = U.put(B.dfields);
   B.d_dblocks = U.put(B.dblocks);
   B.d_dft = U.put(B.dft);
-  B.d_fbp = U.put(B.fbp);
+  B.d_pft = U.put(B.pft);
+  B.d_pfg = U.put(B.pfg);
   B.d_fbs = U.put(B.fbs);
   B.d_nulls = U.put(B.nulls);
   B.d_prec = U.put(B.prec);
@@ -1315,6 +1380,11 @@ namespace {
 int alloc_and_plan(fock_ctx* ctx, Batch& B, bool own) {
   Slab S0, U0;
   plan(B, S0, U0);
+  if (ctx->budget && S0.off + U0.off + 512 > ctx->budget && !B.pft.empty()) {
+    B.pf_limit = 0;
+    S0 = Slab(); U0 = Slab();
+    plan(B, S0, U0);
+  }
   size_t need = S0.off + 256, uneed = U0.off + 256;
   if (ctx->budget && need + uneed > ctx->budget)
     return set_err(ctx, FOCK_ENOMEM, "batch needs " + std::to_string(need + uneed) + " bytes, budget " +
@@ -1412,13 +1482,26 @@ void run_periodic_head(fock_ctx* ctx, Batch& B, cudaStream_t st) {
   { PROF("k_axis_dft", 1); launch_axis_dft(B.d_probs, B.d_dft, (int)B.dft.size(), B.maxLdft, st); }
   { PROF("k_null_tau", 1); launch_null_tau(B.d_nulls, (int)B.nulls.size(), st); }
 }
-// the next nx local indices of every periodic task (nx < 0: all that remain)
-void run_periodic_piece(fock_ctx* ctx, Batch& B, int nx, cudaStream_t st) {
-  if (B.fbp.empty() || B.pchunk_next >= B.maxnj_p) return;
-  const int w = (nx < 0) ? B.maxnj_p - B.pchunk_next : std::min(nx, B.maxnj_p - B.pchunk_next);
+// the spectra of the groups g[0 .. n) on the host and dg[0 .. n) on the device, in chunks
+// of the workspace, each laid out for its first group's blocks (the largest)
+void run_pf(Batch& B, const PfTask* tasks, const PfGroup* g, const PfGroup* dg, int n, char* work, size_t bytes,
+            cudaStream_t st) {
+  for (int i = 0; i < n;) {
+    const int m = B.hp[B.pft[g[i].task].prob].m0;
+    const size_t fit = bytes / pf_bytes_for(m, 1) * (32 / kPfGroup);
+    const int c = (int)std::min<size_t>(n - i, std::max<size_t>(fit, 32 / kPfGroup));
+    PfWork W;
+    pf_layout(work, m, (size_t)c * kPfGroup, &W);
+    launch_pf(B.d_probs, tasks, dg + i, c, W, st);
+    i += c;
+  }
+}
+// the next n groups of the periodic spectra (n < 0: all that remain)
+void run_periodic_piece(fock_ctx* ctx, Batch& B, int n, cudaStream_t st) {
+  const int left = (int)B.pfg.size() - B.pchunk_next, w = (n < 0) ? left : std::min(n, left);
+  if (w <= 0) return;
   { PROF("k_fblocks_eig", 1);
-    launch_fblocks(B.d_probs, B.d_fbp, (int)B.fbp.size(), B.maxnj_p, B.maxm0, st, false, B.pchunk_next, w,
-                   B.odd_m0); }
+    run_pf(B, B.d_pft, B.pfg.data() + B.pchunk_next, B.d_pfg + B.pchunk_next, w, B.pf_work, B.pf_bytes, st); }
   B.pchunk_next += w;
 }
 void run_periodic_tail(fock_ctx* ctx, Batch& B, cudaStream_t st) {
@@ -1733,7 +1816,7 @@ int run_lobpcg(fock_ctx* ctx, Batch& B, double tol, int maxit, std::vector<int>&
     // (lower-priority) stream, started when this stream reaches the
     // Rayleigh-Ritz launch, which occupies one SM per box chain: the piece fills
     // the other SMs meanwhile and is sized to end about when it does
-    if (ctx->pstream && B.pchunk_next < B.maxnj_p) {
+    if (ctx->pstream && B.pchunk_next < (int)B.pfg.size()) {
       CUDA_TRY(ctx, cudaEventRecord(ctx->ev_chunk, st));
       CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->pstream, ctx->ev_chunk, 0));
       run_periodic_piece(ctx, B, B.pchunk_w, ctx->pstream);
@@ -1783,9 +1866,9 @@ int plan_execute(fock_plan& P, double tol, int maxit) {
     CUDA_TRY(ctx, cudaEventRecord(ctx->ev_fork, user));
     CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->hi, ctx->ev_fork, 0));
     run_periodic_head(ctx, B, user);
-    // pieces of about kPeriodicPieceCTAs Fourier blocks ride along with the
+    // pieces of about kPeriodicPiece Fourier blocks ride along with the
     // iteration's Rayleigh-Ritz launches; the rest, and the sorts, follow it
-    B.pchunk_w = std::max(1, kPeriodicPieceCTAs / std::max(1, (int)B.fbp.size()));
+    B.pchunk_w = kPeriodicPiece / kPfGroup;
     ctx->pstream = user;
     ctx->stream = ctx->hi;
     run_struct_setup(ctx, B);
@@ -1909,7 +1992,7 @@ void set_ctx_error(fock_ctx* c, const char* msg) { if (c) c->err = msg; }
 // with host outputs.
 namespace fock {
 
-int detail_estimate(const fock_problem& p, size_t* bytes, int* n_evals, std::string& why) {
+int detail_estimate(const fock_problem& p, size_t budget, size_t* bytes, int* n_evals, std::string& why) {
   Batch B;
   B.nprob = 1;
   B.hp.assign(1, HostProb());
@@ -1917,9 +2000,13 @@ int detail_estimate(const fock_problem& p, size_t* bytes, int* n_evals, std::str
   int rc = validate(p, B.hp[0], why);
   if (rc) return rc;
   for (int a = 0; a < 3; ++a) axis_plan(B.hp[0], a, B.ap[a]);
-  Slab S0, U0;
-  plan(B, S0, U0);
-  *bytes = S0.off + U0.off + 512;
+  for (;;) {
+    Slab S0, U0;
+    plan(B, S0, U0);
+    *bytes = S0.off + U0.off + 512;
+    if (*bytes <= budget || B.pft.empty() || !B.pf_limit) break;
+    B.pf_limit = 0;   // as the plan of a batch that does not fit does
+  }
   *n_evals = B.pp[0].nev;
   return FOCK_OK;
 }
@@ -2388,19 +2475,41 @@ int periodic_range(fock_ctx* ctx, Batch& B, int j0, int j1, double* evals, int* 
   const size_t off_pv = off_blk + (((size_t)n * 4 + 255) & ~(size_t)255);
   const size_t off_pi = off_pv + (size_t)n2 * 8;
   const size_t off_t = (off_pi + (size_t)n2 * 4 + 255) & ~(size_t)255;
-  const size_t off_v = (off_t + sizeof(FBlockTask) + 255) & ~(size_t)255;
+  // eigenvalues by the chunked pipeline, on the representatives of the range
+  const std::vector<int> reps = pf_reps(H.L, j0, nj);
+  const size_t off_r = (off_t + sizeof(FBlockTask) + sizeof(PfTask) + 255) & ~(size_t)255;
+  std::vector<PfGroup> groups;
+  pf_groups(0, (int)reps.size(), groups);
+  const size_t off_g = (off_r + reps.size() * sizeof(int) + 255) & ~(size_t)255;
+  const size_t off_v = (off_g + groups.size() * sizeof(PfGroup) + 255) & ~(size_t)255;
   const size_t vbytes = vecs ? (size_t)n * H.m0 * sizeof(cplx) : 0;
-  CUDA_TRY(ctx, cudaMalloc(&mem, off_v + vbytes));
+  const size_t off_w = (off_v + vbytes + 255) & ~(size_t)255, least = pf_bytes_for(H.m0, 1);
+  size_t wbytes = std::max(least, std::min(kPfWorkBytes, pf_bytes_for(H.m0, groups.size())));
+  if (cudaMalloc(&mem, off_w + wbytes) != cudaSuccess) {
+    cudaGetLastError();
+    wbytes = least;
+    CUDA_TRY(ctx, cudaMalloc(&mem, off_w + wbytes));
+  }
   double* ev = (double*)mem;
   int* blk = (int*)(mem + off_blk);
   FBlockTask f = B.fbp[0];
-  f.j0 = j0; f.nj = nj; f.outH = nullptr; f.outS = nullptr; f.want = 1; f.ev = ev; f.blk = blk; f.fail = nullptr;
+  f.j0 = j0; f.nj = nj; f.outH = nullptr; f.outS = nullptr; f.want = 1; f.ev = nullptr; f.blk = nullptr; f.fail = nullptr;
   f.vecs = vecs ? (cplx*)(mem + off_v) : nullptr;
   int rc = FOCK_OK;
+  PfTask pt = B.pft[0];
+  pt.j0 = j0; pt.nj = nj; pt.nrep = (int)reps.size(); pt.rep = (const int*)(mem + off_r);
+  pt.ev = ev; pt.blk = blk; pt.neig = nullptr;
+  char* const dpt = mem + off_t + sizeof(FBlockTask);
   cudaError_t e = cudaMemcpyAsync(mem + off_t, &f, sizeof(f), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(dpt, &pt, sizeof(pt), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(mem + off_r, reps.data(), reps.size() * sizeof(int), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(mem + off_g, groups.data(), groups.size() * sizeof(PfGroup), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
     { PROF("k_fblocks_eig", 1);
-      launch_fblocks(B.d_probs, (const FBlockTask*)(mem + off_t), 1, nj, H.m0, st, vecs != nullptr); }
+      if (vecs) launch_fblocks(B.d_probs, (const FBlockTask*)(mem + off_t), 1, nj, H.m0, st, true);
+      run_pf(B, (const PfTask*)dpt, groups.data(), (const PfGroup*)(mem + off_g), (int)groups.size(), mem + off_w, wbytes, st); }
     { PROF("k_sort_global", 1); launch_sort_global(ev, blk, n, (double*)(mem + off_pv), (int*)(mem + off_pi), st); }
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(evals, ev, (size_t)n * 8, cudaMemcpyDeviceToHost, st);

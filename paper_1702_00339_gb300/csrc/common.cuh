@@ -201,7 +201,7 @@ struct FBlockTask {
   cplx* outH;                    // optional [nj][m0*m0]: store Hbar_j
   cplx* outS;                    // optional [nj][m0*m0]: store Sbar_j
   int want;                      // 0: no eigenvalues, 1: all, 2: only the lowest
-  double* ev;                    // [nj*m0] (want 1) or [nj] (want 2)
+  double* ev;                    // [nj*m0] (want 1; null: vectors only) or [nj] (want 2)
   int* blk;                      // optional [nj*m0] Fourier index of each eigenvalue
   int* fail;                     // set to 1 if a block's Sbar is not positive definite
   const double* tau;             // FACTORS: the problem's dependency cut (k_null_tau); TOEPLITZ:
@@ -210,6 +210,36 @@ struct FBlockTask {
                                  // [j][i][mu], Sbar_j-orthonormal, ascending; removed directions zero
   int* neig;                     // optional: counts the blocks solved by the overlap's
                                  // eigendecomposition (the Cholesky certificate failed)
+};
+
+// Whole spectrum of a periodic problem, or of a range of its Fourier indices: the
+// blocks solved (one of each conjugate pair the range holds) in chunks.
+struct PfTask {
+  int prob, j0, nj, nrep;        // Fourier indices j0 .. j0 + nj - 1, representatives
+  int L[3];
+  const cplx* Xh[3];             // per-axis DFT'd factors [L_l][nF][m0*m0]
+  const int* rep;                // [nrep] local index of each representative, ascending
+  double* ev;                    // [nj*m0]
+  int* blk;                      // optional [nj*m0] Fourier index of each eigenvalue
+  const double* tau;             // the problem's dependency cut
+  int* neig;                     // counts the blocks solved by the overlap's eigendecomposition
+};
+// kPfGroup consecutive representatives of a task (the last group of a task may be short)
+constexpr int kPfGroup = 8;
+struct PfGroup { int task, rep; };
+// rotations recorded per block of order m (0.8 to 1.2 m^2 were seen; a block that needs
+// more takes the Jacobi method)
+__host__ __device__ inline int pf_rot_cap(int m) { return m * m * 3 / 2 + 4 * m; }
+// Workspace of a chunk (k_eig.cu), per slot (a block of the chunk): lower triangles
+// of Hbar and Sbar and the overlap's reflectors (nup entries), tridiagonals and
+// rotations with 32 slots side by side.
+struct PfWork {
+  int mm, nup;                   // largest block order, mm (mm + 1) / 2
+  cplx *H, *S, *R;
+  double *sd, *se, *td, *te;     // tridiagonals of the overlap and of the reduced matrix
+  double* rtau; cplx* rph;       // [slot][mm] the overlap's reflector factors and phases
+  cplx* rot; unsigned char* roti;   // recorded rotations (c, s) and their column
+  int *nrot, *order, *status;
 };
 
 // Dependency cut of a periodic problem: B[mu nu] = prod over axes of the sum

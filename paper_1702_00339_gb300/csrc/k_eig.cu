@@ -792,15 +792,16 @@ __global__ void k_fblocks(const ProbDev* __restrict__ probs, const FBlockTask* _
     for (int it = threadIdx.x; it < r * r; it += blockDim.x) Vc[(it / r) * ldr + it % r] = H[it];
     __syncthreads();
   }
-  if (r > 0) cta_tridiag(H, r, dd, ee, v, pv);
-  for (int i = threadIdx.x; i < r; i += blockDim.x) {
+  const bool values = F.want != 1 || F.ev;      // vectors alone: no eigenvalues
+  if (values && r > 0) cta_tridiag(H, r, dd, ee, v, pv);
+  for (int i = threadIdx.x; values && i < r; i += blockDim.x) {
     const double e2i = (i + 1 < r) ? ee[i] * ee[i] : 0.0;
     e2[i] = e2i;
     df[i] = (float)dd[i];
     e2f[i] = (float)e2i;
   }
   __syncthreads();
-  if (F.want == 1) {
+  if (F.want == 1 && F.ev) {
     for (int i = threadIdx.x; i < m0; i += blockDim.x) {
       const double lam = (i < r) ? tridiag_eig_fast(df, e2f, dd, e2, r, i, 0.0) : INFINITY;
       F.ev[(size_t)jl * m0 + i] = lam;
@@ -810,7 +811,7 @@ __global__ void k_fblocks(const ProbDev* __restrict__ probs, const FBlockTask* _
         if (F.blk) F.blk[(size_t)(jm - F.j0) * m0 + i] = jm;
       }
     }
-  } else if (threadIdx.x == 0) {
+  } else if (F.want == 2 && threadIdx.x == 0) {
     // the lowest eigenvalue of an embedding block only sets the preconditioner
     // shift (lowered by 2e-5 relative afterwards): 1e-9 relative suffices
     F.ev[jl] = (r > 0) ? tridiag_eig_fast(df, e2f, dd, e2, r, 0, 1e-9) : INFINITY;
@@ -847,6 +848,593 @@ __global__ void k_fblocks(const ProbDev* __restrict__ probs, const FBlockTask* _
       }
       F.vecs[(size_t)jl * np + it] = y;
       if (jm >= 0) F.vecs[(size_t)(jm - F.j0) * np + it] = cconj(y);
+    }
+  }
+}
+
+// ---- periodic spectra (factors, eigenvalues only): a pipeline over Fourier blocks ----
+//
+// k_fblocks above takes a block through every phase in one CTA.  Its time went to
+// FP64 instructions that half-empty warps issued and to phases that one warp or
+// one thread ran while the CTA waited: three products per quadrature term and
+// block in the formation, the QL sweeps with their rotations, FP64 bisection,
+// serial triangular inverses.  For whole spectra the phases are kernels of their
+// own over a chunk of blocks (conjugate pairs once), each spread as it likes:
+//
+//  k_pf_form    Hbar_j, Sbar_j, lower triangles: a thread per entry, eight blocks j
+//               with the same (j1, j2) at a time, so the product of the first two
+//               axes' factors is formed once for them: 38 FP64 instructions per
+//               term and eight blocks instead of 80
+//  k_pf_reduce  elimination of Sbar_j applied to Hbar_j from both sides and to L^-1 as
+//               it goes (entries in registers); when L^-1 certifies that nothing is
+//               numerically singular: the reduced matrix to tridiagonal form.
+//               Otherwise Sbar_j to tridiagonal form, reflectors kept
+//  k_pf_ql      one thread per block: QL on the overlaps' tridiagonals, rotations recorded
+//  k_pf_cut     the recorded rotations applied, the cut, X = Q_K diag(s_K)^-1/2,
+//               X^H Hbar X to tridiagonal form
+//  k_pf_values  one thread per block: QL for the eigenvalues
+//
+// All are bound by the FP64 pipe or, the two QL kernels, by a thread's chain of
+// about 850 cycles per rotation with every SM holding a few warps.  Measured: two
+// lattices of 16^3 cells of 16 functions 3.06 -> 1.7 ms, one of 32^3 cells of 32
+// functions, four of them cut in every block, 86.5 -> 38 ms.
+
+// lower-triangle position t = a (a + 1) / 2 + b, b <= a
+__device__ inline void tri_pos(int t, int& a, int& b) {
+  a = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+  while ((a + 1) * (a + 2) / 2 <= t) ++a;
+  while (a * (a + 1) / 2 > t) --a;
+  b = t - a * (a + 1) / 2;
+}
+// element i of slot's tridiagonal arrays: 32 slots side by side
+__device__ inline size_t pf_ix(int slot, int i, int mm) { return ((size_t)(slot >> 5) * mm + i) * 32 + (slot & 31); }
+
+// G: blocks per thread at a time (8; 2 where there are too few blocks to fill the GPU)
+// A warp per CTA: 32 entries of the triangle waste least, and warps of 160 000 cycles
+// fill the SMs evenly (two lattices of 16^3 cells: 840 us with CTAs of 160 threads).
+template <int G>
+__global__ void __launch_bounds__(32) k_pf_form(const ProbDev* __restrict__ probs, const PfTask* __restrict__ tasks,
+                                                const PfGroup* __restrict__ groups, PfWork W) {
+  const PfGroup grp = groups[blockIdx.x * G / kPfGroup];
+  const PfTask F = tasks[grp.task];
+  const ProbDev& P = probs[F.prob];
+  const int m0 = P.m0, np = m0 * m0, nup = m0 * (m0 + 1) / 2, R = P.R, T = P.T;
+  const int t0 = blockIdx.y * blockDim.x + threadIdx.x, s0 = blockIdx.x * G, r0 = grp.rep + s0 % kPfGroup;
+  const int cnt = min(G, F.nrep - r0);
+  if (t0 >= nup || cnt <= 0) return;
+  int a, b;
+  tri_pos(t0, a, b);
+  const int pr = b * m0 + a;                 // the upper entry (b, a); the lower one is its conjugate
+  const int nfe = P.nF * np;
+  const double *Zq = P.Z, *cq = P.cq;
+  // the inner axis, along which consecutive blocks run: the last one with more than one cell
+  const int in = (F.L[2] > 1) ? 2 : (F.L[1] > 1) ? 1 : 0, o0 = (in == 0) ? 1 : 0, o1 = (in == 2) ? 1 : 2;
+  const int Lin = F.L[in];
+  for (int g0 = 0; g0 < cnt;) {
+    // a run of blocks with the same indices on the other two axes
+    const int j = F.j0 + F.rep[r0 + g0], jo = j / Lin;   // (axes after the inner one have one cell)
+    int n = 1;
+    while (g0 + n < cnt && (F.j0 + F.rep[r0 + g0 + n]) / Lin == jo) ++n;
+    const int i0 = (in == 2) ? jo / F.L[1] : (in == 1) ? jo : 0, i1 = (in == 2) ? jo % F.L[1] : 0;
+    const cplx* f0 = F.Xh[o0] + (size_t)i0 * nfe + pr;
+    const cplx* f1 = F.Xh[o1] + (size_t)i1 * nfe + pr;
+    const cplx* f2[G];
+    cplx v[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      const int jg = F.j0 + F.rep[r0 + g0 + min(g, n - 1)];
+      f2[g] = F.Xh[in] + (size_t)(jg % Lin) * nfe + pr;
+      v[g] = cmk(0.0, 0.0);
+    }
+    for (int nu = 0; nu < T / R; ++nu) {
+      const double zw = Zq[nu];
+#pragma unroll 2
+      for (int q = 0; q < R; ++q) {
+        const size_t o = (size_t)(2 + nu * R + q) * np;
+        const cplx p = cscale(cmul(f0[o], f1[o]), zw * cq[q]);
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+          if (g < n) v[g] = cfma(p, f2[g][o], v[g]);
+      }
+    }
+    const cplx s0v = f0[0], s1 = f1[0], a0 = f0[np], a1 = f1[np];
+    const cplx s01 = cmul(s0v, s1), k01 = cadd(cmul(a0, s1), cmul(s0v, a1));
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+      if (g < n) {
+        const cplx s2 = f2[g][0], a2 = f2[g][np];
+        cplx h = csub(cscale(cadd(cmul(k01, s2), cmul(s01, a2)), 0.5), v[g]);
+        cplx s = cmul(s01, s2);
+        if (a == b) { h.y = 0.0; s.y = 0.0; }
+        const size_t o = (size_t)(s0 + g0 + g) * W.nup + t0;
+        W.H[o] = cconj(h);
+        W.S[o] = cconj(s);
+      }
+    g0 += n;
+  }
+}
+
+// The warp that does what one warp does, different in the CTAs that share an SM
+// (CTAs b, b + 152, ...): warps of one number share a sub-partition.
+__device__ inline int pf_lead(int nw) { return (int)((blockIdx.x / 152 + blockIdx.x) % (unsigned)nw); }
+
+// Householder reduction of the Hermitian m x m matrix A (lower triangle, pitch ld,
+// shared memory) to tridiagonal form: d, e = |subdiagonal|, and of each step the
+// reflector I - tau v v^H (v left in A's column below the diagonal) and the
+// subdiagonal's phase.  v, w: m entries each.  lw: the warp that makes the reflectors.
+__device__ void cta_tridiag_lower(cplx* A, int ld, int m, double* d, double* e, double* tau, cplx* ph, cplx* v, cplx* w,
+                                  int lw) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int k = 0; k + 1 < m; ++k) {
+    const int n = m - k - 1;
+    if (warp == lw) {
+      const cplx x = (lane < n) ? A[(k + 1 + lane) * ld + k] : cmk(0.0, 0.0);
+      double tail = (lane >= 1) ? cabs2(x) : 0.0;
+      for (int o = 16; o > 0; o >>= 1) tail += __shfl_xor_sync(0xffffffffu, tail, o);
+      const cplx x1 = cmk(__shfl_sync(0xffffffffu, x.x, 0), __shfl_sync(0xffffffffu, x.y, 0));
+      const double a2 = cabs2(x1);
+      const double r1 = (__double_as_longlong(a2) > 0) ? rsqrt_nr(a2) : 0.0;
+      const double ax = a2 * r1;
+      const cplx p1 = (__double_as_longlong(a2) > 0) ? cscale(x1, r1) : cmk(1.0, 0.0);
+      double ek = ax, tk = 0.0;
+      cplx phase = p1, vi = x;
+      if (__double_as_longlong(tail) > 0) {      // (no tail for the last column)
+        const double s = a2 + tail, xn = s * rsqrt_nr(s);
+        tk = rcp_nr(fma(ax, xn, s));
+        ek = xn;
+        phase = cmk(-p1.x, -p1.y);
+        if (lane == 0) vi = cscale(p1, ax + xn);
+      }
+      if (lane < n) { v[lane] = vi; if (lane == 0) A[(k + 1) * ld + k] = vi; }
+      if (lane == 0) { d[k] = A[k * ld + k].x; e[k] = ek; tau[k] = tk; ph[k] = phase; }
+    }
+    __syncthreads();
+    const double tk = tau[k];
+    if (__double_as_longlong(tk) == 0) continue;   // uniform
+    const cplx* B = A + (size_t)(k + 1) * ld + (k + 1);   // trailing block
+    for (int it = threadIdx.x; it < ((4 * n + 31) & ~31); it += blockDim.x) {   // w = tau B v, 4 threads per row
+      const int i = it >> 2, o = it & 3;
+      cplx s = cmk(0.0, 0.0);
+      if (i < n)
+        for (int j = o; j < n; j += 4) {
+          // the entry or its mirror's conjugate (sign bit flipped: no FP64, no divergence)
+          const bool low = j <= i;
+          cplx x = B[low ? i * ld + j : j * ld + i];
+          x.y = __longlong_as_double(__double_as_longlong(x.y) ^ (low ? 0ll : (long long)0x8000000000000000ull));
+          s = cfma(x, v[j], s);
+        }
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, 1);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, 1);
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, 2);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, 2);
+      if (i < n && o == 0) w[i] = cscale(s, tk);
+    }
+    __syncthreads();
+    if (warp == lw) {                               // w -= (tau / 2) Re(v^H w) v
+      const cplx vi = (lane < n) ? v[lane] : cmk(0.0, 0.0), wi = (lane < n) ? w[lane] : cmk(0.0, 0.0);
+      double s = fma(vi.x, wi.x, vi.y * wi.y);
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      const double K = -0.5 * tk * s;
+      if (lane < n) w[lane] = cmk(fma(K, vi.x, wi.x), fma(K, vi.y, wi.y));
+    }
+    __syncthreads();
+    // B -= v w^H + w v^H, lower triangle: rows n-1-p and p together are n + 1 entries
+    const int half = (n + 1) >> 1;
+    for (int it = threadIdx.x; it < half * (n + 1); it += blockDim.x) {
+      const int p = it / (n + 1), q = it - p * (n + 1);
+      int i = n - 1 - p, j = q;
+      if (q > i) { if (i == p) continue; j = q - i - 1; i = p; }
+      cplx* x = A + (size_t)(k + 1 + i) * ld + (k + 1 + j);
+      *x = crank2(*x, v[i], w[j], w[i], v[j]);
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
+    d[m - 1] = A[(m - 1) * ld + (m - 1)].x;
+    e[m - 1] = 0.0;
+  }
+  __syncthreads();
+}
+
+// NT threads, NS entries of the lower triangle per thread.
+template <int NT, int NS>
+__global__ void __launch_bounds__(NT) k_pf_reduce(const ProbDev* __restrict__ probs, const PfTask* __restrict__ tasks,
+                                                  const PfGroup* __restrict__ groups, PfWork W) {
+  extern __shared__ __align__(16) cplx psm[];
+  const int slot = blockIdx.x;
+  const PfGroup grp = groups[slot / kPfGroup];
+  const PfTask F = tasks[grp.task];
+  if (grp.rep + slot % kPfGroup >= F.nrep) { if (threadIdx.x == 0) W.status[slot] = -1; return; }
+  const int m = probs[F.prob].m0, nup = m * (m + 1) / 2, ld = m | 1, tid = threadIdx.x;
+  cplx* A = psm;                               // m x ld
+  __shared__ cplx cS[2][MAXM0], cH[2][MAXM0], lv[MAXM0], uv[MAXM0], xs[MAXM0], yh[MAXM0], zl[MAXM0];
+  __shared__ double dl[MAXM0], dd[MAXM0], ee[MAXM0], tt[MAXM0], red[4];
+  __shared__ cplx ph[MAXM0];
+  const int lane = tid & 31, lw = pf_lead(NT / 32);
+  const cplx* Hg = W.H + (size_t)slot * W.nup;
+  const cplx* Sg = W.S + (size_t)slot * W.nup;
+  cplx S[NS], H[NS];
+  int ea[NS], eb[NS];
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    const int t = s * NT + tid;
+    ea[s] = -1;
+    eb[s] = 0;
+    if (t < nup) { tri_pos(t, ea[s], eb[s]); S[s] = Sg[t]; H[s] = Hg[t]; }
+  }
+  bool ok = true;
+  const double cut = fmax(*F.tau, 0.0);
+  // Step j: l = S(:, j) / S_jj for rows a > j; S and L^-1 (in S's eliminated columns)
+  // lose l times row j, H loses l u^H + u l^H with u = H(:, j) - l H_jj / 2 in the
+  // columns still to come and l times its row j in those already eliminated.  Column
+  // b's multipliers of -l_a and -u_a stand in xs, yh and zl whatever b's case, so the
+  // lanes of a warp do not diverge.
+  for (int j = 0; j < m; ++j) {
+    const int par = j & 1;
+    // entry t of column j where t >= j, of row j where t < j
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      if (eb[s] == j && ea[s] >= j) { cS[par][ea[s]] = S[s]; cH[par][ea[s]] = H[s]; }
+      if (ea[s] == j && eb[s] < j) { cS[par][eb[s]] = S[s]; cH[par][eb[s]] = H[s]; }
+    }
+    __syncthreads();
+    const double dj = cS[par][j].x, hjj = cH[par][j].x;
+    // a pivot at or below the cut bounds lambda_min(Sbar): no certificate (uniform)
+    if (!(dj > cut)) { ok = false; break; }
+    if ((tid >> 5) == lw && lane < m) {
+      const cplx c = cS[par][lane], h = cH[par][lane];
+      if (lane > j) {
+        const cplx l = cscale(c, rcp_nr(dj));
+        const cplx u = cmk(fma(-0.5 * hjj, l.x, h.x), fma(-0.5 * hjj, l.y, h.y));
+        lv[lane] = cmk(-l.x, -l.y);
+        uv[lane] = cmk(-u.x, -u.y);
+        xs[lane] = cconj(c);
+        yh[lane] = cconj(u);
+        zl[lane] = cconj(l);
+      } else {
+        if (lane == j) dl[j] = dj;
+        xs[lane] = (lane == j) ? cmk(1.0, 0.0) : c;
+        yh[lane] = (lane == j) ? cmk(hjj, 0.0) : h;
+        zl[lane] = cmk(0.0, 0.0);
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      const int a = ea[s], b = eb[s];
+      if (a <= j) continue;
+      const cplx l = lv[a];
+      S[s] = cfma(l, xs[b], (b == j) ? cmk(0.0, 0.0) : S[s]);
+      H[s] = cfma(uv[a], zl[b], cfma(l, yh[b], H[s]));
+    }
+  }
+  __syncthreads();
+  if (ok) {
+    // certificate: lambda_min(Sbar) >= 1 / ||L^-1||_F^2 > tau (Cholesky's L^-1 = delta^-1/2 times ours)
+    double part = 0.0;
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+      if (ea[s] >= 0) part = fma((ea[s] == eb[s]) ? 1.0 : cabs2(S[s]), rcp_nr(dl[ea[s]]), part);
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    if ((tid & 31) == 0) red[tid >> 5] = part;
+    __syncthreads();
+    double t = 0.0;
+    for (int w = 0; w < NT / 32; ++w) t += red[w];
+    ok = t > 0.0 && t * cut < 1.0;             // uniform
+  }
+  const int mm = W.mm;
+  if (ok) {
+    for (int t = tid; t < m; t += NT) tt[t] = rsqrt_nr(dl[t]);
+    __syncthreads();
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+      if (ea[s] >= 0) {
+        const cplx x = cscale(H[s], tt[ea[s]] * tt[eb[s]]);
+        A[ea[s] * ld + eb[s]] = (ea[s] == eb[s]) ? cmk(x.x, 0.0) : x;
+      }
+  } else {
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+      if (ea[s] >= 0) A[ea[s] * ld + eb[s]] = Sg[s * NT + tid];
+    if (tid == 0 && F.neig) atomicAdd(F.neig, 1);
+  }
+  __syncthreads();
+  cta_tridiag_lower(A, ld, m, dd, ee, tt, ph, cS[0], cS[1], lw);
+  double* od = ok ? W.td : W.sd;
+  double* oe = ok ? W.te : W.se;
+  for (int i = tid; i < m; i += NT) {
+    od[pf_ix(slot, i, mm)] = dd[i];
+    oe[pf_ix(slot, i, mm)] = ee[i];
+  }
+  if (tid == 0) { W.status[slot] = ok ? 0 : 1; W.order[slot] = m; }
+  if (!ok) {
+    for (int i = tid; i + 1 < m; i += NT) { W.rtau[(size_t)slot * mm + i] = tt[i]; W.rph[(size_t)slot * mm + i] = ph[i]; }
+    cplx* R = W.R + (size_t)slot * W.nup;
+    for (int t = tid; t < nup; t += NT) {
+      int a, b;
+      tri_pos(t, a, b);
+      R[t] = A[a * ld + b];
+    }
+  }
+}
+
+// Implicit QL with Wilkinson's shift (Bowdler, Martin, Reinsch and Wilkinson, Numer.
+// Math. 11 (1968)) on one thread's tridiagonal: D(i), E(i) at D[32 i], E[32 i].  An
+// off-diagonal is negligible at eps ||T||_inf.  rec(i, c, s) is told each rotation
+// of columns i, i + 1.  False when an eigenvalue takes more than 60 iterations.
+template <class Rec>
+__device__ bool lane_ql(double* D, double* E, int n, Rec rec) {
+  double tn = 0.0, em = 0.0;
+  for (int i = 0; i < n; ++i) {
+    const double e = (i + 1 < n) ? E[32 * i] : 0.0;
+    tn = fmax(tn, fabs(D[32 * i]) + e + em);
+    em = e;
+  }
+  const double small = 2.220446049250313e-16 * tn;
+  const long long small_bits = __double_as_longlong(small);
+  for (int l = 0; l < n; ++l) {
+    for (int iter = 0;; ++iter) {
+      int m = l;
+      while (m + 1 < n && abs_bits(E[32 * m]) > small_bits) ++m;
+      if (m == l) break;                               // D(l) is an eigenvalue
+      if (iter == 60) return false;
+      // shift: the eigenvalue of the leading 2 x 2 of block l..m nearer D(l)
+      const double el = E[32 * l], dl = D[32 * l];
+      double g = (D[32 * (l + 1)] - dl) * rcp_nr(2.0 * el);
+      const double q1 = fma(g, g, 1.0);
+      const double r1 = q1 * rsqrt_nr(q1);
+      g = D[32 * m] - dl + el * rcp_nr(g + copysign(r1, g));
+      double s = 1.0, c = 1.0, p = 0.0, dn = D[32 * m];
+      bool split = false;
+      for (int i = m - 1; i >= l; --i) {
+        const double ei = E[32 * i], di = D[32 * i];
+        const double f = s * ei, b = c * ei;
+        const double q2 = fma(f, f, g * g);
+        if (__double_as_longlong(q2) == 0) {           // the chase stopped: restart
+          D[32 * (i + 1)] = dn - p;
+          E[32 * m] = 0.0;
+          split = true;
+          break;
+        }
+        const double ir = rsqrt_nr(q2);
+        E[32 * (i + 1)] = q2 * ir;
+        s = f * ir;
+        c = g * ir;
+        g = dn - p;
+        const double r = fma(di - g, s, 2.0 * c * b);
+        p = s * r;
+        D[32 * (i + 1)] = g + p;
+        g = fma(c, r, -b);
+        dn = di;
+        rec(i, c, s);
+      }
+      if (split) continue;
+      D[32 * l] = dn - p;
+      E[32 * l] = g;
+      E[32 * m] = 0.0;
+    }
+  }
+  return true;
+}
+
+__global__ void __launch_bounds__(32) k_pf_ql(PfWork W, int nslot) {
+  extern __shared__ __align__(16) cplx psm[];
+  double* D = reinterpret_cast<double*>(psm) + threadIdx.x;
+  double* E = D + 32 * W.mm;
+  const int slot = blockIdx.x * 32 + threadIdx.x;
+  if (slot >= nslot || W.status[slot] != 1) return;
+  const int m = W.order[slot], cap = pf_rot_cap(W.mm);
+  for (int i = 0; i < m; ++i) { D[32 * i] = W.sd[pf_ix(slot, i, W.mm)]; E[32 * i] = W.se[pf_ix(slot, i, W.mm)]; }
+  int k = 0;
+  const size_t base = (size_t)(slot >> 5) * cap * 32 + (slot & 31);
+  const bool ok = lane_ql(D, E, m, [&](int i, double c, double s) {
+    if (k < cap) { W.rot[base + (size_t)k * 32] = cmk(c, s); W.roti[base + (size_t)k * 32] = (unsigned char)i; }
+    ++k;
+  });
+  W.nrot[slot] = k;
+  if (!ok || k > pf_rot_cap(m)) W.status[slot] = 2;    // the Jacobi method (not cap: no choice of the chunk)
+  for (int i = 0; i < m; ++i) W.sd[pf_ix(slot, i, W.mm)] = D[32 * i];
+}
+
+// Blocks whose overlap has directions at or below the cut (or no certificate
+// against them): Sbar = Q diag(s) Q^H with Q = H_0 ... H_{m-3} D Z (reflectors, phases
+// and rotations recorded above), K = {s > tau}, C = X^H Hbar X, X = Q_K diag(s_K)^-1/2.
+__global__ void __launch_bounds__(128) k_pf_cut(const ProbDev* __restrict__ probs, const PfTask* __restrict__ tasks,
+                                                const PfGroup* __restrict__ groups, PfWork W) {
+  extern __shared__ __align__(16) cplx psm[];
+  const int slot = blockIdx.x;
+  const int status = W.status[slot];
+  if (status != 1 && status != 2) return;
+  const PfTask F = tasks[groups[slot / kPfGroup].task];
+  const int m = probs[F.prob].m0, nup = m * (m + 1) / 2, ld = m | 1, mm = W.mm, cap = pf_rot_cap(mm);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nth = blockDim.x, nw = nth >> 5;
+  cplx* V = psm;                               // m x ld: eigenvectors, then X
+  cplx* H = V + (m + 1) * (m + 1);             // m x ld: Hbar, then C
+  cplx* U = H + (m + 1) * (m + 1);             // reflectors (packed) and Z, then Hbar X
+  double* Z = reinterpret_cast<double*>(U + nup);   // column i, row r: Z[i ld + r]
+  __shared__ double sv[MAXM0], dd[MAXM0], ee[MAXM0], tt[MAXM0];
+  __shared__ cplx hw[MAXM0], ph[MAXM0], vv[MAXM0];
+  __shared__ cplx rot[128];
+  __shared__ unsigned char roti[128];
+  __shared__ int keep[MAXM0], s_r;
+  __shared__ double rsq[MAXM0];
+  // the kept directions, in ascending index, and s^-1/2
+  auto choose = [&]() {
+    if (tid == 0) {
+      int r = 0;
+      const double tau = *F.tau;
+      for (int i = 0; i < m; ++i)
+        if (sv[i] > tau && sv[i] > 0.0) { keep[r] = i; rsq[r] = rsqrt_nr(sv[i]); ++r; }
+      s_r = r;
+    }
+  };
+  if (status == 1) {
+    for (int it = tid; it < m * m; it += nth) Z[(it / m) * ld + it % m] = (it / m == it % m) ? 1.0 : 0.0;
+    for (int t = tid; t < nup; t += nth) U[t] = W.R[(size_t)slot * W.nup + t];
+    // rotations on the rows of Z, a lane per row, on a warp that differs from CTA to
+    // CTA (the CTAs of an SM then use different sub-partitions' FP64 units)
+    const int zw = pf_lead(nw), cnt = W.nrot[slot];
+    const size_t base = (size_t)(slot >> 5) * cap * 32 + (slot & 31);
+    int last = -1;
+    double zc = 0.0;                           // column `last` of this lane's row, in a register
+    for (int k0 = 0; k0 < cnt; k0 += 128) {
+      const int nk = min(128, cnt - k0);
+      for (int k = tid; k < nk; k += nth) { rot[k] = W.rot[base + (size_t)(k0 + k) * 32]; roti[k] = W.roti[base + (size_t)(k0 + k) * 32]; }
+      __syncthreads();
+      if (warp == zw && lane < m)
+        for (int k = 0; k < nk; ++k) {
+          const int i = roti[k];
+          const double c = rot[k].x, s = rot[k].y;
+          double zj = zc;
+          if (i + 1 != last) {                 // a new sweep: column `last` goes back first
+            if (last >= 0) Z[last * ld + lane] = zc;
+            zj = Z[(i + 1) * ld + lane];
+          }
+          const double zi = Z[i * ld + lane];
+          Z[(i + 1) * ld + lane] = fma(s, zi, c * zj);
+          zc = fma(c, zi, -s * zj);
+          last = i;
+        }
+      __syncthreads();
+    }
+    if (warp == zw && lane < m && last >= 0) Z[last * ld + lane] = zc;
+    if (tid == 0) {                            // phases: phi_0 = 1, phi_{k+1} = phi_k times the subdiagonal's
+      cplx phi = cmk(1.0, 0.0);
+      for (int k = 0; k < m; ++k) {
+        ph[k] = phi;
+        if (k + 1 < m) phi = cmul(phi, W.rph[(size_t)slot * mm + k]);
+      }
+    }
+    for (int i = tid; i + 1 < m; i += nth) tt[i] = W.rtau[(size_t)slot * mm + i];
+    for (int i = tid; i < m; i += nth) sv[i] = W.sd[pf_ix(slot, i, mm)];
+    __syncthreads();
+    choose();
+    __syncthreads();
+    for (int it = tid; it < m * s_r; it += nth) {   // the kept columns alone, scaled
+      const int i = it % m, c = it / m;
+      V[i * ld + c] = cscale(ph[i], Z[keep[c] * ld + i] * rsq[c]);
+    }
+    __syncthreads();
+    for (int k = m - 3; k >= 0; --k) {         // V loses tau v (v^H V)
+      const double tk = tt[k];
+      if (__double_as_longlong(tk) == 0) continue;
+      const int n = m - k - 1;
+      auto vk = [&](int i) { const int a = k + 1 + i; return U[a * (a + 1) / 2 + k]; };
+      const int nk = s_r;
+      for (int it = tid; it < ((4 * nk + 31) & ~31); it += nth) {
+        const int c = it >> 2, o = it & 3;
+        cplx s = cmk(0.0, 0.0);
+        if (c < nk)
+          for (int i = o; i < n; i += 4) s = cfmac(V[(k + 1 + i) * ld + c], vk(i), s);
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, 1);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, 1);
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, 2);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, 2);
+        if (c < nk && o == 0) hw[c] = cscale(s, -tk);
+      }
+      __syncthreads();
+      for (int it = tid; it < n * nk; it += nth) {
+        const int i = it / nk, c = it - i * nk;
+        V[(k + 1 + i) * ld + c] = cfma(vk(i), hw[c], V[(k + 1 + i) * ld + c]);
+      }
+      __syncthreads();
+    }
+  } else {
+    // QL ran out of iterations or rotations: cyclic Jacobi on Sbar
+    const int lj = m + (m & 1);
+    cplx* a = U;                               // lj x lj
+    for (int t = tid; t < nup; t += nth) {
+      int i, j;
+      tri_pos(t, i, j);
+      const cplx x = W.S[(size_t)slot * W.nup + t];
+      a[i * lj + j] = x;
+      a[j * lj + i] = cconj(x);
+    }
+    __syncthreads();
+    cta_jacobi_herm(a, H, m, lj);              // (H is loaded below)
+    for (int i = tid; i < m; i += nth) sv[i] = a[i * lj + i].x;
+    __syncthreads();
+    choose();
+    __syncthreads();
+    for (int it = tid; it < m * s_r; it += nth) {
+      const int i = it / s_r, c = it - i * s_r;
+      V[i * ld + c] = cscale(H[i * lj + keep[c]], rsq[c]);
+    }
+    __syncthreads();
+  }
+  for (int t = tid; t < nup; t += nth) {
+    int a, b;
+    tri_pos(t, a, b);
+    const cplx x = W.H[(size_t)slot * W.nup + t];
+    H[a * ld + b] = x;
+    H[b * ld + a] = cconj(x);
+  }
+  __syncthreads();
+  const int r = s_r;
+  cplx* Y = U;                                 // m x r, pitch ld: Hbar X
+  for (int it = tid; it < m * r; it += nth) {
+    const int i = it / r, c = it - i * r;
+    cplx s = cmk(0.0, 0.0);
+    for (int q = 0; q < m; ++q) s = cfma(H[i * ld + q], V[q * ld + c], s);
+    Y[i * ld + c] = s;
+  }
+  __syncthreads();
+  for (int t = tid; t < r * (r + 1) / 2; t += nth) {   // C = X^H Y, lower triangle
+    int a, b;
+    tri_pos(t, a, b);
+    cplx s = cmk(0.0, 0.0);
+    for (int q = 0; q < m; ++q) s = cfmac(Y[q * ld + b], V[q * ld + a], s);
+    if (a == b) s.y = 0.0;
+    H[a * ld + b] = s;
+  }
+  __syncthreads();
+  if (r > 0) cta_tridiag_lower(H, ld, r, dd, ee, tt, ph, vv, hw, pf_lead(nw));
+  for (int i = tid; i < r; i += nth) {
+    W.td[pf_ix(slot, i, mm)] = dd[i];
+    W.te[pf_ix(slot, i, mm)] = ee[i];
+  }
+  if (tid == 0) { W.order[slot] = r; W.status[slot] = 0; }
+}
+
+__global__ void __launch_bounds__(32) k_pf_values(const ProbDev* __restrict__ probs, const PfTask* __restrict__ tasks,
+                                                  const PfGroup* __restrict__ groups, PfWork W, int nslot) {
+  extern __shared__ __align__(16) cplx psm[];
+  double* D = reinterpret_cast<double*>(psm) + threadIdx.x;
+  double* E = D + 32 * W.mm;
+  const int slot = blockIdx.x * 32 + threadIdx.x;
+  if (slot >= nslot) return;
+  const PfGroup grp = groups[slot / kPfGroup];
+  const PfTask F = tasks[grp.task];
+  const int rep = grp.rep + slot % kPfGroup;
+  if (rep >= F.nrep) return;
+  const int m0 = probs[F.prob].m0, r = W.order[slot];
+  for (int i = 0; i < r; ++i) { D[32 * i] = W.td[pf_ix(slot, i, W.mm)]; E[32 * i] = W.te[pf_ix(slot, i, W.mm)]; }
+  if (!lane_ql(D, E, r, [](int, double, double) {})) {
+    // out of iterations: bisection on the tridiagonal itself
+    double d[MAXM0], e2[MAXM0];
+    float df[MAXM0], e2f[MAXM0];
+    for (int i = 0; i < r; ++i) {
+      d[i] = W.td[pf_ix(slot, i, W.mm)];
+      const double e = W.te[pf_ix(slot, i, W.mm)];
+      e2[i] = (i + 1 < r) ? e * e : 0.0;
+      df[i] = (float)d[i];
+      e2f[i] = (float)e2[i];
+    }
+    for (int i = 0; i < r; ++i) D[32 * i] = tridiag_eig_fast(df, e2f, d, e2, r, i, 0.0);
+  }
+  // the conjugate block's spectrum too, where the task's range holds it
+  const int jl = F.rep[rep], j = F.j0 + jl;
+  const int j3 = j % F.L[2], j2 = (j / F.L[2]) % F.L[1], j1 = j / (F.L[1] * F.L[2]);
+  const int c1 = (F.L[0] - j1) % F.L[0], c2 = (F.L[1] - j2) % F.L[1], c3 = (F.L[2] - j3) % F.L[2];
+  const int jm = (c1 * F.L[1] + c2) * F.L[2] + c3;
+  const bool pair = jm != j && jm >= F.j0 && jm < F.j0 + F.nj;
+  for (int i = 0; i < m0; ++i) {
+    const double lam = (i < r) ? D[32 * i] : INFINITY;
+    F.ev[(size_t)jl * m0 + i] = lam;
+    if (F.blk) F.blk[(size_t)jl * m0 + i] = j;
+    if (pair) {
+      F.ev[(size_t)(jm - F.j0) * m0 + i] = lam;
+      if (F.blk) F.blk[(size_t)(jm - F.j0) * m0 + i] = jm;
     }
   }
 }
@@ -1085,6 +1673,57 @@ void launch_fblocks(const ProbDev* probs, const FBlockTask* tasks, int ntask, in
   // per SM keep the FP64 pipe busy), up to four warps for m0 = 32
   const int threads = (maxm0 <= 8) ? 32 : (maxm0 <= 16) ? 64 : 128;
   k_fblocks<<<dim3(gx, ntask), threads, sm, st>>>(probs, tasks, x0);
+}
+
+// Bytes of workspace for nslot blocks of order at most m, and its layout. The arrays
+// hold multiples of 32 slots.
+size_t pf_layout(char* base, int m, size_t nslot, PfWork* W) {
+  const size_t ns = (nslot + 31) & ~(size_t)31, nup = (size_t)m * (m + 1) / 2, cap = pf_rot_cap(m);
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    char* p = base + off;
+    off += (bytes + 255) & ~(size_t)255;
+    return p;
+  };
+  PfWork w;
+  w.mm = m; w.nup = (int)nup;
+  w.H = (cplx*)take(ns * nup * sizeof(cplx)); w.S = (cplx*)take(ns * nup * sizeof(cplx));
+  w.R = (cplx*)take(ns * nup * sizeof(cplx));
+  w.sd = (double*)take(ns * m * sizeof(double)); w.se = (double*)take(ns * m * sizeof(double));
+  w.td = (double*)take(ns * m * sizeof(double)); w.te = (double*)take(ns * m * sizeof(double));
+  w.rtau = (double*)take(ns * m * sizeof(double)); w.rph = (cplx*)take(ns * m * sizeof(cplx));
+  w.rot = (cplx*)take(ns * cap * sizeof(cplx)); w.roti = (unsigned char*)take(ns * cap);
+  w.nrot = (int*)take(ns * sizeof(int)); w.order = (int*)take(ns * sizeof(int)); w.status = (int*)take(ns * sizeof(int));
+  if (W) *W = w;
+  return off;
+}
+
+// The blocks of ng groups; none of an order above W.mm.
+void launch_pf(const ProbDev* probs, const PfTask* tasks, const PfGroup* groups, int ng, const PfWork& W,
+               cudaStream_t st) {
+  if (ng <= 0) return;
+  const int m = W.mm, nslot = ng * kPfGroup;
+  const size_t qs = (size_t)2 * 32 * m * sizeof(double), rs = (size_t)m * (m | 1) * sizeof(cplx);
+  const size_t cs = (size_t)3 * (m + 1) * (m + 1) * sizeof(cplx);
+  const int tiles = (W.nup + 31) / 32;
+  if ((long long)ng * tiles >= 4 * 152)
+    k_pf_form<kPfGroup><<<dim3(ng, tiles), 32, 0, st>>>(probs, tasks, groups, W);
+  else
+    k_pf_form<2><<<dim3(nslot / 2, tiles), 32, 0, st>>>(probs, tasks, groups, W);
+  if (m <= 8) k_pf_reduce<32, 2><<<nslot, 32, rs, st>>>(probs, tasks, groups, W);
+  else if (m <= 16) k_pf_reduce<64, 3><<<nslot, 64, rs, st>>>(probs, tasks, groups, W);
+  else {
+    FOCK_SMEM_OPTIN((k_pf_reduce<128, 5>));
+    k_pf_reduce<128, 5><<<nslot, 128, rs, st>>>(probs, tasks, groups, W);
+  }
+  k_pf_ql<<<(nslot + 31) / 32, 32, qs, st>>>(W, nslot);
+  FOCK_SMEM_OPTIN(k_pf_cut);
+  {   // the largest shared-memory carveout: four 32 x 32 blocks per SM
+    static std::once_flag carve;
+    std::call_once(carve, [] { cudaFuncSetAttribute(k_pf_cut, cudaFuncAttributePreferredSharedMemoryCarveout, 100); });
+  }
+  k_pf_cut<<<nslot, m <= 8 ? 32 : m <= 16 ? 64 : 128, cs, st>>>(probs, tasks, groups, W);
+  k_pf_values<<<(nslot + 31) / 32, 32, qs, st>>>(probs, tasks, groups, W, nslot);
 }
 
 void launch_precond(const ProbDev* probs, const PrecTask* tasks, int ntask, int maxM, int maxm0,

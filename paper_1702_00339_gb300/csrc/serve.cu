@@ -39,7 +39,7 @@
 #include "admission.h"
 
 namespace fock {
-int detail_estimate(const fock_problem& p, size_t* bytes, int* n_evals, std::string& why);
+int detail_estimate(const fock_problem& p, size_t budget, size_t* bytes, int* n_evals, std::string& why);
 fock_ctx* detail_worker_ctx(int device, cudaMemPool_t pool, size_t budget);
 const char* detail_ctx_error(const fock_ctx* c);
 cudaStream_t detail_ctx_stream(const fock_ctx* c);
@@ -270,7 +270,7 @@ int fock_serve_submit(fock_server* S, const fock_problem* p, uint64_t* ticket) {
   std::unique_ptr<Req> r(new Req());
   r->op.copy_from(*p);
   std::string why;
-  int rc = fock::detail_estimate(r->op.p, &r->bytes, &r->n_evals, why);
+  int rc = fock::detail_estimate(r->op.p, S->cfg.hbm_budget_bytes, &r->bytes, &r->n_evals, why);
   std::lock_guard<std::mutex> lk(S->m);
   if (rc) { S->err = why; return rc; }
   if (S->stopping) { S->err = "server is stopping"; return FOCK_EINVAL; }
