@@ -795,7 +795,8 @@ void plan(Batch& B, Slab& S, Slab& U) {
     sp.A = tab + off; sp.a_m = ld; sp.a_k = 1;
     sp.B = t.Zs; sp.b_k = np; sp.b_n = 1;
     sp.C = t.X + (direct ? 0 : 2 * np); sp.c_m = np; sp.c_n = 1;
-    sp.alpha = 1.0; sp.beta = 0.0;
+    sp.alpha = 1.0; sp.beta = 0.0; sp.ksplit = 1;
+    sp.ex = S.take<int>(sp.n_ex());
     B.splits.push_back(sp);
     B.split_maxm = std::max(B.split_maxm, sp.M);
     B.split_maxn = std::max(B.split_maxn, sp.N);
@@ -1250,6 +1251,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
           t.ksplit = std::min(32, std::max(1, ((t.K + 63) / 64 + 7) / 8));
           t.work = S.take<double>((size_t)t.ksplit * t.M * t.N);
           t.sym = g.sym;
+          t.ex = S.take<int>(t.n_ex());
           out.push_back(t);
           g.split = 1;
         };
@@ -1260,6 +1262,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
           t.A = g.A; t.a_m = 1; t.a_k = g.lda; t.B = g.B; t.b_k = 1; t.b_n = g.ldb;
           t.C = g.C; t.c_m = 1; t.c_n = g.ldc; t.alpha = g.alpha; t.beta = g.beta;
           t.ksplit = 1; t.work = nullptr; t.sym = 0;
+          t.ex = S.take<int>(t.n_ex());
           out.push_back(t);
           g.split = 1;
         };
@@ -2278,8 +2281,8 @@ int fock_plan_split_work(const fock_plan* P, double* tensor_flops, double* fp64_
   if (!P) return FOCK_EINVAL;
   double tf = 0.0, ff = 0.0;
   for (const SplitTask& t : P->B.splits) {
-    const double tiles = (double)((t.M + 127) / 128) * ((t.N + 63) / 64), chunks = (double)((t.K + 63) / 64);
-    tf += tiles * chunks * 28.0 * 4.0 * (128.0 * 64.0 * 16.0 * 2.0);
+    const double tiles = (double)((t.M + 127) / 128) * ((t.N + 63) / 64), chunks = (double)((t.K + 31) / 32);
+    tf += tiles * chunks * 36.0 * 2.0 * (128.0 * 64.0 * 16.0 * 2.0);
     ff += 2.0 * t.M * (double)t.N * t.K;
   }
   if (tensor_flops) *tensor_flops = tf;
@@ -2624,9 +2627,11 @@ int fock_split_dgemm(fock_ctx* ctx, int M, int N, int K, const double* A, long l
   t.ksplit = ksplit; t.sym = sym ? 1 : 0;
   const bool red = ksplit > 1 || sym;
   char* mem = nullptr;
-  const size_t wbytes = red ? (size_t)ksplit * M * N * sizeof(double) : 0;
-  CUDA_TRY(ctx, cudaMalloc(&mem, 256 + sizeof(SplitTask) + 256 + wbytes));
-  if (red) t.work = (double*)(mem + 512 + ((sizeof(SplitTask) + 255) & ~(size_t)255));
+  const size_t off_w = 256 + ((sizeof(SplitTask) + 255) & ~(size_t)255);
+  const size_t wbytes = red ? (((size_t)ksplit * M * N * sizeof(double) + 255) & ~(size_t)255) : 0;
+  CUDA_TRY(ctx, cudaMalloc(&mem, off_w + wbytes + t.n_ex() * sizeof(int) + 256));
+  if (red) t.work = (double*)(mem + off_w);
+  t.ex = (int*)(mem + off_w + wbytes);
   int herr = 0;
   cudaError_t e = cudaMemsetAsync(mem, 0, sizeof(int), st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(mem + 256, &t, sizeof(t), cudaMemcpyHostToDevice, st);

@@ -395,6 +395,26 @@ struct CanonTask {
 // exact split products (k_split.cu): A is M x K with A(m, k) at
 // A[m * a_m + k * a_k], B is K x N with B(k, n) at B[k * b_k + n * b_n],
 // C(m, n) at C[m * c_m + n * c_n].
+// The K ranges of a split product: nks of them by separate CTAs, in whole 64s, each
+// in `per` pieces of at most 512 summands (over which operands are aligned)
+struct SplitRanges {
+  static constexpr int RANGE = 512;
+  int K, nks, cps, per;
+  __host__ __device__ SplitRanges(int K_, int ksplit) : K(K_), nks(ksplit < 1 ? 1 : ksplit) {
+    cps = ((K + 63) / 64 + nks - 1) / nks;
+    per = (cps * 64 + RANGE - 1) / RANGE;
+  }
+  __host__ __device__ int count() const { return nks * per; }
+  __host__ __device__ int end(int e) const {
+    const long long k = (long long)(e / per) * cps * 64;
+    const long long a = k + (e % per + 1) * RANGE, b = k + cps * 64, m = a < b ? a : b;
+    return (int)(m < K ? m : K);
+  }
+  __host__ __device__ int begin(int e) const {
+    const long long k = (long long)(e / per) * cps * 64 + (long long)(e % per) * RANGE;
+    return (int)(k < K ? k : K);
+  }
+};
 struct SplitTask {
   const int* active;           // skip when *active == 0 (null: always)
   int M, N, K;
@@ -406,6 +426,9 @@ struct SplitTask {
   double* work;                // null: C written directly; else [ksplit][M][N] partial sums,
                                // reduced in a fixed order by k_split_reduce
   int sym;                     // (with work) C is symmetric: the upper triangle is reduced, mirrored
+  int* ex;                     // [ranges][M], then [ranges][N]: exponents of A's rows and B's columns
+  __host__ __device__ bool same() const { return A == B && a_m == b_n && a_k == b_k && M == N; }
+  __host__ __device__ size_t n_ex() const { return (size_t)SplitRanges(K, ksplit).count() * ((size_t)M + N); }
 };
 
 // Device pointers and sizes the matvec of an assembled box chain needs.

@@ -3,27 +3,36 @@
 // "Error-free transformations of matrix multiplication by using fast routines
 // of matrix multiplication", Numer. Algorithms 59 (2012)), used by the mixed
 // form for the quadrature contractions of stage (a) (Lemma 2.1 display,
-// Eqs. 2.16-2.17: X_t[mu nu] = sum_r P_t[r] Z[r][mu nu]).
+// Eqs. 2.16-2.17: X_t[mu nu] = sum_r P_t[r] Z[r][mu nu]) and for the dense
+// products of the block iteration.
 //
-// For a chunk of KC = 64 along the summation index, every row of A and every
-// column of B is aligned to its largest binary exponent, and its 53-bit
-// integer mantissas are cut into NDIG = 7 signed base-128 digits (|digit| <=
-// 127, exact in BF16).  For each level g = j + l (2 <= g <= NDIG + 1) the
-// products of digit planes j of A and l of B are summed by tcgen05.mma
-// (kind::f16, BF16 x BF16 -> FP32) into one TMEM accumulator per level; the
-// level sums are integers below 2^24, so FP32 accumulation is exact.  Each
-// thread then combines its row's levels in 64-bit integers and adds the
-// chunk, scaled by the two exponents, into FP64 accumulators.  Truncation:
-// the digits keep 49 of the 53 mantissa bits and the levels above NDIG + 1
-// are dropped, so each product carries a relative error below ~2^-46 of
-// (row maximum x column maximum) per summand.
+// Over a range of up to RANGE = 512 of the summation index, every row of A and
+// every column of B is aligned to its largest binary exponent (k_split_exps) and
+// rounded to 55 bits below it, which are written as NDIG = 8 balanced base-128
+// digits (-64 .. 64, exact in BF16).  For each level g = j + l (2 <= g <= NDIG + 1)
+// the products of digit planes j of A and l of B are summed by tcgen05.mma
+// (kind::f16, BF16 x BF16 -> FP32) into one TMEM accumulator per level: at most
+// 8 x 512 x 64^2 = 2^24, so FP32 accumulation is exact over a whole range.
+// Then each thread combines its row's levels in 64-bit integers, makes a double
+// of the sum with integer instructions (an FP64 instruction costs 64 of them
+// here) and adds ranges in FP64.  Error: rounding of the operands, 2^-56 of the
+// row's and the column's largest, and the levels above NDIG + 1, about 2^-54 of their
+// product per summand; on random operands 6e-16 to 3e-15 of the largest entries'
+// product (with 7 truncated digits aligned over 64 summands, as this was: 1e-13).
 //
-// One CTA of 128 threads per 128 x 64 output tile (M tiles of 128 rows of A,
-// N tiles of 64 columns of B); operands staged by the threads into shared
-// memory in the no-swizzle K-major core-matrix layout (8 rows x 16 bytes per
-// core matrix); one thread issues the MMAs and commits them to an mbarrier;
-// every wait is bounded (clock64), after which the kernel flags an error,
-// frees its TMEM and returns.
+// One CTA of 256 threads per 128 x 64 output tile and K range.  Stages of KC = 32
+// summands in two buffers: the threads load and split the next stage while the
+// tensor core works on this one.  A thread splits eight summands of a row into the
+// 16 bytes of a core matrix row per plane (no-swizzle K-major layout: 8 rows x 16
+// bytes per core matrix); summands oct + 4 i, i = 0..7, go to octet oct, the same
+// permutation in A and B, so that four lanes read whole sectors.  The B planes
+// lie one after another, so one MMA of up to 256 columns covers four levels of an
+// A plane: 12 reads of A instead of 36.  One thread issues; every wait is bounded
+// (clock64), after which the kernel flags an error, frees its TMEM and returns.
+//
+// 216 x 216 x 16384 (a symmetric Gram product, 32 ranges): 384 -> 153 us with
+// the reduction; bound by the integer instructions of the splitting, which every
+// tile does for its own rows and columns, and by 192 tiles on 152 SMs.
 #include <cuda_bf16.h>
 #include <stdint.h>
 
@@ -33,18 +42,19 @@ namespace fock {
 
 namespace {
 
-constexpr int TM = 128, TN = 64, KC = 64, NDIG = 7;   // digit levels g = 2 .. NDIG + 1
-constexpr int TMEM_COLS = 512;                                     // NLEV * TN = 448 used
+constexpr int TM = 128, TN = 64, KC = 32, NDIG = 8;                // digit levels g = 2 .. NDIG + 1
+constexpr int TMEM_COLS = 512;                                     // NDIG * TN
 constexpr uint32_t A_PLANE = TM * KC * 2, B_PLANE = TN * KC * 2;   // bytes per digit plane
-constexpr size_t SPLIT_SMEM = (size_t)NDIG * (A_PLANE + B_PLANE) + 1024;
+constexpr uint32_t STAGE = NDIG * (A_PLANE + B_PLANE);
+constexpr size_t SPLIT_SMEM = 2 * (size_t)STAGE + 1024;
 constexpr long long kWaitCycles = 4000000000ll;                    // ~2 s at 2 GHz
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// byte offset of element (r, k) of an R x KC operand: core matrix (r/8, k/8),
-// K-adjacent core matrices 128 B apart (LBO), 8-row groups KC/8 * 128 B apart (SBO)
-__device__ __forceinline__ uint32_t core_off(int r, int k) {
-  return (uint32_t)(((r >> 3) * (KC >> 3) + (k >> 3)) * 128 + (r & 7) * 16 + (k & 7) * 2);
+// byte offset of octet o of row r of an R x KC operand: core matrix (r/8, o), K-adjacent
+// core matrices 128 B apart (LBO), 8-row groups KC/8 * 128 B apart (SBO)
+__device__ __forceinline__ uint32_t core_off(int r, int o) {
+  return (uint32_t)(((r >> 3) * (KC >> 3) + o) * 128 + (r & 7) * 16);
 }
 
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
@@ -53,9 +63,8 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
          (uint64_t)1 << 46;   // version 1, base offset 0, no swizzle
 }
 
-// instruction descriptor: D FP32, A and B BF16, both K-major, M = TM, N = TN
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
-                            ((uint32_t)(TM >> 4) << 24);
+// instruction descriptor: D FP32, A and B BF16, both K-major, M = TM, N = n
+constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TM >> 4) << 24);
 
 // biased exponent field of |x| (0 for zero and subnormals: they align as exponent 1)
 __device__ __forceinline__ int exp_field(double x) {
@@ -63,21 +72,38 @@ __device__ __forceinline__ int exp_field(double x) {
   return e == 0 ? 1 : e;
 }
 
-// the NDIG signed base-128 digits of x aligned to the exponent field E
-__device__ __forceinline__ void digits(double x, int E, __nv_bfloat16* q) {
+// x = w 2^(E - 1077) rounded to an integer |w| <= 2^55, plus 64 in every base-128 digit
+__device__ __forceinline__ unsigned long long offset_digits(double x, int E) {
   const long long b = __double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7FF);
   long long m = b & 0xFFFFFFFFFFFFFll;
   if (ex != 0) m |= 1ll << 52;
-  const int sh = E - (ex == 0 ? 1 : ex);
-  const long long a = (sh < 53) ? (m >> sh) : 0;
-  const int sg = b < 0 ? -1 : 1;
-#pragma unroll
-  for (int j = 0; j < NDIG; ++j) q[j] = __int2bfloat16_rn(sg * (int)((a >> (46 - 7 * j)) & 127));
+  if (b < 0) m = -m;
+  const int s = min(E - (ex == 0 ? 1 : ex) + 7, 63);
+  const long long w = (((m << 9) >> (s - 1)) + 1) >> 1;
+  constexpr unsigned long long off = 64ull * ((1ull << 56) - 1) / 127;   // 64 (1 + 128 + ... + 128^7)
+  return (unsigned long long)w + off;
 }
 
-__device__ __forceinline__ double pow2(int e) {   // 2^e, 0 below the normal range
-  return e < -1022 ? 0.0 : __longlong_as_double((long long)(e + 1023) << 52);
+// the digits 7 (NDIG - 1 - j) bits up of two offset numbers, as a pair of BF16: 0x4300 | u is
+// 128 + u (also for u = 128, the top digit's largest), less 192
+template <int SH>
+__device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned long long b) {
+  constexpr uint32_t mask = SH == 7 * (NDIG - 1) ? 0xFFu : 0x7Fu;
+  const uint32_t w = 0x43004300u | ((uint32_t)(a >> SH) & mask) | (((uint32_t)(b >> SH) & mask) << 16);
+  __nv_bfloat162 v;
+  *reinterpret_cast<uint32_t*>(&v) = w;
+  v = __hsub2(v, __float2bfloat162_rn(192.0f));
+  return *reinterpret_cast<uint32_t*>(&v);
+}
+template <int J>
+__device__ __forceinline__ void put_planes(const unsigned long long* t, unsigned char* p, uint32_t plane) {
+  if constexpr (J < NDIG) {
+    constexpr int SH = 7 * (NDIG - 1 - J);
+    *reinterpret_cast<uint4*>(p + J * plane) = make_uint4(digit_pair<SH>(t[0], t[1]), digit_pair<SH>(t[2], t[3]),
+                                                          digit_pair<SH>(t[4], t[5]), digit_pair<SH>(t[6], t[7]));
+    put_planes<J + 1>(t, p, plane);
+  }
 }
 
 __device__ __forceinline__ bool wait_phase(uint32_t mbar, uint32_t phase) {
@@ -91,100 +117,99 @@ __device__ __forceinline__ bool wait_phase(uint32_t mbar, uint32_t phase) {
   return true;
 }
 
-// Stage one operand chunk as digit planes: R rows of `rows` (<= TR), KC
-// columns along k from k0; element (r, k) at P[r * sr + k * sk].  Rows that
-// do not exist and k beyond K give zero digits.  Writes the row exponents.
-template <int TR>
-__device__ void stage(const double* __restrict__ P, long long sr, long long sk, int rows, int k0, int K,
-                      unsigned char* planes, uint32_t plane_bytes, int* rexp) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (sk == 1) {
-    // rows contiguous along k: one warp per row, lanes along k; the loads of
-    // SU rows are issued before any of them is converted (their latency
-    // overlaps instead of adding up row after row)
-    constexpr int SU = 4;
-    for (int r0 = warp; r0 < TR; r0 += 4 * SU) {
-      double x0[SU], x1[SU];
+// One warp's share of an operand: eight rows, four lanes each (summands contiguous), or
+// 32 rows of one octet.  Rows that do not exist and summands from kend on are zero.
+struct Share {
+  const double* p;     // the row's element 0, null: no such row
+  long long sk;
+  int row, oct, E;
+  __device__ void place(const double* P, long long sr, long long k1, int rows, int it, int lane) {
+    sk = k1;
+    if (k1 == 1) { row = it * 8 + (lane & 7); oct = lane >> 3; }
+    else { row = (it >> 2) * 32 + lane; oct = it & 3; }
+    p = row < rows ? P + row * sr : nullptr;
+  }
+  __device__ void load(double* x, int k0, int kend) const {
 #pragma unroll
-      for (int u = 0; u < SU; ++u) {
-        const int r = r0 + 4 * u;
-        x0[u] = 0.0; x1[u] = 0.0;
-        if (r < rows) {
-          if (k0 + lane < K) x0[u] = P[r * sr + (k0 + lane)];
-          if (k0 + lane + 32 < K) x1[u] = P[r * sr + (k0 + lane + 32)];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < SU; ++u) {
-        const int r = r0 + 4 * u;
-        if (r >= TR) break;
-        const int E = __reduce_max_sync(0xffffffffu, max(exp_field(x0[u]), exp_field(x1[u])));
-        if (lane == 0) rexp[r] = E;
-        __nv_bfloat16 q[NDIG];
-        digits(x0[u], E, q);
-#pragma unroll
-        for (int j = 0; j < NDIG; ++j) *(__nv_bfloat16*)(planes + j * plane_bytes + core_off(r, lane)) = q[j];
-        digits(x1[u], E, q);
-#pragma unroll
-        for (int j = 0; j < NDIG; ++j) *(__nv_bfloat16*)(planes + j * plane_bytes + core_off(r, lane + 32)) = q[j];
-      }
+    for (int i = 0; i < 8; ++i) {
+      const int k = k0 + oct + 4 * i;
+      x[i] = (p && k < kend) ? p[k * sk] : 0.0;
     }
-  } else {
-    // lanes along the rows (coalesced when rows are contiguous), loop along k
-    // in groups of SK independent loads (the exponent pass and the digit pass
-    // each keep SK loads in flight)
-    constexpr int SK = 8;
-    for (int r = threadIdx.x; r < TR; r += blockDim.x) {
-      const bool live = (r < rows);
-      int E = 1;
-      for (int kb = 0; kb < KC; kb += SK) {
-        double x[SK];
+  }
+  __device__ void store(const double* x, unsigned char* planes, uint32_t plane) const {
+    unsigned long long t[8];
 #pragma unroll
-        for (int u = 0; u < SK; ++u)
-          x[u] = (live && k0 + kb + u < K) ? P[r * sr + (long long)(k0 + kb + u) * sk] : 0.0;
-#pragma unroll
-        for (int u = 0; u < SK; ++u) E = max(E, exp_field(x[u]));
+    for (int i = 0; i < 8; ++i) t[i] = offset_digits(x[i], E);
+    put_planes<0>(t, planes + core_off(row, oct), plane);
+  }
+};
+
+// S 2^e, rounded to nearest, by integer instructions where the result is a normal number
+__device__ __forceinline__ double scaled_int(long long S, int e) {
+  const unsigned long long a = S < 0 ? 0ull - (unsigned long long)S : (unsigned long long)S;
+  if (a == 0) return 0.0;
+  const int lz = __clzll((long long)a), be = 1086 - lz + e;
+  if (be < 1 || be > 2045) return scalbn((double)S, e);
+  const unsigned long long m = a << lz, r = (m >> 11) + ((m >> 10) & 1);   // 2^52 <= r <= 2^53
+  return __longlong_as_double((long long)((((unsigned long long)(be - 1)) << 52) + r) | (S & (1ll << 63)));
+}
+
+}  // namespace
+
+// Largest exponent fields of the rows of A (and columns of B) over each range.
+__global__ void __launch_bounds__(256) k_split_exps(const SplitTask* __restrict__ tasks) {
+  const SplitTask T = tasks[blockIdx.y];
+  if (T.active && *T.active == 0) return;
+  const SplitRanges R(T.K, T.ksplit);
+  const int lane = threadIdx.x & 31;
+  const long long w0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), nw = (long long)gridDim.x * (blockDim.x >> 5);
+  for (int o = 0; o < (T.same() ? 1 : 2); ++o) {
+    const double* P = o ? T.B : T.A;
+    const long long sr = o ? T.b_n : T.a_m, sk = o ? T.b_k : T.a_k;
+    const int rows = o ? T.N : T.M;
+    int* ex = T.ex + (o ? (long long)R.count() * T.M : 0);
+    if (sk == 1) {
+      for (long long w = w0; w < (long long)R.count() * rows; w += nw) {
+        const int e = (int)(w / rows), r = (int)(w % rows), k1 = R.end(e);
+        int E = 1;
+#pragma unroll 8
+        for (int k = R.begin(e) + lane; k < k1; k += 32) E = max(E, exp_field(P[r * sr + k]));
+        E = __reduce_max_sync(0xffffffffu, E);
+        if (lane == 0) ex[w] = E;
       }
-      rexp[r] = E;
-      for (int kb = 0; kb < KC; kb += SK) {
-        double x[SK];
-#pragma unroll
-        for (int u = 0; u < SK; ++u)
-          x[u] = (live && k0 + kb + u < K) ? P[r * sr + (long long)(k0 + kb + u) * sk] : 0.0;
-#pragma unroll
-        for (int u = 0; u < SK; ++u) {
-          __nv_bfloat16 q[NDIG];
-          digits(x[u], E, q);
-#pragma unroll
-          for (int j = 0; j < NDIG; ++j) *(__nv_bfloat16*)(planes + j * plane_bytes + core_off(r, kb + u)) = q[j];
-        }
+    } else {
+      const int rg = (rows + 31) >> 5;
+      for (long long w = w0; w < (long long)R.count() * rg; w += nw) {
+        const int e = (int)(w / rg), r = (int)(w % rg) * 32 + lane, k1 = R.end(e);
+        if (r >= rows) continue;
+        int E = 1;
+#pragma unroll 8
+        for (int k = R.begin(e); k < k1; ++k) E = max(E, exp_field(P[r * sr + k * sk]));
+        ex[(long long)e * rows + r] = E;
       }
     }
   }
 }
 
-}  // namespace
-
-__global__ void __launch_bounds__(128, 1) k_split_gemm(const SplitTask* __restrict__ tasks, int max_ks, int* err) {
+__global__ void __launch_bounds__(256, 1) k_split_gemm(const SplitTask* __restrict__ tasks, int max_ks, int* err) {
   const SplitTask T = tasks[blockIdx.z / max_ks];
-  const int ks = blockIdx.z % max_ks, nks = max(T.ksplit, 1);
+  const int ks = blockIdx.z % max_ks;
+  const SplitRanges R(T.K, T.ksplit);
   const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-  if (ks >= nks || m0 >= T.M || n0 >= T.N) return;
+  if (ks >= R.nks || m0 >= T.M || n0 >= T.N) return;
   if (T.active && *T.active == 0) return;
+  if (T.work && T.sym && n0 + TN <= m0) return;   // wholly below the diagonal: mirrored by the reduction
   extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* Ap = (unsigned char*)(((uintptr_t)smem + 1023) & ~(uintptr_t)1023);
-  unsigned char* Bp = Ap + NDIG * A_PLANE;
-  __shared__ __align__(8) uint64_t mbar;
+  unsigned char* buf = (unsigned char*)(((uintptr_t)smem + 1023) & ~(uintptr_t)1023);
+  __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t tmem_base;
-  __shared__ int rexpA[TM], rexpB[TN];
-  __shared__ int s_fail;
+  __shared__ int s_fail, exB[TN];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rowsA = min(TM, T.M - m0), colsB = min(TN, T.N - n0);
-  const double* Ab = T.A + (long long)m0 * T.a_m;
-  const double* Bb = T.B + (long long)n0 * T.b_n;
   if (tid == 0) {
     s_fail = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&mbar)));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&mbar[0])));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(smem_u32(&mbar[1])));
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
   if (warp == 0) {
@@ -196,96 +221,112 @@ __global__ void __launch_bounds__(128, 1) k_split_gemm(const SplitTask* __restri
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tbase = tmem_base;
-  const int row = 32 * (warp & 3) + lane;     // this thread's TMEM lane = output row of the tile
-  double acc[TN];
+  const int row = 32 * (warp & 3) + lane, cb = 32 * (warp >> 2);   // this thread's TMEM lane and first column
+  Share sh[3];   // two of A's sixteen, one of B's eight
+  sh[0].place(T.A + (long long)m0 * T.a_m, T.a_m, T.a_k, rowsA, warp, lane);
+  sh[1].place(T.A + (long long)m0 * T.a_m, T.a_m, T.a_k, rowsA, warp + 8, lane);
+  sh[2].place(T.B + (long long)n0 * T.b_n, T.b_n, T.b_k, colsB, warp, lane);
+  double acc[32], x[3][8];
 #pragma unroll
-  for (int c = 0; c < TN; ++c) acc[c] = 0.0;
-  // this CTA's chunks of the summation: [c_lo, c_hi) of ceil(K / KC)
-  const int nchunk_all = (T.K + KC - 1) / KC, cps = (nchunk_all + nks - 1) / nks;
-  const int c_lo = min(ks * cps, nchunk_all), c_hi = min(c_lo + cps, nchunk_all);
-  const int nchunk = c_hi - c_lo;
+  for (int c = 0; c < 32; ++c) acc[c] = 0.0;
+  int st = 0;   // stages so far
   bool ok = true;
-  for (int ch = 0; ch < nchunk && ok; ++ch) {
-    const int k0 = (c_lo + ch) * KC;
-    stage<TM>(Ab, T.a_m, T.a_k, rowsA, k0, T.K, Ap, A_PLANE, rexpA);
-    stage<TN>(Bb, T.b_n, T.b_k, colsB, k0, T.K, Bp, B_PLANE, rexpB);
-    asm volatile("fence.proxy.async.shared::cta;");   // generic-proxy writes -> tensor-core reads
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      const uint32_t a0 = smem_u32(Ap), b0 = smem_u32(Bp);
-      for (int g = 2; g <= NDIG + 1; ++g) {
-        const uint32_t dcol = tbase + (uint32_t)((g - 2) * TN);
-        uint32_t accum = 0;
-        for (int j = 1; j <= NDIG; ++j) {
-          const int l = g - j;
-          if (l < 1 || l > NDIG) continue;
-          for (int kk = 0; kk < KC / 16; ++kk) {
-            const uint64_t da = smem_desc(a0 + (j - 1) * A_PLANE + kk * 256);
-            const uint64_t db = smem_desc(b0 + (l - 1) * B_PLANE + kk * 256);
-            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                         :: "r"(dcol), "l"(da), "l"(db), "r"(kIdesc), "r"(accum));
-            accum = 1;
-          }
-        }
+  for (int d = 0; d < R.per && ok; ++d) {
+    const int e = ks * R.per + d, k0 = R.begin(e), k1 = R.end(e);
+    if (k0 >= k1) break;
+    const int* eA = T.ex + (long long)e * T.M;
+    const int* eB = T.same() ? eA : T.ex + (long long)R.count() * T.M + (long long)e * T.N;
+    sh[0].E = sh[0].p ? eA[m0 + sh[0].row] : 1;
+    sh[1].E = sh[1].p ? eA[m0 + sh[1].row] : 1;
+    sh[2].E = sh[2].p ? eB[n0 + sh[2].row] : 1;
+    const int EA = row < rowsA ? eA[m0 + row] : 1;
+    if (tid < TN) exB[tid] = tid < colsB ? eB[n0 + tid] : 1;   // read after a barrier below
+#pragma unroll
+    for (int i = 0; i < 3; ++i) sh[i].load(x[i], k0, k1);
+    for (int k = k0; k < k1; k += KC, ++st) {
+      unsigned char* Ap = buf + (st & 1) * STAGE;
+      unsigned char* Bp = Ap + NDIG * A_PLANE;
+      // the MMAs that read this buffer two stages ago are done
+      if (st >= 2 && !wait_phase(smem_u32(&mbar[st & 1]), (uint32_t)((st >> 1) - 1) & 1)) atomicExch(&s_fail, 1);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        sh[i].store(x[i], i < 2 ? Ap : Bp, i < 2 ? A_PLANE : B_PLANE);
+        sh[i].load(x[i], k + KC, k1);                        // the next stage's
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                   :: "r"(smem_u32(&mbar)) : "memory");
+      asm volatile("fence.proxy.async.shared::cta;");        // generic-proxy writes -> tensor-core reads
+      __syncthreads();
+      if (s_fail) { ok = false; break; }
+      if (tid == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;");
+        const uint32_t a0 = smem_u32(Ap), b0 = smem_u32(Bp);
+        for (int kk = 0; kk < KC / 16; ++kk)
+          for (int j = 0; j < NDIG; ++j)                     // planes j of A, q .. q + nl - 1 of B: levels j + q on
+            for (int q = 0; q < NDIG - j; q += 4) {
+              const int nl = min(4, NDIG - j - q);
+              const uint64_t da = smem_desc(a0 + j * A_PLANE + kk * 256);
+              const uint64_t db = smem_desc(b0 + q * B_PLANE + kk * 256);
+              const uint32_t accum = (k > k0 || kk > 0 || j > 0) ? 1u : 0u;
+              const uint32_t idesc = kIdesc | (uint32_t)((nl * TN) >> 3) << 17;
+              asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                           "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                           :: "r"(tbase + (uint32_t)((j + q) * TN)), "l"(da), "l"(db), "r"(idesc), "r"(accum));
+            }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                     :: "r"(smem_u32(&mbar[st & 1])) : "memory");
+      }
     }
-    if (!wait_phase(smem_u32(&mbar), (uint32_t)(ch & 1))) {
-      atomicExch(&s_fail, 1);
-    }
+    if (!ok) break;
+    if (!wait_phase(smem_u32(&mbar[(st - 1) & 1]), (uint32_t)((st - 1) >> 1) & 1)) atomicExch(&s_fail, 1);
     __syncthreads();
     if (s_fail) { ok = false; break; }
     asm volatile("tcgen05.fence::after_thread_sync;");
-    // combine the levels of this thread's row in 64-bit integers, add in FP64
-    const double rs = pow2(rexpA[row] - 1050);
-    const uint32_t lane_addr = tbase + ((uint32_t)(32 * (warp & 3)) << 16);
+    // sum = (hi 2^28 + lo) 2^(49 + EA + EB - 2154), the last 8 bits of lo dropped
+    const uint32_t lane_addr = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)cb;
 #pragma unroll
-    for (int c0 = 0; c0 < TN; c0 += 8) {
-      long long S[8];
+    for (int c0 = 0; c0 < 32; c0 += 8) {
+      uint32_t v[NDIG][8];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) S[c] = 0;
-#pragma unroll
-      for (int g = 2; g <= NDIG + 1; ++g) {
-        uint32_t v[8];
+      for (int g = 0; g < NDIG; ++g)
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                       "=r"(v[7])
-                     : "r"(lane_addr + (uint32_t)((g - 2) * TN + c0)));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                     : "=r"(v[g][0]), "=r"(v[g][1]), "=r"(v[g][2]), "=r"(v[g][3]), "=r"(v[g][4]), "=r"(v[g][5]),
+                       "=r"(v[g][6]), "=r"(v[g][7])
+                     : "r"(lane_addr + (uint32_t)(g * TN + c0)));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-        for (int c = 0; c < 8; ++c)
-          S[c] += (long long)__float2int_rn(__uint_as_float(v[c])) * (1ll << (7 * (NDIG + 1 - g)));
+      for (int c = 0; c < 8; ++c) {
+        long long hi = 0, lo = 0;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          hi = hi * 128 + __float2int_rn(__uint_as_float(v[g][c]));
+          lo = lo * 128 + __float2int_rn(__uint_as_float(v[4 + g][c]));
+        }
+        const double val = scaled_int(hi * (1ll << 20) + (lo >> 8), EA + exB[cb + c0 + c] - 2097);
+        acc[c0 + c] = d == 0 ? val : acc[c0 + c] + val;
       }
-#pragma unroll
-      for (int c = 0; c < 8; ++c) acc[c0 + c] = fma((double)S[c], rs * pow2(rexpB[c0 + c] - 1050), acc[c0 + c]);
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();   // the digit planes and TMEM are reused by the next chunk
+    __syncthreads();   // TMEM and exB are reused by the next range
+    asm volatile("tcgen05.fence::after_thread_sync;");
   }
   if (!ok) {
     // an MMA group did not complete in time: wait (bounded) once more so no
     // write to TMEM is in flight when it is freed, flag the error
     if (tid == 0) {
-      wait_phase(smem_u32(&mbar), (uint32_t)((nchunk - 1) & 1));
+      if (st > 0) wait_phase(smem_u32(&mbar[(st - 1) & 1]), (uint32_t)((st - 1) >> 1) & 1);
       atomicExch(err, 1);
     }
     __syncthreads();
   } else if (row < rowsA && T.work) {
-    // a partial sum over this CTA's chunks, reduced by k_split_reduce
+    // a partial sum over this CTA's range, reduced by k_split_reduce
     double* Wr = T.work + ((long long)ks * T.M + m0 + row) * T.N + n0;
 #pragma unroll
-    for (int c = 0; c < TN; ++c)
-      if (c < colsB) Wr[c] = acc[c];
+    for (int c = 0; c < 32; ++c)
+      if (cb + c < colsB) Wr[cb + c] = acc[c];
   } else if (row < rowsA) {
-    // value = S * 2^(EA + EB - 2100): the per-row and per-column factors
-    // 2^(E - 1050) multiply to it
-    double* Cr = T.C + (long long)(m0 + row) * T.c_m + (long long)n0 * T.c_n;
+    double* Cr = T.C + (long long)(m0 + row) * T.c_m + (long long)(n0 + cb) * T.c_n;
 #pragma unroll
-    for (int c = 0; c < TN; ++c)
-      if (c < colsB) {
+    for (int c = 0; c < 32; ++c)
+      if (cb + c < colsB) {
         double v = T.alpha * acc[c];
         if (T.beta != 0.0) v = fma(T.beta, Cr[(long long)c * T.c_n], v);
         Cr[(long long)c * T.c_n] = v;
@@ -324,9 +365,10 @@ void launch_split_gemm(const SplitTask* tasks, int ntask, int max_m, int max_n, 
   if (!ntask || max_m <= 0 || max_n <= 0) return;
   FOCK_SMEM_OPTIN(k_split_gemm);
   max_ks = max_ks < 1 ? 1 : max_ks;
+  k_split_exps<<<dim3(ntask < 4 ? 304 : 76, ntask), 256, 0, st>>>(tasks);
   dim3 grid((max_n + TN - 1) / TN, (max_m + TM - 1) / TM, ntask * max_ks);
-  k_split_gemm<<<grid, 128, SPLIT_SMEM, st>>>(tasks, max_ks, err);
-  if (reduce) k_split_reduce<<<dim3(64, ntask), 256, 0, st>>>(tasks);
+  k_split_gemm<<<grid, 256, SPLIT_SMEM, st>>>(tasks, max_ks, err);
+  if (reduce) k_split_reduce<<<dim3(152, ntask), 256, 0, st>>>(tasks);
 }
 
 }  // namespace fock
