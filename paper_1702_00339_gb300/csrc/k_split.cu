@@ -8,14 +8,14 @@
 //
 // Over a range of up to RANGE = 512 of the summation index, every row of A and
 // every column of B is aligned to its largest binary exponent (k_split_exps) and
-// rounded to 55 bits below it, which are written as NDIG = 8 balanced base-128
-// digits (-64 .. 64, exact in BF16).  For each level g = j + l (2 <= g <= NDIG + 1)
+// cut to 55 bits below it, which are written as NDIG = 8 balanced base-128
+// digits (-64 .. 64, exact in FP16).  For each level g = j + l (2 <= g <= NDIG + 1)
 // the products of digit planes j of A and l of B are summed by tcgen05.mma
-// (kind::f16, BF16 x BF16 -> FP32) into one TMEM accumulator per level: at most
+// (kind::f16, FP16 x FP16 -> FP32) into one TMEM accumulator per level: at most
 // 8 x 512 x 64^2 = 2^24, so FP32 accumulation is exact over a whole range.
 // Then each thread combines its row's levels in 64-bit integers, makes a double
 // of the sum with integer instructions (an FP64 instruction costs 64 of them
-// here) and adds ranges in FP64.  Error: rounding of the operands, 2^-56 of the
+// here) and adds ranges in FP64.  Error: cutting the operands, 2^-55 of the
 // row's and the column's largest, and the levels above NDIG + 1, about 2^-54 of their
 // product per summand; on random operands 6e-16 to 3e-15 of the largest entries'
 // product (with 7 truncated digits aligned over 64 summands, as this was: 1e-13).
@@ -30,10 +30,10 @@
 // A plane: 12 reads of A instead of 36.  One thread issues; every wait is bounded
 // (clock64), after which the kernel flags an error, frees its TMEM and returns.
 //
-// 216 x 216 x 16384 (a symmetric Gram product, 32 ranges): 384 -> 153 us with
-// the reduction; bound by the integer instructions of the splitting, which every
+// 216 x 216 x 16384 (a symmetric Gram product, 32 ranges): 384 -> 140 us with
+// the reduction; bound by the splitting, 55 instructions per summand and row that every
 // tile does for its own rows and columns, and by 192 tiles on 152 SMs.
-#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <stdint.h>
 
 #include "common.cuh"
@@ -63,8 +63,8 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
          (uint64_t)1 << 46;   // version 1, base offset 0, no swizzle
 }
 
-// instruction descriptor: D FP32, A and B BF16, both K-major, M = TM, N = n
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TM >> 4) << 24);
+// instruction descriptor: D FP32, A and B FP16, both K-major, M = TM, N = n
+constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(TM >> 4) << 24);
 
 // biased exponent field of |x| (0 for zero and subnormals: they align as exponent 1)
 __device__ __forceinline__ int exp_field(double x) {
@@ -72,38 +72,40 @@ __device__ __forceinline__ int exp_field(double x) {
   return e == 0 ? 1 : e;
 }
 
-// x = w 2^(E - 1077) rounded to an integer |w| <= 2^55, plus 64 in every base-128 digit
-__device__ __forceinline__ unsigned long long offset_digits(double x, int E) {
-  const long long b = __double_as_longlong(x);
-  const int ex = (int)((b >> 52) & 0x7FF);
-  long long m = b & 0xFFFFFFFFFFFFFll;
-  if (ex != 0) m |= 1ll << 52;
-  if (b < 0) m = -m;
-  const int s = min(E - (ex == 0 ? 1 : ex) + 7, 63);
-  const long long w = (((m << 9) >> (s - 1)) + 1) >> 1;
+// x = w 2^(E - 1077), cut to an integer |w| <= 2^55, plus 64 in every base-128 digit: the low
+// and the high word
+__device__ __forceinline__ uint2 offset_digits(double x, int E) {
+  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+  const int ex = (int)((h >> 20) & 0x7FF), s = min(E - max(ex, 1), 63);
+  const uint32_t mh = (h & 0xFFFFFu) + (uint32_t)min(ex, 1) * 0x100000u;
+  uint32_t a = l << 2, b = __funnelshift_l(l, mh, 2);
+  if (s >= 32) { a = b; b = 0; }
+  a = __funnelshift_r(a, b, s & 31);
+  b >>= s & 31;
+  const uint32_t sg = (uint32_t)((int)h >> 31);
   constexpr unsigned long long off = 64ull * ((1ull << 56) - 1) / 127;   // 64 (1 + 128 + ... + 128^7)
-  return (unsigned long long)w + off;
+  const unsigned long long t = ((unsigned long long)(b ^ sg) << 32 | (a ^ sg)) +
+                               ((unsigned long long)(uint32_t)(off >> 32) << 32 | ((uint32_t)off - sg));
+  return make_uint2((uint32_t)t, (uint32_t)(t >> 32));
 }
 
-// the digits 7 (NDIG - 1 - j) bits up of two offset numbers, as a pair of BF16: 0x4300 | u is
-// 128 + u (also for u = 128, the top digit's largest), less 192
-template <int SH>
-__device__ __forceinline__ uint32_t digit_pair(unsigned long long a, unsigned long long b) {
-  constexpr uint32_t mask = SH == 7 * (NDIG - 1) ? 0xFFu : 0x7Fu;
-  const uint32_t w = 0x43004300u | ((uint32_t)(a >> SH) & mask) | (((uint32_t)(b >> SH) & mask) << 16);
-  __nv_bfloat162 v;
+// A digit of two offset numbers as a pair of FP16, from the words a and b that hold it at byte P,
+// bit O (at most 3): a byte permutation and a mask put u 2^O into the mantissas of 1024, one
+// packed FMA takes the offsets off and the scale away (exact).
+template <int P, int O, uint32_t MASK>
+__device__ __forceinline__ uint32_t digit_pair(uint32_t a, uint32_t b) {
+  constexpr uint32_t q = P < 3 ? P + 1 : 3, sel = P | q << 4 | (P + 4) << 8 | (q + 4) << 12;
+  constexpr uint32_t m = MASK << O;
+  const uint32_t w = (__byte_perm(a, b, sel) & (m | m << 16)) | 0x64006400u;
+  __half2 v;
   *reinterpret_cast<uint32_t*>(&v) = w;
-  v = __hsub2(v, __float2bfloat162_rn(192.0f));
+  v = __hfma2(v, __float2half2_rn(1.0f / (1 << O)), __float2half2_rn(-1024.0f / (1 << O) - 64.0f));
   return *reinterpret_cast<uint32_t*>(&v);
 }
-template <int J>
-__device__ __forceinline__ void put_planes(const unsigned long long* t, unsigned char* p, uint32_t plane) {
-  if constexpr (J < NDIG) {
-    constexpr int SH = 7 * (NDIG - 1 - J);
-    *reinterpret_cast<uint4*>(p + J * plane) = make_uint4(digit_pair<SH>(t[0], t[1]), digit_pair<SH>(t[2], t[3]),
-                                                          digit_pair<SH>(t[4], t[5]), digit_pair<SH>(t[6], t[7]));
-    put_planes<J + 1>(t, p, plane);
-  }
+template <int P, int O, uint32_t MASK>
+__device__ __forceinline__ void put_plane(const uint32_t* w, unsigned char* p) {
+  *reinterpret_cast<uint4*>(p) = make_uint4(digit_pair<P, O, MASK>(w[0], w[1]), digit_pair<P, O, MASK>(w[2], w[3]),
+                                            digit_pair<P, O, MASK>(w[4], w[5]), digit_pair<P, O, MASK>(w[6], w[7]));
 }
 
 __device__ __forceinline__ bool wait_phase(uint32_t mbar, uint32_t phase) {
@@ -137,10 +139,23 @@ struct Share {
     }
   }
   __device__ void store(const double* x, unsigned char* planes, uint32_t plane) const {
-    unsigned long long t[8];
+    uint32_t lo[8], hi[8], l4[8];   // l4: the number four bits down, low word
 #pragma unroll
-    for (int i = 0; i < 8; ++i) t[i] = offset_digits(x[i], E);
-    put_planes<0>(t, planes + core_off(row, oct), plane);
+    for (int i = 0; i < 8; ++i) {
+      const uint2 t = offset_digits(x[i], E);
+      lo[i] = t.x;
+      hi[i] = t.y;
+      l4[i] = __funnelshift_r(t.x, t.y, 4);
+    }
+    unsigned char* p = planes + core_off(row, oct);
+    put_plane<2, 1, 0xFF>(hi, p);              // bit 49; up to 128
+    put_plane<1, 2, 0x7F>(hi, p + plane);      // 42
+    put_plane<0, 3, 0x7F>(hi, p + 2 * plane);  // 35
+    put_plane<3, 0, 0x7F>(l4, p + 3 * plane);  // 28
+    put_plane<2, 1, 0x7F>(l4, p + 4 * plane);  // 21
+    put_plane<1, 2, 0x7F>(l4, p + 5 * plane);  // 14
+    put_plane<0, 3, 0x7F>(l4, p + 6 * plane);  // 7
+    put_plane<0, 0, 0x7F>(lo, p + 7 * plane);  // 0
   }
 };
 
@@ -350,6 +365,7 @@ __global__ void k_split_reduce(const SplitTask* __restrict__ tasks) {
     const int m = (int)(it / T.N), n = (int)(it % T.N);
     if (T.sym && m > n) continue;
     double s = 0.0;
+#pragma unroll 8
     for (int ks = 0; ks < nks; ++ks) s += T.work[ks * mn + it];
     double* c = T.C + (long long)m * T.c_m + (long long)n * T.c_n;
     const double v = (T.beta != 0.0) ? fma(T.beta, *c, T.alpha * s) : T.alpha * s;
