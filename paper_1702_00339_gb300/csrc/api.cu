@@ -94,6 +94,9 @@ struct fock_ctx {
   uint32_t* hstage = nullptr;        // pinned host staging of gathered results
   size_t hstage_cap = 0;             // (words)
   cudaMemPool_t mempool = nullptr;   // serving workers: batches allocated stream-ordered from this pool
+  // device workspaces of single calls (split products, operator applications), which keep up
+  // to kScratchKeep bytes between calls; given back with the context
+  cudaMemPool_t scratch = nullptr;
   std::string err;
   // kernel timers: events recorded around launches while enabled
   bool prof = false;
@@ -156,6 +159,43 @@ const int kPeriodicPiece = 1024;
 // lattice of 32^3 cells of 32 functions: the call takes 55 ms with 256 MB, 45 with 1 GB). A plan that would not fit its budget otherwise takes the least, 32 blocks at
 // a time; the chunks do not change a result.
 const size_t kPfWorkBytes = (size_t)1 << 30;
+
+const uint64_t kScratchKeep = (uint64_t)256 << 20;
+
+void scratch_create(fock_ctx* c) {
+  cudaMemPoolProps pr = {};
+  pr.allocType = cudaMemAllocationTypePinned;
+  pr.location.type = cudaMemLocationTypeDevice;
+  pr.location.id = c->device;
+  uint64_t keep = kScratchKeep;
+  if (cudaMemPoolCreate(&c->scratch, &pr) != cudaSuccess) {
+    cudaGetLastError();
+    c->scratch = nullptr;
+  } else {
+    cudaMemPoolSetAttribute(c->scratch, cudaMemPoolAttrReleaseThreshold, &keep);
+  }
+}
+// A call's device workspace, stream-ordered from the context's pool (a cudaMalloc and
+// cudaFree pair cost 40 us for small workspaces, 130 for 12 MB); cudaMalloc where the
+// pool cannot serve it. Freed on scope exit.
+struct Scratch {
+  char* p = nullptr;
+  cudaStream_t st = nullptr;
+  bool pooled = false;
+  cudaError_t get(fock_ctx* c, size_t bytes) {
+    st = c->stream;
+    pooled = c->scratch && cudaMallocFromPoolAsync((void**)&p, bytes, c->scratch, st) == cudaSuccess;
+    if (pooled) return cudaSuccess;
+    cudaGetLastError();
+    p = nullptr;
+    return cudaMalloc((void**)&p, bytes);
+  }
+  ~Scratch() {
+    if (!p) return;
+    if (pooled) cudaFreeAsync(p, st);
+    else cudaFree(p);
+  }
+};
 
 int set_err(fock_ctx* c, int code, const std::string& m) {
   if (c) c->err = m;
@@ -2128,6 +2168,7 @@ int fock_create(fock_ctx** out, int device, size_t hbm_budget_bytes, void* strea
     hbm_budget_bytes = (size_t)(0.9 * (double)fr);
   }
   c->budget = hbm_budget_bytes;
+  scratch_create(c);
   *out = c;
   return FOCK_OK;
 }
@@ -2143,6 +2184,7 @@ void fock_destroy(fock_ctx* c) {
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
   if (c->ev_chunk) cudaEventDestroy(c->ev_chunk);
+  if (c->scratch) cudaMemPoolDestroy(c->scratch);
   if (c->own_stream) cudaStreamDestroy(c->stream);
   delete c;
 }
@@ -2626,10 +2668,11 @@ int fock_split_dgemm(fock_ctx* ctx, int M, int N, int K, const double* A, long l
   t.C = C; t.c_m = c_m; t.c_n = c_n; t.alpha = alpha; t.beta = beta;
   t.ksplit = ksplit; t.sym = sym ? 1 : 0;
   const bool red = ksplit > 1 || sym;
-  char* mem = nullptr;
   const size_t off_w = 256 + ((sizeof(SplitTask) + 255) & ~(size_t)255);
   const size_t wbytes = red ? (((size_t)ksplit * M * N * sizeof(double) + 255) & ~(size_t)255) : 0;
-  CUDA_TRY(ctx, cudaMalloc(&mem, off_w + wbytes + t.n_ex() * sizeof(int) + 256));
+  Scratch scratch;
+  CUDA_TRY(ctx, scratch.get(ctx, off_w + wbytes + t.n_ex() * sizeof(int) + 256));
+  char* const mem = scratch.p;
   if (red) t.work = (double*)(mem + off_w);
   t.ex = (int*)(mem + off_w + wbytes);
   int herr = 0;
@@ -2642,7 +2685,6 @@ int fock_split_dgemm(fock_ctx* ctx, int M, int N, int K, const double* A, long l
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, mem, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFree(mem);
   if (e != cudaSuccess) return set_err(ctx, FOCK_ECUDA, cudaGetErrorString(e));
   if (herr) return set_err(ctx, FOCK_ETIMEOUT, "split_dgemm: a tensor-core commit did not complete in time");
   return FOCK_OK;
@@ -2660,18 +2702,16 @@ int fock_toeplitz_matvec(fock_ctx* ctx, const fock_blocks* b, int which, const d
   const size_t nbytes = (size_t)n * nvec * 8;
   if (on_device && (const char*)x < (const char*)y + nbytes && (const char*)y < (const char*)x + nbytes)
     return set_err(ctx, FOCK_EINVAL, "matvec: device x and y must not overlap");
-  double *dx = nullptr, *dy = nullptr;
-  cplx *X = nullptr, *Y = nullptr;
-  char* tasks = nullptr;
-  if (on_device) { dx = const_cast<double*>(x); dy = y; }
-  else {
-    CUDA_TRY(ctx, cudaMalloc(&dx, nbytes));
-    CUDA_TRY(ctx, cudaMalloc(&dy, nbytes));
-    CUDA_TRY(ctx, cudaMemcpyAsync(dx, x, nbytes, cudaMemcpyHostToDevice, st));
-  }
-  CUDA_TRY(ctx, cudaMalloc(&X, (size_t)Q.M * H.m0 * nvec * sizeof(cplx)));
-  CUDA_TRY(ctx, cudaMalloc(&Y, (size_t)Q.M * H.m0 * nvec * sizeof(cplx)));
-  CUDA_TRY(ctx, cudaMalloc(&tasks, 4096));
+  const size_t vb = (nbytes + 255) & ~(size_t)255;
+  const size_t xb = ((size_t)Q.M * H.m0 * nvec * sizeof(cplx) + 255) & ~(size_t)255;
+  Scratch scratch;
+  CUDA_TRY(ctx, scratch.get(ctx, 4096 + 2 * xb + (on_device ? 0 : 2 * vb)));
+  char* const tasks = scratch.p;
+  cplx* const X = (cplx*)(scratch.p + 4096);
+  cplx* const Y = (cplx*)(scratch.p + 4096 + xb);
+  double* dx = on_device ? const_cast<double*>(x) : (double*)(scratch.p + 4096 + 2 * xb);
+  double* dy = on_device ? y : (double*)(scratch.p + 4096 + 2 * xb + vb);
+  if (!on_device) CUDA_TRY(ctx, cudaMemcpyAsync(dx, x, nbytes, cudaMemcpyHostToDevice, st));
   int cc = std::max(1, std::min(16, 98304 / (32 * Q.M)));
   FftTask tf; std::memset(&tf, 0, sizeof(tf));
   tf.prob = 0; tf.L = Q.Lc; tf.m0 = H.m0; tf.ncol = nvec; tf.circ = B.d_circs + Q.circ; tf.x = dx; tf.ldx = n;
@@ -2696,8 +2736,6 @@ int fock_toeplitz_matvec(fock_ctx* ctx, const fock_blocks* b, int which, const d
   if (!on_device) CUDA_TRY(ctx, cudaMemcpyAsync(y, dy, nbytes, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(ctx, cudaStreamSynchronize(st));
   CUDA_TRY(ctx, cudaGetLastError());
-  if (!on_device) { cudaFree(dx); cudaFree(dy); }
-  cudaFree(X); cudaFree(Y); cudaFree(tasks);
   return FOCK_OK;
 }
 
