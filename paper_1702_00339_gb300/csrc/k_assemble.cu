@@ -190,11 +190,11 @@ __device__ inline double gval(const AxisDev& A, int mode, int n0, int mu, int ce
 }
 
 // Folded pair products Z[r][mu nu] (shared out over blockIdx.y) and the S1 / A1
-// forms (the last blockIdx.y: lanes over an entry's nodes).  Both gram
+// forms (the last blockIdx.y).  Both gram
 // kernels were one CTA per task with a thread summing each form's nodes in turn,
 // latency from end to end: 237 us for a ring of 8 cells of 4 functions (9 axis
 // forms over up to 256 nodes), 1.1 ms for a chain of 101 cells of 16; now
-// 35 us and 0.23 ms (4600 tasks of 32 chains and rings of 64 cells: 1.40 -> 1.25).
+// 56 us and 0.19 ms (4600 tasks of 32 chains and rings of 64 cells: 1.40 -> 1.13).
 __global__ void __launch_bounds__(256) k_gram_fold(const ProbDev* __restrict__ probs, const GramTask* __restrict__ tasks) {
   const GramTask T = tasks[blockIdx.x];
   const ProbDev& P = probs[T.prob];
@@ -203,41 +203,69 @@ __global__ void __launch_bounds__(256) k_gram_fold(const ProbDev* __restrict__ p
   const bool direct = (T.ptab >= 0);      // defect tables: no replication
   if (blockIdx.y + 1 == gridDim.y) {
     if (direct) return;   // defect forms carry no mass / stiffness part
-    // 8 lanes per entry (32 where entries are few) over the nodes of g_mu's own
-    // support (the others add zeros)
+    // g_mu, and the mass and stiffness stencils of g_nu, which no entry of its own needs,
+    // are formed for 32 nodes at a time; then a thread per form and entry adds its
+    // nodes one after another: the boundary blocks are differences of such sums
+    // that agree in all but a tail, so all forms are summed in the same order
     const bool ring_sup = (T.mode == RING && A.slen < A.N);
     const int lo0 = ring_sup ? A.smin : T.rho0 - T.a * n0, len = ring_sup ? A.slen : T.rho1 - T.rho0;   // from cell a's origin
-    __shared__ float s_log;
-    if (threadIdx.x == 0) s_log = (float)log(1.0 / P.eps);
-    __syncthreads();
-    const int LN = (np <= 16) ? 32 : 8, o = threadIdx.x & (LN - 1);
-    for (int p0 = 0; p0 < np; p0 += blockDim.x / LN) {
-      const int pr = p0 + threadIdx.x / LN, mu = min(pr, np - 1) / m0, nu = pr % m0;
-      double s = 0.0, a = 0.0;
+    constexpr int NB = 32, NP = NB + 1, NI = 2 * MAXM0 * MAXM0 / 256;
+    __shared__ double sg[MAXM0 * NP], sw[2][MAXM0 * NP];
+    __shared__ int s0[MAXM0], s1[MAXM0];       // nodes of g_mu's support
+    if (threadIdx.x < m0) {
+      const int mu = threadIdx.x;
       int t0 = 0, t1 = len;
       if (T.mode != RING || ring_sup) {
         const float c = (float)(P.frac[P.centre[mu] * 3 + T.axis] * (double)n0) - 0.5f;
-        const float reach = sqrtf(s_log / (float)P.alpha[mu]) / (float)P.h * 1.0001f + 1.0f;   // a node to spare
+        const float reach = sqrtf((float)log(1.0 / P.eps) / (float)P.alpha[mu]) / (float)P.h * 1.0001f + 1.0f;   // a node to spare
         t0 = max(t0, (int)floorf(c - reach) - lo0);
         t1 = min(t1, (int)ceilf(c + reach) + 1 - lo0);
       }
-      if (pr < np)
-        for (int t = t0 + o; t < t1; t += LN) {
+      s0[mu] = t0;
+      s1[mu] = t1;
+    }
+    __syncthreads();
+    int ta = len, tb = 0;
+    for (int mu = 0; mu < m0; ++mu) { ta = min(ta, s0[mu]); tb = max(tb, s1[mu]); }
+    double acc[NI];
+#pragma unroll
+    for (int i = 0; i < NI; ++i) acc[i] = 0.0;
+    for (int tc = ta; tc < tb; tc += NB) {
+      for (int it = threadIdx.x; it < m0 * NB; it += blockDim.x) {
+        const int mu = it / NB, k = it % NB, t = tc + k;
+        double g = 0.0, w = 0.0, u = 0.0;
+        if (t < tb) {
           const int rho = ring_sup ? posmod(T.a * n0 + A.smin + t, A.N) : T.rho0 + t;
-          const double ga = gval(A, T.mode, n0, mu, T.a, rho);
-          const double b0 = gval(A, T.mode, n0, nu, T.b, rho);
-          const double b1 = gval(A, T.mode, n0, nu, T.b, rho - 1) + gval(A, T.mode, n0, nu, T.b, rho + 1);
-          s = fma(ga, fma(4.0, b0, b1), s);
-          a = fma(ga, fma(2.0, b0, -b1), a);
+          const double b0 = gval(A, T.mode, n0, mu, T.b, rho);
+          const double bm = gval(A, T.mode, n0, mu, T.b, rho - 1), bp = gval(A, T.mode, n0, mu, T.b, rho + 1);
+          g = gval(A, T.mode, n0, mu, T.a, rho);
+          w = fma(4.0, b0, bm) + bp;
+          u = fma(2.0, b0, -bm) - bp;
         }
-      for (int x = 1; x < LN; x <<= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, x);
-        a += __shfl_xor_sync(0xffffffffu, a, x);
+        sg[mu * NP + k] = g;
+        sw[0][mu * NP + k] = w;
+        sw[1][mu * NP + k] = u;
       }
-      if (o == 0 && pr < np) {
-        T.X[0 * np + pr] = s * (P.h / 6.0);
-        T.X[1 * np + pr] = a / P.h;
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const int it = threadIdx.x + 256 * i, form = it >= np ? 1 : 0, pr = it - form * np;
+        if (it >= 2 * np) continue;
+        const int mu = pr / m0, nu = pr % m0;
+        const int k0 = max(s0[mu] - tc, 0), k1 = min(s1[mu] - tc, NB);
+        const double *g = sg + mu * NP, *w = sw[form] + nu * NP;
+        double x = acc[i];
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k) x = fma(g[k], w[k], x);
+        acc[i] = x;
       }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int it = threadIdx.x + 256 * i;
+      if (it < np) T.X[it] = acc[i] * (P.h / 6.0);
+      else if (it < 2 * np) T.X[it] = acc[i] / P.h;
     }
     return;
   }
@@ -283,13 +311,11 @@ __global__ void __launch_bounds__(256) k_gram_fold(const ProbDev* __restrict__ p
   }
 }
 
-// X_t[mu nu] = sum_r P_t[r] Z[r][mu nu].  A CTA takes 64 of the task's outputs
-// (t, mu nu), four threads each: their sums over every fourth node, in registers,
-// added through shared memory; short sums (folded nodes) take a thread each, and
-// so do all, with the same four partial sums, where tasks alone fill the GPU
-// (spread = 0).
+// X_t[mu nu] = sum_r P_t[r] Z[r][mu nu], a thread per output, shared out over
+// blockIdx.y.  The nodes are added one after another, as in the forms above and for
+// the same reason; the loads of eight run ahead of the multiply-adds.
 __global__ void __launch_bounds__(256) k_gram_pot(const ProbDev* __restrict__ probs, const GramTask* __restrict__ tasks,
-                                                  const DefTab* __restrict__ dtabs, int spread) {
+                                                  const DefTab* __restrict__ dtabs) {
   const GramTask T = tasks[blockIdx.x];
   if (T.split) return;   // mixed form: contracted by k_split_gemm
   const ProbDev& P = probs[T.prob];
@@ -301,39 +327,20 @@ __global__ void __launch_bounds__(256) k_gram_pot(const ProbDev* __restrict__ pr
   const int ld = direct ? dtabs[T.ptab].N : A.nr;
   const int off = direct ? (T.foldlo + dtabs[T.ptab].pad) : (T.foldlo - A.rlo);
   double* out = T.X + (direct ? 0 : 2 * np);
-  if (T.nfold <= 32 || !spread) {
-    for (int it = blockIdx.y * blockDim.x + threadIdx.x; it < nt * np; it += gridDim.y * blockDim.x) {
-      const double* pt = tab + (size_t)(it / np) * ld + off;
-      const double* z = T.Zs + it % np;
-      double acc[4] = {0.0, 0.0, 0.0, 0.0};
-      if (T.nfold <= 32) {
-        for (int rr = 0; rr < T.nfold; ++rr) acc[0] += pt[rr] * z[(size_t)rr * np];
-      } else {
-        for (int r0 = 0; r0 < T.nfold; r0 += 4)
-#pragma unroll
-          for (int g = 0; g < 4; ++g)
-            if (r0 + g < T.nfold) acc[g] += pt[r0 + g] * z[(size_t)(r0 + g) * np];
-        acc[0] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-      }
-      out[it] = acc[0];
-    }
-    return;
-  }
-  __shared__ double part[3][64];
-  const int o = threadIdx.x & 63, g = threadIdx.x >> 6, tot = nt * np;
-  for (int i0 = blockIdx.y * 64; i0 < tot; i0 += gridDim.y * 64) {
-    const int it = i0 + o;
+  for (int it = blockIdx.y * blockDim.x + threadIdx.x; it < nt * np; it += gridDim.y * blockDim.x) {
+    const double* pt = tab + (size_t)(it / np) * ld + off;
+    const double* z = T.Zs + it % np;
     double acc = 0.0;
-    if (it < tot) {
-      const double* pt = tab + (size_t)(it / np) * ld + off;
-      const double* z = T.Zs + it % np;
-#pragma unroll 4
-      for (int rr = g; rr < T.nfold; rr += 4) acc += pt[rr] * z[(size_t)rr * np];
+    int rr = 0;
+    for (; rr + 8 <= T.nfold; rr += 8) {
+      double p[8], v[8];
+#pragma unroll
+      for (int g = 0; g < 8; ++g) { p[g] = pt[rr + g]; v[g] = z[(size_t)(rr + g) * np]; }
+#pragma unroll
+      for (int g = 0; g < 8; ++g) acc = fma(p[g], v[g], acc);
     }
-    if (g) part[g - 1][o] = acc;
-    __syncthreads();
-    if (g == 0 && it < tot) out[it] = (acc + part[0][o]) + (part[1][o] + part[2][o]);
-    __syncthreads();
+    for (; rr < T.nfold; ++rr) acc = fma(pt[rr], z[(size_t)rr * np], acc);
+    out[it] = acc;
   }
 }
 
@@ -486,7 +493,8 @@ void launch_gram(const ProbDev* probs, const GramTask* tasks, int ntask, const D
   // fill the GPU
   const int room = std::max(1, 2048 / ntask);
   k_gram_fold<<<dim3(ntask, 1 + std::min(8, room)), 256, 0, st>>>(probs, tasks);
-  k_gram_pot<<<dim3(ntask, std::min(room, (maxout + 63) / 64)), 256, 0, st>>>(probs, tasks, dtabs, room >= 8);
+  const int th = (room >= 8) ? 64 : 256;
+  k_gram_pot<<<dim3(ntask, std::min(room, (maxout + th - 1) / th)), th, 0, st>>>(probs, tasks, dtabs);
 }
 
 void launch_combine(const ProbDev* probs, const CombineTask* tasks, int n, cudaStream_t st) {
