@@ -59,7 +59,7 @@ int fft_max_cc(int);
 void launch_blockmul(const BmulTask*, int, int, int, cudaStream_t, bool);
 void launch_eapply(const EApplyTask*, int, int, int, int, bool, cudaStream_t);
 void launch_band_factor(const BandTask*, int, int, int, cudaStream_t);
-void launch_band_solve(const BandTask*, int, int, int, int, int, cudaStream_t, bool);
+void launch_band_solve(const BandTask*, int, int, int, int, int, int, int, cudaStream_t, bool);
 void launch_cell_canon(const CanonTask*, int, int, int, cudaStream_t);
 void launch_gather(const GatherSeg*, int, uint32_t*, cudaStream_t);
 void launch_cell_back(const double*, int, int, int, const double*, double*, int, cudaStream_t);
@@ -516,7 +516,8 @@ struct Batch {
     int *Erows = nullptr, *Erowptr = nullptr, *Ecols = nullptr; int nErows = 0;
     cplx *CH = nullptr, *CS = nullptr, *K = nullptr;
     double *emin = nullptr, *sigma = nullptr;
-    bool use_band = false;            // preconditioner: banded Cholesky (else circulant inverse)
+    bool use_band = false;            // preconditioner: banded factor (else circulant inverse)
+    bool band_twist = false;          // eliminated from both ends
     // cell canonical orthogonalisation: transformed operator used by the solver
     double *Xc = nullptr, *THc = nullptr, *TSc = nullptr, *EHc = nullptr, *ESc = nullptr;
     int* kept = nullptr;
@@ -549,7 +550,8 @@ struct Batch {
   TL rfwdXP, rinvHXP, rinvSXP, rbmulHS2, reHXP;   // image refresh at the FP32 -> FP64 switch
   TL bandF, bandS;
   int band_col = 0;                  // doubles of the largest block column of a band factorisation
-  int band_row = 0, band_step = 0, band_8 = 0;   // band solves: largest (D + 4) m0, step, 8 (D + 1) m0
+  int band_item = 0, band_row = 0, band_step = 0, band_8 = 0;   // band solves: largest (D + 4) m0, (3 D + 4) m0, step, 8 (D + 1) m0
+  int band_sides = 1;
   int gemm_tiles = 0;                // TN tile sizes in use: bit 0 = 16, bit 1 = 20
   int* gemm_count = nullptr;         // [structured problem][2][kGemmTiles] arrivals of split TN sums, zero between launches
   bool odd_m0 = true;                // some problem has odd m0 (Fourier-block layout, k_fblocks)
@@ -595,7 +597,8 @@ void plan(Batch& B, Slab& S, Slab& U) {
   B.any_mixed = false;
   B.eapply_rows = 0;
   B.band_col = 0;
-  B.band_row = 0;
+  B.band_row = B.band_item = 0;
+  B.band_sides = 1;
   B.band_step = B.band_8 = 0;
   B.gemm_tiles = 0;
   B.ptab_maxT = 0; B.ptab_maxni = 0;
@@ -1030,10 +1033,12 @@ void plan(Batch& B, Slab& S, Slab& U) {
       // against 274 ms, 800 cells with D = 18 (1.7e10) 500 against 346.
       Q.use_band = 2.0 * Q.Lc * (double)Q.D * Q.D * (double)H.m0 * H.m0 * H.m0 <= 8e9;
       if (Q.use_band) {
-        Q.band_win = S.take<double>((size_t)(Q.D + 1) * (Q.D + 1) * m2);
-        Q.band_fwd = S.take<double>((size_t)Q.Lc * std::max<size_t>(band_step(Q.D, H.m0), 2));
-        Q.band_bwd = S.take<double>((size_t)Q.Lc * band_step(Q.D + 1, H.m0));
-        Q.band_dinv = S.take<double>((size_t)Q.Lc * m2);
+        Q.band_twist = Q.D > 0 && Q.Lc >= 2 * Q.D + 2;
+        const size_t rows = Q.Lc + (Q.band_twist ? Q.D : 0);
+        Q.band_win = S.take<double>((size_t)(Q.band_twist ? 2 : 1) * (Q.D + 1) * (Q.D + 1) * m2);
+        Q.band_fwd = S.take<double>(rows * std::max<size_t>(band_step(Q.D, H.m0), 2));
+        Q.band_bwd = S.take<double>(rows * band_step(Q.D + 1, H.m0));
+        Q.band_dinv = S.take<double>(rows * m2);
         Q.sigma_band = S.take<double>(1);
         Q.band_fail = S.take<int>(1);
       }
@@ -1187,7 +1192,10 @@ void plan(Batch& B, Slab& S, Slab& U) {
         bt.fail = Q.band_fail; bt.R = l.R; bt.W = Yw; bt.ld = n; bt.active = l.active;
         bt.fp32 = H.f32;
         B.band_col = std::max(B.band_col, 2 * m0 * m0 + (Q.D + 1) * m0 * (m0 + 1));
-        B.band_row = std::max(B.band_row, (Q.D + 4) * m0);
+        bt.twist = Q.band_twist;
+        if (Q.band_twist) B.band_sides = 2;
+        B.band_item = std::max(B.band_item, (Q.D + 4) * m0);
+        B.band_row = std::max(B.band_row, ((Q.band_twist ? 3 : 1) * Q.D + 4) * m0);
         B.band_step = std::max(B.band_step, (int)band_step(Q.D + 1, m0));
         if (m0 > 8) B.band_8 = std::max(B.band_8, 8 * (Q.D + 1) * m0);
         std::vector<int> ef((size_t)Q.Lc * (Q.D + 1), -1);   // a position's entries lie one after another
@@ -1684,7 +1692,7 @@ void refresh_XP(Batch& B, cudaStream_t st) {
 // Rayleigh-Ritz, P' S-orthogonal to X' in the coefficients, [X | P] <- Y Cc and
 // their fresh images.  Launches only.
 void lobpcg_body_a(Batch& B, cudaStream_t st) {
-  if (B.bandS.n) { PROF("k_band_solve", 1); launch_band_solve(tl<BandTask>(B.bandS), B.bandS.n, B.kmax, B.band_row, B.band_step, B.band_8, st, B.any_mixed); }
+  if (B.bandS.n) { PROF("k_band_solve", 1); launch_band_solve(tl<BandTask>(B.bandS), B.bandS.n, B.kmax, B.band_item, B.band_row, B.band_step, B.band_8, B.band_sides, st, B.any_mixed); }
   if (B.fwdR.n) {
     mv_fwd(B, B.fwdR, st);
     { PROF("k_blockmul", 1); launch_blockmul(tl<BmulTask>(B.bmulK), B.bmulK.n, B.maxM, B.maxm0, st, B.any_mixed); }

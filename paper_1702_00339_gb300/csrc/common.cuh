@@ -360,13 +360,14 @@ struct BandTask {
   const double* EH; const double* ES;      // [nE][m0*m0]
   const double* sigma0;                    // shift from the embedding
   const int* efirst;                       // [L][D+1] first entry at (K, K-d), -1: none
-  double* win;                             // [D+1][D+1][m0*m0] factorisation window
+  double* win;                             // [sides][D+1][D+1][m0*m0] factorisation window
   double* fwd; double* bwd; double* dinv;  // the factor (k_band.cu): [L][band_step], [L][m0*m0]
   double* sigma_used;                      // out
   int* fail;                               // out: 1 if every attempt broke down
   const double* R; double* W; int ld;      // solve: W = A^-1 R (n x k, ld)
   const int* active;
   int fp32;                                // 1: solve in FP32 arithmetic (mixed form)
+  int twist;                               // eliminated from both ends (rows of the factor: L + D)
 };
 
 // Cell basis of a chain on the structured path: Xc (m0 x m0, row-major

@@ -10,6 +10,13 @@
 // of either substitution is one product of a block column with the row just
 // finished, without a triangular solve in between.
 //
+// A chain of L block rows is long, and a step waits for the one before: where L >= 2 D + 2
+// the elimination goes from both ends towards D rows in the middle (twist). Side 0
+// eliminates rows 0 .. a - 1 downwards, side 1 rows L - 1 .. a + D upwards, which is the
+// same procedure on the chain in reverse order; the sum of what both leave of the middle
+// rows is factored by each side for itself, in its own order, so that each goes on into its
+// half without waiting for the other: (L + D) / 2 steps instead of L.
+//
 //  k_band_factor  one thread-block cluster per problem: fill the band from T
 //                 and E, factor it block column by block column; on a
 //                 non-positive pivot lower sigma and start again
@@ -20,7 +27,7 @@
 // blocks (K, K-d) of what is left of A; fwd[J], the coefficients of one step
 // down, [q][d-1][mu] = M_{J+d,J}[mu][q]; bwd[K], those of one step up,
 // [q][d][mu] = M_{K,K-d}[q][mu] for d >= 1 and Delta_{K-D-1}^-1[q][mu] for
-// d = 0; dinv[K] = Delta_K^-1.  A step's coefficients lie one after another in
+// d = 0; dinv[K] = Delta_K^-1; side 1's rows, in its own order, after side 0's.  A step's coefficients lie one after another in
 // the order its threads (d, mu) read them, padded to a multiple of 16 bytes.
 #include <algorithm>
 
@@ -34,6 +41,28 @@ __device__ __forceinline__ void cl_arrive() { asm volatile("barrier.cluster.arri
 __device__ __forceinline__ void cl_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ int cl_rank() { int r; asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
 __device__ __forceinline__ int cl_size() { int r; asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
+
+// the shared memory of another CTA of the cluster at the address of p in this one
+template <typename X> __device__ __forceinline__ uint32_t cl_addr(const X* p, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ int cl_load(const int* p, int rank) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(cl_addr(p, rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ double cl_load(const double* p, int rank) {
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(cl_addr(p, rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ float cl_load(const float* p, int rank) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cl_addr(p, rank)) : "memory");
+  return v;
+}
 
 constexpr int kFactorThreads = 512;   // 256 where blocks are small
 
@@ -57,15 +86,21 @@ __device__ __forceinline__ int pair_row(int p) {
 // waiting for another CTA to do it; the M_d are made by one CTA each.  Every decision depends on values all CTAs
 // compute alike, so all take the same sequence of cluster barriers, and an
 // entry's arithmetic does not depend on the cluster's size.  Measured: 101 cells
-// of 16 functions 22.5 -> 2.5 ms, 64 cells of 8 1.96 -> 0.75 ms (one problem, one
-// factorisation), three rings of 61 cells of 16 with bound states (several
-// shifts) 69 -> 7.7 ms, 512 cells of 32 50 ms.
+// of 16 functions 22.5 -> 1.9 ms (2.5 from one end), 64 cells of 8 1.96 -> 0.55 ms (0.75;
+// one problem, one factorisation), 32 of those 0.94 -> 0.79 ms, 512 cells of 32 50 -> 40.
 __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* __restrict__ tasks, int smem_doubles) {
   extern __shared__ double fsm[];
-  const int C = cl_size(), rank = cl_rank();
-  const BandTask T = tasks[blockIdx.x / C];
-  const int m0 = T.m0, m2 = m0 * m0, D = T.D, L = T.L, mp = m0 + 1, D1 = D + 1;
+  const int CC = cl_size(), crank = cl_rank();
+  const BandTask T = tasks[blockIdx.x / CC];
+  // a side's CTAs; L is the length of its chain, of which it eliminates a rows before
+  // the middle (all of them without twist)
+  const int C = T.twist ? CC / 2 : CC, side = crank / C, rank = crank % C;
+  const int m0 = T.m0, m2 = m0 * m0, D = T.D, LL = T.L, mp = m0 + 1, D1 = D + 1;
+  const int a0 = (LL - D) / 2, a1 = LL - D - a0;   // a0 <= a1 <= a0 + 1
+  const int a = !T.twist ? LL : side ? a1 : a0, L = T.twist ? a + D : LL;
   const size_t fst = band_step(D, m0), bst = band_step(D1, m0);
+  const size_t r0 = side ? a0 + D : 0;       // the side's first row of the factor
+  double *const Tfwd = T.fwd + r0 * fst, *const Tbwd = T.bwd + r0 * bst, *const Tdinv = T.dinv + r0 * m2;
   const int tid = threadIdx.x, nth = blockDim.x, gtid = rank * nth + tid, gnth = C * nth;
   double* g0 = fsm;                          // diagonal block, its inverse in the end
   double* g1 = g0 + m2;
@@ -87,31 +122,69 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
   int nbis = 0;
   bool stop = false;
   // block (K, K-d) of the window; written by any CTA of the cluster: read from L2
-  auto win = [&](int K, int d) { return T.win + ((size_t)(K % D1) * D1 + d) * m2; };
+  auto winS = [&](int sd, int K, int d) { return T.win + ((size_t)(sd * D1 + K % D1) * D1 + d) * m2; };
+  auto win = [&](int K, int d) { return winS(side, K, d); };
   // row K enters the window: Toeplitz part and boundary blocks (a position's
-  // entries lie one after another, its first one in efirst)
+  // entries lie one after another, its first one in efirst); side 1's block (K, K - d)
+  // is the transpose of the one at row LL - 1 - K + d, and its middle starts at zero
   auto enter = [&](int K) {
     for (int it = gtid; it < D1 * m2; it += gnth) {
       const int d = it / m2, e = it % m2;
       if (d > K) continue;
-      double v = T.TH[(size_t)d * m2 + e] - sg * T.TS[(size_t)d * m2 + e];
-      const int q0 = T.efirst[(size_t)K * D1 + d];
-      if (q0 >= 0) {
-        double x = 0.0;
-        for (int q = q0; q < T.nE && T.Ek[q] == K && T.Em[q] == K - d; ++q)
-          x += T.EH[(size_t)q * m2 + e] - sg * T.ES[(size_t)q * m2 + e];
-        v += x;
+      const int Kr = side ? LL - 1 - K + d : K, f = side ? (e % m0) * m0 + e / m0 : e;
+      double v = 0.0;
+      if (!side || K - d < a) {
+        v = T.TH[(size_t)d * m2 + f] - sg * T.TS[(size_t)d * m2 + f];
+        const int q0 = T.efirst[(size_t)Kr * D1 + d];
+        if (q0 >= 0) {
+          double x = 0.0;
+          for (int q = q0; q < T.nE && T.Ek[q] == Kr && T.Em[q] == Kr - d; ++q)
+            x += T.EH[(size_t)q * m2 + f] - sg * T.ES[(size_t)q * m2 + f];
+          v += x;
+        }
       }
       win(K, d)[e] = v;
     }
   };
+  // the middle's blocks (a + i, a + j), j <= i: on side 0 the sum of both sides' (its block
+  // is the transpose of side 1's (D - 1 - j, D - 1 - i)), on side 1 a copy of that
+  auto middle = [&](int sd) {
+    for (long long it = gtid; it < (long long)(D * (D + 1) / 2) * m2; it += gnth) {
+      const int p = (int)(it / m2), e = (int)(it % m2), mu = e / m0, nu = e % m0;
+      const int i = pair_row(p) - 1, j = p - i * (i + 1) / 2;
+      if (i == j && nu > mu) continue;         // diagonal blocks: lower triangle
+      const int f = i == j ? e : nu * m0 + mu;
+      const double x = __ldcg(winS(1 - sd, (sd ? a0 : a1) + D - 1 - j, i - j) + f);
+      double* out = win(a + i, i - j) + e;
+      *out = sd ? x : __ldcg(out) + x;
+    }
+  };
+  const int steps = T.twist ? a1 + D : L, late = T.twist ? a1 - a : 0;   // side 0 may start one step late
   for (int attempt = 0; attempt < 24; ++attempt) {
     for (int K = 0; K < min(D1, L); ++K) enter(K);
     if (tid == 0) s_bad = 0;
     cl_arrive();
     cl_wait();
     bool bad = false;
-    for (int J = 0; J < L; ++J) {
+    for (int t = 0; t < steps; ++t) {
+      if (T.twist && t == a1) {                // both sides are at their first middle row
+        bad = bad || cl_load(&s_bad, (crank + C) % CC) != 0;
+        if (!side && !bad) middle(0);
+        cl_arrive();
+        cl_wait();
+        if (side && !bad) middle(1);
+        cl_arrive();
+        cl_wait();
+        if (bad) break;
+      }
+      const int J = t - late;
+      if (J < 0 || (T.twist && bad)) {         // nothing to do: the step's barriers
+        cl_arrive();
+        cl_wait();
+        cl_arrive();
+        cl_wait();
+        continue;
+      }
       const int dmax = min(D, L - 1 - J);
       auto Acol = [&](int d, int nu, int q) { return __ldcg(win(J + d, d) + nu * m0 + q); };
       for (int e = tid; e < m2; e += nth) {   // lower triangle mirrored: exactly symmetric
@@ -151,7 +224,7 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
           }
         }
         __syncthreads();
-        double* t = cur; cur = nxt; nxt = t;
+        double* swp = cur; cur = nxt; nxt = swp;
       }
       const double* Di = cur;
       bad = s_bad != 0;
@@ -172,8 +245,8 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
         __syncthreads();
       };
       auto store_M = [&](int d1) {
-        double* f = T.fwd + (size_t)J * fst + (d1 - 1) * m0;
-        double* u = T.bwd + (size_t)(J + d1) * bst + d1 * m0;
+        double* f = Tfwd + (size_t)J * fst + (d1 - 1) * m0;
+        double* u = Tbwd + (size_t)(J + d1) * bst + d1 * m0;
         for (int e = tid; e < m2; e += nth) {
           const int q = e / m0, mu = e % m0;
           f[(size_t)q * D * m0 + mu] = Ms[mu * mp + q];
@@ -196,17 +269,17 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
         const int p0 = (int)((long long)np * rank / C), p1 = (int)((long long)np * (rank + 1) / C);
         for (int p = p0; p < p1;) {
           const int d1 = pair_row(p), base = d1 * (d1 - 1) / 2;
-          const int a = p - base + 1, b = min(d1, p1 - base);   // d2 in a..b
+          const int da = p - base + 1, db = min(d1, p1 - base);   // d2 in da..db
           if (fits) {
-            const double* f = T.fwd + (size_t)J * fst + (d1 - 1) * m0;
+            const double* f = Tfwd + (size_t)J * fst + (d1 - 1) * m0;
             for (int e = tid; e < m2; e += nth) Ms[(e % m0) * mp + e / m0] = __ldcg(f + (size_t)(e / m0) * D * m0 + e % m0);
             __syncthreads();
           } else {
             make_M(d1);
-            if (a == 1) store_M(d1);           // the owner of (d1, 1)
+            if (da == 1) store_M(d1);          // the owner of (d1, 1)
           }
-          for (int it = tid; it < (b - a + 1) * m2; it += nth) {
-            const int d2 = a + it / m2, e = it % m2, mu = e / m0, nu = e % m0;
+          for (int it = tid; it < (db - da + 1) * m2; it += nth) {
+            const int d2 = da + it / m2, e = it % m2, mu = e / m0, nu = e % m0;
             if (d1 == d2 && nu > mu) continue;   // diagonal block: lower triangle suffices
             double* out = win(J + d1, d1 - d2) + e;
             const double old = __ldcg(out);
@@ -220,12 +293,12 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
             *out = old - s;
           }
           __syncthreads();
-          p = base + b;
+          p = base + db;
         }
         if (rank == 0)
           for (int e = tid; e < m2; e += nth) {
-            T.dinv[(size_t)J * m2 + e] = Di[e];
-            if (J + D1 < L) T.bwd[(size_t)(J + D1) * bst + (size_t)(e / m0) * D1 * m0 + e % m0] = Di[e];
+            Tdinv[(size_t)J * m2 + e] = Di[e];
+            if (J + D1 < L) Tbwd[(size_t)(J + D1) * bst + (size_t)(e / m0) * D1 * m0 + e % m0] = Di[e];
           }
       }
       if (!fits) {
@@ -235,7 +308,14 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
       if (!bad && J + D1 < L) enter(J + D1);
       cl_arrive();
       cl_wait();                              // the trailing update and the new row are visible to all
-      if (bad) break;
+      if (bad && !T.twist) break;
+    }
+    if (T.twist) {                             // one decision for both sides
+      cl_arrive();
+      cl_wait();
+      bad = bad || cl_load(&s_bad, (crank + C) % CC) != 0;
+      cl_arrive();
+      cl_wait();
     }
     if (!bad) {
       sg_ok = sg;
@@ -248,7 +328,7 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
     else if (nbis < 3) { sg = 0.5 * (sg_ok + sg_bad); ++nbis; }
     else { sg = sg_ok - (sg_bad - sg_ok); nbis = 99; }   // refactor one bracket below
   }
-  if (rank == 0 && tid == 0) {
+  if (crank == 0 && tid == 0) {
     *T.sigma_used = sg;
     if (!stop && T.fail) *T.fail = 1;
   }
@@ -279,27 +359,37 @@ __host__ __device__ inline int band_rows(int nd, int m0, int stage) {
 // multiply-adds.  Per step an SM's FP64 pipe takes (D + 1) m0^2 / 2 cycles, the
 // bound; hence one column per CTA (two, which read the coefficients half as often,
 // were slower from 20 columns to 2560).  Measured per launch,
-// 20 columns a problem: one chain of 64 cells of 8 functions (D = 13) 941 -> 97 us,
-// 32 of them 945 -> 200 us, three rings of 61 cells of 16 4320 -> 166 us; with one
-// step of coefficients ahead in registers instead of shared memory the first took
-// 205 us.  72 columns of 512 cells of 32: 4.9 ms (6.9 without the stages).
+// 20 columns a problem: one chain of 64 cells of 8 functions (D = 13) 941 -> 97 us from
+// one end, 64 us from two (a cluster of two CTAs per column, which meet once);
+// 32 of them 945 -> 185 and 215 us (the middle is done twice, and here the FP64 pipe
+// is full; their factor gains as much); with one step of coefficients ahead in
+// registers instead of shared memory the first took 205 us.  72 columns of 512 cells
+// of 32: 4.9 ms from one end (6.9 without the stages), 2.5 from two.
 template <typename R, bool MULTI>
-__global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict__ tasks, int maxrow, int maxstage) {
+__global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict__ tasks, int sides, int maxstage) {
   extern __shared__ __align__(16) double bsm[];
   const BandTask T = tasks[blockIdx.y];
   if (T.active && *T.active == 0) return;
   if ((T.fp32 != 0) != (sizeof(R) == 4)) return;
-  if (blockIdx.x >= (unsigned)T.k) return;
-  const double* Rc = T.R + (size_t)T.ld * blockIdx.x;   // this CTA's column
-  double* Wc = T.W + (size_t)T.ld * blockIdx.x;
-  const int m0 = T.m0, m2 = m0 * m0, D = T.D, L = T.L, nslot = D + 2, D1 = D + 1;
+  const int col = blockIdx.x / sides, side = blockIdx.x % sides;
+  if (col >= T.k || (side && !T.twist)) return;
+  const double* Rc = T.R + (size_t)T.ld * col;   // this CTA's column
+  double* Wc = T.W + (size_t)T.ld * col;
+  const int m0 = T.m0, m2 = m0 * m0, D = T.D, LL = T.L, nslot = D + 2, D1 = D + 1;
+  const int a0 = (LL - D) / 2, a = !T.twist ? LL : side ? LL - D - a0 : a0, L = T.twist ? a + D : LL;
+  // the side's row r in the column; its part of the factor
+  auto at = [&](int r, int mu) { return (size_t)(side ? LL - 1 - r : r) * m0 + mu; };
+  const size_t r0 = side ? a0 + D : 0;
   const int tid = threadIdx.x, nth = blockDim.x, items = D1 * m0, fit = D * m0;
   const int fst = (int)band_step(D, m0), bst = (int)band_step(D1, m0);   // doubles per step
+  const double *const Tfwd = T.fwd + r0 * fst, *const Tbwd = T.bwd + r0 * bst, *const Tdinv = T.dinv + r0 * m2;
   // rows of coefficients per stage: all m0, or a multiple of 8 that fits
   const int qc = MULTI ? band_rows(D1, m0, maxstage) : m0, nch = MULTI ? (m0 + qc - 1) / qc : 1;
   double* cf = bsm;                           // two stages of maxstage doubles
   R* acc = reinterpret_cast<R*>(bsm + (size_t)2 * maxstage);   // nslot rows, then two of the forward solution
   R* zb = acc + (size_t)nslot * m0;
+  R* xm = zb + 2 * m0;                        // twist: what the side leaves of the middle rows, then
+  R* zm = xm + (size_t)D * m0;                // their forward solution
   // rows [h qc, ...) of a step of `width` entries a row into stage `slot`
   auto stage = [&](const double* step, int total, int width, int h, int slot) {
     const double* src = step + (size_t)h * qc * width;
@@ -310,31 +400,46 @@ __global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict_
   const int mu0 = tid % m0;
   const bool zero = tid < m0;                 // this thread is (d = 0, mu0)
   // ---- M z = r, downwards ----
-  stage(T.fwd, fst, fit, 0, 0);
+  stage(Tfwd, fst, fit, 0, 0);
   cp_async_commit();
   for (int it = tid; it < items; it += nth) {   // rows 0 .. D enter
     const int r = it / m0, mu = it % m0;
-    if (r < L)
-      acc[(r % nslot) * m0 + mu] = (R)Rc[(size_t)r * m0 + mu];
+    if (r < L) acc[(r % nslot) * m0 + mu] = (side && r >= a) ? (R)0 : (R)Rc[at(r, mu)];
   }
-  R nr = 0;                                    // the row that enters next
-  if (zero && D1 < L) nr = (R)Rc[(size_t)D1 * m0 + mu0];
+  // the row that enters next (side 1's middle starts at zero)
+  auto next = [&](int r) { return (side && r >= a) ? (R)0 : (R)Rc[at(r, mu0)]; };
+  R nr = 0;
+  if (zero && D1 < L) nr = next(D1);
   cp_async_wait0();
   __syncthreads();
   int st = 0;
   for (int J = 0, js = 0; J < L; ++J) {
+    if (J == a) {                              // (twist) the middle rows: both sides' partial sums
+      auto mid = [&](int it) { return acc + (js + it / m0 >= nslot ? js + it / m0 - nslot : js + it / m0) * m0 + it % m0; };
+      for (int it = tid; it < fit; it += nth) xm[it] = *mid(it);
+      __syncthreads();
+      cl_arrive();
+      cl_wait();
+      for (int it = tid; it < fit; it += nth) {
+        const R o = cl_load(xm + (D - 1 - it / m0) * m0 + it % m0, side ^ 1);
+        *mid(it) = side ? o + xm[it] : xm[it] + o;
+      }
+      __syncthreads();
+      cl_arrive();                             // waited for at the end: xm stays until the other side has read it
+    }
     const R* y = acc + js * m0;
     const int live = min(D, L - 1 - J) * m0;
     for (int h = 0; h < nch; ++h, st ^= 1) {
       const double* cs = cf + (size_t)st * maxstage;
-      if (h + 1 < nch) stage(T.fwd + (size_t)J * fst, fst, fit, h + 1, st ^ 1);
-      else if (J + 1 < L) stage(T.fwd + (size_t)(J + 1) * fst, fst, fit, 0, st ^ 1);
+      if (h + 1 < nch) stage(Tfwd + (size_t)J * fst, fst, fit, h + 1, st ^ 1);
+      else if (J + 1 < L) stage(Tfwd + (size_t)(J + 1) * fst, fst, fit, 0, st ^ 1);
       cp_async_commit();
       if (zero && h == 0) {
         const int r = J + D1, sl = js + D1 >= nslot ? js + D1 - nslot : js + D1;
-        Wc[(size_t)J * m0 + mu0] = (double)y[mu0];
+        if (J < a) Wc[at(J, mu0)] = (double)y[mu0];
+        else zm[(J - a) * m0 + mu0] = y[mu0];
         if (r < L) acc[sl * m0 + mu0] = nr;
-        if (r + 1 < L) nr = (R)Rc[(size_t)(r + 1) * m0 + mu0];
+        if (r + 1 < L) nr = next(r + 1);
       }
       const int qa = h * qc, qn = min(qc, m0 - qa);
       // (from the last thread down: the threads of d = 0 are busy with the rows)
@@ -352,21 +457,21 @@ __global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict_
     js = (js + 1 == nslot) ? 0 : js + 1;
   }
   // ---- M^T x = Delta^-1 z, upwards ----
-  stage(T.bwd + (size_t)(L - 1) * bst, bst, items, 0, st);
+  stage(Tbwd + (size_t)(L - 1) * bst, bst, items, 0, st);
   cp_async_commit();
   for (int it = tid; it < items; it += nth) {   // rows L-1 .. L-1-D enter
     const int r = L - 1 - it / m0, mu = it % m0;
     if (r >= 0) {
       R s = 0;
-      for (int q = 0; q < m0; ++q) s += (R)T.dinv[(size_t)r * m2 + q * m0 + mu] * (R)Wc[(size_t)r * m0 + q];
+      for (int q = 0; q < m0; ++q) s += (R)Tdinv[(size_t)r * m2 + q * m0 + mu] * (r < a ? (R)Wc[at(r, q)] : zm[(r - a) * m0 + q]);
       acc[(r % nslot) * m0 + mu] = s;
     }
   }
   // row that enters at step K: K - D - 1; its z waits in zb, the one after it in nr
   if (zero) {
     const int r = L - 1 - D1;
-    if (r >= 0) zb[((L - 1) & 1) * m0 + mu0] = (R)Wc[(size_t)r * m0 + mu0];
-    nr = (r - 1 >= 0) ? (R)Wc[(size_t)(r - 1) * m0 + mu0] : (R)0;
+    if (r >= 0) zb[((L - 1) & 1) * m0 + mu0] = (R)Wc[at(r, mu0)];
+    nr = (r - 1 >= 0) ? (R)Wc[at(r - 1, mu0)] : (R)0;
   }
   cp_async_wait0();
   __syncthreads();
@@ -376,13 +481,13 @@ __global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict_
     const int live = (K >= D1) ? items : (K + 1) * m0;
     for (int h = 0; h < nch; ++h, st ^= 1) {
       const double* cs = cf + (size_t)st * maxstage;
-      if (h + 1 < nch) stage(T.bwd + (size_t)K * bst, bst, items, h + 1, st ^ 1);
-      else if (K > 0) stage(T.bwd + (size_t)(K - 1) * bst, bst, items, 0, st ^ 1);
+      if (h + 1 < nch) stage(Tbwd + (size_t)K * bst, bst, items, h + 1, st ^ 1);
+      else if (K > 0) stage(Tbwd + (size_t)(K - 1) * bst, bst, items, 0, st ^ 1);
       cp_async_commit();
       if (zero && h == 0) {
-        Wc[(size_t)K * m0 + mu0] = (double)x[mu0];
+        if (K < a || !side) Wc[at(K, mu0)] = (double)x[mu0];   // (the middle by side 0)
         if (K - D1 - 1 >= 0) zb[((K - 1) & 1) * m0 + mu0] = nr;
-        if (K - D1 - 2 >= 0) nr = (R)Wc[(size_t)(K - D1 - 2) * m0 + mu0];
+        if (K - D1 - 2 >= 0) nr = (R)Wc[at(K - D1 - 2, mu0)];
       }
       const int qa = h * qc, qn = min(qc, m0 - qa);
       for (int it = nth - 1 - tid; it < live; it += nth) {
@@ -400,6 +505,7 @@ __global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict_
     }
     ks = (ks == 0) ? nslot - 1 : ks - 1;
   }
+  if (T.twist) cl_wait();
 }
 
 // maxcol: the largest m0 (m0 + 1) (D + 3) among the tasks (shared doubles that
@@ -446,17 +552,28 @@ void launch_band_factor(const BandTask* t, int n, int maxcol, int maxm0, cudaStr
   cudaLaunchKernelEx(&cfg, k_band_factor, t, doubles);
 }
 
-// maxrow: the largest (D + 4) m0 among the tasks (ring and z rows of a column),
-// maxstep: the largest step (coefficient doubles), max8: the largest 8 (D + 1) m0
-// of the steps that are taken in pieces
+// maxitem: the largest (D + 4) m0 among the tasks, maxrow: the largest (3 D + 4) m0 (ring, z
+// and middle rows of a column), maxstep: the largest step (coefficient doubles), max8: the
+// largest 8 (D + 1) m0 of the steps that are taken in pieces, sides: 2 if any task is twisted
 template <typename R, bool MULTI>
-static void solve_go(const BandTask* t, int n, int kmax, int maxrow, int maxstage, cudaStream_t st) {
+static void solve_go(const BandTask* t, int n, int kmax, int maxitem, int maxrow, int maxstage, int sides, cudaStream_t st) {
   FOCK_SMEM_OPTIN((k_band_solve<R, MULTI>));
-  const size_t sm = ((size_t)2 * maxstage + (size_t)maxrow) * sizeof(double);
-  const int threads = std::min(1024, std::max(64, (maxrow + 31) & ~31));
-  k_band_solve<R, MULTI><<<dim3(kmax, n), threads, sm, st>>>(t, maxrow, maxstage);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(kmax * sides), (unsigned)n);
+  cfg.blockDim = dim3(std::min(1024, std::max(64, (maxitem + 31) & ~31)));
+  cfg.dynamicSmemBytes = ((size_t)2 * maxstage + (size_t)maxrow) * sizeof(double);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = sides;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_band_solve<R, MULTI>, t, sides, maxstage);
 }
-void launch_band_solve(const BandTask* t, int n, int kmax, int maxrow, int maxstep, int max8, cudaStream_t st, bool mixed) {
+void launch_band_solve(const BandTask* t, int n, int kmax, int maxitem, int maxrow, int maxstep, int max8, int sides,
+                       cudaStream_t st, bool mixed) {
   if (!n) return;
   // A stage holds a step up to 64 KB, or as many rows of one (at least 8).  Two
   // stages are enough and leave room for several CTAs per SM: eight give the same
@@ -465,11 +582,11 @@ void launch_band_solve(const BandTask* t, int n, int kmax, int maxrow, int maxst
   // of 32 functions 5.8 ms against 4.9.
   const int maxstage = std::max(std::min(maxstep, 8192), max8);
   if (maxstep <= maxstage) {
-    solve_go<double, false>(t, n, kmax, maxrow, maxstage, st);
-    if (mixed) solve_go<float, false>(t, n, kmax, maxrow, maxstage, st);
+    solve_go<double, false>(t, n, kmax, maxitem, maxrow, maxstage, sides, st);
+    if (mixed) solve_go<float, false>(t, n, kmax, maxitem, maxrow, maxstage, sides, st);
   } else {
-    solve_go<double, true>(t, n, kmax, maxrow, maxstage, st);
-    if (mixed) solve_go<float, true>(t, n, kmax, maxrow, maxstage, st);
+    solve_go<double, true>(t, n, kmax, maxitem, maxrow, maxstage, sides, st);
+    if (mixed) solve_go<float, true>(t, n, kmax, maxitem, maxrow, maxstage, sides, st);
   }
 }
 
