@@ -58,7 +58,7 @@ void launch_fft_cc(const FftTask*, int, int, int, int, int, cudaStream_t, bool);
 int fft_max_cc(int);
 void launch_blockmul(const BmulTask*, int, int, int, cudaStream_t, bool);
 void launch_eapply(const EApplyTask*, int, int, int, int, bool, cudaStream_t);
-void launch_band_factor(const BandTask*, int, int, int, cudaStream_t);
+void launch_band_factor(const BandTask*, int, int, int, const BandSteps&, cudaStream_t);
 void launch_band_solve(const BandTask*, int, int, int, int, int, int, int, cudaStream_t, bool);
 void launch_cell_canon(const CanonTask*, int, int, int, cudaStream_t);
 void launch_gather(const GatherSeg*, int, uint32_t*, cudaStream_t);
@@ -552,6 +552,7 @@ struct Batch {
   int band_col = 0;                  // doubles of the largest block column of a band factorisation
   int band_item = 0, band_row = 0, band_step = 0, band_8 = 0;   // band solves: largest (D + 4) m0, (3 D + 4) m0, step, 8 (D + 1) m0
   int band_sides = 1;
+  BandSteps band_cs;
   int gemm_tiles = 0;                // TN tile sizes in use: bit 0 = 16, bit 1 = 20
   int* gemm_count = nullptr;         // [structured problem][2][kGemmTiles] arrivals of split TN sums, zero between launches
   bool odd_m0 = true;                // some problem has odd m0 (Fourier-block layout, k_fblocks)
@@ -599,6 +600,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
   B.band_col = 0;
   B.band_row = B.band_item = 0;
   B.band_sides = 1;
+  B.band_cs = BandSteps();
   B.band_step = B.band_8 = 0;
   B.gemm_tiles = 0;
   B.ptab_maxT = 0; B.ptab_maxni = 0;
@@ -1025,22 +1027,22 @@ void plan(Batch& B, Slab& S, Slab& U) {
       Q.K = S.take<cplx>((size_t)Q.M * m2);
       Q.emin = S.take<double>(Q.M);
       Q.sigma = S.take<double>(1);
-      // Banded factor of H - sigma S up to ~8 GFLOP (70 ms), above that the circulant
-      // inverse.  512 cells of 32 functions (5.7e9, D = 13), 64 eigenpairs, three draws:
-      // banded 13 iterations and 185 ms in the mixed form, 350 in the FP64 form;
-      // circulant 31, 50, 37 iterations and 207, 320, 243 ms (FP64 718 ms and more).
-      // Beyond, an iteration no longer repays the factor: 1000 cells (1.1e10) 359
+      // Banded factor of H - sigma S up to ~8 GFLOP, above that the circulant inverse.
+      // 512 cells of 32 functions (5.7e9, D = 13), 64 eigenpairs, three draws: banded 13
+      // iterations and 124 ms in the mixed form; circulant 31, 50, 37 iterations and
+      // 207, 320, 243 ms (FP64 718 ms and more). Beyond, with the factor made from one
+      // end by one cluster, an iteration no longer repaid it: 1000 cells (1.1e10) 359
       // against 274 ms, 800 cells with D = 18 (1.7e10) 500 against 346.
       Q.use_band = 2.0 * Q.Lc * (double)Q.D * Q.D * (double)H.m0 * H.m0 * H.m0 <= 8e9;
       if (Q.use_band) {
         Q.band_twist = Q.D > 0 && Q.Lc >= 2 * Q.D + 2;
         const size_t rows = Q.Lc + (Q.band_twist ? Q.D : 0);
-        Q.band_win = S.take<double>((size_t)(Q.band_twist ? 2 : 1) * (Q.D + 1) * (Q.D + 1) * m2);
+        Q.band_win = S.take<double>((size_t)(Q.band_twist ? 2 : 1) * (Q.D + 2) * (Q.D + 1) * m2);
         Q.band_fwd = S.take<double>(rows * std::max<size_t>(band_step(Q.D, H.m0), 2));
         Q.band_bwd = S.take<double>(rows * band_step(Q.D + 1, H.m0));
         Q.band_dinv = S.take<double>(rows * m2);
         Q.sigma_band = S.take<double>(1);
-        Q.band_fail = S.take<int>(1);
+        Q.band_fail = S.take<int>(4);   // [0] no shift worked, [1..3] BandTask::sync
       }
       Q.fail = S.take<int>(1);
       FBlockTask fb;
@@ -1193,6 +1195,13 @@ void plan(Batch& B, Slab& S, Slab& U) {
         bt.fp32 = H.f32;
         B.band_col = std::max(B.band_col, 2 * m0 * m0 + (Q.D + 1) * m0 * (m0 + 1));
         bt.twist = Q.band_twist;
+        bt.sync = Q.band_fail + 1;
+        if (band_columns(m0, Q.D)) {
+          const int joins = Q.Lc - Q.D - (Q.Lc - Q.D) / 2;
+          B.band_cs.steps = std::max(B.band_cs.steps, Q.band_twist ? joins + Q.D : Q.Lc);
+          B.band_cs.pairs = std::max(B.band_cs.pairs, Q.D * (Q.D + 1) / 2);
+          if (Q.band_twist) { B.band_cs.sides = 2; B.band_cs.middles.push_back(joins); }
+        }
         if (Q.band_twist) B.band_sides = 2;
         B.band_item = std::max(B.band_item, (Q.D + 4) * m0);
         B.band_row = std::max(B.band_row, ((Q.band_twist ? 3 : 1) * Q.D + 4) * m0);
@@ -1368,6 +1377,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
     TLp(nP, B.normP);
     TLp(nW, B.normW);
     TLp(bnd, B.bandF);
+    std::sort(B.band_cs.middles.begin(), B.band_cs.middles.end());
     B.bandS = B.bandF;
     TLp(rs, B.resid, kk);
   }
@@ -1577,9 +1587,9 @@ void run_struct_setup(fock_ctx* ctx, Batch& B) {
     launch_fblocks(B.d_probs, B.d_fbs, (int)B.fbs.size(), B.maxnj_s, B.maxm0, st, false, 0, -1, B.odd_m0); }
   { PROF("k_precond", 2); launch_precond(B.d_probs, B.d_prec, (int)B.prec.size(), B.maxM, B.maxm0, st); }
   for (auto& Q : B.pp)
-    if (Q.band_fail) cudaMemsetAsync(Q.band_fail, 0, sizeof(int), st);
+    if (Q.band_fail) cudaMemsetAsync(Q.band_fail, 0, 4 * sizeof(int), st);
   if (B.bandF.n) { PROF("k_band_factor", 1);
-    launch_band_factor(reinterpret_cast<const BandTask*>(B.bandF.d), B.bandF.n, B.band_col, B.maxm0, st); }
+    launch_band_factor(reinterpret_cast<const BandTask*>(B.bandF.d), B.bandF.n, B.band_col, B.maxm0, B.band_cs, st); }
 }
 
 template <class T> const T* tl(const Batch::TL& t) { return reinterpret_cast<const T*>(t.d); }

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <mutex>
+#include <vector>
 
 // Raises a kernel's dynamic shared memory limit, once per process, to the
 // device's opt-in maximum minus the kernel's static shared memory.  The
@@ -360,7 +361,7 @@ struct BandTask {
   const double* EH; const double* ES;      // [nE][m0*m0]
   const double* sigma0;                    // shift from the embedding
   const int* efirst;                       // [L][D+1] first entry at (K, K-d), -1: none
-  double* win;                             // [sides][D+1][D+1][m0*m0] factorisation window
+  double* win;                             // [sides][D+2][D+1][m0*m0] factorisation window
   double* fwd; double* bwd; double* dinv;  // the factor (k_band.cu): [L][band_step], [L][m0*m0]
   double* sigma_used;                      // out
   int* fail;                               // out: 1 if every attempt broke down
@@ -368,7 +369,21 @@ struct BandTask {
   const int* active;
   int fp32;                                // 1: solve in FP32 arithmetic (mixed form)
   int twist;                               // eliminated from both ends (rows of the factor: L + D)
+  int* sync;                               // [3] progress of the factorisation by columns (k_band.cu), zero before it
 };
+// What the launches of a factorisation by columns need of its tasks: the most steps and pairs
+// of blocks of a column, sides (2 if any is twisted), the steps before which a task joins its sides.
+struct BandSteps {
+  int steps = 0, pairs = 1, sides = 1;
+  std::vector<int> middles;                // ascending
+};
+constexpr int kColumnProblems = 4;         // most problems factored by columns
+// Whether a chain's block products are worth a launch per column: more of them than a side's
+// CTAs in a cluster, and multiply-adds for 5 us there.
+__host__ __device__ inline bool band_columns(int m0, int D) {
+  const int pairs = D * (D + 1) / 2;
+  return pairs >= 16 && (long long)pairs * m0 * m0 * m0 >= 150000;
+}
 
 // Cell basis of a chain on the structured path: Xc (m0 x m0, row-major
 // Xc[mu][j]) = Q_K diag(s_K)^-1/2 from the eigenpairs of the cell overlap

@@ -17,6 +17,7 @@
 // rows is factored by each side for itself, in its own order, so that each goes on into its
 // half without waiting for the other: (L + D) / 2 steps instead of L.
 //
+//  k_band_column  few problems of large blocks: a launch per block column, all SMs
 //  k_band_factor  one thread-block cluster per problem: fill the band from T
 //                 and E, factor it block column by block column; on a
 //                 non-positive pivot lower sigma and start again
@@ -76,6 +77,170 @@ __device__ __forceinline__ int pair_row(int p) {
 
 }  // namespace
 
+namespace {
+
+// One side of a factorisation (the whole chain without twist): L rows in its order, a of
+// them before the middle; sg the shift.
+struct BandSide {
+  const BandTask& T;
+  int side, m0, m2, D, D1, LL, a0, a1, a, L, late, steps;
+  size_t fst, bst;
+  double *fwd, *bwd, *dinv, sg;
+  __device__ BandSide(const BandTask& t, int sd) : T(t), side(sd), m0(t.m0), m2(t.m0 * t.m0), D(t.D), D1(t.D + 1), LL(t.L) {
+    a0 = (LL - D) / 2;
+    a1 = LL - D - a0;                          // a0 <= a1 <= a0 + 1
+    a = !T.twist ? LL : side ? a1 : a0;
+    L = T.twist ? a + D : LL;
+    steps = T.twist ? a1 + D : LL;
+    late = T.twist ? a1 - a : 0;               // side 0 may start one step late
+    fst = band_step(D, m0);
+    bst = band_step(D1, m0);
+    const size_t r0 = side ? a0 + D : 0;       // the side's first row of the factor
+    fwd = T.fwd + r0 * fst; bwd = T.bwd + r0 * bst; dinv = T.dinv + r0 * m2;
+  }
+  // block (K, K-d) of the window, a ring of D + 2 rows; written by any CTA: read from L2
+  __device__ double* winS(int sd, int K, int d) const { return T.win + ((size_t)(sd * (D1 + 1) + K % (D1 + 1)) * D1 + d) * m2; }
+  __device__ double* win(int K, int d) const { return winS(side, K, d); }
+  __device__ double at(int J, int d, int nu, int q) const { return __ldcg(win(J + d, d) + nu * m0 + q); }   // column J
+  // row K enters the window: Toeplitz part and boundary blocks (a position's
+  // entries lie one after another, its first one in efirst); side 1's block (K, K - d)
+  // is the transpose of the one at row LL - 1 - K + d, and its middle starts at zero.
+  // Shared out over gnth threads.
+  __device__ void enter(int K, int gtid, int gnth) const {
+    for (int it = gtid; it < D1 * m2; it += gnth) {
+      const int d = it / m2, e = it % m2;
+      if (d > K) continue;
+      const int Kr = side ? LL - 1 - K + d : K, f = side ? (e % m0) * m0 + e / m0 : e;
+      double v = 0.0;
+      if (!side || K - d < a) {
+        v = fma(-sg, T.TS[(size_t)d * m2 + f], T.TH[(size_t)d * m2 + f]);
+        const int q0 = T.efirst[(size_t)Kr * D1 + d];
+        if (q0 >= 0) {
+          double x = 0.0;
+          for (int q = q0; q < T.nE && T.Ek[q] == Kr && T.Em[q] == Kr - d; ++q)
+            x += fma(-sg, T.ES[(size_t)q * m2 + f], T.EH[(size_t)q * m2 + f]);
+          v += x;
+        }
+      }
+      win(K, d)[e] = v;
+    }
+  }
+  // the middle's blocks (a + i, a + j), j <= i: on side 0 the sum of both sides' (its block
+  // is the transpose of side 1's (D - 1 - j, D - 1 - i)), on side 1 a copy of that
+  __device__ void middle(int gtid, int gnth) const {
+    for (long long it = gtid; it < (long long)(D * (D + 1) / 2) * m2; it += gnth) {
+      const int p = (int)(it / m2), e = (int)(it % m2), mu = e / m0, nu = e % m0;
+      const int i = pair_row(p) - 1, j = p - i * (i + 1) / 2;
+      if (i == j && nu > mu) continue;         // diagonal blocks: lower triangle
+      const int f = i == j ? e : nu * m0 + mu;
+      const double x = __ldcg(winS(1 - side, (side ? a0 : a1) + D - 1 - j, i - j) + f);
+      double* out = win(a + i, i - j) + e;
+      *out = side ? x : __ldcg(out) + x;
+    }
+  }
+  // column J into shared memory: the diagonal block (lower triangle mirrored: exactly
+  // symmetric) into g0, and where it fits [d-1][q][nu] = A_{J+d,J}[nu][q], rows mp apart
+  __device__ void load(int J, int dmax, double* g0, double* col, bool fits) const {
+    const int mp = m0 + 1;
+    for (int e = threadIdx.x; e < m2; e += blockDim.x) {
+      const int i = e / m0, j = e % m0;
+      g0[e] = at(J, 0, max(i, j), min(i, j));
+    }
+    if (fits)
+      for (int it = threadIdx.x; it < dmax * m2; it += blockDim.x) {
+        const int d = 1 + it / m2, e = it % m2, nu = e / m0, q = e % m0;
+        col[((d - 1) * m0 + q) * mp + nu] = at(J, d, nu, q);
+      }
+    __syncthreads();
+  }
+  // M_{J+d1,J} = A_{J+d1,J} Delta_J^-1 into Ms (rows mp apart)
+  __device__ void make_M(int J, int d1, const double* col, const double* Di, double* Ms, bool fits) const {
+    const int mp = m0 + 1;
+    for (int e = threadIdx.x; e < m2; e += blockDim.x) {
+      const int mu = e / m0, q = e % m0;
+      double s = 0.0;
+      if (fits) {
+        const double* c = col + (d1 - 1) * m0 * mp + mu;
+        for (int t = 0; t < m0; ++t) s = fma(c[t * mp], Di[t * m0 + q], s);
+      } else {
+        for (int t = 0; t < m0; ++t) s = fma(at(J, d1, mu, t), Di[t * m0 + q], s);
+      }
+      Ms[mu * mp + q] = s;
+    }
+    __syncthreads();
+  }
+  __device__ void store_M(int J, int d1, const double* Ms) const {
+    const int mp = m0 + 1;
+    double* f = fwd + (size_t)J * fst + (d1 - 1) * m0;
+    double* u = bwd + (size_t)(J + d1) * bst + d1 * m0;
+    for (int e = threadIdx.x; e < m2; e += blockDim.x) {
+      const int q = e / m0, mu = e % m0;
+      f[(size_t)q * D * m0 + mu] = Ms[mu * mp + q];
+      u[(size_t)q * D1 * m0 + mu] = Ms[q * mp + mu];
+    }
+  }
+  // A_{J+d1,J+d2} -= M_{d1} A_{d2}^T, d2 = da .. db
+  __device__ void update(int J, int d1, int da, int db, const double* col, const double* Ms, bool fits) const {
+    const int mp = m0 + 1;
+    for (int it = threadIdx.x; it < (db - da + 1) * m2; it += blockDim.x) {
+      const int d2 = da + it / m2, e = it % m2, mu = e / m0, nu = e % m0;
+      if (d1 == d2 && nu > mu) continue;       // diagonal block: lower triangle suffices
+      double* out = win(J + d1, d1 - d2) + e;
+      const double old = __ldcg(out);
+      double s = 0.0;
+      if (fits) {
+        const double* c = col + (d2 - 1) * m0 * mp + nu;
+        for (int q = 0; q < m0; ++q) s = fma(Ms[mu * mp + q], c[q * mp], s);
+      } else {
+        for (int q = 0; q < m0; ++q) s = fma(Ms[mu * mp + q], at(J, d2, nu, q), s);
+      }
+      *out = old - s;
+    }
+  }
+  __device__ void store_inverse(int J, const double* Di) const {
+    for (int e = threadIdx.x; e < m2; e += blockDim.x) {
+      dinv[(size_t)J * m2 + e] = Di[e];
+      if (J + D1 < L) bwd[(size_t)(J + D1) * bst + (size_t)(e / m0) * D1 * m0 + e % m0] = Di[e];
+    }
+  }
+};
+
+// Delta_J^-1 by Gauss-Jordan elimination without pivoting (positive definite exactly
+// when every pivot is positive, else *s_bad is set), between g0 and g1; returns the one
+// that holds it.
+__device__ double* band_invert(double* g0, double* g1, int m0, double* s_r, int* s_bad) {
+  const int tid = threadIdx.x, nth = blockDim.x, m2 = m0 * m0;
+  if (tid == 0) {
+    const double p = g0[0];
+    const bool pos = __double_as_longlong(p) > 0;
+    if (!pos || !(p == p)) *s_bad = 1;
+    s_r[0] = rcp_nr(pos ? p : 1.0);
+  }
+  __syncthreads();
+  double *cur = g0, *nxt = g1;
+  const int step = nth - nth % m0, j = tid % m0;   // a thread's entries lie in one column j
+  for (int k = 0; k < m0; ++k) {
+    const double r = s_r[k & 1];
+    if (tid < step) {
+      const double g = (j == k) ? r : cur[k * m0 + j] * r;   // row k of the next matrix
+      for (int e = tid, i = tid / m0; e < m2; e += step, i += step / m0) {
+        const double v = (i == k) ? g : fma(-cur[i * m0 + k], g, (j == k) ? 0.0 : cur[e]);
+        nxt[e] = v;
+        if (i == k + 1 && j == k + 1) {        // the next pivot
+          const bool pos = __double_as_longlong(v) > 0;
+          if (!pos || !(v == v)) *s_bad = 1;
+          s_r[(k + 1) & 1] = rcp_nr(pos ? v : 1.0);
+        }
+      }
+    }
+    __syncthreads();
+    double* swp = cur; cur = nxt; nxt = swp;
+  }
+  return cur;
+}
+
+}  // namespace
+
 // Bound by the chain of block columns, not by arithmetic throughput: column J
 // needs Delta_J^-1 (m0 dependent pivots), M_d = A_d Delta_J^-1, and the trailing
 // update A_{J+d1,J+d2} -= M_{d1} A_{d2}^T, D (D + 1) / 2 block products.  One SM
@@ -85,27 +250,24 @@ __device__ __forceinline__ int pair_row(int p) {
 // barrier per pivot, half of a Cholesky factor and its inverse) instead of
 // waiting for another CTA to do it; the M_d are made by one CTA each.  Every decision depends on values all CTAs
 // compute alike, so all take the same sequence of cluster barriers, and an
-// entry's arithmetic does not depend on the cluster's size.  Measured: 101 cells
-// of 16 functions 22.5 -> 1.9 ms (2.5 from one end), 64 cells of 8 1.96 -> 0.55 ms (0.75;
-// one problem, one factorisation), 32 of those 0.94 -> 0.79 ms, 512 cells of 32 50 -> 40.
+// entry's arithmetic does not depend on the cluster's size.  Measured: 64 cells
+// of 8 functions 1.96 -> 0.55 ms (0.75 from one end; one problem, one factorisation), 32 of
+// those 0.94 -> 0.79 ms.  Few problems of larger blocks go through k_band_column
+// first and leave to this kernel only those that need another shift.
 __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* __restrict__ tasks, int smem_doubles) {
   extern __shared__ double fsm[];
   const int CC = cl_size(), crank = cl_rank();
   const BandTask T = tasks[blockIdx.x / CC];
-  // a side's CTAs; L is the length of its chain, of which it eliminates a rows before
-  // the middle (all of them without twist)
+  if (T.sync[0] == 1) return;                  // factored by k_band_column
+  // a side's CTAs
   const int C = T.twist ? CC / 2 : CC, side = crank / C, rank = crank % C;
-  const int m0 = T.m0, m2 = m0 * m0, D = T.D, LL = T.L, mp = m0 + 1, D1 = D + 1;
-  const int a0 = (LL - D) / 2, a1 = LL - D - a0;   // a0 <= a1 <= a0 + 1
-  const int a = !T.twist ? LL : side ? a1 : a0, L = T.twist ? a + D : LL;
-  const size_t fst = band_step(D, m0), bst = band_step(D1, m0);
-  const size_t r0 = side ? a0 + D : 0;       // the side's first row of the factor
-  double *const Tfwd = T.fwd + r0 * fst, *const Tbwd = T.bwd + r0 * bst, *const Tdinv = T.dinv + r0 * m2;
+  BandSide B(T, side);
+  const int m0 = T.m0, m2 = m0 * m0, D = T.D, D1 = D + 1, mp = m0 + 1, L = B.L;
   const int tid = threadIdx.x, nth = blockDim.x, gtid = rank * nth + tid, gnth = C * nth;
   double* g0 = fsm;                          // diagonal block, its inverse in the end
   double* g1 = g0 + m2;
   double* Ms = g1 + m2;                      // M_{J+d1,J}, rows mp apart
-  double* col = Ms + m0 * mp;                // column J: [d-1][q][nu] = A_{J+d,J}[nu][q], rows mp apart
+  double* col = Ms + m0 * mp;                // column J
   const bool fits = 2 * m2 + D1 * m0 * mp <= smem_doubles;   // else the column is read from global memory
   __shared__ double s_r[2];
   __shared__ int s_bad;
@@ -121,63 +283,25 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
   double sg = *T.sigma0, sg_ok = NAN, sg_bad = NAN;
   int nbis = 0;
   bool stop = false;
-  // block (K, K-d) of the window; written by any CTA of the cluster: read from L2
-  auto winS = [&](int sd, int K, int d) { return T.win + ((size_t)(sd * D1 + K % D1) * D1 + d) * m2; };
-  auto win = [&](int K, int d) { return winS(side, K, d); };
-  // row K enters the window: Toeplitz part and boundary blocks (a position's
-  // entries lie one after another, its first one in efirst); side 1's block (K, K - d)
-  // is the transpose of the one at row LL - 1 - K + d, and its middle starts at zero
-  auto enter = [&](int K) {
-    for (int it = gtid; it < D1 * m2; it += gnth) {
-      const int d = it / m2, e = it % m2;
-      if (d > K) continue;
-      const int Kr = side ? LL - 1 - K + d : K, f = side ? (e % m0) * m0 + e / m0 : e;
-      double v = 0.0;
-      if (!side || K - d < a) {
-        v = T.TH[(size_t)d * m2 + f] - sg * T.TS[(size_t)d * m2 + f];
-        const int q0 = T.efirst[(size_t)Kr * D1 + d];
-        if (q0 >= 0) {
-          double x = 0.0;
-          for (int q = q0; q < T.nE && T.Ek[q] == Kr && T.Em[q] == Kr - d; ++q)
-            x += T.EH[(size_t)q * m2 + f] - sg * T.ES[(size_t)q * m2 + f];
-          v += x;
-        }
-      }
-      win(K, d)[e] = v;
-    }
-  };
-  // the middle's blocks (a + i, a + j), j <= i: on side 0 the sum of both sides' (its block
-  // is the transpose of side 1's (D - 1 - j, D - 1 - i)), on side 1 a copy of that
-  auto middle = [&](int sd) {
-    for (long long it = gtid; it < (long long)(D * (D + 1) / 2) * m2; it += gnth) {
-      const int p = (int)(it / m2), e = (int)(it % m2), mu = e / m0, nu = e % m0;
-      const int i = pair_row(p) - 1, j = p - i * (i + 1) / 2;
-      if (i == j && nu > mu) continue;         // diagonal blocks: lower triangle
-      const int f = i == j ? e : nu * m0 + mu;
-      const double x = __ldcg(winS(1 - sd, (sd ? a0 : a1) + D - 1 - j, i - j) + f);
-      double* out = win(a + i, i - j) + e;
-      *out = sd ? x : __ldcg(out) + x;
-    }
-  };
-  const int steps = T.twist ? a1 + D : L, late = T.twist ? a1 - a : 0;   // side 0 may start one step late
   for (int attempt = 0; attempt < 24; ++attempt) {
-    for (int K = 0; K < min(D1, L); ++K) enter(K);
+    B.sg = sg;
+    for (int K = 0; K < min(D1, L); ++K) B.enter(K, gtid, gnth);
     if (tid == 0) s_bad = 0;
     cl_arrive();
     cl_wait();
     bool bad = false;
-    for (int t = 0; t < steps; ++t) {
-      if (T.twist && t == a1) {                // both sides are at their first middle row
+    for (int t = 0; t < B.steps; ++t) {
+      if (T.twist && t == B.a1) {              // both sides are at their first middle row
         bad = bad || cl_load(&s_bad, (crank + C) % CC) != 0;
-        if (!side && !bad) middle(0);
+        if (!side && !bad) B.middle(gtid, gnth);
         cl_arrive();
         cl_wait();
-        if (side && !bad) middle(1);
+        if (side && !bad) B.middle(gtid, gnth);
         cl_arrive();
         cl_wait();
         if (bad) break;
       }
-      const int J = t - late;
+      const int J = t - B.late;
       if (J < 0 || (T.twist && bad)) {         // nothing to do: the step's barriers
         cl_arrive();
         cl_wait();
@@ -186,78 +310,16 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
         continue;
       }
       const int dmax = min(D, L - 1 - J);
-      auto Acol = [&](int d, int nu, int q) { return __ldcg(win(J + d, d) + nu * m0 + q); };
-      for (int e = tid; e < m2; e += nth) {   // lower triangle mirrored: exactly symmetric
-        const int i = e / m0, j = e % m0;
-        g0[e] = Acol(0, max(i, j), min(i, j));
-      }
-      if (fits) {
-        for (int it = tid; it < dmax * m2; it += nth) {
-          const int d = 1 + it / m2, e = it % m2, nu = e / m0, q = e % m0;
-          col[((d - 1) * m0 + q) * mp + nu] = Acol(d, nu, q);
-        }
-      }
-      __syncthreads();
-      // Delta_J^-1 by Gauss-Jordan elimination without pivoting (positive
-      // definite exactly when every pivot is positive)
-      if (tid == 0) {
-        const double p = g0[0];
-        const bool pos = __double_as_longlong(p) > 0;
-        if (!pos || !(p == p)) s_bad = 1;
-        s_r[0] = rcp_nr(pos ? p : 1.0);
-      }
-      __syncthreads();
-      double *cur = g0, *nxt = g1;
-      const int step = nth - nth % m0, j = tid % m0;   // a thread's entries lie in one column j
-      for (int k = 0; k < m0; ++k) {
-        const double r = s_r[k & 1];
-        if (tid < step) {
-          const double g = (j == k) ? r : cur[k * m0 + j] * r;   // row k of the next matrix
-          for (int e = tid, i = tid / m0; e < m2; e += step, i += step / m0) {
-            const double v = (i == k) ? g : fma(-cur[i * m0 + k], g, (j == k) ? 0.0 : cur[e]);
-            nxt[e] = v;
-            if (i == k + 1 && j == k + 1) {     // the next pivot
-              const bool pos = __double_as_longlong(v) > 0;
-              if (!pos || !(v == v)) s_bad = 1;
-              s_r[(k + 1) & 1] = rcp_nr(pos ? v : 1.0);
-            }
-          }
-        }
-        __syncthreads();
-        double* swp = cur; cur = nxt; nxt = swp;
-      }
-      const double* Di = cur;
+      B.load(J, dmax, g0, col, fits);
+      const double* Di = band_invert(g0, g1, m0, s_r, &s_bad);
       bad = s_bad != 0;
       // M_{J+d1,J} into Ms, and its storage for the solves: by one CTA each, read by
       // the others after a barrier (made anew where the column does not fit)
-      auto make_M = [&](int d1) {
-        for (int e = tid; e < m2; e += nth) {
-          const int mu = e / m0, q = e % m0;
-          double s = 0.0;
-          if (fits) {
-            const double* c = col + (d1 - 1) * m0 * mp + mu;
-            for (int t = 0; t < m0; ++t) s = fma(c[t * mp], Di[t * m0 + q], s);
-          } else {
-            for (int t = 0; t < m0; ++t) s = fma(Acol(d1, mu, t), Di[t * m0 + q], s);
-          }
-          Ms[mu * mp + q] = s;
-        }
-        __syncthreads();
-      };
-      auto store_M = [&](int d1) {
-        double* f = Tfwd + (size_t)J * fst + (d1 - 1) * m0;
-        double* u = Tbwd + (size_t)(J + d1) * bst + d1 * m0;
-        for (int e = tid; e < m2; e += nth) {
-          const int q = e / m0, mu = e % m0;
-          f[(size_t)q * D * m0 + mu] = Ms[mu * mp + q];
-          u[(size_t)q * D1 * m0 + mu] = Ms[q * mp + mu];
-        }
-      };
       if (fits) {
         if (!bad)
           for (int d1 = 1 + rank; d1 <= dmax; d1 += C) {
-            make_M(d1);
-            store_M(d1);
+            B.make_M(J, d1, col, Di, Ms, true);
+            B.store_M(J, d1, Ms);
             __syncthreads();
           }
         cl_arrive();                          // (and this CTA needs no more of column J)
@@ -271,41 +333,24 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
           const int d1 = pair_row(p), base = d1 * (d1 - 1) / 2;
           const int da = p - base + 1, db = min(d1, p1 - base);   // d2 in da..db
           if (fits) {
-            const double* f = Tfwd + (size_t)J * fst + (d1 - 1) * m0;
+            const double* f = B.fwd + (size_t)J * B.fst + (d1 - 1) * m0;
             for (int e = tid; e < m2; e += nth) Ms[(e % m0) * mp + e / m0] = __ldcg(f + (size_t)(e / m0) * D * m0 + e % m0);
             __syncthreads();
           } else {
-            make_M(d1);
-            if (da == 1) store_M(d1);          // the owner of (d1, 1)
+            B.make_M(J, d1, col, Di, Ms, false);
+            if (da == 1) B.store_M(J, d1, Ms);   // the owner of (d1, 1)
           }
-          for (int it = tid; it < (db - da + 1) * m2; it += nth) {
-            const int d2 = da + it / m2, e = it % m2, mu = e / m0, nu = e % m0;
-            if (d1 == d2 && nu > mu) continue;   // diagonal block: lower triangle suffices
-            double* out = win(J + d1, d1 - d2) + e;
-            const double old = __ldcg(out);
-            double s = 0.0;
-            if (fits) {
-              const double* c = col + (d2 - 1) * m0 * mp + nu;
-              for (int q = 0; q < m0; ++q) s = fma(Ms[mu * mp + q], c[q * mp], s);
-            } else {
-              for (int q = 0; q < m0; ++q) s = fma(Ms[mu * mp + q], Acol(d2, nu, q), s);
-            }
-            *out = old - s;
-          }
+          B.update(J, d1, da, db, col, Ms, fits);
           __syncthreads();
           p = base + db;
         }
-        if (rank == 0)
-          for (int e = tid; e < m2; e += nth) {
-            Tdinv[(size_t)J * m2 + e] = Di[e];
-            if (J + D1 < L) Tbwd[(size_t)(J + D1) * bst + (size_t)(e / m0) * D1 * m0 + e % m0] = Di[e];
-          }
+        if (rank == 0) B.store_inverse(J, Di);
       }
       if (!fits) {
         cl_arrive();
-        cl_wait();                            // every CTA has taken what it needs of row J's slot
+        cl_wait();                            // every CTA has taken what it needs of row J
       }
-      if (!bad && J + D1 < L) enter(J + D1);
+      if (!bad && J + D1 < L) B.enter(J + D1, gtid, gnth);
       cl_arrive();
       cl_wait();                              // the trailing update and the new row are visible to all
       if (bad && !T.twist) break;
@@ -332,6 +377,70 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_factor(const BandTask* 
     *T.sigma_used = sg;
     if (!stop && T.fail) *T.fail = 1;
   }
+}
+
+// The same factorisation at the first shift with a launch per block column, where a
+// cluster is too small for the block products (band_columns) of at most four problems.
+// A launch is a barrier over the whole GPU of about 4 us.  Every CTA inverts the
+// diagonal block and makes the M of its pairs for itself, so a column takes one
+// launch; the row that enters goes to a slot of its own (the window has one row more
+// than the band).  sync[1 + side]: a pivot was not positive, and what follows is
+// skipped; sync[0] = 1: done.  101 cells of 16 functions 1.90 -> 1.36 ms, 512 of 32 40 -> 19
+// ms, three rings of 61 cells of 16 with bound states 1.24 -> 0.98 ms.
+//   phase 0: the first rows; 1: block column t; 2, 3: the middle, side 0 then 1; 4: the end
+__global__ void __launch_bounds__(kFactorThreads) k_band_column(const BandTask* __restrict__ tasks, int phase, int t) {
+  extern __shared__ double fsm[];
+  const BandTask T = tasks[blockIdx.z];
+  if (!band_columns(T.m0, T.D)) return;
+  const int side = blockIdx.y, C = gridDim.x, rank = blockIdx.x;
+  if (side && !T.twist) return;
+  BandSide B(T, side);
+  B.sg = *T.sigma0;
+  const int tid = threadIdx.x, nth = blockDim.x, gtid = rank * nth + tid, gnth = C * nth;
+  if (phase == 0) {
+    for (int K = 0; K < min(B.D1, B.L); ++K) B.enter(K, gtid, gnth);
+    if (rank == 0 && side == 0 && tid < 3) T.sync[tid] = 0;
+    return;
+  }
+  if (phase >= 2 && phase <= 3) {
+    if (!T.twist || t != B.a1 || side != phase - 2 || T.sync[1] || T.sync[2]) return;
+    B.middle(gtid, gnth);
+    return;
+  }
+  if (phase == 4) {
+    if (rank == 0 && side == 0 && tid == 0 && !T.sync[1] && !T.sync[2]) {
+      T.sync[0] = 1;
+      *T.sigma_used = B.sg;
+    }
+    return;
+  }
+  const int J = t - B.late;
+  if (J < 0 || J >= B.L || T.sync[1 + side] || (t >= B.a1 && (T.sync[1] || T.sync[2]))) return;
+  const int m0 = T.m0, m2 = m0 * m0;
+  double *g0 = fsm, *g1 = g0 + m2, *Ms = g1 + m2, *col = Ms + m0 * (m0 + 1);
+  __shared__ double s_r[2];
+  __shared__ int s_bad;
+  const int dmax = min(B.D, B.L - 1 - J), np = dmax * (dmax + 1) / 2;
+  const int p0 = (int)((long long)np * rank / C), p1 = (int)((long long)np * (rank + 1) / C);
+  if (J + B.D1 < B.L) B.enter(J + B.D1, gtid, gnth);
+  if (p0 >= p1 && rank != 0) return;
+  if (tid == 0) s_bad = 0;
+  B.load(J, dmax, g0, col, true);
+  const double* Di = band_invert(g0, g1, m0, s_r, &s_bad);
+  if (s_bad) {                                 // (every CTA finds the same)
+    if (rank == 0 && tid == 0) T.sync[1 + side] = 1;
+    return;
+  }
+  for (int p = p0; p < p1;) {
+    const int d1 = pair_row(p), base = d1 * (d1 - 1) / 2;
+    const int da = p - base + 1, db = min(d1, p1 - base);   // d2 in da..db
+    B.make_M(J, d1, col, Di, Ms, true);
+    if (da == 1) B.store_M(J, d1, Ms);         // the owner of (d1, 1)
+    B.update(J, d1, da, db, col, Ms, true);
+    __syncthreads();
+    p = base + db;
+  }
+  if (rank == 0) B.store_inverse(J, Di);
 }
 
 // 16-byte asynchronous global -> shared copies (L2 only)
@@ -511,7 +620,7 @@ __global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict_
 // maxcol: the largest m0 (m0 + 1) (D + 3) among the tasks (shared doubles that
 // hold a block column; capped at what the device has, the kernel then reads the
 // column from global memory)
-void launch_band_factor(const BandTask* t, int n, int maxcol, int maxm0, cudaStream_t st) {
+void launch_band_factor(const BandTask* t, int n, int maxcol, int maxm0, const BandSteps& cs, cudaStream_t st) {
   if (!n) return;
   FOCK_SMEM_OPTIN(k_band_factor);
   {
@@ -529,6 +638,26 @@ void launch_band_factor(const BandTask* t, int n, int maxcol, int maxm0, cudaStr
   // 0.94 / 1.04 / 1.19, 128 3.7 / 2.3 / 1.65; 64 cells of 16, 32 problems 3.4 / 3.1 /
   // 3.3; 64 cells of 32, 8 problems 16.0 / 11.7 / 18.4.
   int C = (n <= 4) ? 16 : (n <= 64) ? 8 : 4;
+  if (n <= kColumnProblems && cs.steps && maxcol <= cap) {
+    FOCK_SMEM_OPTIN(k_band_column);
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // CTAs per side: no more than the largest share of the pairs needs
+    const int most = std::max(1, sms / (n * cs.sides)), share = (cs.pairs + most - 1) / most;
+    const int cta = (cs.pairs + share - 1) / share;
+    const dim3 grid((unsigned)cta, (unsigned)cs.sides, (unsigned)n);
+    const int th = maxm0 > 16 ? kFactorThreads : 256;
+    const size_t sm = (size_t)doubles * 8;
+    k_band_column<<<grid, th, sm, st>>>(t, 0, 0);
+    for (int i = 0; i < cs.steps; ++i) {
+      if (std::binary_search(cs.middles.begin(), cs.middles.end(), i)) {
+        k_band_column<<<grid, th, sm, st>>>(t, 2, i);
+        k_band_column<<<grid, th, sm, st>>>(t, 3, i);
+      }
+      k_band_column<<<grid, th, sm, st>>>(t, 1, i);
+    }
+    k_band_column<<<dim3(1, 1, n), 32, 0, st>>>(t, 4, 0);
+  }
   cudaLaunchConfig_t cfg = {};
   // (64 cells of 32 functions 6.5 ms with 256 threads, 5.9 with 512; of 8 0.76 and 0.82)
   cfg.blockDim = dim3(maxm0 > 16 ? kFactorThreads : 256);
