@@ -220,7 +220,8 @@ int fock_bloch_vectors(fock_ctx* ctx, const fock_blocks* b, int nsel, const int*
 
 /* y = H x or y = S x (which = FOCK_OP_H / FOCK_OP_S) for an assembled box
  * chain or problem with defects, by the block-circulant embedding FFT
- * matvec plus the boundary/defect blocks (Remark 3.2, Sec. 2.3).  x, y:
+ * matvec plus the boundary/defect blocks (Remark 3.2, Sec. 2.3), small
+ * products block by block.  x, y:
  * N_b x nvec, column-major; device pointers when on_device != 0, else
  * host.  Errors: FOCK_EINVAL (a periodic handle -- its operator is applied
  * through its Fourier blocks -- null pointers, `which`, nvec < 1, device x

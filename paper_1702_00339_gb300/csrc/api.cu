@@ -57,6 +57,7 @@ void launch_fft(const FftTask*, int, int, int, int, int, cudaStream_t, bool);
 void launch_fft_cc(const FftTask*, int, int, int, int, int, cudaStream_t, bool);
 int fft_max_cc(int);
 void launch_blockmul(const BmulTask*, int, int, int, cudaStream_t, bool);
+void launch_band_apply(const BandApply&, cudaStream_t);
 void launch_eapply(const EApplyTask*, int, int, int, int, bool, cudaStream_t);
 void launch_band_factor(const BandTask*, int, int, int, const BandSteps&, cudaStream_t);
 void launch_band_solve(const BandTask*, int, int, int, int, int, int, int, cudaStream_t, bool);
@@ -2720,16 +2721,27 @@ int fock_toeplitz_matvec(fock_ctx* ctx, const fock_blocks* b, int which, const d
   const size_t nbytes = (size_t)n * nvec * 8;
   if (on_device && (const char*)x < (const char*)y + nbytes && (const char*)y < (const char*)x + nbytes)
     return set_err(ctx, FOCK_EINVAL, "matvec: device x and y must not overlap");
+  const bool direct = (double)Q.Lc * (2 * Q.D + 1) * H.m0 * H.m0 * nvec <= kApplyMacs;
   const size_t vb = (nbytes + 255) & ~(size_t)255;
-  const size_t xb = ((size_t)Q.M * H.m0 * nvec * sizeof(cplx) + 255) & ~(size_t)255;
+  const size_t xb = direct ? 0 : ((size_t)Q.M * H.m0 * nvec * sizeof(cplx) + 255) & ~(size_t)255;
+  const size_t need = (direct ? 0 : 4096 + 2 * xb) + (on_device ? 0 : 2 * vb);
   Scratch scratch;
-  CUDA_TRY(ctx, scratch.get(ctx, 4096 + 2 * xb + (on_device ? 0 : 2 * vb)));
+  if (need) CUDA_TRY(ctx, scratch.get(ctx, need));
+  double* dx = on_device ? const_cast<double*>(x) : (double*)(scratch.p + need - 2 * vb);
+  double* dy = on_device ? y : (double*)(scratch.p + need - vb);
+  if (!on_device) CUDA_TRY(ctx, cudaMemcpyAsync(dx, x, nbytes, cudaMemcpyHostToDevice, st));
+  if (direct) {
+    BandApply t = {H.m0, Q.Lc, Q.D, nvec, Q.nE ? Q.nErows : 0, which == FOCK_OP_H ? Q.TH : Q.TS,
+                   Q.Erows, Q.Erowptr, Q.Ecols, which == FOCK_OP_H ? Q.EH : Q.ES, dx, dy, n, n};
+    launch_band_apply(t, st);
+    if (!on_device) CUDA_TRY(ctx, cudaMemcpyAsync(y, dy, nbytes, cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(ctx, cudaStreamSynchronize(st));
+    CUDA_TRY(ctx, cudaGetLastError());
+    return FOCK_OK;
+  }
   char* const tasks = scratch.p;
   cplx* const X = (cplx*)(scratch.p + 4096);
   cplx* const Y = (cplx*)(scratch.p + 4096 + xb);
-  double* dx = on_device ? const_cast<double*>(x) : (double*)(scratch.p + 4096 + 2 * xb);
-  double* dy = on_device ? y : (double*)(scratch.p + 4096 + 2 * xb + vb);
-  if (!on_device) CUDA_TRY(ctx, cudaMemcpyAsync(dx, x, nbytes, cudaMemcpyHostToDevice, st));
   int cc = std::max(1, std::min(16, 98304 / (32 * Q.M)));
   FftTask tf; std::memset(&tf, 0, sizeof(tf));
   tf.prob = 0; tf.L = Q.Lc; tf.m0 = H.m0; tf.ncol = nvec; tf.circ = B.d_circs + Q.circ; tf.x = dx; tf.ldx = n;

@@ -286,6 +286,21 @@ struct BmulTask {
   const int* active;               // as FftTask::active
 };
 
+// A small product with a chain's operator, block by block (k_band_apply): its generators and
+// boundary blocks as in EApplyTask, in the original basis.
+struct BandApply {
+  int m0, L, D, ncol, nrows;
+  const double* T;             // [D+1][m0*m0], T_d = block (k + d, k)
+  const int *rows, *rowptr, *cols;
+  const double* vals;
+  const double* x; double* y;
+  int ldx, ldy;
+};
+constexpr int kApplyCols = 4;
+// Multiply-adds up to which the block-by-block product is taken: 64 cells of 8 functions,
+// 72 vectors (8e6) 38 us against 65 through the transforms, 512 of 8, 8 vectors 38 against 128;
+// 128 of 32, 4 vectors (1.4e7) 119 against 117.
+constexpr double kApplyMacs = 8e6;
 struct EApplyTask {
   int prob, m0, ncol, nrows;
   const int* rows;      // [nrows] block-row ids

@@ -361,4 +361,63 @@ void launch_eapply(const EApplyTask* tasks, int ntask, int maxrows, int maxcols,
   k_eapply<<<dim3(maxrows, (maxcols + kECols - 1) / kECols, ntask), kECols * maxm0, sm, st>>>(tasks);
 }
 
+// y = (BToepl(T) + E) x block by block, for products too small to be worth transforms:
+// four launches and the descriptors' copy took 40 us whatever the size.  A CTA per
+// block row and four columns; thread (slice, mu) adds every S-th block of the row's
+// band, then of its boundary and defect blocks, and the slices are added pairwise.
+// Latency from the first loads to the last sum.  64 cells of 8 functions (D = 13),
+// one vector: 65 -> 18 us a call.
+__global__ void __launch_bounds__(256) k_band_apply(const BandApply T) {
+  __shared__ double part[256][kApplyCols + 1];
+  __shared__ int s_ri;
+  const int m0 = T.m0, k = blockIdx.x, v0 = blockIdx.y * kApplyCols, tid = threadIdx.x;
+  const int S = 256 / m0, mu = tid % m0, s = tid / m0, nv = min(kApplyCols, T.ncol - v0);
+  if (tid == 0) s_ri = -1;
+  __syncthreads();
+  for (int i = tid; i < T.nrows; i += 256)
+    if (T.rows[i] == k) s_ri = i;
+  __syncthreads();
+  const int e0 = s_ri < 0 ? 0 : T.rowptr[s_ri], e1 = s_ri < 0 ? 0 : T.rowptr[s_ri + 1];
+  double acc[kApplyCols];
+#pragma unroll
+  for (int c = 0; c < kApplyCols; ++c) acc[c] = 0.0;
+  if (s < S) {
+    // entry nu of the block's row mu: a[nu sn]; columns of x: xb[nu + c ldx]
+    auto block = [&](const double* a, int sn, int col) {
+      const double* xb = T.x + (size_t)col * m0 + (size_t)T.ldx * v0;
+#pragma unroll 8
+      for (int nu = 0; nu < m0; ++nu) {
+        const double w = a[(size_t)nu * sn];
+#pragma unroll
+        for (int c = 0; c < kApplyCols; ++c)
+          if (c < nv) acc[c] = fma(w, xb[nu + (size_t)T.ldx * c], acc[c]);
+      }
+    };
+    for (int b = max(0, T.D - k) + s; b < min(2 * T.D + 1, T.L - k + T.D); b += S) {
+      const int d = b - T.D;                       // block (k, k + d): T_-d below the diagonal, T_d^T above
+      if (d <= 0) block(T.T + (size_t)(-d) * m0 * m0 + mu * m0, 1, k + d);
+      else block(T.T + (size_t)d * m0 * m0 + mu, m0, k + d);
+    }
+    for (int e = e0 + s; e < e1; e += S) block(T.vals + (size_t)e * m0 * m0 + mu * m0, 1, T.cols[e]);
+#pragma unroll
+    for (int c = 0; c < kApplyCols; ++c) part[tid][c] = acc[c];
+  }
+  __syncthreads();
+  for (int n = S; n > 1;) {
+    const int h = (n + 1) / 2;
+    if (s < n - h)
+#pragma unroll
+      for (int c = 0; c < kApplyCols; ++c) part[tid][c] += part[tid + h * m0][c];
+    __syncthreads();
+    n = h;
+  }
+  for (int it = tid; it < m0 * nv; it += 256) {
+    const int m = it % m0, c = it / m0;
+    T.y[(size_t)k * m0 + m + (size_t)T.ldy * (v0 + c)] = part[m][c];
+  }
+}
+void launch_band_apply(const BandApply& T, cudaStream_t st) {
+  k_band_apply<<<dim3(T.L, (T.ncol + kApplyCols - 1) / kApplyCols), 256, 0, st>>>(T);
+}
+
 }  // namespace fock
