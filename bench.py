@@ -719,8 +719,8 @@ def main():
              "statuses_nonzero": sum(1 for o in mouts if o["status"] != 0),
              "box_iters": [int(o["iters"]) for o in mouts[:args.batch]],
              "form": "FOCK_MIXED: the assembly's quadrature contractions and the block iteration's Gram "
-                     "and basis products as exact split products on tcgen05 tensor cores (BF16 digits, "
-                     "FP32 TMEM sums, FP64 combination); Rayleigh-Ritz, matvecs, preconditioner and "
+                     "and basis products as exact split products on tcgen05 tensor cores (FP16 digits, "
+                     "FP32 TMEM sums, integer combination); Rayleigh-Ritz, matvecs, preconditioner and "
                      "Fourier-block eigensolves FP64"}
 
     # ---- end to end through fock_solve (host inputs and outputs) ----

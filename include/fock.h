@@ -300,9 +300,9 @@ int fock_plan_problem_sizes(const fock_plan* plan, int i, int* Nb, int* mcirc, i
  * returns n, or FOCK_EINVAL. */
 int fock_plan_history(const fock_plan* plan, int i, double* res, int cap);
 /* Tensor-core work of one execution of a plan's mixed-form assembly
- * (fock_split_dgemm products of its gram tasks): the BF16 multiply-add
- * flops the MMAs execute (128 x 64 output tiles, 64-long chunks, 28 digit
- * pairs, 4 MMAs of K = 16 each) and the FP64 flops they stand for (2 M N K).
+ * (fock_split_dgemm products of its gram tasks): the FP16 multiply-add
+ * flops the MMAs execute (128 x 64 output tiles, stages of 32 summands, 36
+ * digit pairs) and the FP64 flops they stand for (2 M N K).
  * Zero for a plan without mixed problems. */
 int fock_plan_split_work(const fock_plan* plan, double* tensor_flops, double* fp64_flops);
 void fock_plan_free(fock_plan* plan);
@@ -317,14 +317,14 @@ int fock_profile_reset(fock_ctx* ctx);
 int fock_profile_read(fock_ctx* ctx, int cap, char* names, int* launches, double* ms);
 
 /* C = alpha A B + beta C in FP64 on the tensor cores: the exact split
- * products (base-128 digits of the 53-bit mantissas, BF16 x BF16 -> FP32
- * tcgen05 products, integer level sums combined in FP64) that the mixed
+ * products (base-128 digits of the mantissas, FP16 x FP16 -> FP32 tcgen05
+ * products, integer level sums) that the mixed
  * form uses for the quadrature contractions of stage (a) (Lemma 2.1
  * display; X_t = sum_r P_t[r] Z[r]).  A: M x K with element (m, k) at
  * A[m*a_m + k*a_k]; B: K x N, (k, n) at B[k*b_k + n*b_n]; C: (m, n) at
  * C[m*c_m + n*c_n]; all device pointers, strides in elements.  Each product
- * carries a relative error below ~2^-46 of |row max of A| |column max of B|
- * per summand.  ksplit (1..1024): the summation is split into that many
+ * carries a relative error below ~2^-50 of |row max of A| |column max of B|
+ * per summand (largest over ranges of at most 512 summands).  ksplit (1..1024): the summation is split into that many
  * ranges computed by separate CTAs and added in a fixed order (a work array
  * is allocated for them); sym != 0 (M = N): C is taken as symmetric, its
  * upper triangle computed and mirrored (the Gram products of the block

@@ -162,6 +162,7 @@ const int kPeriodicPiece = 1024;
 const size_t kPfWorkBytes = (size_t)1 << 30;
 
 const uint64_t kScratchKeep = (uint64_t)256 << 20;
+const size_t kScratchFirst = (size_t)16 << 20;
 
 void scratch_create(fock_ctx* c) {
   cudaMemPoolProps pr = {};
@@ -174,6 +175,10 @@ void scratch_create(fock_ctx* c) {
     c->scratch = nullptr;
   } else {
     cudaMemPoolSetAttribute(c->scratch, cudaMemPoolAttrReleaseThreshold, &keep);
+    // the first pages, which a first small call would otherwise wait 100 us for
+    void* p = nullptr;
+    if (cudaMallocFromPoolAsync(&p, kScratchFirst, c->scratch, c->stream) == cudaSuccess) cudaFreeAsync(p, c->stream);
+    else cudaGetLastError();
   }
 }
 // A call's device workspace, stream-ordered from the context's pool (a cudaMalloc and
