@@ -45,7 +45,7 @@ void launch_axis_dft(const ProbDev*, const DftTask*, int, int, cudaStream_t);
 size_t pf_layout(char*, int, size_t, PfWork*);
 void launch_pf(const ProbDev*, const PfTask*, const PfGroup*, int, const PfWork&, cudaStream_t);
 void launch_fblocks(const ProbDev*, const FBlockTask*, int, int, int, cudaStream_t, bool vectors = false,
-                    int x0 = 0, int nx = -1, bool any_odd = true);
+                    bool any_odd = true);
 void launch_bloch_vectors(int, int, int, int, int, const int*, const cplx*, const int*, cplx*, cudaStream_t);
 void launch_split_gemm(const SplitTask*, int, int, int, int*, cudaStream_t, int max_ks = 1, bool reduce = false);
 void launch_null_tau(const NullTask*, int, cudaStream_t);
@@ -1590,7 +1590,7 @@ void run_struct_setup(fock_ctx* ctx, Batch& B) {
   { PROF("k_cell_canon", 2); launch_cell_canon(B.d_canon, (int)B.canon.size(), B.maxm0, B.maxcblk, st); }
   { PROF("k_twiddle", 1); launch_twiddles(B.d_circs, (int)B.circs.size(), st); }
   { PROF("k_fblocks_embed", 1);
-    launch_fblocks(B.d_probs, B.d_fbs, (int)B.fbs.size(), B.maxnj_s, B.maxm0, st, false, 0, -1, B.odd_m0); }
+    launch_fblocks(B.d_probs, B.d_fbs, (int)B.fbs.size(), B.maxnj_s, B.maxm0, st, false, B.odd_m0); }
   { PROF("k_precond", 2); launch_precond(B.d_probs, B.d_prec, (int)B.prec.size(), B.maxM, B.maxm0, st); }
   for (auto& Q : B.pp)
     if (Q.band_fail) cudaMemsetAsync(Q.band_fail, 0, 4 * sizeof(int), st);
@@ -2646,8 +2646,7 @@ int fock_bloch_vectors(fock_ctx* ctx, const fock_blocks* b, int nsel, const int*
   { PROF("k_null_tau", 1); launch_null_tau(B.d_nulls, (int)B.nulls.size(), st); }
   std::vector<FBlockTask> tasks(nd);
   const size_t nbv = (size_t)ncell * m0;
-  const size_t off_ev = 0, off_y = ((size_t)nd * m0 * 8 + 255) & ~(size_t)255;
-  const size_t off_t = (off_y + (size_t)nd * m0 * m0 * sizeof(cplx) + 255) & ~(size_t)255;
+  const size_t off_t = ((size_t)nd * m0 * m0 * sizeof(cplx) + 255) & ~(size_t)255;
   const size_t off_i = (off_t + nd * sizeof(FBlockTask) + 255) & ~(size_t)255;
   const size_t off_u = (off_i + 2 * (size_t)nsel * sizeof(int) + 255) & ~(size_t)255;
   char* mem = nullptr;
@@ -2655,8 +2654,8 @@ int fock_bloch_vectors(fock_ctx* ctx, const fock_blocks* b, int nsel, const int*
   for (int q = 0; q < nd; ++q) {
     FBlockTask f = B.fbp[0];
     f.j0 = blocks_needed[q]; f.nj = 1; f.outH = nullptr; f.outS = nullptr; f.want = 1;
-    f.ev = (double*)(mem + off_ev) + (size_t)q * m0; f.blk = nullptr; f.fail = nullptr;
-    f.vecs = (cplx*)(mem + off_y) + (size_t)q * m0 * m0;
+    f.ev = nullptr; f.blk = nullptr; f.fail = nullptr;
+    f.vecs = (cplx*)mem + (size_t)q * m0 * m0;
     tasks[q] = f;
   }
   std::vector<int> ibuf(2 * (size_t)nsel);
@@ -2667,7 +2666,7 @@ int fock_bloch_vectors(fock_ctx* ctx, const fock_blocks* b, int nsel, const int*
   if (e == cudaSuccess) {
     { PROF("k_fblocks_eig", 1); launch_fblocks(B.d_probs, (const FBlockTask*)(mem + off_t), nd, 1, m0, st, true); }
     { PROF("k_bloch_vectors", 1);
-      launch_bloch_vectors(H.L[0], H.L[1], H.L[2], m0, nsel, (const int*)(mem + off_i), (const cplx*)(mem + off_y),
+      launch_bloch_vectors(H.L[0], H.L[1], H.L[2], m0, nsel, (const int*)(mem + off_i), (const cplx*)mem,
                            (const int*)(mem + off_i) + nsel, (cplx*)(mem + off_u), st); }
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(U, mem + off_u, nbv * nsel * sizeof(cplx), cudaMemcpyDeviceToHost, st);

@@ -1,8 +1,8 @@
 // Stage (b) and the Fourier side of stage (c).
 //
 //  k_fblocks   one CTA per Fourier index j: forms the m0 x m0 Hermitian pair
-//              (Hbar_j, Sbar_j) and, on request, stores it and/or solves the
-//              generalized eigenproblem Hbar u = l Sbar u in FP64.
+//              (Hbar_j, Sbar_j) and, on request, stores it, finds its lowest
+//              eigenvalue or its eigenvectors, Hbar u = l Sbar u, in FP64.
 //     source FACTORS (periodic lattice, Thm. 3.3 with the CP rank of the
 //       potential, Remark 3.5): Hbar_j = 1/2 sum_p (prod_{l!=p} Shat_l) Ahat_p
 //       - sum_t w_t prod_l Mhat_{l,t}, Sbar_j = prod_l Shat_l, elementwise in
@@ -18,12 +18,13 @@
 //       X = Q_K diag(s_K)^-1/2 over the kept directions K = {s > tau} (tau the
 //       problem's dependency cut: every direction when none is numerically
 //       singular, so C = X^H Hbar X has the pencil's eigenvalues exactly) --
-//       then Householder reduction of C to a real tridiagonal and
-//       Sturm-sequence bisection per eigenvalue, FP32 first then FP64 with
-//       division-free counts (ascending, so the block spectrum comes out
-//       sorted); the removed directions report +inf.  The lowest eigenvalue
-//       of an embedding block (preconditioner shift only) stops at 1e-9
-//       relative.  One warp per block for m0 <= 8.
+//       then the eigenvectors of C by Jacobi, or Householder reduction to a real
+//       tridiagonal and Sturm-sequence bisection for the lowest eigenvalue of an
+//       embedding block (preconditioner shift only: 1e-9 relative). One warp
+//       per block for m0 <= 8.
+//  k_pf_*       the spectra of periodic lattices by the same reductions: a
+//               pipeline over chunks of blocks, described there. Eigenvalues
+//               ascend within a block, removed directions report +inf.
 //  k_sigma      shift of the preconditioner: min_j lambda_min(Chat_j) - delta.
 //  k_precond    K_j = (Chat_H,j - sigma Chat_S,j)^-1 per Fourier index.
 //  k_sort_*     ascending sort of (eigenvalue, Fourier index) pairs.
@@ -630,10 +631,10 @@ __device__ void reform_S(const FBlockTask& F, const ProbDev& P, int j, int m0, c
   }
 }
 
-__global__ void k_fblocks(const ProbDev* __restrict__ probs, const FBlockTask* __restrict__ tasks, int x0) {
+__global__ void k_fblocks(const ProbDev* __restrict__ probs, const FBlockTask* __restrict__ tasks) {
   extern __shared__ cplx sm[];
   const FBlockTask F = tasks[blockIdx.y];
-  const int jl = x0 + blockIdx.x; // local output index (a launch may cover a range of them)
+  const int jl = blockIdx.x;      // local output index
   if (jl >= F.nj) return;
   const int j = F.j0 + jl;        // Fourier index
   // Real generators: the block at -j (componentwise mod L) is the complex
@@ -792,7 +793,7 @@ __global__ void k_fblocks(const ProbDev* __restrict__ probs, const FBlockTask* _
     for (int it = threadIdx.x; it < r * r; it += blockDim.x) Vc[(it / r) * ldr + it % r] = H[it];
     __syncthreads();
   }
-  const bool values = F.want != 1 || F.ev;      // vectors alone: no eigenvalues
+  const bool values = F.want == 2;
   if (values && r > 0) cta_tridiag(H, r, dd, ee, v, pv);
   for (int i = threadIdx.x; values && i < r; i += blockDim.x) {
     const double e2i = (i + 1 < r) ? ee[i] * ee[i] : 0.0;
@@ -801,17 +802,7 @@ __global__ void k_fblocks(const ProbDev* __restrict__ probs, const FBlockTask* _
     e2f[i] = (float)e2i;
   }
   __syncthreads();
-  if (F.want == 1 && F.ev) {
-    for (int i = threadIdx.x; i < m0; i += blockDim.x) {
-      const double lam = (i < r) ? tridiag_eig_fast(df, e2f, dd, e2, r, i, 0.0) : INFINITY;
-      F.ev[(size_t)jl * m0 + i] = lam;
-      if (F.blk) F.blk[(size_t)jl * m0 + i] = j;
-      if (jm >= 0) {   // the conjugate block's spectrum
-        F.ev[(size_t)(jm - F.j0) * m0 + i] = lam;
-        if (F.blk) F.blk[(size_t)(jm - F.j0) * m0 + i] = jm;
-      }
-    }
-  } else if (F.want == 2 && threadIdx.x == 0) {
+  if (F.want == 2 && threadIdx.x == 0) {
     // the lowest eigenvalue of an embedding block only sets the preconditioner
     // shift (lowered by 2e-5 relative afterwards): 1e-9 relative suffices
     F.ev[jl] = (r > 0) ? tridiag_eig_fast(df, e2f, dd, e2, r, 0, 1e-9) : INFINITY;
@@ -1656,12 +1647,9 @@ size_t fblocks_smem(int m0, bool vectors, bool any_odd) {
          (vectors ? 16 + 2 * ldj * ldj * sizeof(cplx) : 0);
 }
 
-// x0, nx: the launch covers local indices x0 .. x0 + nx - 1 of every task
-// (nx < 0: up to maxnj), so that a large solve can be issued in pieces
 void launch_fblocks(const ProbDev* probs, const FBlockTask* tasks, int ntask, int maxnj, int maxm0,
-                    cudaStream_t st, bool vectors, int x0, int nx, bool any_odd) {
-  const int gx = (nx < 0) ? maxnj - x0 : std::min(nx, maxnj - x0);
-  if (!ntask || gx <= 0) return;
+                    cudaStream_t st, bool vectors, bool any_odd) {
+  if (!ntask || maxnj <= 0) return;
   size_t sm = fblocks_smem(maxm0, vectors, any_odd);
   FOCK_SMEM_OPTIN(k_fblocks);
   {   // the largest shared-memory carveout: four 32 x 32 blocks (~54 KB each) per SM
@@ -1672,7 +1660,7 @@ void launch_fblocks(const ProbDev* probs, const FBlockTask* tasks, int ntask, in
   // parallel items: one warp for m0 <= 8 (more independent blocks resident
   // per SM keep the FP64 pipe busy), up to four warps for m0 = 32
   const int threads = (maxm0 <= 8) ? 32 : (maxm0 <= 16) ? 64 : 128;
-  k_fblocks<<<dim3(gx, ntask), threads, sm, st>>>(probs, tasks, x0);
+  k_fblocks<<<dim3(maxnj, ntask), threads, sm, st>>>(probs, tasks);
 }
 
 // Bytes of workspace for nslot blocks of order at most m, and its layout. The arrays
