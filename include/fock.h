@@ -324,8 +324,9 @@ int fock_profile_read(fock_ctx* ctx, int cap, char* names, int* launches, double
  * A[m*a_m + k*a_k]; B: K x N, (k, n) at B[k*b_k + n*b_n]; C: (m, n) at
  * C[m*c_m + n*c_n]; all device pointers, strides in elements.  Each product
  * carries a relative error below ~2^-50 of |row max of A| |column max of B|
- * per summand (largest over ranges of at most 512 summands).  ksplit (1..1024): the summation is split into that many
- * ranges computed by separate CTAs and added in a fixed order (a work array
+ * per summand (largest over ranges of at most 512 summands).  ksplit
+ * (1..1024): the summation is split into at most that many ranges, computed
+ * by separate CTAs and added in a fixed order (a work array
  * is allocated for them); sym != 0 (M = N): C is taken as symmetric, its
  * upper triangle computed and mirrored (the Gram products of the block
  * iteration).  Synchronous on the context's stream.  Errors: FOCK_EINVAL,

@@ -47,6 +47,7 @@ void launch_pf(const ProbDev*, const PfTask*, const PfGroup*, int, const PfWork&
 void launch_fblocks(const ProbDev*, const FBlockTask*, int, int, int, cudaStream_t, bool vectors = false,
                     bool any_odd = true);
 void launch_bloch_vectors(int, int, int, int, int, const int*, const cplx*, const int*, cplx*, cudaStream_t);
+int split_ranges(const SplitTask&, int, int);
 void launch_split_gemm(const SplitTask*, int, int, int, int*, cudaStream_t, int max_ks = 1, bool reduce = false);
 void launch_null_tau(const NullTask*, int, cudaStream_t);
 void launch_precond(const ProbDev*, const PrecTask*, int, int, int, cudaStream_t);
@@ -2689,8 +2690,11 @@ int fock_split_dgemm(fock_ctx* ctx, int M, int N, int K, const double* A, long l
   std::memset(&t, 0, sizeof(t));
   t.M = M; t.N = N; t.K = K; t.A = A; t.a_m = a_m; t.a_k = a_k; t.B = B; t.b_k = b_k; t.b_n = b_n;
   t.C = C; t.c_m = c_m; t.c_n = c_n; t.alpha = alpha; t.beta = beta;
-  t.ksplit = ksplit; t.sym = sym ? 1 : 0;
+  t.sym = sym ? 1 : 0;
   const bool red = ksplit > 1 || sym;
+  int sms = 1;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+  ksplit = t.ksplit = split_ranges(t, ksplit, std::max(sms, 1));
   const size_t off_w = 256 + ((sizeof(SplitTask) + 255) & ~(size_t)255);
   const size_t wbytes = red ? (((size_t)ksplit * M * N * sizeof(double) + 255) & ~(size_t)255) : 0;
   Scratch scratch;

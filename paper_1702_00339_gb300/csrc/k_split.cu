@@ -20,7 +20,7 @@
 // product per summand; on random operands 6e-16 to 3e-15 of the largest entries'
 // product (with 7 truncated digits aligned over 64 summands, as this was: 1e-13).
 //
-// One CTA of 256 threads per 128 x 64 output tile and K range.  Stages of KC = 32
+// One CTA of 384 threads per 128 x 64 output tile and K range.  Stages of KC = 32
 // summands in two buffers: the threads load and split the next stage while the
 // tensor core works on this one.  A thread splits eight summands of a row into the
 // 16 bytes of a core matrix row per plane (no-swizzle K-major layout: 8 rows x 16
@@ -30,9 +30,9 @@
 // A plane: 12 reads of A instead of 36.  One thread issues; every wait is bounded
 // (clock64), after which the kernel flags an error, frees its TMEM and returns.
 //
-// 216 x 216 x 16384 (a symmetric Gram product, 32 ranges): 384 -> 140 us with
-// the reduction; bound by the splitting, 55 instructions per summand and row that every
-// tile does for its own rows and columns, and by 192 tiles on 152 SMs.
+// 216 x 216 x 16384 (a symmetric Gram product, at most 32 ranges): 384 -> 119 us with
+// the reduction; bound by the ALU pipe of the splitting (84 % where CTAs run), about 55
+// instructions per summand and row that every tile does for its own rows and columns.
 #include <cuda_fp16.h>
 #include <stdint.h>
 
@@ -43,6 +43,7 @@ namespace fock {
 namespace {
 
 constexpr int TM = 128, TN = 64, KC = 32, NDIG = 8;                // digit levels g = 2 .. NDIG + 1
+constexpr int kSplitThreads = 384;   // three warps a sub-partition split the operands, eight of the twelve read TMEM
 constexpr int TMEM_COLS = 512;                                     // NDIG * TN
 constexpr uint32_t A_PLANE = TM * KC * 2, B_PLANE = TN * KC * 2;   // bytes per digit plane
 constexpr uint32_t STAGE = NDIG * (A_PLANE + B_PLANE);
@@ -206,7 +207,7 @@ __global__ void __launch_bounds__(256) k_split_exps(const SplitTask* __restrict_
   }
 }
 
-__global__ void __launch_bounds__(256, 1) k_split_gemm(const SplitTask* __restrict__ tasks, int max_ks, int* err) {
+__global__ void __launch_bounds__(kSplitThreads, 1) k_split_gemm(const SplitTask* __restrict__ tasks, int max_ks, int* err) {
   const SplitTask T = tasks[blockIdx.z / max_ks];
   const int ks = blockIdx.z % max_ks;
   const SplitRanges R(T.K, T.ksplit);
@@ -237,11 +238,15 @@ __global__ void __launch_bounds__(256, 1) k_split_gemm(const SplitTask* __restri
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tbase = tmem_base;
   const int row = 32 * (warp & 3) + lane, cb = 32 * (warp >> 2);   // this thread's TMEM lane and first column
-  Share sh[3];   // two of A's sixteen, one of B's eight
-  sh[0].place(T.A + (long long)m0 * T.a_m, T.a_m, T.a_k, rowsA, warp, lane);
-  sh[1].place(T.A + (long long)m0 * T.a_m, T.a_m, T.a_k, rowsA, warp + 8, lane);
-  sh[2].place(T.B + (long long)n0 * T.b_n, T.b_n, T.b_k, colsB, warp, lane);
-  double acc[32], x[3][8];
+  Share sh[2];   // of A's sixteen, then B's eight
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int it = warp + 12 * i;
+    if (it < 16) sh[i].place(T.A + (long long)m0 * T.a_m, T.a_m, T.a_k, rowsA, it, lane);
+    else sh[i].place(T.B + (long long)n0 * T.b_n, T.b_n, T.b_k, colsB, it - 16, lane);
+  }
+  const bool b1 = warp + 12 >= 16;   // the second share is B's (the first is A's)
+  double acc[32], x[2][8];
 #pragma unroll
   for (int c = 0; c < 32; ++c) acc[c] = 0.0;
   int st = 0;   // stages so far
@@ -252,20 +257,19 @@ __global__ void __launch_bounds__(256, 1) k_split_gemm(const SplitTask* __restri
     const int* eA = T.ex + (long long)e * T.M;
     const int* eB = T.same() ? eA : T.ex + (long long)R.count() * T.M + (long long)e * T.N;
     sh[0].E = sh[0].p ? eA[m0 + sh[0].row] : 1;
-    sh[1].E = sh[1].p ? eA[m0 + sh[1].row] : 1;
-    sh[2].E = sh[2].p ? eB[n0 + sh[2].row] : 1;
+    sh[1].E = sh[1].p ? (b1 ? eB[n0 + sh[1].row] : eA[m0 + sh[1].row]) : 1;
     const int EA = row < rowsA ? eA[m0 + row] : 1;
     if (tid < TN) exB[tid] = tid < colsB ? eB[n0 + tid] : 1;   // read after a barrier below
 #pragma unroll
-    for (int i = 0; i < 3; ++i) sh[i].load(x[i], k0, k1);
+    for (int i = 0; i < 2; ++i) sh[i].load(x[i], k0, k1);
     for (int k = k0; k < k1; k += KC, ++st) {
       unsigned char* Ap = buf + (st & 1) * STAGE;
       unsigned char* Bp = Ap + NDIG * A_PLANE;
       // the MMAs that read this buffer two stages ago are done
       if (st >= 2 && !wait_phase(smem_u32(&mbar[st & 1]), (uint32_t)((st >> 1) - 1) & 1)) atomicExch(&s_fail, 1);
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        sh[i].store(x[i], i < 2 ? Ap : Bp, i < 2 ? A_PLANE : B_PLANE);
+      for (int i = 0; i < 2; ++i) {
+        sh[i].store(x[i], i && b1 ? Bp : Ap, i && b1 ? B_PLANE : A_PLANE);
         sh[i].load(x[i], k + KC, k1);                        // the next stage's
       }
       asm volatile("fence.proxy.async.shared::cta;");        // generic-proxy writes -> tensor-core reads
@@ -297,6 +301,7 @@ __global__ void __launch_bounds__(256, 1) k_split_gemm(const SplitTask* __restri
     asm volatile("tcgen05.fence::after_thread_sync;");
     // sum = (hi 2^28 + lo) 2^(49 + EA + EB - 2154), the last 8 bits of lo dropped
     const uint32_t lane_addr = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)cb;
+    if (warp < 8)
 #pragma unroll
     for (int c0 = 0; c0 < 32; c0 += 8) {
       uint32_t v[NDIG][8];
@@ -331,13 +336,13 @@ __global__ void __launch_bounds__(256, 1) k_split_gemm(const SplitTask* __restri
       atomicExch(err, 1);
     }
     __syncthreads();
-  } else if (row < rowsA && T.work) {
+  } else if (warp < 8 && row < rowsA && T.work) {
     // a partial sum over this CTA's range, reduced by k_split_reduce
     double* Wr = T.work + ((long long)ks * T.M + m0 + row) * T.N + n0;
 #pragma unroll
     for (int c = 0; c < 32; ++c)
       if (cb + c < colsB) Wr[cb + c] = acc[c];
-  } else if (row < rowsA) {
+  } else if (warp < 8 && row < rowsA) {
     double* Cr = T.C + (long long)(m0 + row) * T.c_m + (long long)(n0 + cb) * T.c_n;
 #pragma unroll
     for (int c = 0; c < 32; ++c)
@@ -374,7 +379,23 @@ __global__ void k_split_reduce(const SplitTask* __restrict__ tasks) {
   }
 }
 
-size_t split_gemm_smem() { return SPLIT_SMEM; }
+// The number of K ranges, at most `most`, that a product alone on sms SMs (a CTA each) should
+// take: the fewest rounds of stages, a range's reading of TMEM counted as one. 216 x 216 x
+// 16384, symmetric, at most 32 ranges: six tiles by 25 ranges fill one round, 32 take two
+// with the second a quarter full, 119 against 137 us.
+int split_ranges(const SplitTask& T, int most, int sms) {
+  const int tm = (T.M + TM - 1) / TM, tn = (T.N + TN - 1) / TN;
+  int tiles = 0, best = most;
+  for (int i = 0; i < tm; ++i)
+    for (int j = 0; j < tn; ++j) tiles += !(T.sym && (j + 1) * TN <= i * TM);
+  double least = 0.0;
+  for (int n = most; n >= 1; --n) {
+    const SplitRanges R(T.K, n);
+    const double rounds = (double)(((long long)tiles * n + sms - 1) / sms), cost = rounds * (2.0 * R.cps + R.per);
+    if (n == most || cost < least) { least = cost; best = n; }
+  }
+  return best;
+}
 
 void launch_split_gemm(const SplitTask* tasks, int ntask, int max_m, int max_n, int* err, cudaStream_t st,
                        int max_ks, bool reduce) {
@@ -383,7 +404,7 @@ void launch_split_gemm(const SplitTask* tasks, int ntask, int max_m, int max_n, 
   max_ks = max_ks < 1 ? 1 : max_ks;
   k_split_exps<<<dim3(ntask < 4 ? 304 : 76, ntask), 256, 0, st>>>(tasks);
   dim3 grid((max_n + TN - 1) / TN, (max_m + TM - 1) / TM, ntask * max_ks);
-  k_split_gemm<<<grid, 256, SPLIT_SMEM, st>>>(tasks, max_ks, err);
+  k_split_gemm<<<grid, kSplitThreads, SPLIT_SMEM, st>>>(tasks, max_ks, err);
   if (reduce) k_split_reduce<<<dim3(152, ntask), 256, 0, st>>>(tasks);
 }
 
