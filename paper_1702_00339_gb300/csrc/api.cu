@@ -96,9 +96,11 @@ struct fock_ctx {
   uint32_t* hstage = nullptr;        // pinned host staging of gathered results
   size_t hstage_cap = 0;             // (words)
   cudaMemPool_t mempool = nullptr;   // serving workers: batches allocated stream-ordered from this pool
-  // device workspaces of single calls (split products, operator applications), which keep up
-  // to kScratchKeep bytes between calls; given back with the context
-  cudaMemPool_t scratch = nullptr;
+  // the device workspace of the last single call (split product, operator application), kept
+  // for the next one up to kScratchKeep bytes; given back with the context
+  std::mutex scratch_mu;
+  char* scratch = nullptr;
+  size_t scratch_cap = 0;
   std::string err;
   // kernel timers: events recorded around launches while enabled
   bool prof = false;
@@ -162,45 +164,44 @@ const int kPeriodicPiece = 1024;
 // a time; the chunks do not change a result.
 const size_t kPfWorkBytes = (size_t)1 << 30;
 
-const uint64_t kScratchKeep = (uint64_t)256 << 20;
-const size_t kScratchFirst = (size_t)16 << 20;
+const size_t kScratchKeep = (size_t)256 << 20;
 
-void scratch_create(fock_ctx* c) {
-  cudaMemPoolProps pr = {};
-  pr.allocType = cudaMemAllocationTypePinned;
-  pr.location.type = cudaMemLocationTypeDevice;
-  pr.location.id = c->device;
-  uint64_t keep = kScratchKeep;
-  if (cudaMemPoolCreate(&c->scratch, &pr) != cudaSuccess) {
-    cudaGetLastError();
-    c->scratch = nullptr;
-  } else {
-    cudaMemPoolSetAttribute(c->scratch, cudaMemPoolAttrReleaseThreshold, &keep);
-    // the first pages, which a first small call would otherwise wait 100 us for
-    void* p = nullptr;
-    if (cudaMallocFromPoolAsync(&p, kScratchFirst, c->scratch, c->stream) == cudaSuccess) cudaFreeAsync(p, c->stream);
-    else cudaGetLastError();
-  }
-}
-// A call's device workspace, stream-ordered from the context's pool (a cudaMalloc and
-// cudaFree pair cost 40 us for small workspaces, 130 for 12 MB); cudaMalloc where the
-// pool cannot serve it. Freed on scope exit.
+// A call's device workspace: the context's, where it is large enough and no other thread
+// has it, else its own (a cudaMalloc and cudaFree pair cost 40 us for small workspaces, 130
+// for 12 MB). After done(), which says that nothing in flight uses it, it stays with the
+// context; otherwise it is freed on scope exit.
 struct Scratch {
+  fock_ctx* c = nullptr;
   char* p = nullptr;
-  cudaStream_t st = nullptr;
-  bool pooled = false;
-  cudaError_t get(fock_ctx* c, size_t bytes) {
-    st = c->stream;
-    pooled = c->scratch && cudaMallocFromPoolAsync((void**)&p, bytes, c->scratch, st) == cudaSuccess;
-    if (pooled) return cudaSuccess;
-    cudaGetLastError();
+  size_t cap = 0;
+  bool idle = false;
+  cudaError_t get(fock_ctx* ctx, size_t bytes) {
+    c = ctx;
+    {
+      std::lock_guard<std::mutex> lk(c->scratch_mu);
+      std::swap(p, c->scratch);
+      std::swap(cap, c->scratch_cap);
+    }
+    if (cap >= bytes) return cudaSuccess;
+    if (p) cudaFree(p);
     p = nullptr;
-    return cudaMalloc((void**)&p, bytes);
+    cap = bytes;
+    const cudaError_t e = cudaMalloc((void**)&p, bytes);
+    if (e != cudaSuccess) p = nullptr;
+    return e;
   }
+  void done() { idle = true; }
   ~Scratch() {
     if (!p) return;
-    if (pooled) cudaFreeAsync(p, st);
-    else cudaFree(p);
+    if (idle && cap <= kScratchKeep) {
+      std::lock_guard<std::mutex> lk(c->scratch_mu);
+      if (!c->scratch) {
+        c->scratch = p;
+        c->scratch_cap = cap;
+        return;
+      }
+    }
+    cudaFree(p);
   }
 };
 
@@ -2193,7 +2194,6 @@ int fock_create(fock_ctx** out, int device, size_t hbm_budget_bytes, void* strea
     hbm_budget_bytes = (size_t)(0.9 * (double)fr);
   }
   c->budget = hbm_budget_bytes;
-  scratch_create(c);
   *out = c;
   return FOCK_OK;
 }
@@ -2209,7 +2209,7 @@ void fock_destroy(fock_ctx* c) {
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
   if (c->ev_chunk) cudaEventDestroy(c->ev_chunk);
-  if (c->scratch) cudaMemPoolDestroy(c->scratch);
+  if (c->scratch) cudaFree(c->scratch);
   if (c->own_stream) cudaStreamDestroy(c->stream);
   delete c;
 }
@@ -2713,6 +2713,7 @@ int fock_split_dgemm(fock_ctx* ctx, int M, int N, int K, const double* A, long l
   if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, mem, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return set_err(ctx, FOCK_ECUDA, cudaGetErrorString(e));
+  scratch.done();
   if (herr) return set_err(ctx, FOCK_ETIMEOUT, "split_dgemm: a tensor-core commit did not complete in time");
   return FOCK_OK;
 }
@@ -2745,6 +2746,7 @@ int fock_toeplitz_matvec(fock_ctx* ctx, const fock_blocks* b, int which, const d
     if (!on_device) CUDA_TRY(ctx, cudaMemcpyAsync(y, dy, nbytes, cudaMemcpyDeviceToHost, st));
     CUDA_TRY(ctx, cudaStreamSynchronize(st));
     CUDA_TRY(ctx, cudaGetLastError());
+    scratch.done();
     return FOCK_OK;
   }
   char* const tasks = scratch.p;
@@ -2774,6 +2776,7 @@ int fock_toeplitz_matvec(fock_ctx* ctx, const fock_blocks* b, int which, const d
   if (!on_device) CUDA_TRY(ctx, cudaMemcpyAsync(y, dy, nbytes, cudaMemcpyDeviceToHost, st));
   CUDA_TRY(ctx, cudaStreamSynchronize(st));
   CUDA_TRY(ctx, cudaGetLastError());
+  scratch.done();
   return FOCK_OK;
 }
 
