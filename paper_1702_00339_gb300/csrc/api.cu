@@ -158,10 +158,11 @@ const int kGemmTiles = 256;   // output tiles of a TN product: at most (255 / 16
 // Fourier blocks (conjugate pairs once) per piece launched beside a Rayleigh-Ritz
 // launch: a few milliseconds of 32 x 32 blocks on the SMs the iteration leaves free
 const int kPeriodicPiece = 1024;
-// bound of the workspace of the periodic spectra's chunks (55 KB a block of order 32):
+// Bound of the workspace of the periodic spectra's chunks (55 KB a block of order 32):
 // the kernels that give a block one thread take as long for a block as for 19 000 (a
-// lattice of 32^3 cells of 32 functions: the call takes 55 ms with 256 MB, 45 with 1 GB). A plan that would not fit its budget otherwise takes the least, 32 blocks at
-// a time; the chunks do not change a result.
+// lattice of 32^3 cells of 32 functions: the call takes 55 ms with 256 MB, 45 with
+// 1 GB). A plan that would not fit its budget otherwise takes the least, 32 blocks at a
+// time; the chunks do not change a result.
 const size_t kPfWorkBytes = (size_t)1 << 30;
 
 const size_t kScratchKeep = (size_t)256 << 20;
