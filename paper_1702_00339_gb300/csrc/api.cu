@@ -559,7 +559,7 @@ struct Batch {
   TL rfwdXP, rinvHXP, rinvSXP, rbmulHS2, reHXP;   // image refresh at the FP32 -> FP64 switch
   TL bandF, bandS;
   int band_col = 0;                  // doubles of the largest block column of a band factorisation
-  int band_item = 0, band_row = 0, band_step = 0, band_8 = 0;   // band solves: largest (D + 4) m0, (3 D + 4) m0, step, 8 (D + 1) m0
+  int band_item = 0, band_row = 0, band_step = 0, band_8 = 0;   // band solves: largest (D + 4) m0, band_side_rows, step, band_stage_rows8
   int band_sides = 1;
   BandSteps band_cs;
   int gemm_tiles = 0;                // TN tile sizes in use: bit 0 = 16, bit 1 = 20
@@ -1042,7 +1042,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
       // 207, 320, 243 ms (FP64 718 ms and more). Beyond, with the factor made from one
       // end by one cluster, an iteration no longer repaid it: 1000 cells (1.1e10) 359
       // against 274 ms, 800 cells with D = 18 (1.7e10) 500 against 346.
-      Q.use_band = 2.0 * Q.Lc * (double)Q.D * Q.D * (double)H.m0 * H.m0 * H.m0 <= 8e9;
+      Q.use_band = band_rule(Q.Lc, Q.D, H.m0);
       if (Q.use_band) {
         Q.band_twist = Q.D > 0 && Q.Lc >= 2 * Q.D + 2;
         const size_t rows = Q.Lc + (Q.band_twist ? Q.D : 0);
@@ -1213,9 +1213,9 @@ void plan(Batch& B, Slab& S, Slab& U) {
         }
         if (Q.band_twist) B.band_sides = 2;
         B.band_item = std::max(B.band_item, (Q.D + 4) * m0);
-        B.band_row = std::max(B.band_row, ((Q.band_twist ? 3 : 1) * Q.D + 4) * m0);
+        B.band_row = std::max(B.band_row, band_side_rows(Q.D, m0, Q.band_twist));
         B.band_step = std::max(B.band_step, (int)band_step(Q.D + 1, m0));
-        if (m0 > 8) B.band_8 = std::max(B.band_8, 8 * (Q.D + 1) * m0);
+        B.band_8 = std::max(B.band_8, band_stage_rows8(Q.D, m0));
         std::vector<int> ef((size_t)Q.Lc * (Q.D + 1), -1);   // a position's entries lie one after another
         for (int e = Q.nE - 1; e >= 0; --e)
           if (Q.Ek[e] >= Q.Em[e] && Q.Ek[e] - Q.Em[e] <= Q.D) ef[(size_t)Q.Ek[e] * (Q.D + 1) + Q.Ek[e] - Q.Em[e]] = e;

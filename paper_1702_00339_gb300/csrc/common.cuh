@@ -7,6 +7,8 @@
 #include <mutex>
 #include <vector>
 
+#include "band_plan.h"
+
 // Raises a kernel's dynamic shared memory limit, once per process, to the
 // device's opt-in maximum minus the kernel's static shared memory.  The
 // attribute is a per-function upper bound (a launch still occupies only the
@@ -364,9 +366,6 @@ struct CopyTask { const int* active; int n, ncols; const double* src; int lds; d
 // One piece of a batch's results gathered into a contiguous staging buffer
 // (4-byte words) for a single device-to-host copy.
 struct GatherSeg { const uint32_t* src; unsigned int words; unsigned int dst; };
-
-// doubles of one step of the banded solves with nd block coefficients, padded to 16 bytes
-__host__ __device__ inline size_t band_step(int nd, int m0) { return ((size_t)nd * m0 * m0 + 1) & ~(size_t)1; }
 
 struct BandTask {
   int m0, L, D, k, n;

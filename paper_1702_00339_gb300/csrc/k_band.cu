@@ -450,11 +450,6 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-// coefficient rows per stage of at most `stage` doubles: the whole step, or a
-// multiple of 8 (a stage then starts on a 16-byte boundary)
-__host__ __device__ inline int band_rows(int nd, int m0, int stage) {
-  return ((int)band_step(nd, m0) <= stage) ? m0 : max(8, (stage / (nd * m0)) & ~7);
-}
 
 // W = (M Delta M^T)^-1 R, one column of R per CTA.  Right-looking: once row J of
 // the solution is final, its contribution to rows J+1 .. J+D is subtracted from
@@ -492,7 +487,7 @@ __global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict_
   const int tid = threadIdx.x, nth = blockDim.x, items = D1 * m0, fit = D * m0;
   const int fst = (int)band_step(D, m0), bst = (int)band_step(D1, m0);   // doubles per step
   const double *const Tfwd = T.fwd + r0 * fst, *const Tbwd = T.bwd + r0 * bst, *const Tdinv = T.dinv + r0 * m2;
-  // rows of coefficients per stage: all m0, or a multiple of 8 that fits
+  // rows of coefficients per stage: all m0, or as many as fit
   const int qc = MULTI ? band_rows(D1, m0, maxstage) : m0, nch = MULTI ? (m0 + qc - 1) / qc : 1;
   double* cf = bsm;                           // two stages of maxstage doubles
   R* acc = reinterpret_cast<R*>(bsm + (size_t)2 * maxstage);   // nslot rows, then two of the forward solution
@@ -502,7 +497,7 @@ __global__ void __launch_bounds__(1024) k_band_solve(const BandTask* __restrict_
   // rows [h qc, ...) of a step of `width` entries a row into stage `slot`
   auto stage = [&](const double* step, int total, int width, int h, int slot) {
     const double* src = step + (size_t)h * qc * width;
-    const int n = min(qc * width, total - h * qc * width);
+    const int n = band_piece(qc, width, total, h);
     double* dst = cf + (size_t)slot * maxstage;
     for (int i = 2 * tid; i < n; i += 2 * nth) cp_async16(dst + i, src + i);
   };
@@ -681,9 +676,8 @@ void launch_band_factor(const BandTask* t, int n, int maxcol, int maxm0, const B
   cudaLaunchKernelEx(&cfg, k_band_factor, t, doubles);
 }
 
-// maxitem: the largest (D + 4) m0 among the tasks, maxrow: the largest (3 D + 4) m0 (ring, z
-// and middle rows of a column), maxstep: the largest step (coefficient doubles), max8: the
-// largest 8 (D + 1) m0 of the steps that are taken in pieces, sides: 2 if any task is twisted
+// maxitem: the largest (D + 4) m0 among the tasks, maxrow: the largest band_side_rows,
+// maxstep: the largest step (coefficient doubles), max8: the largest band_stage_rows8, sides: 2 if any task is twisted
 template <typename R, bool MULTI>
 static void solve_go(const BandTask* t, int n, int kmax, int maxitem, int maxrow, int maxstage, int sides, cudaStream_t st) {
   FOCK_SMEM_OPTIN((k_band_solve<R, MULTI>));
@@ -704,12 +698,15 @@ static void solve_go(const BandTask* t, int n, int kmax, int maxitem, int maxrow
 void launch_band_solve(const BandTask* t, int n, int kmax, int maxitem, int maxrow, int maxstep, int max8, int sides,
                        cudaStream_t st, bool mixed) {
   if (!n) return;
-  // A stage holds a step up to 64 KB, or as many rows of one (at least 8).  Two
+  // A stage holds a step up to 64 KB, or as many rows of one (8 where there is room).  Two
   // stages are enough and leave room for several CTAs per SM: eight give the same
   // 98 us on one chain of 64 cells of 8 functions, three 929 us against 674 on 32
   // chains of 64 cells of 16.  Pieces of 32 KB instead of 64: 72 columns of 512 cells
   // of 32 functions 5.8 ms against 4.9.
-  const int maxstage = std::max(std::min(maxstep, 8192), max8);
+  int dev = 0, mx = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&mx, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  const int maxstage = band_stage(maxstep, max8, maxrow, (mx - 1024) / 8);
   if (maxstep <= maxstage) {
     solve_go<double, false>(t, n, kmax, maxitem, maxrow, maxstage, sides, st);
     if (mixed) solve_go<float, false>(t, n, kmax, maxitem, maxrow, maxstage, sides, st);
