@@ -415,16 +415,23 @@ __global__ void __launch_bounds__(kFactorThreads) k_band_column(const BandTask* 
     return;
   }
   const int J = t - B.late;
-  if (J < 0 || J >= B.L || T.sync[1 + side] || (t >= B.a1 && (T.sync[1] || T.sync[2]))) return;
+  if (J < 0 || J >= B.L) return;
   const int m0 = T.m0, m2 = m0 * m0;
   double *g0 = fsm, *g1 = g0 + m2, *Ms = g1 + m2, *col = Ms + m0 * (m0 + 1);
   __shared__ double s_r[2];
-  __shared__ int s_bad;
+  __shared__ int s_bad, s_skip;
+  // one read for the whole CTA: a CTA of this launch that started earlier may set the
+  // flags meanwhile, and the threads of this one have to go on, or leave, together
+  if (tid == 0) {
+    s_bad = 0;
+    s_skip = T.sync[1 + side] || (t >= B.a1 && (T.sync[1] || T.sync[2]));
+  }
+  __syncthreads();
+  if (s_skip) return;
   const int dmax = min(B.D, B.L - 1 - J), np = dmax * (dmax + 1) / 2;
   const int p0 = (int)((long long)np * rank / C), p1 = (int)((long long)np * (rank + 1) / C);
   if (J + B.D1 < B.L) B.enter(J + B.D1, gtid, gnth);
   if (p0 >= p1 && rank != 0) return;
-  if (tid == 0) s_bad = 0;
   B.load(J, dmax, g0, col, true);
   const double* Di = band_invert(g0, g1, m0, s_r, &s_bad);
   if (s_bad) {                                 // (every CTA finds the same)
