@@ -242,11 +242,11 @@ __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
 }
-__global__ void __launch_bounds__(256) k_eapply(const EApplyTask* __restrict__ tasks) {
-  const EApplyTask T = tasks[blockIdx.z];
+__global__ void __launch_bounds__(256) k_eapply(const EApplyTask* __restrict__ tasks, int maxrows) {
+  const EApplyTask T = tasks[blockIdx.y];
   if (T.mode && *T.mode != 0) return;
   if (T.active && *T.active == 0) return;
-  const int m0 = T.m0, np = m0 * m0, mp = m0 + 1, ri = blockIdx.x, v0 = blockIdx.y * kECols;
+  const int m0 = T.m0, np = m0 * m0, mp = m0 + 1, ri = blockIdx.x % maxrows, v0 = blockIdx.x / maxrows * kECols;
   if (ri >= T.nrows || v0 >= T.ncol) return;
   extern __shared__ double esm[];
   const int stage = (T.vals2 ? 2 : 1) * m0 * mp + kECols * m0;   // doubles: blocks (transposed), rows of x
@@ -358,7 +358,8 @@ void launch_eapply(const EApplyTask* tasks, int ntask, int maxrows, int maxcols,
   if (!ntask || maxrows <= 0) return;
   const size_t sm = 2 * ((size_t)(both ? 2 : 1) * maxm0 * (maxm0 + 1) + (size_t)kECols * maxm0) * sizeof(double);
   FOCK_SMEM_OPTIN(k_eapply);
-  k_eapply<<<dim3(maxrows, (maxcols + kECols - 1) / kECols, ntask), kECols * maxm0, sm, st>>>(tasks);
+  const unsigned groups = (maxcols + kECols - 1) / kECols;   // (grid.y ends at 65535: rows and columns share x)
+  k_eapply<<<dim3(maxrows * groups, ntask), kECols * maxm0, sm, st>>>(tasks, maxrows);
 }
 
 // y = (BToepl(T) + E) x block by block, for products too small to be worth transforms:
@@ -370,7 +371,7 @@ void launch_eapply(const EApplyTask* tasks, int ntask, int maxrows, int maxcols,
 __global__ void __launch_bounds__(256) k_band_apply(const BandApply T) {
   __shared__ double part[256][kApplyCols + 1];
   __shared__ int s_ri;
-  const int m0 = T.m0, k = blockIdx.x, v0 = blockIdx.y * kApplyCols, tid = threadIdx.x;
+  const int m0 = T.m0, k = blockIdx.x % T.L, v0 = blockIdx.x / T.L * kApplyCols, tid = threadIdx.x;
   const int S = 256 / m0, mu = tid % m0, s = tid / m0, nv = min(kApplyCols, T.ncol - v0);
   if (tid == 0) s_ri = -1;
   __syncthreads();
@@ -417,7 +418,8 @@ __global__ void __launch_bounds__(256) k_band_apply(const BandApply T) {
   }
 }
 void launch_band_apply(const BandApply& T, cudaStream_t st) {
-  k_band_apply<<<dim3(T.L, (T.ncol + kApplyCols - 1) / kApplyCols), 256, 0, st>>>(T);
+  // (rows and columns share grid.x: grid.y would end at 65535 groups of columns)
+  k_band_apply<<<(unsigned)T.L * ((T.ncol + kApplyCols - 1) / kApplyCols), 256, 0, st>>>(T);
 }
 
 }  // namespace fock
