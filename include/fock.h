@@ -324,7 +324,9 @@ int fock_profile_read(fock_ctx* ctx, int cap, char* names, int* launches, double
  * A[m*a_m + k*a_k]; B: K x N, (k, n) at B[k*b_k + n*b_n]; C: (m, n) at
  * C[m*c_m + n*c_n]; all device pointers, strides in elements.  Each product
  * carries a relative error below ~2^-50 of |row max of A| |column max of B|
- * per summand (largest over ranges of at most 512 summands).  ksplit
+ * per summand, largest over its range of at most 512 summands, and where rows and
+ * columns have their largest entries apart below ~2^-44 of those over 64
+ * summands; ranges are added in FP64.  ksplit
  * (1..1024): the summation is split into at most that many ranges, computed
  * by separate CTAs and added in a fixed order (a work array
  * is allocated for them); sym != 0 (M = N): C is taken as symmetric, its

@@ -426,9 +426,10 @@ struct CanonTask {
 // A[m * a_m + k * a_k], B is K x N with B(k, n) at B[k * b_k + n * b_n],
 // C(m, n) at C[m * c_m + n * c_n].
 // The K ranges of a split product: nks of them by separate CTAs, in whole 64s, each
-// in `per` pieces of at most 512 summands (over which operands are aligned)
+// in `per` pieces of at most 512 summands (over which operands are aligned, or over
+// their blocks of 64: k_split.cu)
 struct SplitRanges {
-  static constexpr int RANGE = 512;
+  static constexpr int RANGE = 512, BLOCK = 64, BLOCKS = RANGE / BLOCK;
   int K, nks, cps, per;
   __host__ __device__ SplitRanges(int K_, int ksplit) : K(K_), nks(ksplit < 1 ? 1 : ksplit) {
     cps = ((K + 63) / 64 + nks - 1) / nks;
@@ -456,9 +457,21 @@ struct SplitTask {
   double* work;                // null: C written directly; else [ksplit][M][N] partial sums,
                                // reduced in a fixed order by k_split_reduce
   int sym;                     // (with work) C is symmetric: the upper triangle is reduced, mirrored
-  int* ex;                     // [ranges][M], then [ranges][N]: exponents of A's rows and B's columns
+  int* ex;                     // exponents of A's rows, then of B's columns (SplitExps)
   __host__ __device__ bool same() const { return A == B && a_m == b_n && a_k == b_k && M == N; }
-  __host__ __device__ size_t n_ex() const { return (size_t)SplitRanges(K, ksplit).count() * ((size_t)M + N); }
+  __host__ __device__ size_t n_ex() const { return (size_t)SplitRanges(K, ksplit).count() * ((size_t)M + N) * (2 + SplitRanges::BLOCKS); }
+};
+// Exponents of one operand of a split product, `rows` rows (or columns): for each range
+// the largest exponent field of a row, a byte for each i = 0 .. 3 with the range's blocks of
+// 64 summands whose largest is within i of it, and the blocks' own.
+struct SplitExps {
+  int *wide, *near, *block;    // [ranges][rows], [ranges][rows], [ranges][BLOCKS][rows]
+  __host__ __device__ SplitExps(const SplitTask& T, int count, bool b) {
+    const size_t nA = (size_t)count * T.M, n = b ? (size_t)count * T.N : nA;
+    wide = T.ex + (b ? nA * (2 + SplitRanges::BLOCKS) : 0);
+    near = wide + n;
+    block = near + n;
+  }
 };
 
 // Device pointers and sizes the matvec of an assembled box chain needs.

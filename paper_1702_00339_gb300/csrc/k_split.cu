@@ -15,10 +15,19 @@
 // 8 x 512 x 64^2 = 2^24, so FP32 accumulation is exact over a whole range.
 // Then each thread combines its row's levels in 64-bit integers, makes a double
 // of the sum with integer instructions (an FP64 instruction costs 64 of them
-// here) and adds ranges in FP64.  Error: cutting the operands, 2^-55 of the
-// row's and the column's largest, and the levels above NDIG + 1, about 2^-54 of their
-// product per summand; on random operands 6e-16 to 3e-15 of the largest entries'
-// product (with 7 truncated digits aligned over 64 summands, as this was: 1e-13).
+// here) and adds ranges in FP64.  With 2^a, 2^b the powers of two at or below the largest
+// of the row and of the column, a summand's error is below 2^(a + b) times 2^-52 (the cut
+// operands) and 2^-51.2 (the levels above NDIG + 1): 2^-50.5.  On random operands 6e-16
+// to 3e-15 of the largest entries' product (with 7 truncated digits, 49 bits, aligned over
+// 64 summands, as this was: 2^-44 and 1e-13).
+//
+// Where a row falls while a column rises, the largest over a range say little about the
+// products: with both over 2^40 the sum would keep 20 bits.  So a tile's range is aligned as a
+// whole only if every row and column of it has a block of 64 summands in which the
+// two, together, are within 2^3 of their largest over the range: 512 summands' errors of
+// 2^(a + b - 50.5) are then below what that one block's 64 of 2^(a' + b' - 44) may be. Else the
+// range is taken in its blocks of 64, each aligned for itself.  Looking costs nothing that can
+// be measured (the product below 145.6 us a call with and without).
 //
 // One CTA of 384 threads per 128 x 64 output tile and K range.  Stages of KC = 32
 // summands in two buffers: the threads load and split the next stage while the
@@ -172,36 +181,61 @@ __device__ __forceinline__ double scaled_int(long long S, int e) {
 
 }  // namespace
 
-// Largest exponent fields of the rows of A (and columns of B) over each range.
+// Exponents of the rows of A (and columns of B) over each range and its blocks (SplitExps).
 __global__ void __launch_bounds__(256) k_split_exps(const SplitTask* __restrict__ tasks) {
   const SplitTask T = tasks[blockIdx.y];
   if (T.active && *T.active == 0) return;
   const SplitRanges R(T.K, T.ksplit);
+  constexpr int NB = SplitRanges::BLOCKS, KB = SplitRanges::BLOCK;
   const int lane = threadIdx.x & 31;
   const long long w0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), nw = (long long)gridDim.x * (blockDim.x >> 5);
   for (int o = 0; o < (T.same() ? 1 : 2); ++o) {
     const double* P = o ? T.B : T.A;
     const long long sr = o ? T.b_n : T.a_m, sk = o ? T.b_k : T.a_k;
     const int rows = o ? T.N : T.M;
-    int* ex = T.ex + (o ? (long long)R.count() * T.M : 0);
+    const SplitExps X(T, R.count(), o != 0);
     if (sk == 1) {
       for (long long w = w0; w < (long long)R.count() * rows; w += nw) {
-        const int e = (int)(w / rows), r = (int)(w % rows), k1 = R.end(e);
-        int E = 1;
-#pragma unroll 8
-        for (int k = R.begin(e) + lane; k < k1; k += 32) E = max(E, exp_field(P[r * sr + k]));
-        E = __reduce_max_sync(0xffffffffu, E);
-        if (lane == 0) ex[w] = E;
+        const int e = (int)(w / rows), r = (int)(w % rows), k0 = R.begin(e) + lane, k1 = R.end(e);
+        int Eb = 1;                            // lane c: block c's
+#pragma unroll
+        for (int c = 0; c < NB; ++c) {
+          int E = 1;
+#pragma unroll
+          for (int k = k0 + c * KB, i = 0; i < KB / 32; k += 32, ++i)
+            if (k < k1) E = max(E, exp_field(P[r * sr + k]));
+          E = __reduce_max_sync(0xffffffffu, E);
+          if (lane == c) Eb = E;
+        }
+        const int E = __reduce_max_sync(0xffffffffu, Eb);
+        uint32_t near = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) near |= (__ballot_sync(0xffffffffu, lane < NB && E - Eb <= i) & 0xffu) << (8 * i);
+        if (lane < NB) X.block[((long long)e * NB + lane) * rows + r] = Eb;
+        if (lane == 0) { X.wide[w] = E; X.near[w] = (int)near; }
       }
     } else {
       const int rg = (rows + 31) >> 5;
       for (long long w = w0; w < (long long)R.count() * rg; w += nw) {
-        const int e = (int)(w / rg), r = (int)(w % rg) * 32 + lane, k1 = R.end(e);
+        const int e = (int)(w / rg), r = (int)(w % rg) * 32 + lane, k0 = R.begin(e), k1 = R.end(e);
         if (r >= rows) continue;
-        int E = 1;
+        int Eb[NB], E = 1;
+#pragma unroll
+        for (int c = 0; c < NB; ++c) {
+          const int kc = min(k0 + (c + 1) * KB, k1);
+          Eb[c] = 1;
 #pragma unroll 8
-        for (int k = R.begin(e); k < k1; ++k) E = max(E, exp_field(P[r * sr + k * sk]));
-        ex[(long long)e * rows + r] = E;
+          for (int k = k0 + c * KB; k < kc; ++k) Eb[c] = max(Eb[c], exp_field(P[r * sr + k * sk]));
+          X.block[((long long)e * NB + c) * rows + r] = Eb[c];
+          E = max(E, Eb[c]);
+        }
+        uint32_t near = 0;
+#pragma unroll
+        for (int c = 0; c < NB; ++c)
+#pragma unroll
+          for (int i = 0; i < 4; ++i) near |= (E - Eb[c] <= i ? 1u : 0u) << (8 * i + c);
+        X.wide[(long long)e * rows + r] = E;
+        X.near[(long long)e * rows + r] = (int)near;
       }
     }
   }
@@ -220,6 +254,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_split_gemm(const SplitTask
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t tmem_base;
   __shared__ int s_fail, exB[TN];
+  __shared__ uint32_t nearB[TN];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rowsA = min(TM, T.M - m0), colsB = min(TN, T.N - n0);
   if (tid == 0) {
@@ -250,83 +285,100 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_split_gemm(const SplitTask
 #pragma unroll
   for (int c = 0; c < 32; ++c) acc[c] = 0.0;
   int st = 0;   // stages so far
-  bool ok = true;
+  bool ok = true, first = true;
+  const SplitExps XA(T, R.count(), false), XB(T, R.count(), !T.same());
   for (int d = 0; d < R.per && ok; ++d) {
-    const int e = ks * R.per + d, k0 = R.begin(e), k1 = R.end(e);
-    if (k0 >= k1) break;
-    const int* eA = T.ex + (long long)e * T.M;
-    const int* eB = T.same() ? eA : T.ex + (long long)R.count() * T.M + (long long)e * T.N;
-    sh[0].E = sh[0].p ? eA[m0 + sh[0].row] : 1;
-    sh[1].E = sh[1].p ? (b1 ? eB[n0 + sh[1].row] : eA[m0 + sh[1].row]) : 1;
-    const int EA = row < rowsA ? eA[m0 + row] : 1;
-    if (tid < TN) exB[tid] = tid < colsB ? eB[n0 + tid] : 1;   // read after a barrier below
+    const int e = ks * R.per + d, r0 = R.begin(e), r1 = R.end(e);
+    if (r0 >= r1) break;
+    // a row and a column agree in block c for some i if c is among the row's within i and
+    // the column's within 3 - i: one AND with the column's bytes in reverse
+    int apart = 0;
+    if (r1 - r0 > SplitRanges::BLOCK) {
+      if (tid < TN) nearB[tid] = tid < colsB ? __byte_perm((uint32_t)XB.near[(long long)e * T.N + n0 + tid], 0, 0x0123) : ~0u;
+      const int ra = tid % TM;
+      const uint32_t nearA = ra < rowsA ? (uint32_t)XA.near[(long long)e * T.M + m0 + ra] : ~0u;
+      __syncthreads();
+      for (int c = tid / TM; c < TN; c += kSplitThreads / TM) apart |= (nearA & nearB[c]) == 0;
+    }
+    const bool fine = __syncthreads_or(apart);
+    for (int k0 = r0, k1; k0 < r1 && ok; k0 = k1) {
+      k1 = fine ? min(k0 + SplitRanges::BLOCK, r1) : r1;
+      const long long xr = fine ? (long long)e * SplitRanges::BLOCKS + (k0 - r0) / SplitRanges::BLOCK : e;
+      const int* eA = (fine ? XA.block : XA.wide) + xr * T.M;
+      const int* eB = (fine ? XB.block : XB.wide) + xr * T.N;
+      sh[0].E = sh[0].p ? eA[m0 + sh[0].row] : 1;
+      sh[1].E = sh[1].p ? (b1 ? eB[n0 + sh[1].row] : eA[m0 + sh[1].row]) : 1;
+      const int EA = row < rowsA ? eA[m0 + row] : 1;
+      if (tid < TN) exB[tid] = tid < colsB ? eB[n0 + tid] : 1;   // read after a barrier below
 #pragma unroll
-    for (int i = 0; i < 2; ++i) sh[i].load(x[i], k0, k1);
-    for (int k = k0; k < k1; k += KC, ++st) {
-      unsigned char* Ap = buf + (st & 1) * STAGE;
-      unsigned char* Bp = Ap + NDIG * A_PLANE;
-      // the MMAs that read this buffer two stages ago are done
-      if (st >= 2 && !wait_phase(smem_u32(&mbar[st & 1]), (uint32_t)((st >> 1) - 1) & 1)) atomicExch(&s_fail, 1);
+      for (int i = 0; i < 2; ++i) sh[i].load(x[i], k0, k1);
+      for (int k = k0; k < k1; k += KC, ++st) {
+        unsigned char* Ap = buf + (st & 1) * STAGE;
+        unsigned char* Bp = Ap + NDIG * A_PLANE;
+        // the MMAs that read this buffer two stages ago are done
+        if (st >= 2 && !wait_phase(smem_u32(&mbar[st & 1]), (uint32_t)((st >> 1) - 1) & 1)) atomicExch(&s_fail, 1);
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        sh[i].store(x[i], i && b1 ? Bp : Ap, i && b1 ? B_PLANE : A_PLANE);
-        sh[i].load(x[i], k + KC, k1);                        // the next stage's
+        for (int i = 0; i < 2; ++i) {
+          sh[i].store(x[i], i && b1 ? Bp : Ap, i && b1 ? B_PLANE : A_PLANE);
+          sh[i].load(x[i], k + KC, k1);                        // the next stage's
+        }
+        asm volatile("fence.proxy.async.shared::cta;");        // generic-proxy writes -> tensor-core reads
+        __syncthreads();
+        if (s_fail) { ok = false; break; }
+        if (tid == 0) {
+          asm volatile("tcgen05.fence::after_thread_sync;");
+          const uint32_t a0 = smem_u32(Ap), b0 = smem_u32(Bp);
+          for (int kk = 0; kk < KC / 16; ++kk)
+            for (int j = 0; j < NDIG; ++j)                     // planes j of A, q .. q + nl - 1 of B: levels j + q on
+              for (int q = 0; q < NDIG - j; q += 4) {
+                const int nl = min(4, NDIG - j - q);
+                const uint64_t da = smem_desc(a0 + j * A_PLANE + kk * 256);
+                const uint64_t db = smem_desc(b0 + q * B_PLANE + kk * 256);
+                const uint32_t accum = (k > k0 || kk > 0 || j > 0) ? 1u : 0u;
+                const uint32_t idesc = kIdesc | (uint32_t)((nl * TN) >> 3) << 17;
+                asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                             "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                             :: "r"(tbase + (uint32_t)((j + q) * TN)), "l"(da), "l"(db), "r"(idesc), "r"(accum));
+              }
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                       :: "r"(smem_u32(&mbar[st & 1])) : "memory");
+        }
       }
-      asm volatile("fence.proxy.async.shared::cta;");        // generic-proxy writes -> tensor-core reads
+      if (!ok) break;
+      if (!wait_phase(smem_u32(&mbar[(st - 1) & 1]), (uint32_t)((st - 1) >> 1) & 1)) atomicExch(&s_fail, 1);
       __syncthreads();
       if (s_fail) { ok = false; break; }
-      if (tid == 0) {
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const uint32_t a0 = smem_u32(Ap), b0 = smem_u32(Bp);
-        for (int kk = 0; kk < KC / 16; ++kk)
-          for (int j = 0; j < NDIG; ++j)                     // planes j of A, q .. q + nl - 1 of B: levels j + q on
-            for (int q = 0; q < NDIG - j; q += 4) {
-              const int nl = min(4, NDIG - j - q);
-              const uint64_t da = smem_desc(a0 + j * A_PLANE + kk * 256);
-              const uint64_t db = smem_desc(b0 + q * B_PLANE + kk * 256);
-              const uint32_t accum = (k > k0 || kk > 0 || j > 0) ? 1u : 0u;
-              const uint32_t idesc = kIdesc | (uint32_t)((nl * TN) >> 3) << 17;
-              asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                           "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                           :: "r"(tbase + (uint32_t)((j + q) * TN)), "l"(da), "l"(db), "r"(idesc), "r"(accum));
-            }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                     :: "r"(smem_u32(&mbar[st & 1])) : "memory");
-      }
-    }
-    if (!ok) break;
-    if (!wait_phase(smem_u32(&mbar[(st - 1) & 1]), (uint32_t)((st - 1) >> 1) & 1)) atomicExch(&s_fail, 1);
-    __syncthreads();
-    if (s_fail) { ok = false; break; }
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    // sum = (hi 2^28 + lo) 2^(49 + EA + EB - 2154), the last 8 bits of lo dropped
-    const uint32_t lane_addr = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)cb;
-    if (warp < 8)
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      // sum = (hi 2^28 + lo) 2^(49 + EA + EB - 2154), the last 8 bits of lo dropped
+      const uint32_t lane_addr = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)cb;
+      if (warp < 8)
 #pragma unroll
-    for (int c0 = 0; c0 < 32; c0 += 8) {
-      uint32_t v[NDIG][8];
+      for (int c0 = 0; c0 < 32; c0 += 8) {
+        uint32_t v[NDIG][8];
 #pragma unroll
-      for (int g = 0; g < NDIG; ++g)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(v[g][0]), "=r"(v[g][1]), "=r"(v[g][2]), "=r"(v[g][3]), "=r"(v[g][4]), "=r"(v[g][5]),
-                       "=r"(v[g][6]), "=r"(v[g][7])
-                     : "r"(lane_addr + (uint32_t)(g * TN + c0)));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        for (int g = 0; g < NDIG; ++g)
+          asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                       : "=r"(v[g][0]), "=r"(v[g][1]), "=r"(v[g][2]), "=r"(v[g][3]), "=r"(v[g][4]), "=r"(v[g][5]),
+                         "=r"(v[g][6]), "=r"(v[g][7])
+                       : "r"(lane_addr + (uint32_t)(g * TN + c0)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        long long hi = 0, lo = 0;
+        for (int c = 0; c < 8; ++c) {
+          long long hi = 0, lo = 0;
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          hi = hi * 128 + __float2int_rn(__uint_as_float(v[g][c]));
-          lo = lo * 128 + __float2int_rn(__uint_as_float(v[4 + g][c]));
+          for (int g = 0; g < 4; ++g) {
+            hi = hi * 128 + __float2int_rn(__uint_as_float(v[g][c]));
+            lo = lo * 128 + __float2int_rn(__uint_as_float(v[4 + g][c]));
+          }
+          const double val = scaled_int(hi * (1ll << 20) + (lo >> 8), EA + exB[cb + c0 + c] - 2097);
+          acc[c0 + c] = first ? val : acc[c0 + c] + val;
         }
-        const double val = scaled_int(hi * (1ll << 20) + (lo >> 8), EA + exB[cb + c0 + c] - 2097);
-        acc[c0 + c] = d == 0 ? val : acc[c0 + c] + val;
       }
+      asm volatile("tcgen05.fence::before_thread_sync;");
+      __syncthreads();   // TMEM and exB are reused by the next range
+      asm volatile("tcgen05.fence::after_thread_sync;");
+      first = false;
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();   // TMEM and exB are reused by the next range
-    asm volatile("tcgen05.fence::after_thread_sync;");
   }
   if (!ok) {
     // an MMA group did not complete in time: wait (bounded) once more so no
