@@ -186,9 +186,9 @@ struct Scratch {
     if (cap >= bytes) return cudaSuccess;
     if (p) cudaFree(p);
     p = nullptr;
-    cap = bytes;
     const cudaError_t e = cudaMalloc((void**)&p, bytes);
     if (e != cudaSuccess) p = nullptr;
+    cap = p ? bytes : 0;
     return e;
   }
   void done() { idle = true; }
@@ -492,6 +492,7 @@ struct Batch {
   std::vector<DftTask> dft; DftTask* d_dft = nullptr; int maxLdft = 1;
   std::vector<PfTask> pft; PfTask* d_pft = nullptr;
   std::vector<PfGroup> pfg; PfGroup* d_pfg = nullptr;   // largest blocks first
+  bool handle = false;               // of fock_assemble: the calls bring the chunk workspace (pf_scratch)
   size_t pf_limit = kPfWorkBytes;    // bound of the workspace below
   char* pf_work = nullptr; size_t pf_bytes = 0;   // chunk workspace of the periodic spectra
   std::vector<FBlockTask> fbp, fbs; FBlockTask* d_fbs = nullptr;   // fbp: templates of the vector solves
@@ -1086,8 +1087,10 @@ void plan(Batch& B, Slab& S, Slab& U) {
       own += pf_bytes_for(B.hp[B.pft[t].prob].m0, B.pfg.size() - n0);
     }
     const size_t least = pf_bytes_for(B.hp[B.pft[by[0]].prob].m0, 1);
-    B.pf_bytes = std::max(least, std::min(own, B.pf_limit));
-    B.pf_work = S.take<char>(B.pf_bytes);
+    if (!B.handle) {
+      B.pf_bytes = std::max(least, std::min(own, B.pf_limit));
+      B.pf_work = S.take<char>(B.pf_bytes);
+    }
   }
   // ---- LOBPCG state ----
   size_t mv_total = 0;
@@ -1566,24 +1569,44 @@ void run_pf(Batch& B, const PfTask* tasks, const PfGroup* g, const PfGroup* dg, 
     i += c;
   }
 }
-// the next n groups of the periodic spectra (n < 0: all that remain)
-void run_periodic_piece(fock_ctx* ctx, Batch& B, int n, cudaStream_t st) {
+// the next n groups of the periodic spectra (n < 0: all that remain), in `bytes` of workspace
+void run_periodic_piece(fock_ctx* ctx, Batch& B, int n, char* work, size_t bytes, cudaStream_t st) {
   const int left = (int)B.pfg.size() - B.pchunk_next, w = (n < 0) ? left : std::min(n, left);
   if (w <= 0) return;
   { PROF("k_fblocks_eig", 1);
-    run_pf(B, B.d_pft, B.pfg.data() + B.pchunk_next, B.d_pfg + B.pchunk_next, w, B.pf_work, B.pf_bytes, st); }
+    run_pf(B, B.d_pft, B.pfg.data() + B.pchunk_next, B.d_pfg + B.pchunk_next, w, work, bytes, st); }
   B.pchunk_next += w;
 }
-void run_periodic_tail(fock_ctx* ctx, Batch& B, cudaStream_t st) {
+void run_periodic_tail(fock_ctx* ctx, Batch& B, char* work, size_t bytes, cudaStream_t st) {
   if (B.fbp.empty()) return;
-  run_periodic_piece(ctx, B, -1, st);
+  run_periodic_piece(ctx, B, -1, work, bytes, st);
   if (!B.sorts.empty()) { PROF("k_sort", 1); launch_sort_small(B.d_sorts, (int)B.sorts.size(), B.maxsort, st); }
   for (int i : B.bigsort) { PROF("k_sort_global", 1);
     launch_sort_global(B.pp[i].ev, B.pp[i].blk, B.pp[i].nev, B.sort_pv, B.sort_pi, st); }
 }
-void run_periodic(fock_ctx* ctx, Batch& B) {
+void run_periodic(fock_ctx* ctx, Batch& B, char* work, size_t bytes) {
   run_periodic_head(ctx, B, ctx->stream);
-  run_periodic_tail(ctx, B, ctx->stream);
+  run_periodic_tail(ctx, B, work, bytes, ctx->stream);
+}
+// Workspace of a call on a handle for the spectra of ng groups, behind `before` bytes of its
+// own: as a plan's, but no more than the budget leaves beside the handle, and the least
+// where the device cannot give that.
+cudaError_t pf_scratch(fock_ctx* ctx, const Batch& B, size_t ng, size_t before, Scratch* s, size_t* bytes) {
+  const int m = B.hp[0].m0;
+  const size_t least = pf_bytes_for(m, 1), used = B.bytes + B.ubytes, page = (size_t)2 << 20;
+  size_t room = kPfWorkBytes;
+  if (ctx->budget) {
+    const size_t left = ctx->budget > used ? (ctx->budget - used) & ~(page - 1) : 0;   // (allocations take whole pages)
+    room = std::min(room, left > before ? left - before : 0);
+  }
+  *bytes = std::max(least, std::min(pf_bytes_for(m, ng), room));
+  cudaError_t e = s->get(ctx, before + *bytes);
+  if (e != cudaSuccess && *bytes > least) {
+    cudaGetLastError();
+    *bytes = least;
+    e = s->get(ctx, before + *bytes);
+  }
+  return e;
 }
 
 void run_struct_setup(fock_ctx* ctx, Batch& B) {
@@ -1889,7 +1912,7 @@ int run_lobpcg(fock_ctx* ctx, Batch& B, double tol, int maxit, std::vector<int>&
     if (ctx->pstream && B.pchunk_next < (int)B.pfg.size()) {
       CUDA_TRY(ctx, cudaEventRecord(ctx->ev_chunk, st));
       CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->pstream, ctx->ev_chunk, 0));
-      run_periodic_piece(ctx, B, B.pchunk_w, ctx->pstream);
+      run_periodic_piece(ctx, B, B.pchunk_w, B.pf_work, B.pf_bytes, ctx->pstream);
     }
     if (graphs) CUDA_TRY(ctx, cudaGraphLaunch(B.iter_graph_b, st));
     else lobpcg_body_b(B, st);
@@ -1927,7 +1950,7 @@ int plan_execute(fock_plan& P, double tol, int maxit) {
   run_assemble(ctx, B);
   const bool overlap = ctx->hi && !ctx->prof && !B.fbp.empty() && !B.fbs.empty();
   if (!overlap) {
-    run_periodic(ctx, B);
+    run_periodic(ctx, B, B.pf_work, B.pf_bytes);
     run_struct_setup(ctx, B);
     int rc = run_lobpcg(ctx, B, tol, maxit, P.iters, P.resid, P.conv, &P.hist, &P.on_left);
     if (rc) return rc;
@@ -1945,7 +1968,7 @@ int plan_execute(fock_plan& P, double tol, int maxit) {
     int rc = run_lobpcg(ctx, B, tol, maxit, P.iters, P.resid, P.conv, &P.hist, &P.on_left);
     ctx->stream = user;
     ctx->pstream = nullptr;
-    run_periodic_tail(ctx, B, user);
+    run_periodic_tail(ctx, B, B.pf_work, B.pf_bytes, user);
     // joined on every path: later work on the context's stream sees both
     cudaError_t e = cudaEventRecord(ctx->ev_join, ctx->hi);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(user, ctx->ev_join, 0);
@@ -2422,6 +2445,7 @@ int fock_assemble(fock_ctx* ctx, const fock_problem* p, fock_blocks** out) {
   ProfBind pb(ctx);
   fock_blocks* b = new fock_blocks();
   b->ctx = ctx;
+  b->B.handle = true;
   int rc = build_batch(ctx, 1, p, b->B, true);
   if (rc) { free_batch(b->B); delete b; return rc; }
   run_assemble(ctx, b->B);
@@ -2541,7 +2565,6 @@ int periodic_range(fock_ctx* ctx, Batch& B, int j0, int j1, double* evals, int* 
   { PROF("k_null_tau", 1); launch_null_tau(B.d_nulls, (int)B.nulls.size(), st); }
   int n2 = 1;
   while (n2 < n) n2 <<= 1;
-  char* mem = nullptr;
   const size_t off_blk = ((size_t)n * 8 + 255) & ~(size_t)255;
   const size_t off_pv = off_blk + (((size_t)n * 4 + 255) & ~(size_t)255);
   const size_t off_pi = off_pv + (size_t)n2 * 8;
@@ -2554,19 +2577,16 @@ int periodic_range(fock_ctx* ctx, Batch& B, int j0, int j1, double* evals, int* 
   const size_t off_g = (off_r + reps.size() * sizeof(int) + 255) & ~(size_t)255;
   const size_t off_v = (off_g + groups.size() * sizeof(PfGroup) + 255) & ~(size_t)255;
   const size_t vbytes = vecs ? (size_t)n * H.m0 * sizeof(cplx) : 0;
-  const size_t off_w = (off_v + vbytes + 255) & ~(size_t)255, least = pf_bytes_for(H.m0, 1);
-  size_t wbytes = std::max(least, std::min(kPfWorkBytes, pf_bytes_for(H.m0, groups.size())));
-  if (cudaMalloc(&mem, off_w + wbytes) != cudaSuccess) {
-    cudaGetLastError();
-    wbytes = least;
-    CUDA_TRY(ctx, cudaMalloc(&mem, off_w + wbytes));
-  }
+  const size_t off_w = (off_v + vbytes + 255) & ~(size_t)255;
+  Scratch scratch;
+  size_t wbytes = 0;
+  CUDA_TRY(ctx, pf_scratch(ctx, B, groups.size(), off_w, &scratch, &wbytes));
+  char* const mem = scratch.p;
   double* ev = (double*)mem;
   int* blk = (int*)(mem + off_blk);
   FBlockTask f = B.fbp[0];
   f.j0 = j0; f.nj = nj; f.outH = nullptr; f.outS = nullptr; f.want = 1; f.ev = nullptr; f.blk = nullptr; f.fail = nullptr;
   f.vecs = vecs ? (cplx*)(mem + off_v) : nullptr;
-  int rc = FOCK_OK;
   PfTask pt = B.pft[0];
   pt.j0 = j0; pt.nj = nj; pt.nrep = (int)reps.size(); pt.rep = (const int*)(mem + off_r);
   pt.ev = ev; pt.blk = blk; pt.neig = nullptr;
@@ -2588,9 +2608,9 @@ int periodic_range(fock_ctx* ctx, Batch& B, int j0, int j1, double* evals, int* 
     if (e == cudaSuccess && vecs) e = cudaMemcpyAsync(vecs, mem + off_v, vbytes, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   }
-  if (e != cudaSuccess) rc = set_err(ctx, FOCK_ECUDA, cudaGetErrorString(e));
-  cudaFree(mem);
-  return rc;
+  if (e != cudaSuccess) return set_err(ctx, FOCK_ECUDA, cudaGetErrorString(e));
+  scratch.done();
+  return FOCK_OK;
 }
 }  // namespace
 
@@ -2601,13 +2621,17 @@ int fock_circulant_eig(fock_ctx* ctx, const fock_blocks* b, double* evals, int* 
   const HostProb& H = B.hp[0];
   if (evecs) return periodic_range(ctx, B, 0, H.L[0] * H.L[1] * H.L[2], evals, block_of, evecs);
   ProfBind pb(ctx);
-  run_periodic(ctx, B);
+  Scratch scratch;
+  size_t wbytes = 0;
+  CUDA_TRY(ctx, pf_scratch(ctx, B, B.pfg.size(), 0, &scratch, &wbytes));
+  run_periodic(ctx, B, scratch.p, wbytes);
   const Batch::PerProb& Q = B.pp[0];
   int fail = 0;
   CUDA_TRY(ctx, cudaMemcpyAsync(evals, Q.ev, Q.nev * 8, cudaMemcpyDeviceToHost, ctx->stream));
   if (block_of) CUDA_TRY(ctx, cudaMemcpyAsync(block_of, Q.blk, Q.nev * 4, cudaMemcpyDeviceToHost, ctx->stream));
   CUDA_TRY(ctx, cudaMemcpyAsync(&fail, Q.fail, 4, cudaMemcpyDeviceToHost, ctx->stream));
   CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+  scratch.done();
   if (fail) return set_err(ctx, FOCK_EINVAL, "a Fourier-block mass matrix was not positive definite");
   return FOCK_OK;
 }
