@@ -112,8 +112,10 @@ typedef struct fock_ctx fock_ctx;
 typedef struct fock_blocks fock_blocks;
 
 /* Context: owns device memory (a growable arena) and one CUDA stream.
- * device: CUDA ordinal.  hbm_budget_bytes: cap on the arena (0: 90% of the
- * free memory at creation).  stream: a cudaStream_t to run on, or NULL to
+ * device: CUDA ordinal.  hbm_budget_bytes: cap on the arena and on each plan
+ * or handle (0: 90% of the free memory at creation); a single call's workspace
+ * comes on top while it runs, and up to 256 MB of it stay with the context for the
+ * next call where they fit the budget beside all of those.  stream: a cudaStream_t to run on, or NULL to
  * create a private one.  Errors: FOCK_EINVAL, FOCK_ECUDA. */
 int fock_create(fock_ctx** ctx, int device, size_t hbm_budget_bytes, void* stream);
 /* Frees the context; every fock_blocks / fock_plan made from it must be

@@ -5,6 +5,7 @@
 // the device slab, once with the real base address to fill the descriptors.
 // Every array of the path lives in that slab; all arithmetic of the method
 // runs in the kernels (k_assemble.cu, k_eig.cu, k_matvec.cu, k_lobpcg.cu).
+#include <atomic>
 #include <chrono>
 #include <algorithm>
 #include <cmath>
@@ -96,11 +97,13 @@ struct fock_ctx {
   uint32_t* hstage = nullptr;        // pinned host staging of gathered results
   size_t hstage_cap = 0;             // (words)
   cudaMemPool_t mempool = nullptr;   // serving workers: batches allocated stream-ordered from this pool
-  // the device workspace of the last single call (split product, operator application), kept
-  // for the next one up to kScratchKeep bytes; given back with the context
+  // the device workspace of the last single call (split product, operator application,
+  // spectrum of a handle), kept for the next one up to kScratchKeep bytes and within the budget
+  // beside the arena and what plans and handles hold; given back with the context
   std::mutex scratch_mu;
   char* scratch = nullptr;
   size_t scratch_cap = 0;
+  std::atomic<size_t> held{0};       // bytes of the context's plans and handles
   std::string err;
   // kernel timers: events recorded around launches while enabled
   bool prof = false;
@@ -196,7 +199,7 @@ struct Scratch {
     if (!p) return;
     if (idle && cap <= kScratchKeep) {
       std::lock_guard<std::mutex> lk(c->scratch_mu);
-      if (!c->scratch) {
+      if (!c->scratch && (!c->budget || c->held + c->arena_cap + cap <= c->budget)) {
         c->scratch = p;
         c->scratch_cap = cap;
         return;
@@ -205,6 +208,20 @@ struct Scratch {
     cudaFree(p);
   }
 };
+
+// Gives the kept workspace back if it does not fit the budget beside `used` bytes; whether
+// there was one to give.
+bool drop_scratch(fock_ctx* c, size_t used) {
+  char* p = nullptr;
+  {
+    std::lock_guard<std::mutex> lk(c->scratch_mu);
+    if (c->budget && used <= c->budget && c->scratch_cap <= c->budget - used) return false;
+    std::swap(p, c->scratch);
+    c->scratch_cap = 0;
+  }
+  if (p) cudaFree(p);
+  return p != nullptr;
+}
 
 int set_err(fock_ctx* c, int code, const std::string& m) {
   if (c) c->err = m;
@@ -466,7 +483,8 @@ struct Batch {
   std::vector<AxisPlan> ap;          // [nprob*3]
   size_t bytes = 0;
   char* base = nullptr;
-  bool own = false;                  // slab owned by the batch (fock_blocks)
+  bool own = false;                  // slab owned by the batch (fock_plan, fock_blocks)
+  fock_ctx* owner = nullptr; size_t held = 0;   // its context, the slab's bytes counted there
   cudaStream_t pooled = nullptr;     // slab allocated from a memory pool on this stream
   // device descriptors
   ProbDev* d_probs = nullptr;
@@ -1462,6 +1480,7 @@ int alloc_and_plan(fock_ctx* ctx, Batch& B, bool own) {
   if (ctx->budget && need + uneed > ctx->budget)
     return set_err(ctx, FOCK_ENOMEM, "batch needs " + std::to_string(need + uneed) + " bytes, budget " +
                                          std::to_string(ctx->budget));
+  drop_scratch(ctx, ctx->held + (own ? ctx->arena_cap + need + uneed : std::max(ctx->arena_cap, need + uneed)));
   char *mb = nullptr, *ub = nullptr;
   if (ctx->mempool) {
     CUDA_TRY(ctx, cudaMallocFromPoolAsync((void**)&mb, need, ctx->mempool, ctx->stream));
@@ -1471,6 +1490,8 @@ int alloc_and_plan(fock_ctx* ctx, Batch& B, bool own) {
     CUDA_TRY(ctx, cudaMalloc(&mb, need));
     CUDA_TRY(ctx, cudaMalloc(&ub, uneed));
     B.own = true;
+    B.owner = ctx;
+    ctx->held += B.held = need + uneed;
   } else {
     if (ctx->arena_cap < need + uneed) {
       if (ctx->arena) { cudaStreamSynchronize(ctx->stream); cudaFree(ctx->arena); ctx->arena = nullptr; ctx->arena_cap = 0; }
@@ -1503,6 +1524,8 @@ void free_batch(Batch& B) {
   } else if (B.own) {
     cudaFree(B.base);
     cudaFree(B.ubase);
+    B.owner->held -= B.held;
+    B.held = 0;
   }
   B.base = B.ubase = nullptr;
 }
