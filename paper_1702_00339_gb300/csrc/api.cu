@@ -104,6 +104,7 @@ struct fock_ctx {
   char* scratch = nullptr;
   size_t scratch_cap = 0;
   std::atomic<size_t> held{0};       // bytes of the context's plans and handles
+  size_t pf_cap = SIZE_MAX;          // bound of a batch's chunk workspace (serving workers)
   std::string err;
   // kernel timers: events recorded around launches while enabled
   bool prof = false;
@@ -164,8 +165,8 @@ const int kPeriodicPiece = 1024;
 // Bound of the workspace of the periodic spectra's chunks (55 KB a block of order 32):
 // the kernels that give a block one thread take as long for a block as for 19 000 (a
 // lattice of 32^3 cells of 32 functions: the call takes 55 ms with 256 MB, 45 with
-// 1 GB). A plan that would not fit its budget otherwise takes the least, 32 blocks at a
-// time; the chunks do not change a result.
+// 1 GB). A plan that would not fit otherwise takes what there is room for, at least 32
+// blocks at a time; the chunks do not change a result.
 const size_t kPfWorkBytes = (size_t)1 << 30;
 
 const size_t kScratchKeep = (size_t)256 << 20;
@@ -209,13 +210,13 @@ struct Scratch {
   }
 };
 
-// Gives the kept workspace back if it does not fit the budget beside `used` bytes; whether
-// there was one to give.
+// Gives the kept workspace back if it does not fit the budget beside `used` bytes (SIZE_MAX:
+// in any case); whether there was one to give.
 bool drop_scratch(fock_ctx* c, size_t used) {
   char* p = nullptr;
   {
     std::lock_guard<std::mutex> lk(c->scratch_mu);
-    if (c->budget && used <= c->budget && c->scratch_cap <= c->budget - used) return false;
+    if (used != SIZE_MAX && (!c->budget || (used <= c->budget && c->scratch_cap <= c->budget - used))) return false;
     std::swap(p, c->scratch);
     c->scratch_cap = 0;
   }
@@ -510,9 +511,15 @@ struct Batch {
   std::vector<DftTask> dft; DftTask* d_dft = nullptr; int maxLdft = 1;
   std::vector<PfTask> pft; PfTask* d_pft = nullptr;
   std::vector<PfGroup> pfg; PfGroup* d_pfg = nullptr;   // largest blocks first
+  // What the structured problems of a plan that does not fit its budget, or the device, give up,
+  // one after the other: 1 the split sums of the Gram products, 2 the factor from both ends,
+  // 3 the factor (the circulant inverse in its place).  It then takes no more memory than the
+  // least form of a problem does; more iterations at 3, slower ones at 1 and 2.
+  int tight = 0;
   bool handle = false;               // of fock_assemble: the calls bring the chunk workspace (pf_scratch)
   size_t pf_limit = kPfWorkBytes;    // bound of the workspace below
   char* pf_work = nullptr; size_t pf_bytes = 0;   // chunk workspace of the periodic spectra
+  size_t pf_extra = 0;               // what of the slab the least workspace would not take
   std::vector<FBlockTask> fbp, fbs; FBlockTask* d_fbs = nullptr;   // fbp: templates of the vector solves
   std::vector<NullTask> nulls; NullTask* d_nulls = nullptr;   // dependency cut of each periodic problem
   int maxnj_p = 0, maxnj_s = 0, maxm0 = 1;
@@ -521,7 +528,7 @@ struct Batch {
   std::vector<FBlockTask> fbo; FBlockTask* d_fbo = nullptr;
   std::vector<SortTask> sorts; SortTask* d_sorts = nullptr; int maxsort = 0;
   std::vector<int> bigsort;          // problems whose eigenvalues need the global sort
-  double* sort_pv = nullptr; int* sort_pi = nullptr;
+  double* sort_pv = nullptr; int* sort_pi = nullptr; int sort_n2 = 0;
   std::vector<CircDev> circs; CircDev* d_circs = nullptr;
   // per-problem outputs / structured operators
   struct PerProb {
@@ -582,7 +589,7 @@ struct Batch {
   int band_sides = 1;
   BandSteps band_cs;
   int gemm_tiles = 0;                // TN tile sizes in use: bit 0 = 16, bit 1 = 20
-  int* gemm_count = nullptr;         // [structured problem][2][kGemmTiles] arrivals of split TN sums, zero between launches
+  int* gemm_count = nullptr;         // [structured problem][2][kGemmTiles] arrivals of split TN sums, zero between launches (null: none)
   bool odd_m0 = true;                // some problem has odd m0 (Fourier-block layout, k_fblocks)
   int ptab_maxT = 0, ptab_maxni = 0; // potential tables: largest term count, endpoint count
   TL init, tnCx, nnW, pcG, pcM, pcZ, g1, g3, rr1, rr3, u1, u3, cp2k, resid, normP, normW;
@@ -621,7 +628,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
   B.dtabs.clear(); B.dfields.clear(); B.dblocks.clear();
   B.dft.clear(); B.fbp.clear(); B.pft.clear(); B.pfg.clear(); B.fbs.clear(); B.nulls.clear(); B.prec.clear(); B.canon.clear(); B.fbo.clear(); B.maxcblk = 0; B.sorts.clear(); B.bigsort.clear();
   B.circs.clear(); B.lob.clear(); B.sidx.clear(); B.mv_off.clear();
-  B.maxnj_p = B.maxnj_s = 0; B.maxm0 = 1; B.maxM = 0; B.maxsort = 0; B.kmax = 0; B.maxLdft = 1;
+  B.maxnj_p = B.maxnj_s = 0; B.maxm0 = 1; B.maxM = 0; B.maxsort = 0; B.sort_n2 = 0; B.kmax = 0; B.maxLdft = 1;
   B.odd_m0 = false;
   B.any_mixed = false;
   B.eapply_rows = 0;
@@ -842,7 +849,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
     Q.nE = (int)n;
   }
   // fold scratch (shared by all tasks of the batch)
-  double* zs = S.take<double>(std::max<size_t>(zs_total, 1));
+  double* const zs = S.take<double>(std::max<size_t>(zs_total, 1));
   {
     size_t o = 0;
     for (auto& t : B.gram) {
@@ -853,6 +860,8 @@ void plan(Batch& B, Slab& S, Slab& U) {
   // mixed form: X_t[mu nu] = sum_r P_t[r] Z[r][mu nu] (T x nfold times nfold x m0^2) on the
   // tensor cores for the gram tasks of mixed problems
   B.splits.clear(); B.split_maxm = B.split_maxn = 0;
+  std::vector<int> split_prob;
+  std::vector<size_t> split_used(np, 0);
   for (auto& t : B.gram) {
     if (!B.hp[t.prob].mixed) continue;
     const ProbDev& P = B.probs[t.prob];
@@ -869,8 +878,8 @@ void plan(Batch& B, Slab& S, Slab& U) {
     sp.B = t.Zs; sp.b_k = np; sp.b_n = 1;
     sp.C = t.X + (direct ? 0 : 2 * np); sp.c_m = np; sp.c_n = 1;
     sp.alpha = 1.0; sp.beta = 0.0; sp.ksplit = 1;
-    sp.ex = S.take<int>(sp.n_ex());
     B.splits.push_back(sp);
+    split_prob.push_back(t.prob);
     B.split_maxm = std::max(B.split_maxm, sp.M);
     B.split_maxn = std::max(B.split_maxn, sp.N);
     t.split = 1;
@@ -1061,9 +1070,9 @@ void plan(Batch& B, Slab& S, Slab& U) {
       // 207, 320, 243 ms (FP64 718 ms and more). Beyond, with the factor made from one
       // end by one cluster, an iteration no longer repaid it: 1000 cells (1.1e10) 359
       // against 274 ms, 800 cells with D = 18 (1.7e10) 500 against 346.
-      Q.use_band = band_rule(Q.Lc, Q.D, H.m0);
+      Q.use_band = B.tight < 3 && band_rule(Q.Lc, Q.D, H.m0);
       if (Q.use_band) {
-        Q.band_twist = Q.D > 0 && Q.Lc >= 2 * Q.D + 2;
+        Q.band_twist = B.tight < 2 && Q.D > 0 && Q.Lc >= 2 * Q.D + 2;
         const size_t rows = Q.Lc + (Q.band_twist ? Q.D : 0);
         Q.band_win = S.take<double>((size_t)(Q.band_twist ? 2 : 1) * (Q.D + 2) * (Q.D + 1) * m2);
         Q.band_fwd = S.take<double>(rows * std::max<size_t>(band_step(Q.D, H.m0), 2));
@@ -1093,6 +1102,8 @@ void plan(Batch& B, Slab& S, Slab& U) {
     }
   }
   // ---- groups and chunk workspace of the periodic spectra ----
+  size_t pf_least = 0;
+  B.pf_bytes = 0;
   if (!B.pft.empty()) {
     std::vector<int> by(B.pft.size());
     for (size_t i = 0; i < by.size(); ++i) by[i] = (int)i;
@@ -1105,10 +1116,8 @@ void plan(Batch& B, Slab& S, Slab& U) {
       own += pf_bytes_for(B.hp[B.pft[t].prob].m0, B.pfg.size() - n0);
     }
     const size_t least = pf_bytes_for(B.hp[B.pft[by[0]].prob].m0, 1);
-    if (!B.handle) {
-      B.pf_bytes = std::max(least, std::min(own, B.pf_limit));
-      B.pf_work = S.take<char>(B.pf_bytes);
-    }
+    B.pf_bytes = B.handle ? 0 : std::max(least, std::min(own, B.pf_limit));
+    pf_least = std::min(B.pf_bytes, least);
   }
   // ---- LOBPCG state ----
   size_t mv_total = 0;
@@ -1133,10 +1142,10 @@ void plan(Batch& B, Slab& S, Slab& U) {
   }
   if (!B.sidx.empty()) {
     const int ns = (int)B.sidx.size();
-    B.d_active = S.take<int>(ns);
-    B.d_mode = S.take<int>(ns);
-    B.d_refresh = S.take<int>(ns);
-    B.d_fail = S.take<int>(ns);
+    B.d_active = S.take<int>(4 * (size_t)ns);
+    B.d_mode = B.d_active + ns;
+    B.d_refresh = B.d_mode + ns;
+    B.d_fail = B.d_refresh + ns;
     B.d_res = S.take<double>((size_t)ns * B.kmax);
     B.d_lam = S.take<double>((size_t)ns * B.kmax);
     for (int s = 0; s < ns; ++s) {
@@ -1149,13 +1158,35 @@ void plan(Batch& B, Slab& S, Slab& U) {
     B.mvY1 = S.take<cplx>(mv_total);
     B.mvY2 = S.take<cplx>(mv_total);
   }
+  // the exponents of the assembly's split products, in the problem's memory that is written
+  // after the assembly: its Fourier factors, or its part of the transforms' work
+  for (size_t q = 0; q < B.splits.size();) {
+    const int i = split_prob[q];
+    size_t end = q, words = 0;
+    for (; end < B.splits.size() && split_prob[end] == i; ++end) words += B.splits[end].n_ex();
+    const HostProb& H = B.hp[i];
+    char* at = (char*)B.pp[i].Xh[0];
+    size_t room = (size_t)(H.L[0] + H.L[1] + H.L[2]) * H.nF * H.m0 * H.m0 * sizeof(cplx);
+    if (H.kind == 1) {
+      const size_t s = std::find(B.sidx.begin(), B.sidx.end(), i) - B.sidx.begin();
+      at = (char*)(B.mvX + B.mv_off[s]);
+      room = (size_t)B.pp[i].M * H.m0 * 2 * B.lob[s].k * sizeof(cplx);
+    }
+    // (a problem's tasks need not lie together: what another run of them took is left out)
+    const size_t before = split_used[i] * sizeof(int);
+    int* ex = before + words * sizeof(int) <= room ? (int*)at + split_used[i] : S.take<int>(words);
+    split_used[i] += words;
+    for (; q < end; ++q) {
+      B.splits[q].ex = ex;
+      ex += B.splits[q].n_ex();
+    }
+  }
   if (!B.bigsort.empty()) {
     int mx = 0;
     for (int i : B.bigsort) mx = std::max(mx, B.pp[i].nev);
     int n2 = 1;
     while (n2 < mx) n2 <<= 1;
-    B.sort_pv = S.take<double>(n2);
-    B.sort_pi = S.take<int>(n2);
+    B.sort_n2 = n2;
   }
   B.d_circs = U.put(B.circs);
   // ---- LOBPCG task lists (fixed addresses, built once) ----
@@ -1176,7 +1207,16 @@ void plan(Batch& B, Slab& S, Slab& U) {
     std::vector<ResidTask> rs;
     std::vector<BandTask> bnd;
     std::vector<int> ones(ns, 1);
-    B.gemm_count = S.take<int>((size_t)ns * 2 * kGemmTiles);
+    // mixed problems whose dense products are split products (with sums of their own); ranges of
+    // the other problems' sums over n
+    auto tensor_of = [&](int i, int n) { return B.hp[i].mixed && n >= kSplitMinRows; };
+    auto ks_of = [&](int i, int n) { return (tensor_of(i, n) || B.tight >= 1) ? 1 : gemm_tn_ksplit(n); };
+    B.gemm_count = nullptr;
+    for (int s2 = 0; s2 < ns; ++s2)
+      if (ks_of(B.sidx[s2], B.lob[s2].n) > 1) {
+        B.gemm_count = S.take<int>((size_t)ns * 2 * kGemmTiles);
+        break;
+      }
     B.d_ones = U.put(ones);
     for (int s2 = 0; s2 < ns; ++s2) {
       const int i = B.sidx[s2];
@@ -1286,7 +1326,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
       };
       // TN products over n with their sums split (the projection; the two Gram
       // matrices, whose start on X alone reuses the same partial sums)
-      const int ks = gemm_tn_ksplit(n);
+      const int ks = ks_of(i, n);
       const size_t pgram = (size_t)ks * 9 * k * k;
       double* part = (ks > 1) ? S.take<double>(2 * pgram) : nullptr;
       auto tn = [&](GemmTask g, int which) {
@@ -1326,10 +1366,19 @@ void plan(Batch& B, Slab& S, Slab& U) {
       nP.push_back({l.active, n, k, nullptr, n, l.Y + nk, n});
       nW.push_back({l.active, n, k, nullptr, n, l.Y + 2 * nk, n});
       rs.push_back({l.active, n, k, n, l.Y, l.HY, l.SY, l.lam, l.R, l.res});
-      if (H.mixed && n >= kSplitMinRows) {
+      if (tensor_of(i, n)) {
         // mixed form: the block iteration's dense products on the tensor cores
         // (exact split products; the Gram sums over n split into K ranges)
-        auto to_tn = [&](GemmTask& g, std::vector<SplitTask>& out) {
+        // the lists run one after another, and not while a matvec is under way: their exponents
+        // share the transforms' work (at most 2.2 n k or 6 (n + 2 k) words of its 8 n k)
+        std::vector<std::pair<std::vector<SplitTask>*, size_t>> exs;   // task and where in it
+        size_t ex_at = 0;
+        auto to_ex = [&](std::vector<SplitTask>& out, bool second) {
+          if (!second) ex_at = 0;
+          exs.push_back({&out, ex_at});
+          ex_at += out.back().n_ex();
+        };
+        auto to_tn = [&](GemmTask& g, std::vector<SplitTask>& out, bool second = false) {
           SplitTask t;
           std::memset(&t, 0, sizeof(t));
           t.active = g.active; t.M = g.a; t.N = g.b; t.K = g.n;
@@ -1338,8 +1387,8 @@ void plan(Batch& B, Slab& S, Slab& U) {
           t.ksplit = std::min(32, std::max(1, ((t.K + 63) / 64 + 7) / 8));
           t.work = S.take<double>((size_t)t.ksplit * t.M * t.N);
           t.sym = g.sym;
-          t.ex = S.take<int>(t.n_ex());
           out.push_back(t);
+          to_ex(out, second);
           g.split = 1;
         };
         auto to_nn = [&](GemmTask& g, std::vector<SplitTask>& out) {
@@ -1349,15 +1398,21 @@ void plan(Batch& B, Slab& S, Slab& U) {
           t.A = g.A; t.a_m = 1; t.a_k = g.lda; t.B = g.B; t.b_k = 1; t.b_n = g.ldb;
           t.C = g.C; t.c_m = 1; t.c_n = g.ldc; t.alpha = g.alpha; t.beta = g.beta;
           t.ksplit = 1; t.work = nullptr; t.sym = 0;
-          t.ex = S.take<int>(t.n_ex());
           out.push_back(t);
+          to_ex(out, false);
           g.split = 1;
         };
         to_tn(tcx.back(), s_tcx);
         to_nn(nw.back(), s_nw);
-        to_tn(gg1[gg1.size() - 2], s_gg1); to_tn(gg1.back(), s_gg1);
-        to_tn(gg3[gg3.size() - 2], s_gg3); to_tn(gg3.back(), s_gg3);
+        to_tn(gg1[gg1.size() - 2], s_gg1); to_tn(gg1.back(), s_gg1, true);
+        to_tn(gg3[gg3.size() - 2], s_gg3); to_tn(gg3.back(), s_gg3, true);
         to_nn(uu1.back(), s_uu1); to_nn(uu3.back(), s_uu3);
+        int* const ex = (int*)X;
+        for (size_t q = exs.size(); q-- > 0;) {   // each list's last tasks are this problem's
+          std::vector<SplitTask>& out = *exs[q].first;
+          const bool last = q + 1 == exs.size() || exs[q + 1].first != &out;
+          out[out.size() - (last ? 1 : 2)].ex = ex + exs[q].second;
+        }
       }
     }
     B.fft_chunks = (maxcols + B.fft_cc - 1) / B.fft_cc;
@@ -1456,7 +1511,17 @@ void plan(Batch& B, Slab& S, Slab& U) {
     }
     B.o_split_err = B.d_split_err ? seg(B.d_split_err, 1) : -1;
     B.ostage_words = w;
-    B.d_ostage = S.take<uint32_t>(std::max<size_t>(w, 2));
+    // the chunks, a global sort and the gathered results come one after another, behind the
+    // assembly: they share memory, the assembly's fold scratch where that is large enough
+    const size_t fold = zs_total * sizeof(double), sort = (size_t)B.sort_n2 * (sizeof(double) + sizeof(int));
+    const size_t late = std::max(sort, std::max<size_t>(w, 2) * sizeof(uint32_t));
+    const size_t most = std::max(late, B.pf_bytes), least = std::max(late, pf_least);
+    char* const at = most <= fold ? (char*)zs : S.take<char>(most);
+    B.pf_extra = (most <= fold ? 0 : most) - (least <= fold ? 0 : least);
+    B.pf_work = at;
+    B.sort_pv = (double*)at;
+    B.sort_pi = (int*)(B.sort_pv + B.sort_n2);
+    B.d_ostage = (uint32_t*)at;
     B.d_gseg = U.put(B.gseg);
   }
   B.bytes = S.off;
@@ -1468,27 +1533,32 @@ void plan(Batch& B, Slab& S, Slab& U) {
 // ------------------------------------------------------------------ drivers
 namespace {
 
-int alloc_and_plan(fock_ctx* ctx, Batch& B, bool own) {
-  Slab S0, U0;
-  plan(B, S0, U0);
-  if (ctx->budget && S0.off + U0.off + 512 > ctx->budget && !B.pft.empty()) {
-    B.pf_limit = 0;
-    S0 = Slab(); U0 = Slab();
-    plan(B, S0, U0);
+// The next smaller form of a plan that is `over` bytes too large: less chunk workspace, then
+// what Batch::tight lists; false when there is none.
+bool tighten(Batch& B, size_t over) {
+  if (B.pf_extra) {
+    B.pf_limit = over + 512 < B.pf_extra ? B.pf_bytes - over - 512 : 0;
+    return true;
   }
-  size_t need = S0.off + 256, uneed = U0.off + 256;
-  if (ctx->budget && need + uneed > ctx->budget)
-    return set_err(ctx, FOCK_ENOMEM, "batch needs " + std::to_string(need + uneed) + " bytes, budget " +
-                                         std::to_string(ctx->budget));
-  drop_scratch(ctx, ctx->held + (own ? ctx->arena_cap + need + uneed : std::max(ctx->arena_cap, need + uneed)));
-  char *mb = nullptr, *ub = nullptr;
+  if (B.sidx.empty() || B.tight == 3) return false;
+  ++B.tight;
+  return true;
+}
+
+// device memory of a batch: from the context's pool, its own, or the context's arena
+cudaError_t alloc_slabs(fock_ctx* ctx, Batch& B, bool own, size_t need, size_t uneed, char** mb, char** ub) {
+  cudaError_t e;
   if (ctx->mempool) {
-    CUDA_TRY(ctx, cudaMallocFromPoolAsync((void**)&mb, need, ctx->mempool, ctx->stream));
-    CUDA_TRY(ctx, cudaMallocFromPoolAsync((void**)&ub, uneed, ctx->mempool, ctx->stream));
+    e = cudaMallocFromPoolAsync((void**)mb, need, ctx->mempool, ctx->stream);
+    if (e != cudaSuccess) return e;
+    e = cudaMallocFromPoolAsync((void**)ub, uneed, ctx->mempool, ctx->stream);
+    if (e != cudaSuccess) { cudaFreeAsync(*mb, ctx->stream); return e; }
     B.pooled = ctx->stream;
   } else if (own) {
-    CUDA_TRY(ctx, cudaMalloc(&mb, need));
-    CUDA_TRY(ctx, cudaMalloc(&ub, uneed));
+    e = cudaMalloc((void**)mb, need);
+    if (e != cudaSuccess) return e;
+    e = cudaMalloc((void**)ub, uneed);
+    if (e != cudaSuccess) { cudaFree(*mb); return e; }
     B.own = true;
     B.owner = ctx;
     ctx->held += B.held = need + uneed;
@@ -1496,11 +1566,39 @@ int alloc_and_plan(fock_ctx* ctx, Batch& B, bool own) {
     if (ctx->arena_cap < need + uneed) {
       if (ctx->arena) { cudaStreamSynchronize(ctx->stream); cudaFree(ctx->arena); ctx->arena = nullptr; ctx->arena_cap = 0; }
       size_t cap = (need + uneed) + (need + uneed) / 4;
-      CUDA_TRY(ctx, cudaMalloc(&ctx->arena, cap));
+      e = cudaMalloc((void**)&ctx->arena, cap);
+      if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        e = cudaMalloc((void**)&ctx->arena, cap = need + uneed);
+      }
+      if (e != cudaSuccess) { ctx->arena = nullptr; return e; }
       ctx->arena_cap = cap;
     }
-    mb = ctx->arena;
-    ub = ctx->arena + ((need + 255) & ~(size_t)255);
+    *mb = ctx->arena;
+    *ub = ctx->arena + ((need + 255) & ~(size_t)255);
+  }
+  return cudaSuccess;
+}
+
+int alloc_and_plan(fock_ctx* ctx, Batch& B, bool own) {
+  Slab S0, U0;
+  char *mb = nullptr, *ub = nullptr;
+  B.pf_limit = std::min(B.pf_limit, ctx->pf_cap);
+  for (;;) {
+    S0 = Slab(); U0 = Slab();
+    plan(B, S0, U0);
+    const size_t need = S0.off + 256, uneed = U0.off + 256, both = need + uneed;
+    if (ctx->budget && both > ctx->budget) {
+      if (tighten(B, both - ctx->budget)) continue;
+      return set_err(ctx, FOCK_ENOMEM, "batch needs " + std::to_string(both) + " bytes, budget " + std::to_string(ctx->budget));
+    }
+    drop_scratch(ctx, ctx->held + (own ? ctx->arena_cap + both : std::max(ctx->arena_cap, both)));
+    cudaError_t e = alloc_slabs(ctx, B, own, need, uneed, &mb, &ub);
+    if (e == cudaSuccess) break;
+    cudaGetLastError();
+    // the device is fuller than the budget says: without the kept workspace, then smaller
+    if (e != cudaErrorMemoryAllocation || !(drop_scratch(ctx, SIZE_MAX) || tighten(B, B.pf_bytes / 4 * 3)))
+      return set_err(ctx, FOCK_ECUDA, "batch of " + std::to_string(both) + " bytes: " + cudaGetErrorString(e));
   }
   B.base = mb;
   B.ubase = ub;
@@ -1798,7 +1896,7 @@ int run_lobpcg(fock_ctx* ctx, Batch& B, double tol, int maxit, std::vector<int>&
   if (!ns) return FOCK_OK;
   CUDA_TRY(ctx, cudaMemcpyAsync(B.d_active, B.d_ones, ns * sizeof(int), cudaMemcpyDeviceToDevice, st));
   CUDA_TRY(ctx, cudaMemsetAsync(B.d_fail, 0, ns * sizeof(int), st));
-  CUDA_TRY(ctx, cudaMemsetAsync(B.gemm_count, 0, (size_t)ns * 2 * kGemmTiles * sizeof(int), st));
+  if (B.gemm_count) CUDA_TRY(ctx, cudaMemsetAsync(B.gemm_count, 0, (size_t)ns * 2 * kGemmTiles * sizeof(int), st));
   // mixed form: matvecs in FP32 until the wanted residual falls below
   // kMixedSwitch, FP64 from then on (monotone), so that the converged pairs
   // come from FP64 images; no convergence decision during the FP32 phase
@@ -2116,13 +2214,11 @@ int detail_estimate(const fock_problem& p, size_t budget, size_t* bytes, int* n_
   int rc = validate(p, B.hp[0], why);
   if (rc) return rc;
   for (int a = 0; a < 3; ++a) axis_plan(B.hp[0], a, B.ap[a]);
-  for (;;) {
+  do {   // as the plan of a batch that does not fit does
     Slab S0, U0;
     plan(B, S0, U0);
     *bytes = S0.off + U0.off + 512;
-    if (*bytes <= budget || B.pft.empty() || !B.pf_limit) break;
-    B.pf_limit = 0;   // as the plan of a batch that does not fit does
-  }
+  } while (*bytes > budget && tighten(B, *bytes - budget));
   *n_evals = B.pp[0].nev;
   return FOCK_OK;
 }

@@ -436,6 +436,7 @@ struct SplitRanges {
     per = (cps * 64 + RANGE - 1) / RANGE;
   }
   __host__ __device__ int count() const { return nks * per; }
+  __host__ __device__ int blocks() const { return cps < BLOCKS ? cps : BLOCKS; }   // of a range, at most
   __host__ __device__ int end(int e) const {
     const long long k = (long long)(e / per) * cps * 64;
     const long long a = k + (e % per + 1) * RANGE, b = k + cps * 64, m = a < b ? a : b;
@@ -459,16 +460,19 @@ struct SplitTask {
   int sym;                     // (with work) C is symmetric: the upper triangle is reduced, mirrored
   int* ex;                     // exponents of A's rows, then of B's columns (SplitExps)
   __host__ __device__ bool same() const { return A == B && a_m == b_n && a_k == b_k && M == N; }
-  __host__ __device__ size_t n_ex() const { return (size_t)SplitRanges(K, ksplit).count() * ((size_t)M + N) * (2 + SplitRanges::BLOCKS); }
+  __host__ __device__ size_t n_ex() const {
+    const SplitRanges R(K, ksplit);
+    return (size_t)R.count() * ((size_t)M + N) * (2 + R.blocks());
+  }
 };
 // Exponents of one operand of a split product, `rows` rows (or columns): for each range
 // the largest exponent field of a row, a byte for each i = 0 .. 3 with the range's blocks of
 // 64 summands whose largest is within i of it, and the blocks' own.
 struct SplitExps {
-  int *wide, *near, *block;    // [ranges][rows], [ranges][rows], [ranges][BLOCKS][rows]
-  __host__ __device__ SplitExps(const SplitTask& T, int count, bool b) {
-    const size_t nA = (size_t)count * T.M, n = b ? (size_t)count * T.N : nA;
-    wide = T.ex + (b ? nA * (2 + SplitRanges::BLOCKS) : 0);
+  int *wide, *near, *block;    // [ranges][rows], [ranges][rows], [ranges][blocks()][rows]
+  __host__ __device__ SplitExps(const SplitTask& T, const SplitRanges& R, bool b) {
+    const size_t nA = (size_t)R.count() * T.M, n = b ? (size_t)R.count() * T.N : nA;
+    wide = T.ex + (b ? nA * (2 + R.blocks()) : 0);
     near = wide + n;
     block = near + n;
   }

@@ -193,7 +193,8 @@ __global__ void __launch_bounds__(256) k_split_exps(const SplitTask* __restrict_
     const double* P = o ? T.B : T.A;
     const long long sr = o ? T.b_n : T.a_m, sk = o ? T.b_k : T.a_k;
     const int rows = o ? T.N : T.M;
-    const SplitExps X(T, R.count(), o != 0);
+    const SplitExps X(T, R, o != 0);
+    const int nb = R.blocks();
     if (sk == 1) {
       for (long long w = w0; w < (long long)R.count() * rows; w += nw) {
         const int e = (int)(w / rows), r = (int)(w % rows), k0 = R.begin(e) + lane, k1 = R.end(e);
@@ -211,7 +212,7 @@ __global__ void __launch_bounds__(256) k_split_exps(const SplitTask* __restrict_
         uint32_t near = 0;
 #pragma unroll
         for (int i = 0; i < 4; ++i) near |= (__ballot_sync(0xffffffffu, lane < NB && E - Eb <= i) & 0xffu) << (8 * i);
-        if (lane < NB) X.block[((long long)e * NB + lane) * rows + r] = Eb;
+        if (lane < nb) X.block[((long long)e * nb + lane) * rows + r] = Eb;
         if (lane == 0) { X.wide[w] = E; X.near[w] = (int)near; }
       }
     } else {
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(256) k_split_exps(const SplitTask* __restrict_
           Eb[c] = 1;
 #pragma unroll 8
           for (int k = k0 + c * KB; k < kc; ++k) Eb[c] = max(Eb[c], exp_field(P[r * sr + k * sk]));
-          X.block[((long long)e * NB + c) * rows + r] = Eb[c];
+          if (c < nb) X.block[((long long)e * nb + c) * rows + r] = Eb[c];
           E = max(E, Eb[c]);
         }
         uint32_t near = 0;
@@ -286,7 +287,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_split_gemm(const SplitTask
   for (int c = 0; c < 32; ++c) acc[c] = 0.0;
   int st = 0;   // stages so far
   bool ok = true, first = true;
-  const SplitExps XA(T, R.count(), false), XB(T, R.count(), !T.same());
+  const SplitExps XA(T, R, false), XB(T, R, !T.same());
   for (int d = 0; d < R.per && ok; ++d) {
     const int e = ks * R.per + d, r0 = R.begin(e), r1 = R.end(e);
     if (r0 >= r1) break;
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_split_gemm(const SplitTask
     const bool fine = __syncthreads_or(apart);
     for (int k0 = r0, k1; k0 < r1 && ok; k0 = k1) {
       k1 = fine ? min(k0 + SplitRanges::BLOCK, r1) : r1;
-      const long long xr = fine ? (long long)e * SplitRanges::BLOCKS + (k0 - r0) / SplitRanges::BLOCK : e;
+      const long long xr = fine ? (long long)e * R.blocks() + (k0 - r0) / SplitRanges::BLOCK : e;
       const int* eA = (fine ? XA.block : XA.wide) + xr * T.M;
       const int* eB = (fine ? XB.block : XB.wide) + xr * T.N;
       sh[0].E = sh[0].p ? eA[m0 + sh[0].row] : 1;

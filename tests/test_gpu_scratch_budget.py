@@ -2,8 +2,8 @@
 budget, beside its plans and handles, and is given back to a plan that needs the room."""
 import pytest
 
-from tests.test_gpu_band import _chain
 from tests.test_gpu_handle_memory import _needs
+from tests.test_gpu_periodic_blocks import _lattice
 
 pytestmark = pytest.mark.gpu
 
@@ -21,7 +21,7 @@ def _product(torch, ctx):
 def test_kept_workspace_counts_against_the_budget():
     torch = pytest.importorskip("torch")
     from paper_1702_00339_gb300 import fock
-    p = _chain(L=40, m0=8, k=4)
+    p = _lattice((9, 5, 7), 12)                      # (a lattice's handle takes the same in every budget)
     need = _needs(fock, p)
     warm = fock.Context(0)                           # the kernels' own memory
     _product(torch, warm)
