@@ -158,7 +158,8 @@ int fock_problem_layout(const fock_problem* p, int* Nb, int* mcirc, int* D, int*
  * Evals pointers are device pointers when outputs_on_device != 0.
  * Returns the first non-zero per-problem status, or FOCK_OK.  Errors:
  * FOCK_EINVAL (no problems, a malformed problem: see fock_problem_check),
- * FOCK_ENOMEM (the batch exceeds the context's budget), FOCK_ECUDA; per
+ * FOCK_ENOMEM (the batch exceeds the context's budget; one that does in its
+ * fast form is solved in a smaller one, with more or slower iterations), FOCK_ECUDA; per
  * problem, out->status FOCK_ENOCONV when the block iteration hit its cap
  * (best estimates written).  The block iteration stops at a relative
  * residual of 1e-10 (or its rounding floor) or after FOCK_DEFAULT_MAXIT

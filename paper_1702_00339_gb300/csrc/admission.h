@@ -15,6 +15,22 @@
 
 namespace fock {
 
+// Device bytes of a request: with the least chunk workspace of its spectrum, the part of them
+// that this workspace shares with other steps of the batch, and the workspace it would like.
+struct ServeSize {
+  size_t bytes = 0, region = 0, chunks = 0;
+};
+
+// Chunk workspace of a batch whose requests' regions and wishes add up to `region` and
+// `chunks`, with `room` bytes beside those admitted; *extra: what of it comes from the room
+// (the batch's shared region is at most its requests' together).
+inline size_t chunk_share(size_t region, size_t chunks, size_t most, size_t room, size_t* extra) {
+  const size_t want = chunks < most ? chunks : most;
+  *extra = want > region ? want - region : 0;
+  if (*extra > room) *extra = room;
+  return region + *extra;
+}
+
 // Moves the admitted requests from `pending` into the returned batch (queue
 // order) and adds their bytes to *taken.  kind_of(r) -> bool, bytes_of(r) ->
 // size_t.  An empty batch means the head does not fit `free_bytes`.

@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "../../include/fock.h"
+#include "admission.h"
 #include "common.cuh"
 
 namespace fock {
@@ -519,7 +520,8 @@ struct Batch {
   bool handle = false;               // of fock_assemble: the calls bring the chunk workspace (pf_scratch)
   size_t pf_limit = kPfWorkBytes;    // bound of the workspace below
   char* pf_work = nullptr; size_t pf_bytes = 0;   // chunk workspace of the periodic spectra
-  size_t pf_extra = 0;               // what of the slab the least workspace would not take
+  // it shares memory with other steps (plan): least bytes of that, and what it takes beyond
+  size_t pf_region = 0, pf_extra = 0;
   std::vector<FBlockTask> fbp, fbs; FBlockTask* d_fbs = nullptr;   // fbp: templates of the vector solves
   std::vector<NullTask> nulls; NullTask* d_nulls = nullptr;   // dependency cut of each periodic problem
   int maxnj_p = 0, maxnj_s = 0, maxm0 = 1;
@@ -848,15 +850,6 @@ void plan(Batch& B, Slab& S, Slab& U) {
     Q.Ek = k2; Q.Em = m2v; Q.Ekind = kd; Q.Esrc = sr;
     Q.nE = (int)n;
   }
-  // fold scratch (shared by all tasks of the batch)
-  double* const zs = S.take<double>(std::max<size_t>(zs_total, 1));
-  {
-    size_t o = 0;
-    for (auto& t : B.gram) {
-      t.Zs = zs + o;
-      o += (size_t)t.nfold * B.probs[t.prob].m0 * B.probs[t.prob].m0;
-    }
-  }
   // mixed form: X_t[mu nu] = sum_r P_t[r] Z[r][mu nu] (T x nfold times nfold x m0^2) on the
   // tensor cores for the gram tasks of mixed problems
   B.splits.clear(); B.split_maxm = B.split_maxn = 0;
@@ -875,7 +868,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
     std::memset(&sp, 0, sizeof(sp));
     sp.M = direct ? P.R : P.T; sp.N = np; sp.K = t.nfold;
     sp.A = tab + off; sp.a_m = ld; sp.a_k = 1;
-    sp.B = t.Zs; sp.b_k = np; sp.b_n = 1;
+    sp.b_k = np; sp.b_n = 1;   // (B: t.Zs, below)
     sp.C = t.X + (direct ? 0 : 2 * np); sp.c_m = np; sp.c_n = 1;
     sp.alpha = 1.0; sp.beta = 0.0; sp.ksplit = 1;
     B.splits.push_back(sp);
@@ -1466,26 +1459,6 @@ void plan(Batch& B, Slab& S, Slab& U) {
     B.bandS = B.bandF;
     TLp(rs, B.resid, kk);
   }
-  // ---- descriptor arrays (uploaded in one copy with the parameters) ----
-  B.d_probs = U.put(B.probs);
-  B.d_gsegs = U.put(B.gsegs);
-  B.d_psegs = U.put(B.psegs);
-  B.d_gram = U.put(B.gram);
-  B.d_splits = U.put(B.splits);
-  B.d_combT = U.put(B.combT);
-  B.d_combE = U.put(B.combE);
-  B.d_dtabs = U.put(B.dtabs);
-  B.d_dfields = U.put(B.dfields);
-  B.d_dblocks = U.put(B.dblocks);
-  B.d_dft = U.put(B.dft);
-  B.d_pft = U.put(B.pft);
-  B.d_pfg = U.put(B.pfg);
-  B.d_fbs = U.put(B.fbs);
-  B.d_nulls = U.put(B.nulls);
-  B.d_prec = U.put(B.prec);
-  B.d_canon = U.put(B.canon);
-  B.d_fbo = U.put(B.fbo);
-  B.d_sorts = U.put(B.sorts);
   // ---- result gather: eigenvalues, block indices and fail flags of every problem ----
   B.gseg.clear();
   B.o_ev.assign(np, -1); B.o_blk.assign(np, -1); B.o_fail.assign(np, -1);
@@ -1511,19 +1484,46 @@ void plan(Batch& B, Slab& S, Slab& U) {
     }
     B.o_split_err = B.d_split_err ? seg(B.d_split_err, 1) : -1;
     B.ostage_words = w;
-    // the chunks, a global sort and the gathered results come one after another, behind the
-    // assembly: they share memory, the assembly's fold scratch where that is large enough
-    const size_t fold = zs_total * sizeof(double), sort = (size_t)B.sort_n2 * (sizeof(double) + sizeof(int));
-    const size_t late = std::max(sort, std::max<size_t>(w, 2) * sizeof(uint32_t));
-    const size_t most = std::max(late, B.pf_bytes), least = std::max(late, pf_least);
-    char* const at = most <= fold ? (char*)zs : S.take<char>(most);
-    B.pf_extra = (most <= fold ? 0 : most) - (least <= fold ? 0 : least);
+    // the assembly's fold scratch (shared by all its tasks), the chunks, a global sort and the
+    // gathered results come one after another: they share memory
+    const size_t sort = (size_t)B.sort_n2 * (sizeof(double) + sizeof(int));
+    B.pf_region = std::max({zs_total * sizeof(double), sort, std::max<size_t>(w, 2) * sizeof(uint32_t), pf_least});
+    const size_t most = std::max(B.pf_region, B.pf_bytes);
+    char* const at = S.take<char>(most);
+    B.pf_extra = most - B.pf_region;
     B.pf_work = at;
     B.sort_pv = (double*)at;
     B.sort_pi = (int*)(B.sort_pv + B.sort_n2);
     B.d_ostage = (uint32_t*)at;
+    double* zs = (double*)at;
+    size_t q = 0;
+    for (auto& t : B.gram) {
+      t.Zs = zs;
+      zs += (size_t)t.nfold * B.probs[t.prob].m0 * B.probs[t.prob].m0;
+      if (t.split) B.splits[q++].B = t.Zs;
+    }
     B.d_gseg = U.put(B.gseg);
   }
+  // ---- descriptor arrays (uploaded in one copy with the parameters) ----
+  B.d_probs = U.put(B.probs);
+  B.d_gsegs = U.put(B.gsegs);
+  B.d_psegs = U.put(B.psegs);
+  B.d_gram = U.put(B.gram);
+  B.d_splits = U.put(B.splits);
+  B.d_combT = U.put(B.combT);
+  B.d_combE = U.put(B.combE);
+  B.d_dtabs = U.put(B.dtabs);
+  B.d_dfields = U.put(B.dfields);
+  B.d_dblocks = U.put(B.dblocks);
+  B.d_dft = U.put(B.dft);
+  B.d_pft = U.put(B.pft);
+  B.d_pfg = U.put(B.pfg);
+  B.d_fbs = U.put(B.fbs);
+  B.d_nulls = U.put(B.nulls);
+  B.d_prec = U.put(B.prec);
+  B.d_canon = U.put(B.canon);
+  B.d_fbo = U.put(B.fbo);
+  B.d_sorts = U.put(B.sorts);
   B.bytes = S.off;
   B.ubytes = U.off;
 }
@@ -2206,7 +2206,9 @@ void set_ctx_error(fock_ctx* c, const char* msg) { if (c) c->err = msg; }
 // with host outputs.
 namespace fock {
 
-int detail_estimate(const fock_problem& p, size_t budget, size_t* bytes, int* n_evals, std::string& why) {
+size_t detail_chunk_bytes() { return kPfWorkBytes; }
+
+int detail_estimate(const fock_problem& p, size_t budget, ServeSize* z, int* n_evals, std::string& why) {
   Batch B;
   B.nprob = 1;
   B.hp.assign(1, HostProb());
@@ -2214,11 +2216,14 @@ int detail_estimate(const fock_problem& p, size_t budget, size_t* bytes, int* n_
   int rc = validate(p, B.hp[0], why);
   if (rc) return rc;
   for (int a = 0; a < 3; ++a) axis_plan(B.hp[0], a, B.ap[a]);
-  do {   // as the plan of a batch that does not fit does
+  for (;; ++B.tight) {   // in the form that the plan of its batch will have
     Slab S0, U0;
     plan(B, S0, U0);
-    *bytes = S0.off + U0.off + 512;
-  } while (*bytes > budget && tighten(B, *bytes - budget));
+    z->bytes = S0.off + U0.off + 512 - B.pf_extra;
+    if (z->bytes <= budget || B.sidx.empty() || B.tight == 3) break;
+  }
+  z->region = B.pf_region;
+  z->chunks = B.pf_bytes;
   *n_evals = B.pp[0].nev;
   return FOCK_OK;
 }
@@ -2257,8 +2262,9 @@ cudaStream_t detail_ctx_stream(const fock_ctx* c) { return c->stream; }
 // caller may hand it back to its owner at once).  A mixed problem is released
 // early only while the batch's tensor-core completion flag is clear; else its
 // status (FOCK_ETIMEOUT) is decided with the batch's.
-int detail_solve(fock_ctx* w, int n, const fock_problem* probs, fock_output* outs, double tol, int maxit,
+int detail_solve(fock_ctx* w, int n, const fock_problem* probs, fock_output* outs, double tol, int maxit, size_t chunks,
                  const std::function<void(int, const fock_output&)>* release) {
+  w->pf_cap = chunks;   // bytes of chunk workspace that the server has room for
   fock_plan P;
   P.ctx = w;
   if (release && *release) {

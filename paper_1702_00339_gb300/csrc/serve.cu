@@ -39,11 +39,12 @@
 #include "admission.h"
 
 namespace fock {
-int detail_estimate(const fock_problem& p, size_t budget, size_t* bytes, int* n_evals, std::string& why);
+int detail_estimate(const fock_problem& p, size_t budget, ServeSize* z, int* n_evals, std::string& why);
+size_t detail_chunk_bytes();
 fock_ctx* detail_worker_ctx(int device, cudaMemPool_t pool, size_t budget);
 const char* detail_ctx_error(const fock_ctx* c);
 cudaStream_t detail_ctx_stream(const fock_ctx* c);
-int detail_solve(fock_ctx* w, int n, const fock_problem* probs, fock_output* outs, double tol, int maxit,
+int detail_solve(fock_ctx* w, int n, const fock_problem* probs, fock_output* outs, double tol, int maxit, size_t chunks,
                  const std::function<void(int, const fock_output&)>* release);
 }  // namespace fock
 
@@ -85,7 +86,7 @@ struct OwnedProblem {
 struct Req {
   uint64_t ticket = 0;
   OwnedProblem op;
-  size_t bytes = 0;
+  fock::ServeSize size;
   int n_evals = 0;
   int64_t t_submit = 0, t_admit = -1, t_done = -1;
   int status = FOCK_EAGAIN;
@@ -135,7 +136,7 @@ void fock_server::worker(int slot) {
   fock_ctx* w = wctx[slot];
   for (;;) {
     std::vector<Req*> batch;
-    size_t bytes = 0;
+    size_t bytes = 0, chunks = 0;
     int bid = 0;
     {
       std::unique_lock<std::mutex> lk(m);
@@ -146,8 +147,15 @@ void fock_server::worker(int slot) {
           const size_t free_bytes = cfg.hbm_budget_bytes > reserved ? cfg.hbm_budget_bytes - reserved : 0;
           batch = fock::admit_batch(
               pending, [](const Req* r) { return structured(r->op.p); },
-              [](const Req* r) { return r->bytes; }, free_bytes, cfg.max_batch, &bytes);
-          if (!batch.empty()) break;
+              [](const Req* r) { return r->size.bytes; }, free_bytes, cfg.max_batch, &bytes);
+          if (!batch.empty()) {
+            // chunk workspace in what the requests themselves leave of the budget
+            size_t region = 0, want = 0, extra = 0;
+            for (const Req* r : batch) { region += r->size.region; want += r->size.chunks; }
+            chunks = fock::chunk_share(region, want, fock::detail_chunk_bytes(), free_bytes - bytes, &extra);
+            bytes += extra;
+            break;
+          }
         } else if (stopping) {
           return;
         }
@@ -199,7 +207,7 @@ void fock_server::worker(int slot) {
       ++completed;
       cv_done.notify_all();
     };
-    int rc = fock::detail_solve(w, n, probs.data(), outs.data(), cfg.tol, cfg.maxit, &publish);
+    int rc = fock::detail_solve(w, n, probs.data(), outs.data(), cfg.tol, cfg.maxit, chunks, &publish);
     {
       std::lock_guard<std::mutex> lk(m);
       const int64_t td = now_ns();
@@ -270,12 +278,12 @@ int fock_serve_submit(fock_server* S, const fock_problem* p, uint64_t* ticket) {
   std::unique_ptr<Req> r(new Req());
   r->op.copy_from(*p);
   std::string why;
-  int rc = fock::detail_estimate(r->op.p, S->cfg.hbm_budget_bytes, &r->bytes, &r->n_evals, why);
+  int rc = fock::detail_estimate(r->op.p, S->cfg.hbm_budget_bytes, &r->size, &r->n_evals, why);
   std::lock_guard<std::mutex> lk(S->m);
   if (rc) { S->err = why; return rc; }
   if (S->stopping) { S->err = "server is stopping"; return FOCK_EINVAL; }
-  if (r->bytes > S->cfg.hbm_budget_bytes) {
-    S->err = "request needs " + std::to_string(r->bytes) + " bytes, budget " +
+  if (r->size.bytes > S->cfg.hbm_budget_bytes) {
+    S->err = "request needs " + std::to_string(r->size.bytes) + " bytes, budget " +
              std::to_string(S->cfg.hbm_budget_bytes);
     return FOCK_ENOMEM;
   }
