@@ -373,10 +373,8 @@ uint64_t problem_seed(const HostProb& H) {
   return h;
 }
 
-// Representatives of the Fourier indices j0 .. j0 + nj - 1 of an L1 x L2 x L3 lattice,
-// as local indices: with real generators the block at -j (componentwise mod L) is the
-// conjugate of the block at j, with the same spectrum; where the range holds both,
-// the lower index stands for the pair.
+// Representatives of the Fourier indices j0 .. j0 + nj - 1 of a lattice (pf_index.h), as local
+// indices, where the range holds both of a pair the lower.
 std::vector<int> pf_reps(const int* L, int j0, int nj) {
   std::vector<int> rep;
   rep.reserve(nj / 2 + 8);
@@ -922,9 +920,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
       std::memset(&pt, 0, sizeof(pt));
       pt.prob = i; pt.nj = ncell;
       for (int a = 0; a < 3; ++a) { pt.L[a] = H.L[a]; pt.Xh[a] = Q.Xh[a]; }
-      const std::vector<int> reps = pf_reps(H.L, 0, ncell);
-      pt.nrep = (int)reps.size();
-      pt.rep = U.put(reps);
+      pt.nrep = pf_count(H.L);
       pt.ev = Q.ev; pt.blk = Q.blk; pt.tau = f.tau; pt.neig = f.neig;
       B.pft.push_back(pt);
       B.maxnj_p = std::max(B.maxnj_p, ncell);
@@ -2695,10 +2691,12 @@ int periodic_range(fock_ctx* ctx, Batch& B, int j0, int j1, double* evals, int* 
   const size_t off_pi = off_pv + (size_t)n2 * 8;
   const size_t off_t = (off_pi + (size_t)n2 * 4 + 255) & ~(size_t)255;
   // eigenvalues by the chunked pipeline, on the representatives of the range
-  const std::vector<int> reps = pf_reps(H.L, j0, nj);
+  const bool whole = j0 == 0 && nj == H.L[0] * H.L[1] * H.L[2];
+  const std::vector<int> reps = whole ? std::vector<int>() : pf_reps(H.L, j0, nj);
+  const int nrep = whole ? pf_count(H.L) : (int)reps.size();
   const size_t off_r = (off_t + sizeof(FBlockTask) + sizeof(PfTask) + 255) & ~(size_t)255;
   std::vector<PfGroup> groups;
-  pf_groups(0, (int)reps.size(), groups);
+  pf_groups(0, nrep, groups);
   const size_t off_g = (off_r + reps.size() * sizeof(int) + 255) & ~(size_t)255;
   const size_t off_v = (off_g + groups.size() * sizeof(PfGroup) + 255) & ~(size_t)255;
   const size_t vbytes = vecs ? (size_t)n * H.m0 * sizeof(cplx) : 0;
@@ -2713,12 +2711,12 @@ int periodic_range(fock_ctx* ctx, Batch& B, int j0, int j1, double* evals, int* 
   f.j0 = j0; f.nj = nj; f.outH = nullptr; f.outS = nullptr; f.want = 1; f.ev = nullptr; f.blk = nullptr; f.fail = nullptr;
   f.vecs = vecs ? (cplx*)(mem + off_v) : nullptr;
   PfTask pt = B.pft[0];
-  pt.j0 = j0; pt.nj = nj; pt.nrep = (int)reps.size(); pt.rep = (const int*)(mem + off_r);
+  pt.j0 = j0; pt.nj = nj; pt.nrep = nrep; pt.rep = whole ? nullptr : (const int*)(mem + off_r);
   pt.ev = ev; pt.blk = blk; pt.neig = nullptr;
   char* const dpt = mem + off_t + sizeof(FBlockTask);
   cudaError_t e = cudaMemcpyAsync(mem + off_t, &f, sizeof(f), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dpt, &pt, sizeof(pt), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && !whole)
     e = cudaMemcpyAsync(mem + off_r, reps.data(), reps.size() * sizeof(int), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(mem + off_g, groups.data(), groups.size() * sizeof(PfGroup), cudaMemcpyHostToDevice, st);

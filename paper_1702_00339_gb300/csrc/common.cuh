@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "band_plan.h"
+#include "pf_index.h"
 
 // Raises a kernel's dynamic shared memory limit, once per process, to the
 // device's opt-in maximum minus the kernel's static shared memory.  The
@@ -221,11 +222,13 @@ struct PfTask {
   int prob, j0, nj, nrep;        // Fourier indices j0 .. j0 + nj - 1, representatives
   int L[3];
   const cplx* Xh[3];             // per-axis DFT'd factors [L_l][nF][m0*m0]
-  const int* rep;                // [nrep] local index of each representative, ascending
+  const int* rep;                // [nrep] local index of each representative, ascending; null: the whole
+                                 // lattice's (pf_index)
   double* ev;                    // [nj*m0]
   int* blk;                      // optional [nj*m0] Fourier index of each eigenvalue
   const double* tau;             // the problem's dependency cut
   int* neig;                     // counts the blocks solved by the overlap's eigendecomposition
+  __device__ int index(int r) const { return rep ? rep[r] : pf_index(L, r); }
 };
 // kPfGroup consecutive representatives of a task (the last group of a task may be short)
 constexpr int kPfGroup = 8;

@@ -903,9 +903,9 @@ __global__ void __launch_bounds__(32) k_pf_form(const ProbDev* __restrict__ prob
   const int Lin = F.L[in];
   for (int g0 = 0; g0 < cnt;) {
     // a run of blocks with the same indices on the other two axes
-    const int j = F.j0 + F.rep[r0 + g0], jo = j / Lin;   // (axes after the inner one have one cell)
+    const int j = F.j0 + F.index(r0 + g0), jo = j / Lin;   // (axes after the inner one have one cell)
     int n = 1;
-    while (g0 + n < cnt && (F.j0 + F.rep[r0 + g0 + n]) / Lin == jo) ++n;
+    while (g0 + n < cnt && (F.j0 + F.index(r0 + g0 + n)) / Lin == jo) ++n;
     const int i0 = (in == 2) ? jo / F.L[1] : (in == 1) ? jo : 0, i1 = (in == 2) ? jo % F.L[1] : 0;
     const cplx* f0 = F.Xh[o0] + (size_t)i0 * nfe + pr;
     const cplx* f1 = F.Xh[o1] + (size_t)i1 * nfe + pr;
@@ -913,7 +913,7 @@ __global__ void __launch_bounds__(32) k_pf_form(const ProbDev* __restrict__ prob
     cplx v[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      const int jg = F.j0 + F.rep[r0 + g0 + min(g, n - 1)];
+      const int jg = F.j0 + F.index(r0 + g0 + min(g, n - 1));
       f2[g] = F.Xh[in] + (size_t)(jg % Lin) * nfe + pr;
       v[g] = cmk(0.0, 0.0);
     }
@@ -1414,7 +1414,7 @@ __global__ void __launch_bounds__(32) k_pf_values(const ProbDev* __restrict__ pr
     for (int i = 0; i < r; ++i) D[32 * i] = tridiag_eig_fast(df, e2f, d, e2, r, i, 0.0);
   }
   // the conjugate block's spectrum too, where the task's range holds it
-  const int jl = F.rep[rep], j = F.j0 + jl;
+  const int jl = F.index(rep), j = F.j0 + jl;
   const int j3 = j % F.L[2], j2 = (j / F.L[2]) % F.L[1], j1 = j / (F.L[1] * F.L[2]);
   const int c1 = (F.L[0] - j1) % F.L[0], c2 = (F.L[1] - j2) % F.L[1], c3 = (F.L[2] - j3) % F.L[2];
   const int jm = (c1 * F.L[1] + c2) * F.L[2] + c3;
