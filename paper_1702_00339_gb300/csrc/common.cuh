@@ -463,23 +463,25 @@ struct SplitTask {
   int sym;                     // (with work) C is symmetric: the upper triangle is reduced, mirrored
   int* ex;                     // exponents of A's rows, then of B's columns (SplitExps)
   __host__ __device__ bool same() const { return A == B && a_m == b_n && a_k == b_k && M == N; }
-  __host__ __device__ size_t n_ex() const {
-    const SplitRanges R(K, ksplit);
-    return (size_t)R.count() * ((size_t)M + N) * (2 + R.blocks());
-  }
+  __host__ __device__ size_t n_ex() const;   // words of ex
 };
-// Exponents of one operand of a split product, `rows` rows (or columns): for each range
-// the largest exponent field of a row, a byte for each i = 0 .. 3 with the range's blocks of
-// 64 summands whose largest is within i of it, and the blocks' own.
+// Exponents of the rows of A and of the columns of B (b) of a split product, for each range:
+// [range][row] the largest exponent field; [range][row] of its blocks of 64 summands, four
+// bits each, whether the block's largest is within 0, 1, 2, 3 of it; [range][block][row] the
+// blocks' own.
 struct SplitExps {
-  int *wide, *near, *block;    // [ranges][rows], [ranges][rows], [ranges][blocks()][rows]
-  __host__ __device__ SplitExps(const SplitTask& T, const SplitRanges& R, bool b) {
-    const size_t nA = (size_t)R.count() * T.M, n = b ? (size_t)R.count() * T.N : nA;
-    wide = T.ex + (b ? nA * (2 + R.blocks()) : 0);
-    near = wide + n;
-    block = near + n;
-  }
+  const SplitTask& T;
+  size_t ranges;
+  __host__ __device__ SplitExps(const SplitTask& t, const SplitRanges& R) : T(t), ranges(R.count()) {}
+  __host__ __device__ size_t rows() const { return (size_t)T.M + T.N; }
+  __host__ __device__ int* wide(bool b) const { return T.ex + (b ? ranges * T.M : 0); }
+  __host__ __device__ int* near(bool b) const { return wide(b) + ranges * rows(); }
+  __host__ __device__ int* block(bool b, int blocks) const { return T.ex + ranges * (2 * rows() + (b ? (size_t)blocks * T.M : 0)); }
 };
+__host__ __device__ inline size_t SplitTask::n_ex() const {
+  const SplitRanges R(K, ksplit);
+  return (size_t)R.count() * ((size_t)M + N) * (2 + R.blocks());
+}
 
 // Device pointers and sizes the matvec of an assembled box chain needs.
 struct MatvecView {

@@ -26,8 +26,9 @@
 // whole only if every row and column of it has a block of 64 summands in which the
 // two, together, are within 2^3 of their largest over the range: 512 summands' errors of
 // 2^(a + b - 50.5) are then below what that one block's 64 of 2^(a' + b' - 44) may be. Else the
-// range is taken in its blocks of 64, each aligned for itself.  Looking costs nothing that can
-// be measured (the product below 145.6 us a call with and without).
+// range is taken in its blocks of 64, each aligned for itself.  The look is taken before the
+// loop over the ranges: inside it, where all registers are in use, it made long sums 5 % slower.
+// 216 x 216 x 16384, not symmetric: 146 us a call, 257 where every range is graded.
 //
 // One CTA of 384 threads per 128 x 64 output tile and K range.  Stages of KC = 32
 // summands in two buffers: the threads load and split the next stage while the
@@ -56,6 +57,7 @@ constexpr int kSplitThreads = 384;   // three warps a sub-partition split the op
 constexpr int TMEM_COLS = 512;                                     // NDIG * TN
 constexpr uint32_t A_PLANE = TM * KC * 2, B_PLANE = TN * KC * 2;   // bytes per digit plane
 constexpr uint32_t STAGE = NDIG * (A_PLANE + B_PLANE);
+constexpr int kFineRanges = 2048;    // ranges of a CTA looked at; any more (past 2^20 summands) are taken in blocks
 constexpr size_t SPLIT_SMEM = 2 * (size_t)STAGE + 1024;
 constexpr long long kWaitCycles = 4000000000ll;                    // ~2 s at 2 GHz
 
@@ -76,11 +78,8 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
 // instruction descriptor: D FP32, A and B FP16, both K-major, M = TM, N = n
 constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(TM >> 4) << 24);
 
-// biased exponent field of |x| (0 for zero and subnormals: they align as exponent 1)
-__device__ __forceinline__ int exp_field(double x) {
-  const int e = (int)((__double_as_longlong(x) >> 52) & 0x7FF);
-  return e == 0 ? 1 : e;
-}
+// biased exponent field of |x| from its high word (0 for zero and subnormals: they align as exponent 1)
+__device__ __forceinline__ int exp_field(int hi) { return max((hi >> 20) & 0x7FF, 1); }
 
 // x = w 2^(E - 1077), cut to an integer |w| <= 2^55, plus 64 in every base-128 digit: the low
 // and the high word
@@ -181,65 +180,78 @@ __device__ __forceinline__ double scaled_int(long long S, int e) {
 
 }  // namespace
 
-// Exponents of the rows of A (and columns of B) over each range and its blocks (SplitExps).
+// Exponents of the rows of A (and columns of B) over each range, and where ranges have more
+// than one block over those (SplitExps): a warp per row, or where summands are apart a lane.
 __global__ void __launch_bounds__(256) k_split_exps(const SplitTask* __restrict__ tasks) {
   const SplitTask T = tasks[blockIdx.y];
   if (T.active && *T.active == 0) return;
   const SplitRanges R(T.K, T.ksplit);
+  const SplitExps X(T, R);
   constexpr int NB = SplitRanges::BLOCKS, KB = SplitRanges::BLOCK;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, nb = R.blocks();
   const long long w0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), nw = (long long)gridDim.x * (blockDim.x >> 5);
   for (int o = 0; o < (T.same() ? 1 : 2); ++o) {
     const double* P = o ? T.B : T.A;
     const long long sr = o ? T.b_n : T.a_m, sk = o ? T.b_k : T.a_k;
     const int rows = o ? T.N : T.M;
-    const SplitExps X(T, R, o != 0);
-    const int nb = R.blocks();
+    int *const wide = X.wide(o), *const near = X.near(o), *const block = X.block(o, nb);
     if (sk == 1) {
       for (long long w = w0; w < (long long)R.count() * rows; w += nw) {
         const int e = (int)(w / rows), r = (int)(w % rows), k0 = R.begin(e) + lane, k1 = R.end(e);
-        int Eb = 1;                            // lane c: block c's
+        const int* p = reinterpret_cast<const int*>(P + r * sr) + 1;   // (high words; all loads before the first use)
+        int h[NB][2], Eb = 1;
 #pragma unroll
-        for (int c = 0; c < NB; ++c) {
-          int E = 1;
+        for (int c = 0; c < NB; ++c)
+          if (c < nb) {                        // uniform
+            h[c][0] = k0 + c * KB < k1 ? p[2 * (k0 + c * KB)] : 0;
+            h[c][1] = k0 + c * KB + 32 < k1 ? p[2 * (k0 + c * KB + 32)] : 0;
+          }
 #pragma unroll
-          for (int k = k0 + c * KB, i = 0; i < KB / 32; k += 32, ++i)
-            if (k < k1) E = max(E, exp_field(P[r * sr + k]));
-          E = __reduce_max_sync(0xffffffffu, E);
-          if (lane == c) Eb = E;
+        for (int c = 0; c < NB; ++c)
+          if (c < nb) {
+            const int E = __reduce_max_sync(0xffffffffu, max(exp_field(h[c][0]), exp_field(h[c][1])));
+            if (lane >> 2 == c) Eb = E;        // four lanes a block
+          }
+        const int E = nb > 1 ? __reduce_max_sync(0xffffffffu, Eb) : __shfl_sync(0xffffffffu, Eb, 0);
+        uint32_t q = 0;
+        if (nb > 1) {
+          for (int i = 0; i < 4; ++i) q |= __ballot_sync(0xffffffffu, E - Eb <= i) & (0x11111111u << i);
+          if ((lane & 3) == 0 && lane >> 2 < nb) block[((long long)e * nb + (lane >> 2)) * rows + r] = Eb;
         }
-        const int E = __reduce_max_sync(0xffffffffu, Eb);
-        uint32_t near = 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) near |= (__ballot_sync(0xffffffffu, lane < NB && E - Eb <= i) & 0xffu) << (8 * i);
-        if (lane < nb) X.block[((long long)e * nb + lane) * rows + r] = Eb;
-        if (lane == 0) { X.wide[w] = E; X.near[w] = (int)near; }
+        if (lane == 0) {
+          wide[w] = E;
+          if (nb > 1) near[w] = (int)q;
+        }
       }
     } else {
       const int rg = (rows + 31) >> 5;
       for (long long w = w0; w < (long long)R.count() * rg; w += nw) {
-        const int e = (int)(w / rg), r = (int)(w % rg) * 32 + lane, k0 = R.begin(e), k1 = R.end(e);
+        const int e = (int)(w / rg), r = (int)(w % rg) * 32 + lane;
         if (r >= rows) continue;
         int Eb[NB], E = 1;
-#pragma unroll
-        for (int c = 0; c < NB; ++c) {
-          const int kc = min(k0 + (c + 1) * KB, k1);
-          Eb[c] = 1;
+#pragma unroll 1
+        for (int c = 0; c < nb; ++c) {
+          const int k0 = R.begin(e) + c * KB, k1 = min(k0 + KB, R.end(e));
+          int x = 1;
 #pragma unroll 8
-          for (int k = k0 + c * KB; k < kc; ++k) Eb[c] = max(Eb[c], exp_field(P[r * sr + k * sk]));
-          if (c < nb) X.block[((long long)e * nb + c) * rows + r] = Eb[c];
-          E = max(E, Eb[c]);
+          for (int k = k0; k < k1; ++k) x = max(x, exp_field(__double2hiint(P[r * sr + k * sk])));
+          block[((long long)e * nb + c) * rows + r] = Eb[c] = x;
+          E = max(E, x);
         }
-        uint32_t near = 0;
-#pragma unroll
-        for (int c = 0; c < NB; ++c)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) near |= (E - Eb[c] <= i ? 1u : 0u) << (8 * i + c);
-        X.wide[(long long)e * rows + r] = E;
-        X.near[(long long)e * rows + r] = (int)near;
+        uint32_t q = 0;
+#pragma unroll 1
+        for (int c = 0; c < nb; ++c) q |= (0xfu << min(E - Eb[c], 4) & 0xfu) << (4 * c);   // bits E - Eb[c] .. 3
+        wide[(long long)e * rows + r] = E;
+        near[(long long)e * rows + r] = (int)q;
       }
     }
   }
+}
+
+// the four bits of each block in reverse
+__device__ __forceinline__ uint32_t near_rev(uint32_t x) {
+  x = (x & 0x55555555u) << 1 | (x >> 1 & 0x55555555u);
+  return (x & 0x33333333u) << 2 | (x >> 2 & 0x33333333u);
 }
 
 __global__ void __launch_bounds__(kSplitThreads, 1) k_split_gemm(const SplitTask* __restrict__ tasks, int max_ks, int* err) {
@@ -255,7 +267,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_split_gemm(const SplitTask
   __shared__ __align__(8) uint64_t mbar[2];
   __shared__ uint32_t tmem_base;
   __shared__ int s_fail, exB[TN];
-  __shared__ uint32_t nearB[TN];
+  __shared__ uint32_t s_fine[kFineRanges / 32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rowsA = min(TM, T.M - m0), colsB = min(TN, T.N - n0);
   if (tid == 0) {
@@ -268,6 +280,36 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_split_gemm(const SplitTask
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                  :: "r"(smem_u32(&tmem_base)), "r"(TMEM_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  // The ranges to be taken in blocks, a warp each, before the loop (whose registers are all in
+  // use).  A row and a column agree in block c for some i if c is among the row's within i
+  // and the column's within 3 - i: one AND with the column's bits in reverse.  Mostly all
+  // rows and columns of the tile agree in one block and i; else each pair is looked at.
+  const SplitExps X(T, R);
+  if (R.blocks() > 1) {
+    if (tid < kFineRanges / 32) s_fine[tid] = 0;
+    __syncthreads();
+    for (int d = warp; d < min(R.per, kFineRanges); d += kSplitThreads / 32) {
+      const int e = ks * R.per + d;
+      const int* nA = X.near(false) + (long long)e * T.M + m0;
+      const int* nB = X.near(!T.same()) + (long long)e * T.N + n0;
+      uint32_t a[TM / 32], b[TN / 32], common = ~0u;
+#pragma unroll
+      for (int j = 0; j < TM / 32; ++j) common &= a[j] = lane + 32 * j < rowsA ? (uint32_t)nA[lane + 32 * j] : ~0u;
+#pragma unroll
+      for (int j = 0; j < TN / 32; ++j) common &= b[j] = lane + 32 * j < colsB ? near_rev((uint32_t)nB[lane + 32 * j]) : ~0u;
+      if (__reduce_and_sync(0xffffffffu, common)) continue;
+      bool apart = false;
+#pragma unroll 1
+      for (int c = 0; c < 32; ++c)
+#pragma unroll
+        for (int i = 0; i < TN / 32; ++i) {
+          const uint32_t x = __shfl_sync(0xffffffffu, b[i], c);
+#pragma unroll
+          for (int j = 0; j < TM / 32; ++j) apart |= (a[j] & x) == 0;
+        }
+      if (__any_sync(0xffffffffu, apart) && lane == 0) atomicOr(&s_fine[d >> 5], 1u << (d & 31));
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
@@ -287,26 +329,18 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_split_gemm(const SplitTask
   for (int c = 0; c < 32; ++c) acc[c] = 0.0;
   int st = 0;   // stages so far
   bool ok = true, first = true;
-  const SplitExps XA(T, R, false), XB(T, R, !T.same());
   for (int d = 0; d < R.per && ok; ++d) {
     const int e = ks * R.per + d, r0 = R.begin(e), r1 = R.end(e);
     if (r0 >= r1) break;
-    // a row and a column agree in block c for some i if c is among the row's within i and
-    // the column's within 3 - i: one AND with the column's bytes in reverse
-    int apart = 0;
-    if (r1 - r0 > SplitRanges::BLOCK) {
-      if (tid < TN) nearB[tid] = tid < colsB ? __byte_perm((uint32_t)XB.near[(long long)e * T.N + n0 + tid], 0, 0x0123) : ~0u;
-      const int ra = tid % TM;
-      const uint32_t nearA = ra < rowsA ? (uint32_t)XA.near[(long long)e * T.M + m0 + ra] : ~0u;
-      __syncthreads();
-      for (int c = tid / TM; c < TN; c += kSplitThreads / TM) apart |= (nearA & nearB[c]) == 0;
-    }
-    const bool fine = __syncthreads_or(apart);
+    const bool fine = R.blocks() > 1 && (d >= kFineRanges || (s_fine[d >> 5] >> (d & 31) & 1));
     for (int k0 = r0, k1; k0 < r1 && ok; k0 = k1) {
       k1 = fine ? min(k0 + SplitRanges::BLOCK, r1) : r1;
-      const long long xr = fine ? (long long)e * R.blocks() + (k0 - r0) / SplitRanges::BLOCK : e;
-      const int* eA = (fine ? XA.block : XA.wide) + xr * T.M;
-      const int* eB = (fine ? XB.block : XB.wide) + xr * T.N;
+      const int *eA = X.wide(false) + (long long)e * T.M, *eB = X.wide(!T.same()) + (long long)e * T.N;
+      if (fine) {
+        const long long x = (long long)e * R.blocks() + (k0 - r0) / SplitRanges::BLOCK;
+        eA = X.block(false, R.blocks()) + x * T.M;
+        eB = X.block(!T.same(), R.blocks()) + x * T.N;
+      }
       sh[0].E = sh[0].p ? eA[m0 + sh[0].row] : 1;
       sh[1].E = sh[1].p ? (b1 ? eB[n0 + sh[1].row] : eA[m0 + sh[1].row]) : 1;
       const int EA = row < rowsA ? eA[m0 + row] : 1;

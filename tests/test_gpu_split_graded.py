@@ -63,3 +63,13 @@ def test_gram_of_localised_columns(ctx):
     C = _run(ctx, Y, Y.T.copy(), True, True, ksplit=4, sym=True)
     assert np.array_equal(C, C.T)
     _check(C, Y, Y.T)
+
+
+def test_more_ranges_than_are_looked_at(ctx):
+    """One CTA with more than 2048 ranges takes those past them in blocks, graded or not."""
+    rng = np.random.default_rng(11)
+    K = 2048 * 512 + 700
+    A, B = rng.standard_normal((3, K)), rng.standard_normal((K, 2))
+    B[-600:] *= 2.0 ** (-60.0 * np.arange(600) / 600)[:, None]
+    A[:, -600:] *= 2.0 ** (60.0 * np.arange(600) / 600)
+    _check(_run(ctx, A, B, True, True), A, B)
