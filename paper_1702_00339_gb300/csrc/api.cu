@@ -522,7 +522,7 @@ struct Batch {
   size_t pf_region = 0, pf_extra = 0;
   std::vector<FBlockTask> fbp, fbs; FBlockTask* d_fbs = nullptr;   // fbp: templates of the vector solves
   std::vector<NullTask> nulls; NullTask* d_nulls = nullptr;   // dependency cut of each periodic problem
-  int maxnj_p = 0, maxnj_s = 0, maxm0 = 1;
+  int maxnj_s = 0, maxm0 = 1;
   std::vector<PrecTask> prec; PrecTask* d_prec = nullptr; int maxM = 0;
   std::vector<CanonTask> canon; CanonTask* d_canon = nullptr; int maxcblk = 0;
   std::vector<FBlockTask> fbo; FBlockTask* d_fbo = nullptr;
@@ -628,7 +628,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
   B.dtabs.clear(); B.dfields.clear(); B.dblocks.clear();
   B.dft.clear(); B.fbp.clear(); B.pft.clear(); B.pfg.clear(); B.fbs.clear(); B.nulls.clear(); B.prec.clear(); B.canon.clear(); B.fbo.clear(); B.maxcblk = 0; B.sorts.clear(); B.bigsort.clear();
   B.circs.clear(); B.lob.clear(); B.sidx.clear(); B.mv_off.clear();
-  B.maxnj_p = B.maxnj_s = 0; B.maxm0 = 1; B.maxM = 0; B.maxsort = 0; B.sort_n2 = 0; B.kmax = 0; B.maxLdft = 1;
+  B.maxnj_s = 0; B.maxm0 = 1; B.maxM = 0; B.maxsort = 0; B.sort_n2 = 0; B.kmax = 0; B.maxLdft = 1;
   B.odd_m0 = false;
   B.any_mixed = false;
   B.eapply_rows = 0;
@@ -904,7 +904,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
       std::memset(&f, 0, sizeof(f));
       f.prob = i; f.source = 0; f.nj = ncell;
       for (int a = 0; a < 3; ++a) { f.L[a] = H.L[a]; f.Xh[a] = Q.Xh[a]; }
-      f.want = 1; f.ev = Q.ev; f.blk = Q.blk; f.fail = Q.fail; f.neig = Q.fail + 1;
+      f.want = 1; f.fail = Q.fail; f.neig = Q.fail + 1;
       NullTask nt;
       std::memset(&nt, 0, sizeof(nt));
       nt.m0 = H.m0; nt.nF = H.nF; nt.nb = ncell * H.m0;
@@ -923,7 +923,6 @@ void plan(Batch& B, Slab& S, Slab& U) {
       pt.nrep = pf_count(H.L);
       pt.ev = Q.ev; pt.blk = Q.blk; pt.tau = f.tau; pt.neig = f.neig;
       B.pft.push_back(pt);
-      B.maxnj_p = std::max(B.maxnj_p, ncell);
       if (Q.nev <= kSmallSort) {
         B.sorts.push_back({Q.nev, Q.ev, Q.blk});
         B.maxsort = std::max(B.maxsort, Q.nev);
@@ -2708,7 +2707,7 @@ int periodic_range(fock_ctx* ctx, Batch& B, int j0, int j1, double* evals, int* 
   double* ev = (double*)mem;
   int* blk = (int*)(mem + off_blk);
   FBlockTask f = B.fbp[0];
-  f.j0 = j0; f.nj = nj; f.outH = nullptr; f.outS = nullptr; f.want = 1; f.ev = nullptr; f.blk = nullptr; f.fail = nullptr;
+  f.j0 = j0; f.nj = nj; f.outH = nullptr; f.outS = nullptr; f.want = 1; f.ev = nullptr; f.fail = nullptr;
   f.vecs = vecs ? (cplx*)(mem + off_v) : nullptr;
   PfTask pt = B.pft[0];
   pt.j0 = j0; pt.nj = nj; pt.nrep = nrep; pt.rep = whole ? nullptr : (const int*)(mem + off_r);
@@ -2803,7 +2802,7 @@ int fock_bloch_vectors(fock_ctx* ctx, const fock_blocks* b, int nsel, const int*
   for (int q = 0; q < nd; ++q) {
     FBlockTask f = B.fbp[0];
     f.j0 = blocks_needed[q]; f.nj = 1; f.outH = nullptr; f.outS = nullptr; f.want = 1;
-    f.ev = nullptr; f.blk = nullptr; f.fail = nullptr;
+    f.ev = nullptr; f.fail = nullptr;
     f.vecs = (cplx*)mem + (size_t)q * m0 * m0;
     tasks[q] = f;
   }

@@ -206,7 +206,6 @@ struct FBlockTask {
   cplx* outS;                    // optional [nj][m0*m0]: store Sbar_j
   int want;                      // 0: no eigenvalues, 1: all, 2: only the lowest
   double* ev;                    // [nj*m0] (want 1; null: vectors only) or [nj] (want 2)
-  int* blk;                      // optional [nj*m0] Fourier index of each eigenvalue
   int* fail;                     // set to 1 if a block's Sbar is not positive definite
   const double* tau;             // FACTORS: the problem's dependency cut (k_null_tau); TOEPLITZ:
                                  // null, the cut is formed from TS in the block kernel
@@ -520,6 +519,12 @@ __device__ inline double rsqrt_nr(double x) {
   const double r = (double)__frsqrt_rn((float)x);
   const double e = fma(-x * r, r, 1.0);          // x^-1/2 = r (1 - e)^-1/2 = r (1 + e/2 + 3 e^2/8 + ...)
   return fma(r * e, fma(0.375, e, 0.5), r);
+}
+__device__ inline uint64_t splitmix64(uint64_t x) {
+  x += 0x9E3779B97F4A7C15ull;
+  x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
+  x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
+  return x ^ (x >> 31);
 }
 // |x| as a bit pattern: orders like |x| (integer compare, no FP64 pipe)
 __device__ inline long long abs_bits(double x) { return __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll; }

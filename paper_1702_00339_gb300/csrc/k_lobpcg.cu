@@ -1,8 +1,9 @@
 // Stage (c): preconditioned block iteration for the lowest k eigenpairs of
 // the box pencil (H, S) -- the paper's "structured iteration on subspace"
 // (Sec. 2.3), read as LOBPCG (Knyazev 2001) with basis Y = [X | P | W],
-// W = K (H X - S X Lambda) and K the shifted inverse of the circulant
-// embedding (a Fourier-block solve).  All dense work is FP64.
+// W = K (H X - S X Lambda) and K the inverse of the banded factor (k_band.cu) or, for the
+// largest chains, the shifted inverse of the circulant embedding (a Fourier-block
+// solve).  All dense work is FP64.
 //
 //  k_init_x     deterministic pseudo-random start X (splitmix64 counter hash), P = W = 0
 //  k_gemm_tn    G = A^T B            (Gram blocks of the Rayleigh-Ritz step; 16- or 20-wide tiles)
@@ -15,22 +16,12 @@
 //               canonical cell basis and the exactly symmetric transformed operator
 #include <float.h>
 #include "common.cuh"
+#include "jacobi.cuh"
 
 namespace fock {
 
 // eigenvalue given to the cell directions dropped by the canonical transform
 constexpr double kDecoupledEig = 1e6;
-
-
-
-__device__ inline uint64_t splitmix64(uint64_t x) {
-  x += 0x9E3779B97F4A7C15ull;
-  x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
-  x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
-  return x ^ (x >> 31);
-}
-
-
 
 __global__ void k_init_x(const InitTask* __restrict__ tasks) {
   const InitTask T = tasks[blockIdx.y];
@@ -45,8 +36,6 @@ __global__ void k_init_x(const InitTask* __restrict__ tasks) {
     T.X[(size_t)i + (size_t)T.ld * c] = v;
   }
 }
-
-
 
 // C = alpha A^T B + beta C on TILE x TILE output tiles, one thread per
 // output; TILE = 20 when the block sizes are multiples of 20 (less padding
@@ -239,96 +228,6 @@ __global__ void k_resid(const ResidTask* __restrict__ tasks, double lock_tol) {
     for (int i = threadIdx.x; i < T.n; i += blockDim.x) T.R[(size_t)i + (size_t)T.ld * c] = 0.0;
 }
 
-
-
-// Parallel cyclic Jacobi on the symmetric n x n matrix a (row-major, stride
-// ld >= n + 1), round-robin pairing, A' = J^T A J; eigenvectors accumulated
-// in v.  Odd n is padded with a decoupled huge diagonal entry.  At exit the
-// eigenvalues are on the diagonal of a (unsorted).
-__device__ void cta_jacobi(double* a, double* v, int n, int ld) {
-  __shared__ double rc[128], rs[128];
-  __shared__ int rp[128], rq[128];
-  __shared__ int nrot;
-  __shared__ double red[32], s_thr;
-  const int ne = n + (n & 1);
-  // rotation threshold: |a_pq| <= 1e-14 ||A||_F leaves the pair alone (rounding level)
-  double part = 0.0;
-  for (int it = threadIdx.x; it < n * n; it += blockDim.x) {
-    double x = a[(it / n) * ld + (it % n)];
-    part += x * x;
-  }
-  for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)((blockDim.x + 31) >> 5); ++w) t += red[w];
-    s_thr = 1e-14 * sqrt(t);
-  }
-  for (int it = threadIdx.x; it < ne * ne; it += blockDim.x) {
-    int i = it / ne, j = it % ne;
-    v[i * ld + j] = (i == j) ? 1.0 : 0.0;
-    if (i == n || j == n) a[i * ld + j] = (i == j) ? 1e300 : 0.0;
-  }
-  __syncthreads();
-  const double thr = s_thr;
-  for (int sweep = 0; sweep < 40; ++sweep) {
-    if (threadIdx.x == 0) nrot = 0;
-    __syncthreads();
-    for (int rnd = 0; rnd < ne - 1; ++rnd) {
-      for (int pi = threadIdx.x; pi < ne / 2; pi += blockDim.x) {
-        int x = (pi == 0) ? 0 : ((pi - 1 + rnd) % (ne - 1)) + 1;
-        int y = ((ne - 2 - pi + rnd) % (ne - 1)) + 1;
-        int p = min(x, y), q = max(x, y);
-        double apq = a[p * ld + q], app = a[p * ld + p], aqq = a[q * ld + q];
-        double c = 1.0, s = 0.0;
-        if (fabs(apq) > thr && apq * apq > 1e-34 * fabs(app * aqq)) {   // |a_pq| > 1e-17 sqrt|a_pp a_qq|
-          // reciprocals and square roots by Newton-Raphson from FP32 seeds
-          const double th = (aqq - app) * (0.5 * rcp_nr(apq));
-          const double y = fma(th, th, 1.0);
-          double t = rcp_nr(fabs(th) + y * rsqrt_nr(y));
-          if (th < 0.0) t = -t;
-          c = rsqrt_nr(fma(t, t, 1.0));
-          s = t * c;
-          atomicAdd(&nrot, 1);
-        }
-        rp[pi] = p; rq[pi] = q; rc[pi] = c; rs[pi] = s;
-      }
-      __syncthreads();
-      const int np2 = ne / 2;
-      for (int it = threadIdx.x; it < np2 * ne; it += blockDim.x) {   // rows p, q
-        int pi = it / ne, jj = it % ne;
-        double s = rs[pi];
-        if (s == 0.0) continue;
-        int p = rp[pi], q = rq[pi];
-        double c = rc[pi];
-        double ap = a[p * ld + jj], aq = a[q * ld + jj];
-        a[p * ld + jj] = c * ap - s * aq;
-        a[q * ld + jj] = s * ap + c * aq;
-      }
-      __syncthreads();
-      for (int it = threadIdx.x; it < np2 * ne; it += blockDim.x) {   // columns p, q and v
-        int pi = it / ne, ii = it % ne;
-        double s = rs[pi];
-        if (s == 0.0) continue;
-        int p = rp[pi], q = rq[pi];
-        double c = rc[pi];
-        double ap = a[ii * ld + p], aq = a[ii * ld + q];
-        a[ii * ld + p] = c * ap - s * aq;
-        a[ii * ld + q] = s * ap + c * aq;
-        double vp = v[ii * ld + p], vq = v[ii * ld + q];
-        v[ii * ld + p] = c * vp - s * vq;
-        v[ii * ld + q] = s * vp + c * vq;
-      }
-      __syncthreads();
-    }
-    int done = (nrot == 0);
-    __syncthreads();
-    if (done) break;
-  }
-}
-
-
 // One CTA per (column, task): scale dst's column to unit 2-norm (zero
 // columns stay zero, non-finite ones become zero).
 __global__ void k_colnorm(const CopyTask* __restrict__ tasks) {
@@ -412,7 +311,7 @@ __global__ void k_cell_canon(const CanonTask* __restrict__ tasks) {
     for (int w = 0; w < (int)((blockDim.x + 31) >> 5); ++w) t += red[w];
     s_tau = null_tau(sqrt(t), (double)T.nb);
   }
-  cta_jacobi(G, Q, m0, ld);
+  const bool turned = cta_jacobi(G, Q, m0, ld);
   if (threadIdx.x == 0) {
     int r = 0;
     for (int i = 0; i < m0; ++i)
@@ -423,7 +322,7 @@ __global__ void k_cell_canon(const CanonTask* __restrict__ tasks) {
   __syncthreads();
   for (int it = threadIdx.x; it < m0 * m0; it += blockDim.x) {
     int mu = it / m0, j = it % m0;
-    T.Xc[it] = (j < s_r) ? Q[mu * ld + keep[j]] / sqrt(sv[j]) : 0.0;
+    T.Xc[it] = (j < s_r) ? (turned ? Q[mu * ld + keep[j]] : mu == keep[j] ? 1.0 : 0.0) / sqrt(sv[j]) : 0.0;
   }
 }
 
@@ -528,9 +427,5 @@ void launch_cell_back(const double* Xc, int m0, int L, int ncol, const double* V
                       cudaStream_t st) {
   k_cell_back<<<64, 256, 0, st>>>(Xc, m0, L, ncol, Vr, V, ld);
 }
-
-}  // namespace fock
-
-namespace fock {
 
 }  // namespace fock

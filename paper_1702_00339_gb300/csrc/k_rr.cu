@@ -35,6 +35,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "jacobi.cuh"
 
 namespace fock {
 
@@ -80,13 +81,6 @@ __device__ inline bool shift_clustered(const double* lam, const float* lo, const
   return gap <= 2.0 * w + 4.0 * FLT_EPSILON * fmax(fabs(lam[q]), fabs(lam[q - 1]));
 }
 
-__device__ inline uint64_t mix64(uint64_t x) {
-  x += 0x9E3779B97F4A7C15ull;
-  x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
-  x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
-  return x ^ (x >> 31);
-}
-
 // One inverse-iteration vector of the symmetric tridiagonal (d, e) of order r
 // for the shift lm: LU with partial pivoting of T - lm I (pivots below eps
 // raised to eps), start vector from a counter hash of (row, c), three sweeps of
@@ -118,7 +112,7 @@ __device__ void inverse_iteration(const double* d, const double* e, int r, doubl
   if (r >= 2) W(r - 2, 3) = 0.0;
   // start vector: counter hash of (row, vector), uniform in [0.5, 1.5)
   for (int i = 0; i < r; ++i) {
-    const uint32_t h = (uint32_t)(mix64(((uint64_t)(c + 1) << 32) | (uint64_t)(i + 1)) >> 40);
+    const uint32_t h = (uint32_t)(splitmix64(((uint64_t)(c + 1) << 32) | (uint64_t)(i + 1)) >> 40);
     W(i, 5) = 0.5 + (double)h * (1.0 / 16777216.0);
   }
   for (int sweep = 0; sweep < 3; ++sweep) {
@@ -157,102 +151,6 @@ __device__ void inverse_iteration(const double* d, const double* e, int r, doubl
     for (int i = 0; i < r; ++i) W(i, 5) *= inv;
   }
   for (int i = 0; i < r; ++i) zs[(size_t)i * kk + c] = W(i, 5);
-}
-
-// Parallel cyclic Jacobi on the symmetric n x n matrix a (row-major, stride
-// ld >= n + 1), round-robin pairing, A' = J^T A J; eigenvectors accumulated in
-// v.  Odd n is padded with a decoupled huge diagonal entry.  At exit the
-// eigenvalues are on the diagonal of a (unsorted).  The matrices met here are
-// nearly diagonal: rounds without a rotation cost one barrier, and a matrix that
-// needs none returns false at once, v untouched (the identity).
-__device__ bool cta_jacobi_near(double* a, double* v, int n, int ld) {
-  __shared__ double rc[kRRMax / 2], rs[kRRMax / 2];
-  __shared__ int rp[kRRMax / 2], rq[kRRMax / 2];
-  __shared__ double red[32], s_thr;
-  const int ne = n + (n & 1);
-  // rotation threshold: |a_pq| <= 1e-14 ||A||_F leaves the pair alone (rounding level)
-  double part = 0.0;
-  for (int it = threadIdx.x; it < n * n; it += blockDim.x) {
-    const double x = a[(it / n) * ld + (it % n)];
-    part = fma(x, x, part);
-  }
-  for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)((blockDim.x + 31) >> 5); ++w) t += red[w];
-    s_thr = 1e-14 * sqrt(t);
-  }
-  __syncthreads();
-  const double thr = s_thr;
-  auto rotates = [&](int p, int q) {   // |a_pq| above the threshold and > 1e-17 sqrt|a_pp a_qq|
-    const double apq = a[p * ld + q];
-    return fabs(apq) > thr && apq * apq > 1e-34 * fabs(a[p * ld + p] * a[q * ld + q]);
-  };
-  int need = 0;
-  for (int it = threadIdx.x; it < n * n; it += blockDim.x)
-    if (it / n < it % n) need |= rotates(it / n, it % n);
-  if (!__syncthreads_or(need)) return false;
-  for (int it = threadIdx.x; it < ne * ne; it += blockDim.x) {
-    int i = it / ne, j = it % ne;
-    v[i * ld + j] = (i == j) ? 1.0 : 0.0;
-    if (i == n || j == n) a[i * ld + j] = (i == j) ? 1e300 : 0.0;
-  }
-  __syncthreads();
-  for (int sweep = 0; sweep < 40; ++sweep) {
-    bool any = false;
-    for (int rnd = 0; rnd < ne - 1; ++rnd) {
-      int rot = 0;
-      for (int pi = threadIdx.x; pi < ne / 2; pi += blockDim.x) {
-        int x = (pi == 0) ? 0 : ((pi - 1 + rnd) % (ne - 1)) + 1;
-        int y = ((ne - 2 - pi + rnd) % (ne - 1)) + 1;
-        int p = min(x, y), q = max(x, y);
-        double c = 1.0, s = 0.0;
-        if (rotates(p, q)) {
-          // reciprocals and square roots by Newton-Raphson from FP32 seeds
-          const double th = (a[q * ld + q] - a[p * ld + p]) * (0.5 * rcp_nr(a[p * ld + q]));
-          const double yy = fma(th, th, 1.0);
-          double t = rcp_nr(fabs(th) + yy * rsqrt_nr(yy));
-          if (th < 0.0) t = -t;
-          c = rsqrt_nr(fma(t, t, 1.0));
-          s = t * c;
-          rot = 1;
-        }
-        rp[pi] = p; rq[pi] = q; rc[pi] = c; rs[pi] = s;
-      }
-      if (!__syncthreads_or(rot)) continue;
-      any = true;
-      const int np2 = ne / 2;
-      for (int it = threadIdx.x; it < np2 * ne; it += blockDim.x) {   // rows p, q
-        int pi = it / ne, jj = it % ne;
-        double s = rs[pi];
-        if (s == 0.0) continue;
-        int p = rp[pi], q = rq[pi];
-        double c = rc[pi];
-        double ap = a[p * ld + jj], aq = a[q * ld + jj];
-        a[p * ld + jj] = c * ap - s * aq;
-        a[q * ld + jj] = s * ap + c * aq;
-      }
-      __syncthreads();
-      for (int it = threadIdx.x; it < np2 * ne; it += blockDim.x) {   // columns p, q and v
-        int pi = it / ne, ii = it % ne;
-        double s = rs[pi];
-        if (s == 0.0) continue;
-        int p = rp[pi], q = rq[pi];
-        double c = rc[pi];
-        double ap = a[ii * ld + p], aq = a[ii * ld + q];
-        a[ii * ld + p] = c * ap - s * aq;
-        a[ii * ld + q] = s * ap + c * aq;
-        double vp = v[ii * ld + p], vq = v[ii * ld + q];
-        v[ii * ld + p] = c * vp - s * vq;
-        v[ii * ld + q] = s * vp + c * vq;
-      }
-      __syncthreads();
-    }
-    if (!any) break;      // uniform
-  }
-  return true;
 }
 
 // Barrier of the cluster (of the CTA alone for C = 1).  The hardware cluster
@@ -308,7 +206,7 @@ __global__ void __launch_bounds__(kRRThreads) k_rr(const RRTask* __restrict__ ta
   __shared__ double bufA[2][kRRMax], bufB[2][kRRMax], bufC[2][kRRMax], bufD[2][kRRMax], xr[kRRMax];
   __shared__ double td[kRRMax], te[kRRMax], ttau[kRRMax], tlam[kRRMax];
   __shared__ int perm[kRRMax], pos[kRRMax], act[kRRMax], apos[kRRMax];
-  __shared__ int s_p[2], s_flag;
+  __shared__ int s_p[2];
   __shared__ double s_rd[2], s_K;
   // ---- 1. scaled Gram matrices, pivoted elimination ----
   for (int i = tid; i < n; i += NT) {
@@ -535,7 +433,7 @@ __global__ void __launch_bounds__(kRRThreads) k_rr(const RRTask* __restrict__ ta
   }
   // ---- 3. the kk lowest eigenvalues of T: FP32 Sturm multisection, a warp per
   // eigenvalue (each round the lanes count below 32 interior points of its
-    // bracket, which becomes 33 times narrower); eigenvalue c on CTA c mod C ----
+  // bracket, which becomes 33 times narrower); eigenvalue c on CTA c mod C ----
   __shared__ float s_lo[kRRMax / 2], s_hi[kRRMax / 2], s_g[2], s_e2;
   float* df = reinterpret_cast<float*>(bufC[0]);   // d and e^2 in FP32
   float* e2f = df + kRRMax;
@@ -719,7 +617,7 @@ __global__ void __launch_bounds__(kRRThreads) k_rr(const RRTask* __restrict__ ta
     }
     group_sync<C>();
     products(tz, R2);
-    const bool turned = cta_jacobi_near(R2, R1, kk, kj);
+    const bool turned = cta_jacobi(R2, R1, kk, kj);
     for (int i = tid; i < kk; i += NT) {           // ascending order, ties by index, NaN last:
       double di = R2[i * kj + i];                  // the ranks are always a permutation
       if (isnan(di)) di = DBL_MAX;
