@@ -868,7 +868,7 @@ void plan(Batch& B, Slab& S, Slab& U) {
     sp.A = tab + off; sp.a_m = ld; sp.a_k = 1;
     sp.b_k = np; sp.b_n = 1;   // (B: t.Zs, below)
     sp.C = t.X + (direct ? 0 : 2 * np); sp.c_m = np; sp.c_n = 1;
-    sp.alpha = 1.0; sp.beta = 0.0; sp.ksplit = 1;
+    sp.alpha = 1.0; sp.beta = 0.0; sp.ksplit = 1; sp.graded = 1;
     B.splits.push_back(sp);
     split_prob.push_back(t.prob);
     B.split_maxm = std::max(B.split_maxm, sp.M);
@@ -2838,6 +2838,7 @@ int fock_split_dgemm(fock_ctx* ctx, int M, int N, int K, const double* A, long l
   t.M = M; t.N = N; t.K = K; t.A = A; t.a_m = a_m; t.a_k = a_k; t.B = B; t.b_k = b_k; t.b_n = b_n;
   t.C = C; t.c_m = c_m; t.c_n = c_n; t.alpha = alpha; t.beta = beta;
   t.sym = sym ? 1 : 0;
+  t.graded = 1;
   const bool red = ksplit > 1 || sym;
   int sms = 1;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);

@@ -460,12 +460,19 @@ struct SplitTask {
   double* work;                // null: C written directly; else [ksplit][M][N] partial sums,
                                // reduced in a fixed order by k_split_reduce
   int sym;                     // (with work) C is symmetric: the upper triangle is reduced, mirrored
+  // 1: pairs of a row and a column whose largest entries lie apart are looked for (k_split.cu).
+  // 0 for the block iteration's products: their errors count against the columns' norms, and
+  // a Gram matrix whose every entry is the exact product of the same cut columns serves it
+  // better than one with some entries more exact (512 cells of 32 functions, four draws: 22, 28,
+  // 24, 24 iterations against 30, 33, 36, 27).
+  int graded;
   int* ex;                     // exponents of A's rows, then of B's columns (SplitExps)
+  __host__ __device__ int blocks() const;   // of a range, to be looked at: 1 for none
   __host__ __device__ bool same() const { return A == B && a_m == b_n && a_k == b_k && M == N; }
   __host__ __device__ size_t n_ex() const;   // words of ex
 };
 // Exponents of the rows of A and of the columns of B (b) of a split product, for each range:
-// [range][row] the largest exponent field; [range][row] of its blocks of 64 summands, four
+// [range][row] the largest exponent field; where there are blocks: [range][row] of its blocks of 64 summands, four
 // bits each, whether the block's largest is within 0, 1, 2, 3 of it; [range][block][row] the
 // blocks' own.
 struct SplitExps {
@@ -477,9 +484,9 @@ struct SplitExps {
   __host__ __device__ int* near(bool b) const { return wide(b) + ranges * rows(); }
   __host__ __device__ int* block(bool b, int blocks) const { return T.ex + ranges * (2 * rows() + (b ? (size_t)blocks * T.M : 0)); }
 };
+__host__ __device__ inline int SplitTask::blocks() const { return graded ? SplitRanges(K, ksplit).blocks() : 1; }
 __host__ __device__ inline size_t SplitTask::n_ex() const {
-  const SplitRanges R(K, ksplit);
-  return (size_t)R.count() * ((size_t)M + N) * (2 + R.blocks());
+  return (size_t)SplitRanges(K, ksplit).count() * ((size_t)M + N) * (blocks() > 1 ? 2 + blocks() : 1);
 }
 
 // Device pointers and sizes the matvec of an assembled box chain needs.

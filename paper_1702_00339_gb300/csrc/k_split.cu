@@ -22,7 +22,8 @@
 // 64 summands, as this was: 2^-44 and 1e-13).
 //
 // Where a row falls while a column rises, the largest over a range say little about the
-// products: with both over 2^40 the sum would keep 20 bits.  So a tile's range is aligned as a
+// products: with both over 2^40 the sum would keep 20 bits.  So, where the task asks for it
+// (SplitTask::graded), a tile's range is aligned as a
 // whole only if every row and column of it has a block of 64 summands in which the
 // two, together, are within 2^3 of their largest over the range: 512 summands' errors of
 // 2^(a + b - 50.5) are then below what that one block's 64 of 2^(a' + b' - 44) may be. Else the
@@ -189,6 +190,7 @@ __global__ void __launch_bounds__(256) k_split_exps(const SplitTask* __restrict_
   const SplitExps X(T, R);
   constexpr int NB = SplitRanges::BLOCKS, KB = SplitRanges::BLOCK;
   const int lane = threadIdx.x & 31, nb = R.blocks();
+  const bool looked = T.blocks() > 1;
   const long long w0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), nw = (long long)gridDim.x * (blockDim.x >> 5);
   for (int o = 0; o < (T.same() ? 1 : 2); ++o) {
     const double* P = o ? T.B : T.A;
@@ -214,13 +216,13 @@ __global__ void __launch_bounds__(256) k_split_exps(const SplitTask* __restrict_
           }
         const int E = nb > 1 ? __reduce_max_sync(0xffffffffu, Eb) : __shfl_sync(0xffffffffu, Eb, 0);
         uint32_t q = 0;
-        if (nb > 1) {
+        if (looked) {
           for (int i = 0; i < 4; ++i) q |= __ballot_sync(0xffffffffu, E - Eb <= i) & (0x11111111u << i);
           if ((lane & 3) == 0 && lane >> 2 < nb) block[((long long)e * nb + (lane >> 2)) * rows + r] = Eb;
         }
         if (lane == 0) {
           wide[w] = E;
-          if (nb > 1) near[w] = (int)q;
+          if (looked) near[w] = (int)q;
         }
       }
     } else {
@@ -235,13 +237,15 @@ __global__ void __launch_bounds__(256) k_split_exps(const SplitTask* __restrict_
           int x = 1;
 #pragma unroll 8
           for (int k = k0; k < k1; ++k) x = max(x, exp_field(__double2hiint(P[r * sr + k * sk])));
-          block[((long long)e * nb + c) * rows + r] = Eb[c] = x;
+          if (looked) block[((long long)e * nb + c) * rows + r] = x;
+          Eb[c] = x;
           E = max(E, x);
         }
+        wide[(long long)e * rows + r] = E;
+        if (!looked) continue;
         uint32_t q = 0;
 #pragma unroll 1
         for (int c = 0; c < nb; ++c) q |= (0xfu << min(E - Eb[c], 4) & 0xfu) << (4 * c);   // bits E - Eb[c] .. 3
-        wide[(long long)e * rows + r] = E;
         near[(long long)e * rows + r] = (int)q;
       }
     }
@@ -286,7 +290,8 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_split_gemm(const SplitTask
   // and the column's within 3 - i: one AND with the column's bits in reverse.  Mostly all
   // rows and columns of the tile agree in one block and i; else each pair is looked at.
   const SplitExps X(T, R);
-  if (R.blocks() > 1) {
+  const int nb = T.blocks();
+  if (nb > 1) {
     if (tid < kFineRanges / 32) s_fine[tid] = 0;
     __syncthreads();
     for (int d = warp; d < min(R.per, kFineRanges); d += kSplitThreads / 32) {
@@ -332,14 +337,14 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_split_gemm(const SplitTask
   for (int d = 0; d < R.per && ok; ++d) {
     const int e = ks * R.per + d, r0 = R.begin(e), r1 = R.end(e);
     if (r0 >= r1) break;
-    const bool fine = R.blocks() > 1 && (d >= kFineRanges || (s_fine[d >> 5] >> (d & 31) & 1));
+    const bool fine = nb > 1 && (d >= kFineRanges || (s_fine[d >> 5] >> (d & 31) & 1));
     for (int k0 = r0, k1; k0 < r1 && ok; k0 = k1) {
       k1 = fine ? min(k0 + SplitRanges::BLOCK, r1) : r1;
       const int *eA = X.wide(false) + (long long)e * T.M, *eB = X.wide(!T.same()) + (long long)e * T.N;
       if (fine) {
-        const long long x = (long long)e * R.blocks() + (k0 - r0) / SplitRanges::BLOCK;
-        eA = X.block(false, R.blocks()) + x * T.M;
-        eB = X.block(!T.same(), R.blocks()) + x * T.N;
+        const long long x = (long long)e * nb + (k0 - r0) / SplitRanges::BLOCK;
+        eA = X.block(false, nb) + x * T.M;
+        eB = X.block(!T.same(), nb) + x * T.N;
       }
       sh[0].E = sh[0].p ? eA[m0 + sh[0].row] : 1;
       sh[1].E = sh[1].p ? (b1 ? eB[n0 + sh[1].row] : eA[m0 + sh[1].row]) : 1;
