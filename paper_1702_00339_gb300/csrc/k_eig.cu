@@ -892,7 +892,11 @@ __global__ void __launch_bounds__(32) k_pf_form(const ProbDev* __restrict__ prob
   const int m0 = P.m0, np = m0 * m0, nup = m0 * (m0 + 1) / 2, R = P.R, T = P.T;
   const int t0 = blockIdx.y * blockDim.x + threadIdx.x, s0 = blockIdx.x * G, r0 = grp.rep + s0 % kPfGroup;
   const int cnt = min(G, F.nrep - r0);
-  if (t0 >= nup || cnt <= 0) return;
+  if (cnt <= 0) return;
+  __shared__ int sj[G];                      // the blocks' Fourier indices
+  if (threadIdx.x < cnt) sj[threadIdx.x] = F.j0 + F.index(r0 + threadIdx.x);
+  __syncwarp();
+  if (t0 >= nup) return;
   int a, b;
   tri_pos(t0, a, b);
   const int pr = b * m0 + a;                 // the upper entry (b, a); the lower one is its conjugate
@@ -903,9 +907,9 @@ __global__ void __launch_bounds__(32) k_pf_form(const ProbDev* __restrict__ prob
   const int Lin = F.L[in];
   for (int g0 = 0; g0 < cnt;) {
     // a run of blocks with the same indices on the other two axes
-    const int j = F.j0 + F.index(r0 + g0), jo = j / Lin;   // (axes after the inner one have one cell)
+    const int j = sj[g0], jo = j / Lin;   // (axes after the inner one have one cell)
     int n = 1;
-    while (g0 + n < cnt && (F.j0 + F.index(r0 + g0 + n)) / Lin == jo) ++n;
+    while (g0 + n < cnt && sj[g0 + n] / Lin == jo) ++n;
     const int i0 = (in == 2) ? jo / F.L[1] : (in == 1) ? jo : 0, i1 = (in == 2) ? jo % F.L[1] : 0;
     const cplx* f0 = F.Xh[o0] + (size_t)i0 * nfe + pr;
     const cplx* f1 = F.Xh[o1] + (size_t)i1 * nfe + pr;
@@ -913,7 +917,7 @@ __global__ void __launch_bounds__(32) k_pf_form(const ProbDev* __restrict__ prob
     cplx v[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      const int jg = F.j0 + F.index(r0 + g0 + min(g, n - 1));
+      const int jg = sj[g0 + min(g, n - 1)];
       f2[g] = F.Xh[in] + (size_t)(jg % Lin) * nfe + pr;
       v[g] = cmk(0.0, 0.0);
     }

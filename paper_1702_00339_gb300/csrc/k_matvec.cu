@@ -368,10 +368,12 @@ void launch_eapply(const EApplyTask* tasks, int ntask, int maxrows, int maxcols,
 // band, then of its boundary and defect blocks, and the slices are added pairwise.
 // Latency from the first loads to the last sum.  64 cells of 8 functions (D = 13),
 // one vector: 65 -> 18 us a call.
+constexpr unsigned kApplyGroups = 65535;
 __global__ void __launch_bounds__(256) k_band_apply(const BandApply T) {
   __shared__ double part[256][kApplyCols + 1];
   __shared__ int s_ri;
-  const int m0 = T.m0, k = blockIdx.x % T.L, v0 = blockIdx.x / T.L * kApplyCols, tid = threadIdx.x;
+  const int m0 = T.m0, k = blockIdx.x, v0 = (blockIdx.y + kApplyGroups * blockIdx.z) * kApplyCols, tid = threadIdx.x;
+  if (v0 >= T.ncol) return;
   const int S = 256 / m0, mu = tid % m0, s = tid / m0, nv = min(kApplyCols, T.ncol - v0);
   if (tid == 0) s_ri = -1;
   __syncthreads();
@@ -418,8 +420,8 @@ __global__ void __launch_bounds__(256) k_band_apply(const BandApply T) {
   }
 }
 void launch_band_apply(const BandApply& T, cudaStream_t st) {
-  // (rows and columns share grid.x: grid.y would end at 65535 groups of columns)
-  k_band_apply<<<(unsigned)T.L * ((T.ncol + kApplyCols - 1) / kApplyCols), 256, 0, st>>>(T);
+  const unsigned groups = (T.ncol + kApplyCols - 1) / kApplyCols;   // (grid.y ends at 65535: by planes of grid.z)
+  k_band_apply<<<dim3(T.L, std::min(groups, kApplyGroups), (groups + kApplyGroups - 1) / kApplyGroups), 256, 0, st>>>(T);
 }
 
 }  // namespace fock
